@@ -132,7 +132,10 @@ tdgs_status tdgs_context_set_sort_variant(tdgs_context* ctx, int variant);
  * TDGS_ERR_INVALID_ARGUMENT.
  *   TDGS_TUNE_SORT_VARIANT     pass kernel of tdgs_sort_pairs (as above)
  *   TDGS_TUNE_TILE_DIGIT_BITS  widest digit (4..12) of the frame's passes
- *                              over the tile bits (built-in: 8)
+ *                              over the tile bits (built-in: no such passes
+ *                              for one view of at most 4096 x 4096 pixels,
+ *                              whose pairs come from two interval splits;
+ *                              8 otherwise)
  *   TDGS_TUNE_CTAS_PER_SM      CTAs per SM of the persistent radix grids
  *                              (capped by occupancy)
  *   TDGS_TUNE_DEPTH_DIGIT_BITS digit width of the frame's depth sort when

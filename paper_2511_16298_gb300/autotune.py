@@ -5,8 +5,8 @@ workload with CUDA events and keeps the fastest:
 
 * tdgs_sort_pairs: the pass kernel variant (digit width 8..11, threads,
   keys per thread, blocks per SM) and CTAs per SM of the persistent grid;
-* the fused frame / multi-view batch: widest tile digit (6, 8 or 12
-  bits), CTAs per SM and the depth sort's digit width (8 or 11).
+* the fused frame / multi-view batch: the built-in pair path, or tile
+  passes with a widest tile digit of 6 or 12 bits, CTAs per SM and the depth sort's digit width (8 or 11).
 
 Results are stored as JSON keyed by workload shape (pair-count bucket and
 key bits, or Gaussians/tiles buckets), so a server can apply the table
@@ -85,7 +85,7 @@ def tune_views(ctx: tdgs.Context, views: list, reps: int = 3) -> dict:
     # Gaussians or more); below that the built-in choice stands
     dbit_choices = (11, 8) if n >= DEPTH_PER_PASS_MIN else (0,)
     trials = []
-    for bits in (12, 8, 6):
+    for bits in (12, 0, 6):  # 0: the built-in choice (interval splits where they apply, else 8)
         for cps in (0, 1, 2, 3):
             for dbits in dbit_choices:
                 knobs = {"tile_digit_bits": bits, "ctas_per_sm": cps, "depth_digit_bits": dbits}

@@ -63,14 +63,15 @@ struct Buffer {
 enum KernelId {
   kKCount, kKScan, kKDuplicate, kKRanges, kKRadixPass,
   kKFrameCount, kKDepthSort, kKFrameScan, kKDupDepth, kKTilePass, kKTileExpand, kKPreprocess, kKBitonic, kKRender, kKPreCount, kKNormRange, kKNormDup, kKNormPass,
-  kKNormRanges, kKRenderOrder, kKSortHist, kKOnesweep, kKCountDepth, kKNum
+  kKNormRanges, kKRenderOrder, kKSortHist, kKOnesweep, kKCountDepth,
+  kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
 };
 const char* const kKernelNames[kKNum] = {
     "count_tiles",  "scan",       "duplicate_keys",     "tile_ranges",    "radix_pass",
     "frame_count",  "depth_sort", "scan_by_depth", "duplicate_by_depth", "tile_sort_pass",
     "tile_expand_pass", "preprocess", "bitonic_sort", "render", "preprocess_count", "norm_range",
     "norm_duplicate", "norm_sort_pass", "norm_ranges", "render_order", "sort_histogram", "onesweep_pass",
-    "count_depth_sort"};
+    "count_depth_sort", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
 
 // View table as stored in device memory (SoA, fixed maximum size).
 struct ViewBlob {
@@ -81,6 +82,10 @@ struct ViewBlob {
   uint32_t tile_begin[kMaxViews + 1];
   uint32_t pbeg[kMaxViews + 1];
   uint32_t nt[kMaxViews];
+  // the interval splits: first level-1 tile, row and level-1 count of each view
+  uint32_t t1_begin[kMaxViews + 1];
+  uint32_t row_begin[kMaxViews + 1];
+  uint32_t c1_begin[kMaxViews + 1];
 };
 
 struct PendingTime {
@@ -112,8 +117,8 @@ struct tdgs_context {
   // State that kernels keep between launches, to be cleared before its next
   // use after an error was latched on the device (a bounded wait may have
   // given up mid-launch): the depth sort's buffers, the onesweep header, the
-  // radix grid barrier words.
-  bool dsort_dirty = true, dos_dirty = true, os_dirty = false, bar_dirty = false;
+  // radix grid barrier words, the view totals.
+  bool dsort_dirty = true, dos_dirty = true, os_dirty = false, bar_dirty = false, vtot_dirty = true;
   // fused-frame / multi-view buffers
   Buffer f_rec3, f_conic;  // projected records and conics of tdgs_sort_frame_3d
   Buffer d_cams;           // cameras of the 3D calls (device)
@@ -125,6 +130,7 @@ struct tdgs_context {
   Buffer b_keys, b_vals;   // padded scratch of tdgs_sort_pairs_bitonic
   Buffer n_counts, n_offs, n_norm, n_keys[2], n_vals[2], n_ranges;  // tdgs_sort_frame_normalized
   Buffer f_counts, f_dkey[3], f_dval[3], f_soff, f_sdo, f_rminmax, f_stream[2], f_keys, f_values, f_ranges;
+  Buffer f_rects, f_c1, f_rows, f_segs, f_c2, f_b2;  // interval splits
   // depth-key range: accumulators [0..1], result [2..3], passes of the last
   // resident depth sort [4]
   uint32_t* d_range = nullptr;
@@ -135,6 +141,8 @@ struct tdgs_context {
   ViewBlob* d_views = nullptr;  // device view table
   ViewBlob* h_views = nullptr;  // pinned staging of the table
   uint32_t nv = 0, n_all = 0, t_all = 0;
+  uint32_t max_gx = 0, max_gy = 0;  // over the staged views
+  bool split = false;           // pairs by interval splits (else packed elements and tile passes)
   uint64_t capacity = 0;        // pair capacity reserved for the asynchronous path
   bool reserved = false;
   Tuning tuning;
@@ -205,7 +213,7 @@ tdgs_status ensure(tdgs_context* ctx, Buffer& b, size_t bytes, cudaStream_t s,
 uint32_t* err_word(tdgs_context* ctx) { return &ctx->d_status->err; }
 
 void note_device_error(tdgs_context* ctx) {
-  ctx->dsort_dirty = ctx->dos_dirty = ctx->os_dirty = ctx->bar_dirty = true;
+  ctx->dsort_dirty = ctx->dos_dirty = ctx->os_dirty = ctx->bar_dirty = ctx->vtot_dirty = true;
 }
 
 // The radix grid barrier words back to zero if an error was latched since
@@ -546,7 +554,9 @@ void tdgs_context_destroy(tdgs_context* ctx) {
                     &ctx->n_offs,       &ctx->n_norm,       &ctx->n_keys[0],    &ctx->n_keys[1],
                     &ctx->n_vals[0],    &ctx->n_vals[1],    &ctx->n_ranges,
                     &ctx->f_rminmax,    &ctx->f_stream[0],   &ctx->f_stream[1],  &ctx->f_keys,
-                    &ctx->f_values,     &ctx->f_ranges,     &ctx->r_order};
+                    &ctx->f_values,     &ctx->f_ranges,     &ctx->r_order,
+                    &ctx->f_rects,      &ctx->f_c1,         &ctx->f_rows,       &ctx->f_segs,       &ctx->f_c2,
+                    &ctx->f_b2};
   if (ctx->d_views) cudaFree(ctx->d_views);
   if (ctx->h_views) cudaFreeHost(ctx->h_views);
   for (Buffer* b : bufs)
@@ -687,7 +697,8 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
   if (nv == 0 || nv > kMaxViews) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "view count out of range");
   if (!views) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null views");
   ViewBlob* h = ctx->h_views;
-  uint64_t n_all = 0, t_all = 0;
+  uint64_t n_all = 0, t_all = 0, t1 = 0, rows = 0, c1 = 0;
+  ctx->max_gx = ctx->max_gy = 0;
   for (uint32_t v = 0; v < nv; ++v) {
     const tdgs_view& w = views[v];
     if (w.f.width == 0 || w.f.height == 0) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "empty image");
@@ -701,20 +712,38 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
     h->vtot[v] = 0;
     n_all += w.n;
     t_all += h->nt[v];
+    const uint32_t gx = static_cast<uint32_t>(h->geom[v].gx), gy = static_cast<uint32_t>(h->geom[v].gy);
+    const uint32_t tiles1 = static_cast<uint32_t>((static_cast<uint64_t>(w.n) + kSplitTile - 1) / kSplitTile);
+    ctx->max_gx = std::max(ctx->max_gx, gx);
+    ctx->max_gy = std::max(ctx->max_gy, gy);
+    h->t1_begin[v] = static_cast<uint32_t>(t1);
+    h->row_begin[v] = static_cast<uint32_t>(rows);
+    h->c1_begin[v] = static_cast<uint32_t>(c1);
+    t1 += tiles1;
+    rows += gy;
+    c1 += static_cast<uint64_t>(tiles1) * gy;
   }
   if (n_all > 0xffffffffull || t_all > 0xffffffffull)
     return fail(ctx, TDGS_ERR_OVERFLOW, "too many Gaussians or tiles in one batch");
   h->rec_begin[nv] = static_cast<uint32_t>(n_all);
   h->tile_begin[nv] = static_cast<uint32_t>(t_all);
+  h->t1_begin[nv] = static_cast<uint32_t>(t1);
+  h->row_begin[nv] = static_cast<uint32_t>(rows);
+  h->c1_begin[nv] = static_cast<uint32_t>(c1);
   ctx->nv = nv;
   ctx->n_all = static_cast<uint32_t>(n_all);
   ctx->t_all = static_cast<uint32_t>(t_all);
   return TDGS_OK;
 }
 
+// One view through the interval splits: its table goes with the kernel
+// parameters (a copy to the device before the first kernel costs a small
+// frame a twentieth of its time); otherwise it is uploaded.
+bool table_in_params(const tdgs_context* ctx) { return ctx->split && ctx->nv == 1; }
+
 ViewTable device_table(tdgs_context* ctx) {
   ViewBlob* d = ctx->d_views;
-  ViewTable vt;
+  ViewTable vt{};
   vt.g = d->g;
   vt.rec_begin = d->rec_begin;
   vt.tile_begin = d->tile_begin;
@@ -722,7 +751,28 @@ ViewTable device_table(tdgs_context* ctx) {
   vt.vtot = d->vtot;
   vt.pbeg = d->pbeg;
   vt.nv = ctx->nv;
+  if (table_in_params(ctx)) {
+    const ViewBlob* h = ctx->h_views;
+    vt.one = OneView{h->g[0], h->geom[0], ctx->n_all, 1u};
+  }
   return vt;
+}
+
+// Whether the staged views' pairs come from the interval splits: one view,
+// images up to 4096 pixels a side; a tuned tile digit width asks for the
+// tile passes.
+bool splits(const tdgs_context* ctx) {
+  return ctx->nv == 1 && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
+         ctx->tuning.tile_digit_bits == 0;
+}
+
+uint32_t split_pitch(const tdgs_context* ctx) { return (ctx->max_gx + 7u) & ~7u; }
+uint32_t split_rows(const tdgs_context* ctx) { return ctx->h_views->row_begin[ctx->nv]; }
+// Level-2 tiles of at most m segments: full ones, and one ragged one per row.
+uint64_t split_tiles(const tdgs_context* ctx, uint64_t m) { return m / kSplitTile + split_rows(ctx); }
+
+DepthPlan depth_plan(const tdgs_context* ctx) {
+  return plan_depth_sort(ctx->n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm, !ctx->split);
 }
 
 struct Shape {
@@ -762,15 +812,20 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_rminmax, static_cast<size_t>(ctx->t_all) * 8 + 16, s, &grown);
   if (grown) ctx->rminmax_dirty = true;
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_ranges, static_cast<size_t>(ctx->t_all) * 8 + 16, s);
+  if (st == TDGS_OK && ctx->split) {
+    st = ensure(ctx, ctx->f_rects, n4, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_c1, static_cast<size_t>(ctx->h_views->c1_begin[ctx->nv]) * 8 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_rows, (static_cast<size_t>(split_rows(ctx)) + 1) * 20 + 16, s);
+  }
   const uint32_t n_all = ctx->n_all;
   const uint32_t tiles = (n_all + kScanTileItems - 1) / kScanTileItems;
   if (st == TDGS_OK) st = ensure(ctx, ctx->scan_status, static_cast<size_t>(tiles) * 8 + 8, s);
-  const DepthPlan dp = plan_depth_sort(n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm);
+  const DepthPlan dp = depth_plan(ctx);
   if (dp.grid == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the depth sort failed");
   if (st == TDGS_OK) st = ensure(ctx, ctx->sort_scratch, dp.scratch_words * 4, s);
   if (st == TDGS_OK && dp.resident) {
     grown = false;
-    st = ensure(ctx, ctx->f_dsort, depth_sort_scratch_words(dp.grid) * 4, s, &grown);
+    st = ensure(ctx, ctx->f_dsort, depth_sort_scratch_words(depth_sort_grid()) * 4, s, &grown);
     if (st == TDGS_OK && (grown || ctx->dsort_dirty)) {
       TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_dsort.p, 0, ctx->f_dsort.bytes, s));
       ctx->dsort_dirty = false;
@@ -789,12 +844,19 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
 
 // Buffers that depend on the pair count (or capacity) m.
 tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
+  tdgs_status st = ensure(ctx, ctx->f_keys, m * 8 + 16, s);
+  if (st == TDGS_OK) st = ensure(ctx, ctx->f_values, m * 4 + 16, s);
+  if (ctx->split) {
+    // every segment has a pair: at most m segments
+    const size_t entries = static_cast<size_t>(split_tiles(ctx, m)) * split_pitch(ctx);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_segs, m * 8 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_c2, entries * 2 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_b2, entries * 4 + 16, s);
+    return st;
+  }
   const Shape sh = shape_of(ctx);
   const size_t esz = sh.wide ? 8 : 4;
-  tdgs_status st = TDGS_OK;
   for (int b = 0; b < 2 && st == TDGS_OK; ++b) st = ensure(ctx, ctx->f_stream[b], m * esz + 16, s);
-  if (st == TDGS_OK) st = ensure(ctx, ctx->f_keys, m * 8 + 16, s);
-  if (st == TDGS_OK) st = ensure(ctx, ctx->f_values, m * 4 + 16, s);
   const uint32_t mm = static_cast<uint32_t>(m ? m : 1);
   const int cps = ctx->tuning.ctas_per_sm;
   const uint32_t g0 = stream_grid(sh.wide, false, sh.kbits, mm, cps), g1 = stream_grid(sh.wide, true, sh.klast, mm, cps);
@@ -813,13 +875,18 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   const ViewTable vt = device_table(ctx);
   const uint32_t n_all = ctx->n_all;
   if (tdgs_status st0 = clear_barrier_if_dirty(ctx, s); st0 != TDGS_OK) return st0;
-  TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->d_views, ctx->h_views, sizeof(ViewBlob), cudaMemcpyHostToDevice, s));
+  if (!table_in_params(ctx)) {
+    TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->d_views, ctx->h_views, sizeof(ViewBlob), cudaMemcpyHostToDevice, s));
+  } else if (ctx->vtot_dirty) {
+    TDGS_CUDA(ctx, cudaMemsetAsync(ctx->d_views->vtot, 0, sizeof(ctx->d_views->vtot), s));
+  }
+  ctx->vtot_dirty = false;
   uint32_t* counts = static_cast<uint32_t*>(ctx->f_counts.p);
   uint32_t* dk[3] = {static_cast<uint32_t*>(ctx->f_dkey[0].p), static_cast<uint32_t*>(ctx->f_dkey[1].p),
                      static_cast<uint32_t*>(ctx->f_dkey[2].p)};
   uint32_t* dv[3] = {static_cast<uint32_t*>(ctx->f_dval[0].p), static_cast<uint32_t*>(ctx->f_dval[1].p),
                      static_cast<uint32_t*>(ctx->f_dval[2].p)};
-  const DepthPlan dp = plan_depth_sort(n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm);
+  const DepthPlan dp = depth_plan(ctx);
   DepthSortArgs da{};
   da.vt = vt;
   da.total = &ctx->d_status->total;
@@ -828,12 +895,12 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   da.k2 = dk[2];
   da.v2 = dv[2];
   da.counts = counts;
-  da.offsets = static_cast<uint32_t*>(ctx->f_soff.p);
+  da.offsets = ctx->split ? nullptr : static_cast<uint32_t*>(ctx->f_soff.p);  // the interval splits take none
   da.range = ctx->d_range;
   da.n = n_all;
   da.scratch = static_cast<uint32_t*>(ctx->f_dsort.p);
   da.err = err_word(ctx);
-  ctx->early_fused = dp.resident && n_all > 0 && n_all <= depth_sort_count_capacity(dp.grid) && !ctx->proj_on;
+  ctx->early_fused = dp.resident && n_all > 0 && !ctx->proj_on;
   if (ctx->early_fused) {
     // one launch: counts, M (also to the mapped host status, tagged with a
     // fresh seq), the depth sort and the offsets
@@ -843,7 +910,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
       if (ctx->early_seq == 0) ctx->early_seq = 1;  // 0: never written
       da.host_seq = ctx->early_seq;
     }
-    TDGS_TRACED(ctx, kKCountDepth, n_all, s, launch_count_depth_sort(dp.grid, da, s));
+    TDGS_TRACED(ctx, kKCountDepth, n_all, s, launch_count_depth_sort(dp.grid, dp.items, da, s));
     if (early_total) TDGS_CUDA(ctx, cudaEventRecord(ctx->ev_count, s));
     return TDGS_OK;
   }
@@ -861,7 +928,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
   if (dp.resident) {  // one launch: the sort (pass count from the depth range) and the offsets
     da.key0 = dk[0];
-    TDGS_TRACED(ctx, kKDepthSort, n_all, s, launch_depth_sort(dp.grid, da, s));
+    TDGS_TRACED(ctx, kKDepthSort, n_all, s, launch_depth_sort(dp.grid, dp.items, da, s));
   } else if (dp.onesweep) {  // histogram, then the passes the key range needs (result in pair 1)
     if (n_all) {
       uint32_t* dos = static_cast<uint32_t*>(ctx->f_dos.p);
@@ -878,7 +945,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
                                     ctx->d_tickets + 2, err_word(ctx), s));
     }
   }
-  if (n_all && !dp.resident) {
+  if (n_all && !dp.resident && !ctx->split) {
     tdgs_status st = do_scan(ctx, kKFrameScan, counts, nullptr, dv[dp.result], FrameGeom{}, n_all,
                              static_cast<uint32_t*>(ctx->f_soff.p), &ctx->d_status->total, nullptr, s);
     if (st != TDGS_OK) return st;
@@ -888,13 +955,62 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   return TDGS_OK;
 }
 
+// Steps after, as interval splits: rows, columns, ranges and final pairs.
+// m = the exact pair count or the reserved capacity (the kernels read the
+// count on the device).
+tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
+  const uint32_t n_all = ctx->n_all;
+  const uint32_t dres = depth_plan(ctx).result;
+  SplitArgs a{};
+  a.vt = device_table(ctx);
+  a.t1_begin = ctx->d_views->t1_begin;
+  a.row_begin = ctx->d_views->row_begin;
+  a.c1_begin = ctx->d_views->c1_begin;
+  a.sorder = static_cast<uint32_t*>(ctx->f_dval[dres].p);
+  a.rects = static_cast<uint32_t*>(ctx->f_rects.p);
+  a.sdo = static_cast<uint2*>(ctx->f_sdo.p);
+  a.c1 = static_cast<uint2*>(ctx->f_c1.p);
+  a.nrows = split_rows(ctx);
+  a.row_tot = static_cast<uint2*>(ctx->f_rows.p);
+  a.row_seg = reinterpret_cast<uint32_t*>(a.row_tot + a.nrows);
+  a.row_tile = a.row_seg + a.nrows + 1;
+  a.row_pair = a.row_tile + a.nrows + 1;
+  a.info = a.row_pair + a.nrows;
+  a.segs = static_cast<uint2*>(ctx->f_segs.p);
+  a.c2 = static_cast<uint16_t*>(ctx->f_c2.p);
+  a.b2 = static_cast<uint32_t*>(ctx->f_b2.p);
+  a.pitch = split_pitch(ctx);
+  a.ranges = static_cast<uint2*>(ctx->f_ranges.p);
+  a.keys = static_cast<uint64_t*>(ctx->f_keys.p);
+  a.values = static_cast<uint32_t*>(ctx->f_values.p);
+  a.cap = m;
+  a.total = &ctx->d_status->total;
+  a.ticket = ctx->d_tickets;
+  a.ntiles1 = ctx->h_views->t1_begin[ctx->nv];
+  a.err = err_word(ctx);
+  const uint32_t tiles2 = static_cast<uint32_t>(split_tiles(ctx, m));
+  const int cps = ctx->tuning.ctas_per_sm;
+  TDGS_TRACED(ctx, kKRowCount, n_all, s, launch_row_count(a, s));
+  TDGS_TRACED(ctx, kKRowScan, a.nrows, s, launch_row_scan(a, s));
+  TDGS_TRACED(ctx, kKRowSplit, n_all, s, launch_row_split(a, ctx->max_gy, cps, s));
+  TDGS_TRACED(ctx, kKColCount, m, s, launch_col_count(a, tiles2, s));
+  TDGS_TRACED(ctx, kKColScan, a.nrows, s, launch_col_scan(a, s));
+  TDGS_TRACED(ctx, kKColSplit, m, s, launch_col_split(a, ctx->max_gx, tiles2, cps, s));
+  return TDGS_OK;
+}
+
 // Steps after: duplication, tile passes, ranges.  m = exact pair count, or
 // the reserved capacity with m_dev pointing at the device count.
 tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaStream_t s) {
+  if (m == 0) {
+    TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_ranges.p, 0, static_cast<size_t>(ctx->t_all) * 8, s));
+    return TDGS_OK;
+  }
+  if (ctx->split) return run_back_split(ctx, m, s);
   const ViewTable vt = device_table(ctx);
   const Shape sh = shape_of(ctx);
   const uint32_t n_all = ctx->n_all;
-  const uint32_t dres = plan_depth_sort(n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm).result;
+  const uint32_t dres = depth_plan(ctx).result;
   const uint32_t* sorder = static_cast<uint32_t*>(ctx->f_dval[dres].p);
   uint2* sdo = static_cast<uint2*>(ctx->f_sdo.p);
   uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
@@ -903,7 +1019,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
   const size_t half = ctx->f_rminmax.bytes / 8;  // tiles the buffer holds
   uint32_t* rmin = static_cast<uint32_t*>(ctx->f_rminmax.p);
   uint32_t* rmax = rmin + half;
-  TDGS_TRACED(ctx, kKDupDepth, m ? n_all : 0, s,
+  TDGS_TRACED(ctx, kKDupDepth, n_all, s,
               launch_views_dup(vt, sorder, static_cast<uint32_t*>(ctx->f_soff.p), n_all, sh.rbits, st[0],
                                sh.wide, m, sdo, err_word(ctx), s));
   // One pass over the whole tile id writes the ranges from its digit
@@ -911,10 +1027,6 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
   // last position and a small kernel turns them into ranges.
   const bool single = sh.npass == 1;
   uint2* ranges = static_cast<uint2*>(ctx->f_ranges.p);
-  if (m == 0) {
-    TDGS_CUDA(ctx, cudaMemsetAsync(ranges, 0, static_cast<size_t>(ctx->t_all) * 8, s));
-    return TDGS_OK;
-  }
   if (!single) {
     if (ctx->rminmax_dirty) {
       TDGS_CUDA(ctx, cudaMemsetAsync(rmin, 0xff, half * 4, s));
@@ -957,6 +1069,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
 // sort and the scan run; the back half is then enqueued with the exact M
 // before the GPU runs out of work.
 tdgs_status sort_views_exact(tdgs_context* ctx, cudaStream_t s, uint32_t* m_out) {
+  ctx->split = splits(ctx);
   tdgs_status st = ensure_record_buffers(ctx, s);
   if (st != TDGS_OK) return st;
   st = run_front(ctx, s, true);
@@ -1062,7 +1175,8 @@ tdgs_status sort_views_3d(tdgs_context* ctx, const tdgs_gaussian3d* g, const tdg
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_conic, total * 16 + 16, s);
   if (st == TDGS_OK) st = ensure(ctx, ctx->d_cams, sizeof(CameraDev) * nv, s);
   if (st != TDGS_OK) return st;
-  TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->d_cams.p, cd.data(), sizeof(CameraDev) * nv, cudaMemcpyHostToDevice, s));
+  if (nv > 1)  // one camera is a kernel parameter
+    TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->d_cams.p, cd.data(), sizeof(CameraDev) * nv, cudaMemcpyHostToDevice, s));
   // the count kernel projects each view's Gaussians first (preprocessing
   // fused with the count) and stores records and conics view after view
   std::vector<tdgs_view> views(nv);
@@ -1319,6 +1433,7 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
   DeviceGuard dg(ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tdgs_status st = stage_views(ctx, views, num_views);
+  if (st == TDGS_OK) ctx->split = splits(ctx);  // the asynchronous calls keep this choice
   if (st == TDGS_OK) st = ensure_record_buffers(ctx, s);
   if (st == TDGS_OK) st = ensure_pair_buffers(ctx, pair_capacity, s);
   if (st != TDGS_OK) return st;

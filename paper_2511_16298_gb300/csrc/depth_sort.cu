@@ -4,9 +4,9 @@
 // order (the first pair of every Gaussian).  Two forms, both with one
 // 8192-key tile per CTA (larger frames take the onesweep passes over the
 // same compressed keys, onesweep.cu):
-//  * k_depth_sort<true>: the tile count step first (records in, keys kept
+//  * k_depth_sort<true, *>: the tile count step first (records in, keys kept
 //    in registers), then the sort.
-//  * k_depth_sort<false>: keys and counts from the count kernel.
+//  * k_depth_sort<false, *>: keys and counts from the count kernel.
 //
 // The N depth keys (raw float bits; all ones for a Gaussian without pairs)
 // are compressed to key - smallest (all ones -> one past the largest) and
@@ -61,7 +61,7 @@
 namespace tdgs {
 namespace depth {
 
-constexpr int kThreads = 512, kItems = 16, kBits = 9;
+constexpr int kThreads = 512, kBits = 9;
 constexpr uint32_t kBins = 1u << kBits;
 constexpr uint32_t kWarps = kThreads / 32;
 constexpr uint32_t kMaxPasses = 4;  // 32 key bits in digits of at most 9
@@ -69,11 +69,17 @@ constexpr uint32_t kMaxGrid = radix::kMaxGrid;  // chunks (CTAs) at most
 constexpr uint32_t kValueBits = 22; // record indices below 2^22 (N <= kMaxGrid * 8192)
 constexpr uint32_t kRecMask = (1u << kValueBits) - 1u;
 constexpr uint32_t kCntEscape = (1u << (32 - kValueBits)) - 1u;  // 1023: the count is gathered again
-using S = radix::PassShape<uint32_t, true, false, kBits, kThreads, kItems, 1>;
-constexpr uint32_t kTileKeys = S::kTileKeys;
-constexpr size_t kSmem = S::kSmem + kTileKeys * 4;  // + the staged values
-static_assert(S::kSmem % 16 == 0, "the staged values start 16-byte aligned");
-static_assert(kTileKeys == 8192, "one 8192-key chunk per CTA");
+template <int kItems>
+using ShapeOf = radix::PassShape<uint32_t, true, false, kBits, kThreads, kItems, 1>;
+constexpr int kMaxItems = 16;
+constexpr uint32_t kTileKeys = kThreads * kMaxItems;
+constexpr size_t smem_bytes(int items) {  // the pass's own + the staged values
+  return (items == 4 ? ShapeOf<4>::kSmem : items == 8 ? ShapeOf<8>::kSmem : ShapeOf<16>::kSmem) +
+         static_cast<size_t>(kThreads) * items * 4;
+}
+static_assert(ShapeOf<4>::kSmem % 16 == 0 && ShapeOf<8>::kSmem % 16 == 0 && ShapeOf<16>::kSmem % 16 == 0,
+              "the staged values start 16-byte aligned");
+static_assert(kTileKeys == 8192, "one chunk of at most 8192 keys per CTA");
 static_assert(4 * kTileKeys + 1 < (1u << 16), "a chunk's count of one digit, plus one, fits a 16-bit row field");
 static_assert(static_cast<uint64_t>(kMaxGrid) * kTileKeys <= (1ull << kValueBits), "record index bits");
 static_assert(kThreads == static_cast<int>(kBins), "one digit per thread in the base computation");
@@ -214,6 +220,7 @@ __device__ __forceinline__ void sum_rows(const uint32_t* __restrict__ rows, uint
 // adds the counts it writes into the per-output-chunk sums csum (chunks of
 // Sz positions; vstage is free by then and holds per-warp sums).  Returns
 // false if a destination fell outside [0, n).  Ends with a block barrier.
+template <bool kOffsets, int kItems>
 __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm, uint32_t* vstage,
                                                  const uint32_t (&hi)[kItems], const uint32_t (&pos)[kItems],
                                                  uint32_t valid,
@@ -223,6 +230,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
                                                  uint32_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                  const uint32_t* __restrict__ counts, uint32_t Sz, uint32_t G,
                                                  uint32_t* __restrict__ csum) {
+  using S = ShapeOf<kItems>;
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   bool ok = true;
   const uint32_t wbase = warp * 32 * kItems;
@@ -234,26 +242,32 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
     const uint32_t idx = wbase + j * 32 + lane;
     v[j] = 0u;
     if (idx < valid) {
-      const uint32_t x = idx < nstaged ? vstage[idx] : __ldg(vsrc + tb + idx);
-      v[j] = first ? (tb + idx) | (min(x, kCntEscape) << kValueBits) : x;
+      if (!kOffsets && first) {
+        v[j] = tb + idx;
+      } else {
+        const uint32_t x = idx < nstaged ? vstage[idx] : __ldg(vsrc + tb + idx);
+        v[j] = first ? (tb + idx) | (min(x, kCntEscape) << kValueBits) : x;
+      }
     }
   }
   uint64_t* x64 = reinterpret_cast<uint64_t*>(sm.xk);
-  static_assert(S::kXkBytes + S::kXvBytes >= kTileKeys * 8, "the 8-byte exchange spans both buffers");
+  static_assert(S::kXkBytes + S::kXvBytes >= S::kTileKeys * 8, "the 8-byte exchange spans both buffers");
 #pragma unroll
   for (int j = 0; j < kItems; ++j)
     if (wbase + j * 32 + lane < valid) x64[pos[j]] = (static_cast<uint64_t>(hi[j]) << 32) | v[j];
   __syncthreads();
-  if (!last) {
+  if (!kOffsets || !last) {
+    // (in the last pass the high word is the digit, and only the values are kept)
+    const uint32_t sh = last ? 0u : shift;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
       const uint32_t xp = i * kThreads + t;
       if (xp < valid) {
         const uint64_t x = x64[xp];
         const uint32_t key = static_cast<uint32_t>(x >> 32);
-        const uint32_t dst = sm.off[(key >> shift) & mask] + xp;
+        const uint32_t dst = sm.off[(key >> sh) & mask] + xp;
         if (dst < n) {
-          kout[dst] = key;
+          if (kOffsets || !last) kout[dst] = key;
           vout[dst] = static_cast<uint32_t>(x);
         } else {
           ok = false;
@@ -265,7 +279,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
     // Gaussian's tile count (k1); the counts are summed per output chunk
     // per-warp rows of counts per output chunk, over the staged values
     // (read before the exchange barrier above)
-    static_assert(kWarps * kMaxGrid * 4 <= kTileKeys * 4, "per-warp chunk sums fit the staging buffer");
+    static_assert(!kOffsets || kWarps * kMaxGrid * 4 <= S::kTileKeys * 4, "per-warp chunk sums fit the staging buffer");
     uint32_t* w_csum = vstage + warp * kMaxGrid;
     for (uint32_t k = lane; k < G; k += 32) w_csum[k] = 0u;
     __syncwarp();
@@ -350,6 +364,7 @@ __device__ __forceinline__ uint64_t chunks_before(const uint32_t* csum, uint32_t
 // the exclusive scan of the counts k1 from `base`, kItems consecutive
 // positions per thread.  Returns base + their sum; a sum above 2^32 - 1
 // latches TDGS_ERR_OVERFLOW.  Block barriers inside.
+template <int kItems>
 __device__ __forceinline__ uint64_t scan_offsets(const uint32_t* __restrict__ k1, uint32_t* __restrict__ offsets,
                                                  uint32_t b, uint32_t e, uint64_t base, unsigned long long* s_sum,
                                                  uint32_t* err) {
@@ -417,9 +432,18 @@ __device__ __forceinline__ uint64_t scan_offsets(const uint32_t* __restrict__ k1
 
 // kCount: the tile count step runs first in the same launch (records of
 // the view table in, keys kept in registers); else the keys come from the
-// count kernel (key0) with the range it published.
-template <bool kCount>
+// count kernel (key0) with the range it published.  kOffsets: the tile
+// counts travel with the record indices and the launch ends with their scan
+// in depth order; without it the values are the record indices alone and
+// counts, k1 and offsets are not touched after pass 0 (the interval splits
+// take no offsets).
+// kItems: keys per thread.  A pass takes about as long for a few keys per CTA
+// as for a full tile, so fewer keys take a smaller tile and no more CTAs than
+// it needs (plan_depth_sort).
+template <bool kCount, bool kOffsets, int kItems>
 __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
+  using S = ShapeOf<kItems>;
+  constexpr uint32_t kTileKeys = S::kTileKeys;
   const uint32_t* __restrict__ key0 = A.key0;
   uint32_t* __restrict__ k1 = A.k1;
   uint32_t* __restrict__ v1 = A.v1;
@@ -446,9 +470,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     sm.off = sm.lstart + kBins;
   }
   uint32_t* vstage = reinterpret_cast<uint32_t*>(smem + S::kSmem);  // this pass's values, in chunk order
-  // the row sums of the groups share the value exchange buffer (not live then)
-  uint32_t* s_part = sm.xv;
-  static_assert(S::kXvBytes >= kRowGroups * kBins * 4, "row-sum partials fit the value exchange");
+  // the row sums of the groups share the exchange buffers (not live then)
+  uint32_t* s_part = sm.xk;
+  static_assert(S::kXkBytes + S::kXvBytes >= kRowGroups * kBins * 4, "row-sum partials fit the exchange");
   __shared__ uint32_t s_hx[kMaxPasses - 1][kBins];  // pass 0: this chunk's counts of the later digits
   __shared__ uint2 s_warp2[kWarps];
   __shared__ unsigned long long s_sum[kWarps + 1];
@@ -485,12 +509,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     __shared__ uint32_t s_lo, s_hi, s_cull;
     const ViewTable& vt = A.vt;
     const uint32_t nv = vt.nv;
-    for (uint32_t v = t; v <= nv; v += kThreads) s_begin[v] = vt.rec_begin[v];
     for (uint32_t v = t; v < nv; v += kThreads) {
-      s_g[v] = vt.g[v];
-      s_geom[v] = vt.geom[v];
+      const ViewOf w = view_of(vt, v);
+      s_begin[v] = w.rec0;
+      s_g[v] = w.g;
+      s_geom[v] = w.geom;
       s_tot[v] = 0ull;
     }
+    if (t == 0) s_begin[nv] = n;
     s_raw[t] = 0u;
     s_h0[t] = 0u;
     if (t == 0) {
@@ -503,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     uint32_t klo = 0xffffffffu, khi = 0u, nculled = 0u;
     unsigned long long tsum = 0;  // one view: this thread's pairs
     bool bad = false;
-    constexpr int kGroup = 16;  // records in flight per thread
+    constexpr int kGroup = kItems;  // records in flight per thread
 #pragma unroll
     for (int j0 = 0; j0 < kItems; j0 += kGroup) {
       float4 rec[kGroup];
@@ -527,8 +553,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
           const TileRect tr = tile_rect(rec[u], s_geom[vv[u]]);
           bad |= tr.invalid;
           const uint32_t cnt = tr.count;
-          vstage[idx] = cnt;
-          if (cnt >= kCntEscape) counts[beg + idx] = cnt;
+          if constexpr (kOffsets) {
+            vstage[idx] = cnt;
+            if (cnt >= kCntEscape) counts[beg + idx] = cnt;
+          }
           if (cnt) {
             const uint32_t key = __float_as_uint(rec[u].z);
             R.k[j] = key;
@@ -575,6 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
       for (uint32_t v = 0; v < nv; ++v) {
         vt.pbeg[v] = static_cast<uint32_t>(run);
         run += __ldcg(reinterpret_cast<const unsigned long long*>(vt.vtot + v));
+        vt.vtot[v] = 0;  // for the next frame
       }
       vt.pbeg[nv] = static_cast<uint32_t>(run);
       *A.total = run;
@@ -602,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     range[4] = passes;
     scratch[kFinalSlot * kLine] = 0u;  // the previous launch's final barrier
   }
-  if (c == 0)  // this launch's chunk sums (added to after the first barrier)
+  if (kOffsets && c == 0)  // this launch's chunk sums (added to after the first barrier)
     for (uint32_t i = t; i < G; i += kThreads) csum[i] = 0u;
   const uint32_t nbulk = valid & ~3u;  // values by bulk copy; the last 1-3 by plain loads
   if (t == 0) {
@@ -636,12 +665,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     uint32_t* vout = to_one ? v1 : v2;
     a.shift = p * width;
     const uint32_t* vsrc = p == 0 ? counts : vin;
-    const bool counted = kCount && p == 0;  // values (the counts) already staged by the count step
+    const bool counted = kCount && p == 0;  // keys in registers, values (the counts) already staged
+    const bool unstaged = counted || (!kOffsets && p == 0);  // no values to copy in
     const uint32_t nstaged = counted ? valid : nbulk;
     if (t == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      osw::mbar_arrive(&s_mbar, counted ? 0u : nbulk * 4);
-      if (!counted && nbulk) osw::bulk_g2s(vstage, vsrc + beg, nbulk * 4, &s_mbar);
+      osw::mbar_arrive(&s_mbar, unstaged ? 0u : nbulk * 4);
+      if (!unstaged && nbulk) osw::bulk_g2s(vstage, vsrc + beg, nbulk * 4, &s_mbar);
     }
     {
       // this pass's keys: pass 0 compresses them (from the count step's
@@ -731,19 +761,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     uint32_t hk[kItems];  // exchanged with each value: the key, in the last pass its digit
 #pragma unroll
     for (int j = 0; j < kItems; ++j) hk[j] = last ? R.d[j] : R.k[j];
-    ok &= exchange_scatter(sm, vstage, hk, R.r, valid, beg, nstaged, vsrc, p == 0, last, a.shift, mask, n, kout,
+    ok &= exchange_scatter<kOffsets, kItems>(sm, vstage, hk, R.r, valid, beg, nstaged, vsrc, p == 0, last, a.shift, mask, n, kout,
                            vout, k1, v1, counts, Sz, G, csum);
     arrive_and_wait(scratch + (last ? kFinalSlot : 1 + p) * kLine, G, err);
   }
   if (!ok) latch_error(err, TDGS_ERR_CAPACITY, kSiteRadixRange);
   // The pair offsets: counts in depth order (k1) scanned from the sum of
   // the chunks before this one.
-  if (warp == 0) {
-    uint64_t before = chunks_before(csum, c);
-    if (lane == 0) s_base = before;
+  if constexpr (kOffsets) {
+    if (warp == 0) {
+      uint64_t before = chunks_before(csum, c);
+      if (lane == 0) s_base = before;
+    }
+    __syncthreads();
+    scan_offsets<kItems>(k1, offsets, beg, end, s_base, s_sum, err);
   }
-  __syncthreads();
-  scan_offsets(k1, offsets, beg, end, s_base, s_sum, err);
   // Reset for the next launch (every reader of these is past the final
   // barrier): this chunk's rows; CTA 0 the totals, the histogram of the
   // count step, the key range and the mid-launch counters.
@@ -769,31 +801,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
 
 // ------------------------------------------------------------- host side
 namespace {
-enum class Form { kCount, kOne };
-radix::Kernel depth_kernel(Form f) {
-  const void* fn = f == Form::kCount ? reinterpret_cast<const void*>(&depth::k_depth_sort<true>)
-                                     : reinterpret_cast<const void*>(&depth::k_depth_sort<false>);
-  return radix::Kernel{fn, depth::kBits, depth::kThreads, depth::kItems, depth::kSmem, 1};
+// With the count step and with the offsets (always 16 keys per thread), or
+// the order alone (4, 8 or 16).
+radix::Kernel depth_kernel(bool count, bool offsets, int items) {
+  using namespace depth;
+  const void* fn = nullptr;
+  if (offsets)
+    fn = count ? reinterpret_cast<const void*>(&k_depth_sort<true, true, 16>)
+               : reinterpret_cast<const void*>(&k_depth_sort<false, true, 16>);
+  else if (items == 4)
+    fn = count ? reinterpret_cast<const void*>(&k_depth_sort<true, false, 4>)
+               : reinterpret_cast<const void*>(&k_depth_sort<false, false, 4>);
+  else if (items == 8)
+    fn = count ? reinterpret_cast<const void*>(&k_depth_sort<true, false, 8>)
+               : reinterpret_cast<const void*>(&k_depth_sort<false, false, 8>);
+  else
+    fn = count ? reinterpret_cast<const void*>(&k_depth_sort<true, false, 16>)
+               : reinterpret_cast<const void*>(&k_depth_sort<false, false, 16>);
+  return radix::Kernel{fn, kBits, kThreads, items, smem_bytes(items), 1};
 }
 
-cudaError_t launch_depth(Form f, uint32_t grid, const DepthSortArgs& a, cudaStream_t s) {
+cudaError_t launch_depth(bool count, uint32_t grid, int items, const DepthSortArgs& a, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
-  if (grid == 0 || grid > radix::kMaxGrid || a.n > depth_sort_count_capacity(grid))
+  if (a.offsets && items != 16) return cudaErrorInvalidConfiguration;
+  if (grid == 0 || grid > radix::kMaxGrid || a.n > depth_sort_count_capacity(grid, items))
     return cudaErrorInvalidConfiguration;
-  if (f == Form::kCount && a.vt.nv > kMaxViews) return cudaErrorInvalidValue;
+  if (count && a.vt.nv > kMaxViews) return cudaErrorInvalidValue;
   DepthSortArgs args = a;
   void* params[] = {(void*)&args};
+  const radix::Kernel k = depth_kernel(count, a.offsets != nullptr, items);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(depth::kThreads);
-  cfg.dynamicSmemBytes = depth::kSmem;
+  cfg.dynamicSmemBytes = k.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelExC(&cfg, depth_kernel(f).fn, params);
+  return cudaLaunchKernelExC(&cfg, k.fn, params);
 }
 }  // namespace
 
@@ -801,29 +848,33 @@ uint32_t depth_sort_grid() {
   // every form: one CTA per SM (the occupancy query also sets their shared
   // memory limit on this device)
   uint32_t g = radix::kMaxGrid;
-  for (Form f : {Form::kCount, Form::kOne}) {
-    const uint32_t r = radix::resident_ctas(depth_kernel(f), 1);
+  for (bool count : {true, false}) {
+    for (int items : {4, 8, 16}) {
+      const uint32_t r = radix::resident_ctas(depth_kernel(count, false, items), 1);
+      if (r < g) g = r;
+    }
+    const uint32_t r = radix::resident_ctas(depth_kernel(count, true, 16), 1);
     if (r < g) g = r;
   }
   return g;
 }
 
-uint32_t depth_sort_count_capacity(uint32_t grid) {
+uint32_t depth_sort_count_capacity(uint32_t grid, int items) {
   // chunks of ceil(n / G) keys rounded up to a multiple of 4 fit one tile
-  // (8192, itself a multiple of 4) exactly when n <= G * 8192
-  return grid * depth::kTileKeys;
+  // (itself a multiple of 4) exactly when n <= G * tile
+  return grid * static_cast<uint32_t>(depth::kThreads * items);
 }
 
 size_t depth_sort_scratch_words(uint32_t grid) {
   return depth::kRowWord + static_cast<size_t>(depth::kMaxPasses) * grid * depth::kRowWords;
 }
 
-cudaError_t launch_depth_sort(uint32_t grid, const DepthSortArgs& a, cudaStream_t s) {
-  return launch_depth(Form::kOne, grid, a, s);
+cudaError_t launch_depth_sort(uint32_t grid, int items, const DepthSortArgs& a, cudaStream_t s) {
+  return launch_depth(false, grid, items, a, s);
 }
 
-cudaError_t launch_count_depth_sort(uint32_t grid, const DepthSortArgs& a, cudaStream_t s) {
-  return launch_depth(Form::kCount, grid, a, s);
+cudaError_t launch_count_depth_sort(uint32_t grid, int items, const DepthSortArgs& a, cudaStream_t s) {
+  return launch_depth(true, grid, items, a, s);
 }
 
 }  // namespace tdgs

@@ -40,17 +40,21 @@ __global__ void __launch_bounds__(256)
   __shared__ uint32_t s_lo, s_hi;
   __shared__ CameraDev s_cam[kProject ? kMaxViews : 1];
   __shared__ float2 s_lim[kProject ? kMaxViews : 1];
-  for (uint32_t v = threadIdx.x; v <= vt.nv; v += blockDim.x) s_begin[v] = vt.rec_begin[v];
   for (uint32_t v = threadIdx.x; v < vt.nv; v += blockDim.x) {
+    const ViewOf w = view_of(vt, v);
+    s_begin[v] = w.rec0;
     s_tot[v] = 0;
-    s_g[v] = vt.g[v];
-    s_geom[v] = vt.geom[v];
+    s_g[v] = w.g;
+    s_geom[v] = w.geom;
     if constexpr (kProject) {
-      s_cam[v] = pj.cams[v];
-      s_lim[v] = proj::slope_limits(pj.cams[v]);
+      if (vt.nv > 1) {  // one view's camera is a parameter
+        s_cam[v] = pj.cams[v];
+        s_lim[v] = proj::slope_limits(pj.cams[v]);
+      }
     }
   }
   if (threadIdx.x == 0) {
+    s_begin[vt.nv] = n_all;
     s_lo = 0xffffffffu;
     s_hi = 0u;
   }
@@ -143,7 +147,10 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   if (s_last) {
     __threadfence();
-    for (uint32_t v = threadIdx.x; v < vt.nv; v += blockDim.x) s_tot[v] = __ldcg(reinterpret_cast<unsigned long long*>(vt.vtot + v));
+    for (uint32_t v = threadIdx.x; v < vt.nv; v += blockDim.x) {
+      s_tot[v] = __ldcg(reinterpret_cast<unsigned long long*>(vt.vtot + v));
+      vt.vtot[v] = 0;  // for the next frame
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
       uint64_t run = 0;

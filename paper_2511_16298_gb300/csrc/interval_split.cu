@@ -1,0 +1,674 @@
+// Duplication and tile sort of the fused frame (Sec. II-A "Duplication with
+// Tiles" and "Sorting", Identify Range of Sec. IV-B) as two stable splits of
+// intervals.  The Gaussians arrive in depth order (view after view).  A
+// Gaussian's tile rectangle is an interval of tile rows times an interval of
+// tile columns, so the pairs need no sort of their own:
+//   level 1  items = Gaussians in depth order, bins = tile rows: every
+//            Gaussian goes, in order, to the list of each row it covers, as a
+//            segment {depth position, its columns};
+//   level 2  items = a row's segments in order, bins = tile columns: every
+//            segment goes to the list of each column it covers, as the final
+//            (tile << 32 | depth bits, index) pair.
+// Rows are outer and columns inner in the tile id, so the rows' lists one
+// after the other are the sorted pairs, and each tile's list keeps the depth
+// order.  Only level 2 touches every pair, once: no pair is written or read
+// in between.
+//
+// One level is three launches over tiles of 1024 items:
+//   count  per tile and bin, how many items cover it (two shared atomics per
+//          item into a difference array, then a prefix over the bins);
+//   scan   per row: each tile's first position in each bin's list (level 2:
+//          also the tile ranges);
+//   split  ranks and writes the tile (k_split below).
+//
+// Ranks need no sort either.  A warp takes 32 items; per bin, the mask of its
+// items that cover the bin is the prefix XOR over the bins of each item's bit
+// toggled at its first bin and past its last one: two shared atomics per item
+// and one XOR scan over the bins, whatever the intervals.  The rank of item i
+// in a bin is the number of lower bits of that bin's mask, plus the bin's
+// items in the warps before.
+#include "radix.cuh"
+
+namespace tdgs {
+namespace split {
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kPerWarp = 2;                                 // 32-item batches per warp
+constexpr int kBatches = kWarps * kPerWarp;
+constexpr uint32_t kTile = kBatches * 32;                   // items per tile
+constexpr uint32_t kStage = 8192;                           // pairs staged in shared memory at once
+constexpr uint32_t kMaxBins = kSplitMaxBins;
+constexpr int kCountThreads = 256;
+constexpr uint32_t kEmptyRect = 0x00ff0000u;                // first row above the last: no rows
+static_assert(kTile == kSplitTile, "the host sizes the tile tables");
+static_assert(kMaxBins == 256, "bins and columns are packed in bytes");
+static_assert(kTile <= kStage, "one bin of a tile fits the stage");
+
+// Every launch here may start while the one before it on the stream still
+// runs (programmatic dependent launch): its blocks wait for that launch's
+// end, and all of its writes, before they touch memory.  Every block waits,
+// so a launch's end implies the end of all launches before it.
+__device__ __forceinline__ void begin_launch() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Largest i < n with begin[i] <= x (begin ascending, begin[0] <= x), by the
+// whole warp: 32 probes at a time.
+__device__ __forceinline__ uint32_t warp_find(const uint32_t* __restrict__ begin, uint32_t n, uint32_t x) {
+  uint32_t lo = 0, len = n;
+  while (len > 1) {
+    const uint32_t step = (len + 31) / 32, at = lane_id() * step;
+    const bool le = at < len && __ldg(begin + lo + at) <= x;
+    const uint32_t k = 31u - __clz(__ballot_sync(0xffffffffu, le) | 1u);
+    lo += k * step;
+    len = min(step, len - k * step);
+  }
+  return lo;
+}
+
+// 1 << n, 0 for n above 31, and the n lowest bits.
+__device__ __forceinline__ uint32_t bit_or_none(uint32_t n) {
+  uint32_t x;
+  asm("shl.b32 %0, 1, %1;" : "=r"(x) : "r"(n));
+  return x;
+}
+__device__ __forceinline__ uint32_t low_bits(uint32_t n) {
+  uint32_t x;
+  asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(x) : "r"(n));
+  return x;
+}
+
+template <typename T>
+__device__ __forceinline__ T warp_incl_scan(T x) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const T o = __shfl_up_sync(0xffffffffu, x, d);
+    if (lane_id() >= static_cast<uint32_t>(d)) x += o;
+  }
+  return x;
+}
+
+// Inclusive sums over the block of two values at once (s_w: one per warp).
+template <int kW, typename T>
+__device__ __forceinline__ void block_incl_scan2(T& a, T& b, T (*s_w)[2]) {
+  const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+  a = warp_incl_scan(a);
+  b = warp_incl_scan(b);
+  if (lane == 31) {
+    s_w[warp][0] = a;
+    s_w[warp][1] = b;
+  }
+  __syncthreads();
+  T pa = 0, pb = 0;
+#pragma unroll
+  for (int w = 0; w < kW; ++w)
+    if (w < static_cast<int>(warp)) {
+      pa += s_w[w][0];
+      pb += s_w[w][1];
+    }
+  a += pa;
+  b += pb;
+}
+
+// Where view v's level-1 tiles, rows and counts lie among all views'.
+struct Place {
+  uint32_t tile0, tiles, row0, c10;
+};
+__device__ __forceinline__ Place place_of(const SplitArgs& a, uint32_t v) {
+  if (a.vt.one.on) return Place{0u, a.ntiles1, 0u, 0u};
+  const uint32_t t0 = __ldg(a.t1_begin + v);
+  return Place{t0, __ldg(a.t1_begin + v + 1) - t0, __ldg(a.row_begin + v), __ldg(a.c1_begin + v)};
+}
+
+// ------------------------------------------------------------ level 1 count
+// Per tile of 1024 depth positions: each Gaussian's {depth key, index} and
+// rectangle in depth order (coalesced for the later launches; the records
+// are gathered here, once), and per row its Gaussians and its pairs in the
+// tile, as differences at the first row and past the last.
+__global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
+  __shared__ int s_d[kMaxBins + 1][2];
+  __shared__ uint32_t s_w[kCountThreads / 32][2];
+  begin_launch();
+  const uint32_t t = threadIdx.x;
+  const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.t1_begin, a.vt.nv, blockIdx.x);
+  const Place pl = place_of(a, v);
+  const ViewOf vw = view_of(a.vt, v);
+  const uint32_t tl = blockIdx.x - pl.tile0, nt = pl.tiles, rec0 = vw.rec0, nrec = vw.nrec;
+  const FrameGeom fg = vw.geom;
+  const float4* __restrict__ g = vw.g;
+  for (uint32_t b = t; b <= kMaxBins; b += kCountThreads) s_d[b][0] = s_d[b][1] = 0;
+  __syncthreads();
+  constexpr int kPer = kTile / kCountThreads;
+  const uint32_t first = tl * kTile;
+  uint32_t gi[kPer];
+  float4 rec[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint32_t p = first + u * kCountThreads + t;
+    gi[u] = p < nrec ? __ldg(a.sorder + rec0 + p) - rec0 : 0xffffffffu;
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u)  // an order that is not a permutation is never followed out of bounds
+    rec[u] = gi[u] < nrec ? __ldg(g + gi[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint32_t p = first + u * kCountThreads + t;
+    if (p >= nrec) continue;
+    const TileRect q = tile_rect(rec[u], fg);
+    uint32_t pack = kEmptyRect;
+    if (q.count) {
+      const int w = q.x1 - q.x0;
+      pack = static_cast<uint32_t>(q.x0) | (static_cast<uint32_t>(q.x1 - 1) << 8) |
+             (static_cast<uint32_t>(q.y0) << 16) | (static_cast<uint32_t>(q.y1 - 1) << 24);
+      atomicAdd(&s_d[q.y0][0], 1);
+      atomicAdd(&s_d[q.y0][1], w);
+      atomicAdd(&s_d[q.y1][0], -1);
+      atomicAdd(&s_d[q.y1][1], -w);
+    }
+    a.rects[rec0 + p] = pack;
+    a.sdo[rec0 + p] = make_uint2(__float_as_uint(rec[u].z), gi[u]);
+  }
+  __syncthreads();
+  uint32_t c = static_cast<uint32_t>(s_d[t][0]), w = static_cast<uint32_t>(s_d[t][1]);
+  block_incl_scan2<kCountThreads / 32>(c, w, s_w);
+  if (t < static_cast<uint32_t>(fg.gy)) a.c1[pl.c10 + t * nt + tl] = make_uint2(c, w);
+}
+
+// ------------------------------------------------------------- level 1 scan
+// One block per row (of all views): the row's Gaussians before each of its
+// tiles, and the row's segments and pairs.  The last block then gives every
+// row its first segment, first level-2 tile and first pair.  More pairs than
+// the buffers hold (or than the depth order accounts for) latches
+// TDGS_ERR_CAPACITY and leaves nothing for the later launches to do.
+__global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
+  __shared__ uint32_t s_w[kCountThreads / 32][2];
+  __shared__ unsigned long long s_w64[kCountThreads / 32][2];
+  __shared__ bool s_last;
+  begin_launch();
+  constexpr uint32_t kPer = 4;
+  const uint32_t t = threadIdx.x, r = blockIdx.x;
+  const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
+  const Place pl = place_of(a, v);
+  const uint32_t nt = pl.tiles;
+  uint2* __restrict__ col = a.c1 + pl.c10 + static_cast<size_t>(r - pl.row0) * nt;
+  uint32_t segs = 0, pairs = 0;
+  for (uint32_t i0 = 0; i0 < nt; i0 += kCountThreads * kPer) {
+    uint2 x[kPer];
+    uint32_t sum = 0, w = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t i = i0 + t * kPer + u;
+      x[u] = i < nt ? col[i] : make_uint2(0u, 0u);
+      sum += x[u].x;
+      w += x[u].y;
+    }
+    uint32_t run = sum;
+    block_incl_scan2<kCountThreads / 32>(run, w, s_w);
+    uint32_t before = segs + run - sum;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t i = i0 + t * kPer + u;
+      if (i < nt) col[i].y = before;
+      before += x[u].x;
+    }
+    __syncthreads();  // s_w is read
+    if (t == kCountThreads - 1) {
+      s_w[0][0] = run;
+      s_w[0][1] = w;
+    }
+    __syncthreads();
+    segs += s_w[0][0];
+    pairs += s_w[0][1];
+    __syncthreads();
+  }
+  if (t == 0) {
+    a.row_tot[r] = make_uint2(segs, pairs);
+    __threadfence();
+    s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const uint32_t nrows = gridDim.x;
+  uint32_t seg0 = 0, tile0 = 0;
+  unsigned long long pair0 = 0;
+  for (uint32_t i0 = 0; i0 < nrows; i0 += kCountThreads) {
+    const uint32_t i = i0 + t;
+    const uint2 x = i < nrows ? __ldcg(a.row_tot + i) : make_uint2(0u, 0u);
+    const uint32_t nt2 = (x.x + kTile - 1) / kTile;
+    // segments and tiles side by side in 64 bits (neither reaches 2^32)
+    unsigned long long st = (static_cast<unsigned long long>(nt2) << 32) | x.x, pr = x.y;
+    block_incl_scan2<kCountThreads / 32>(st, pr, s_w64);
+    if (i < nrows) {
+      a.row_seg[i] = seg0 + static_cast<uint32_t>(st) - x.x;
+      a.row_tile[i] = tile0 + static_cast<uint32_t>(st >> 32) - nt2;
+      a.row_pair[i] = static_cast<uint32_t>(pair0 + pr - x.y);
+    }
+    __syncthreads();
+    if (t == kCountThreads - 1) {
+      s_w64[0][0] = st;
+      s_w64[0][1] = pr;
+    }
+    __syncthreads();
+    seg0 += static_cast<uint32_t>(s_w64[0][0]);
+    tile0 += static_cast<uint32_t>(s_w64[0][0] >> 32);
+    pair0 += s_w64[0][1];
+    __syncthreads();
+  }
+  if (t == 0) {
+    const bool fits = pair0 == *a.total && pair0 <= a.cap;
+    if (!fits)
+      latch_error(a.err, *a.total > 0xffffffffull ? TDGS_ERR_OVERFLOW : TDGS_ERR_CAPACITY, kSiteViewsDup);
+    a.row_seg[nrows] = seg0;
+    a.row_tile[nrows] = tile0;
+    a.info[0] = fits ? tile0 : 0u;  // level-2 tiles to process
+    a.info[1] = fits ? 1u : 0u;
+    *a.ticket = 0u;
+  }
+}
+
+// ------------------------------------------------------------ level 2 count
+// Per tile of 1024 segments of one row: the segments that cover each column.
+__global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
+  __shared__ int s_d[kMaxBins + 1];
+  __shared__ uint32_t s_w[kCountThreads / 32];
+  begin_launch();
+  const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+  const uint32_t ntiles = __ldg(a.info);
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const uint32_t r = warp_find(a.row_tile, a.nrows, tile);
+    const uint32_t beg = __ldg(a.row_seg + r) + (tile - __ldg(a.row_tile + r)) * kTile;
+    const uint32_t end = min(beg + kTile, __ldg(a.row_seg + r + 1));
+    constexpr int kPer = kTile / kCountThreads;
+    uint32_t x[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint32_t p = beg + u * kCountThreads + t;
+      x[u] = p < end ? __ldg(&a.segs[p].y) : 0xffffffffu;
+    }
+    for (uint32_t b = t; b <= kMaxBins; b += kCountThreads) s_d[b] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      if (x[u] != 0xffffffffu) {
+        atomicAdd(&s_d[x[u] & 0xffu], 1);
+        atomicAdd(&s_d[((x[u] >> 8) & 0xffu) + 1u], -1);
+      }
+    }
+    __syncthreads();
+    uint32_t c = warp_incl_scan(static_cast<uint32_t>(s_d[t]));
+    if (lane == 31) s_w[warp] = c;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kCountThreads / 32; ++w)
+      if (w < static_cast<int>(warp)) c += s_w[w];
+    if (t < a.pitch) a.c2[static_cast<size_t>(tile) * a.pitch + t] = static_cast<uint16_t>(c);
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------- level 2 scan
+// One block per row: the first output position of every tile and column, and
+// the row's tile ranges (relative to the view's first pair; {0, 0} if
+// empty).  Thread (g, c) walks column c over the g-th share of the row's
+// tiles: once for the sums, once for the positions.
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
+  __shared__ uint32_t s_sum[kScanThreads];
+  __shared__ uint32_t s_w[kScanThreads / 32];
+  begin_launch();
+  if (__ldg(a.info + 1) == 0u) return;  // more pairs than the buffers hold
+  const uint32_t t = threadIdx.x, r = blockIdx.x;
+  const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
+  const uint32_t gx = static_cast<uint32_t>(view_of(a.vt, v).geom.gx), y = r - place_of(a, v).row0;
+  const uint32_t lp = gx <= 32 ? 5u : 32u - static_cast<uint32_t>(__clz(gx - 1));  // columns padded to 2^lp
+  const uint32_t c = t & ((1u << lp) - 1u), g = t >> lp, groups = kScanThreads >> lp;
+  const uint32_t tile0 = __ldg(a.row_tile + r), nt = __ldg(a.row_tile + r + 1) - tile0;
+  const uint32_t per = (nt + groups - 1) / groups;
+  const uint32_t lo = min(g * per, nt), hi = min(lo + per, nt);
+  const uint16_t* __restrict__ cnt = a.c2 + static_cast<size_t>(tile0) * a.pitch + c;
+  uint32_t sum = 0;
+  if (c < gx) {
+#pragma unroll 8
+    for (uint32_t i = lo; i < hi; ++i) sum += __ldg(cnt + static_cast<size_t>(i) * a.pitch);
+  }
+  s_sum[t] = sum;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+  for (uint32_t k = 0; k < groups; ++k) {
+    const uint32_t x = s_sum[(k << lp) + c];
+    if (k < g) before += x;
+    total += x;
+  }
+  // columns in order: the first 2^lp threads hold each column once
+  uint32_t incl = warp_incl_scan(t < (1u << lp) ? total : 0u);
+  if (lane_id() == 31) s_w[t >> 5] = incl;
+  __syncthreads();
+  const uint32_t cw = c >> 5;  // the warp that holds column c
+#pragma unroll
+  for (uint32_t w = 0; w < kMaxBins / 32; ++w)
+    if (w < cw && t < (1u << lp)) incl += s_w[w];
+  __syncthreads();
+  if (t < (1u << lp)) {
+    const uint32_t start = __ldg(a.row_pair + r) + incl - total;
+    s_sum[t] = start;
+    if (c < gx) {
+      const uint32_t pb = a.vt.pbeg[v];
+      a.ranges[(a.vt.one.on ? 0u : __ldg(a.vt.tile_begin + v)) + y * gx + c] =
+          total ? make_uint2(start - pb, start + total - pb) : make_uint2(0u, 0u);
+    }
+  }
+  __syncthreads();
+  uint32_t run = s_sum[c] + before;
+  if (c < gx) {
+    uint32_t* __restrict__ out = a.b2 + static_cast<size_t>(tile0) * a.pitch + c;
+#pragma unroll 8
+    for (uint32_t i = lo; i < hi; ++i) {
+      out[static_cast<size_t>(i) * a.pitch] = run;
+      run += __ldg(cnt + static_cast<size_t>(i) * a.pitch);
+    }
+  }
+}
+
+// ------------------------------------------------------------------- split
+// One tile of up to 1024 items at a time.  kLevel 1: items are depth
+// positions, bins the view's rows, the output segments; kLevel 2: items are
+// a row's segments, bins the columns, the output final pairs.  Steps:
+//   load     each lane its items' intervals and payloads; one warp the tile's
+//            counts and positions per bin (their prefix over the bins is
+//            where each bin's pairs start in the tile);
+//   masks    per warp and batch of 32 items, by the XOR scan;
+//   prefix   per bin over the batches, four threads per bin;
+//   expand   the batch's pairs, 32 at a time, staged as {bin, item} at their
+//            positions in bin order;
+//   flush    the staged pairs in bin order: runs of consecutive addresses.
+// A tile with more pairs than the stage holds takes windows of whole bins.
+template <int kWords>  // 32 kWords bins; each lane scans kWords consecutive ones
+struct Smem {
+  static constexpr int kBinsP = 32 * kWords;
+  static constexpr int kPitch = kBinsP + 1;  // odd: (batch, bin) lanes of the prefix step hit different banks
+  uint2 pay[kTile];
+  uint32_t stage[kStage];
+  uint32_t mask[kBatches][kPitch];
+  uint32_t lstart[kBinsP + 1];
+  uint32_t off[kBinsP];
+  uint16_t pos[kBatches][kPitch];
+};
+
+template <int kLevel, int kWords>
+__global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArgs a) {
+  using S = Smem<kWords>;
+  constexpr int kBinsP = S::kBinsP;
+  extern __shared__ __align__(16) unsigned char smem[];
+  S& s = *reinterpret_cast<S*>(smem);
+  begin_launch();
+  const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
+  if (__ldg(a.info + 1) == 0u) return;
+  const uint32_t ntiles = kLevel == 1 ? a.ntiles1 : __ldg(a.info);
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    uint32_t v, beg, cnt, bins, r = 0, tl = 0;
+    Place pl;
+    if constexpr (kLevel == 1) {
+      v = a.vt.nv == 1 ? 0u : warp_find(a.t1_begin, a.vt.nv, tile);
+      pl = place_of(a, v);
+      const ViewOf vw = view_of(a.vt, v);
+      tl = tile - pl.tile0;
+      beg = vw.rec0 + tl * kTile;
+      cnt = min(kTile, vw.nrec - tl * kTile);
+      bins = static_cast<uint32_t>(vw.geom.gy);
+    } else {
+      r = warp_find(a.row_tile, a.nrows, tile);
+      v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
+      pl = place_of(a, v);
+      beg = __ldg(a.row_seg + r) + (tile - __ldg(a.row_tile + r)) * kTile;
+      cnt = min(kTile, __ldg(a.row_seg + r + 1) - beg);
+      bins = static_cast<uint32_t>(view_of(a.vt, v).geom.gx);
+    }
+    // ---- load
+    uint32_t lo[kPerWarp], hi[kPerWarp];  // bins [lo, hi)
+#pragma unroll
+    for (int b = 0; b < kPerWarp; ++b) {
+      const uint32_t i = (warp * kPerWarp + b) * 32 + lane;
+      lo[b] = hi[b] = 0u;
+      if (i < cnt) {
+        if constexpr (kLevel == 1) {
+          const uint32_t q = __ldg(a.rects + beg + i);
+          lo[b] = (q >> 16) & 0xffu;
+          hi[b] = (q >> 24) + 1u;
+          if (hi[b] <= lo[b]) lo[b] = hi[b] = 0u;
+          s.pay[i] = make_uint2(beg + i, q & 0xffffu);
+        } else {
+          const uint2 q = __ldg(a.segs + beg + i);
+          lo[b] = q.y & 0xffu;
+          hi[b] = (q.y >> 8) + 1u;
+          s.pay[i] = __ldg(a.sdo + q.x);
+        }
+      }
+    }
+    if (warp == kWarps - 1) {
+      constexpr int kPer = kWords;
+      uint32_t c[kPer], base[kPer], sum = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const uint32_t b = lane * kPer + i;
+        c[i] = base[i] = 0u;
+        if (b < bins) {
+          if constexpr (kLevel == 1) {
+            const uint2 x = __ldg(a.c1 + pl.c10 + static_cast<size_t>(b) * pl.tiles + tl);
+            c[i] = x.x;
+            base[i] = x.y + __ldg(a.row_seg + pl.row0 + b);
+          } else {
+            c[i] = __ldg(a.c2 + static_cast<size_t>(tile) * a.pitch + b);
+            base[i] = __ldg(a.b2 + static_cast<size_t>(tile) * a.pitch + b);
+          }
+        }
+        sum += c[i];
+      }
+      uint32_t run = warp_incl_scan(sum) - sum;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const uint32_t b = lane * kPer + i;
+        s.lstart[b] = run;
+        s.off[b] = base[i] - run;
+        run += c[i];
+      }
+      if (lane == 31) s.lstart[kBinsP] = run;  // (all pairs; every bin past the last starts here too)
+    }
+    // ---- masks
+#pragma unroll
+    for (int b = 0; b < kPerWarp; ++b) {
+      uint32_t* m = s.mask[warp * kPerWarp + b];
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) m[k * 32 + lane] = 0u;
+      __syncwarp();
+      if (hi[b] > lo[b]) {
+        atomicXor(m + lo[b], 1u << lane);
+        if (hi[b] < bins) atomicXor(m + hi[b], 1u << lane);
+      }
+      __syncwarp();
+      uint32_t x[kWords], own = 0;  // inclusive over this lane's bins, then over the lanes before
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) {
+        own ^= m[lane * kWords + k];
+        x[k] = own;
+      }
+      uint32_t before = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, before, d);
+        if (lane >= static_cast<uint32_t>(d)) before ^= o;
+      }
+      before ^= own;
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) m[lane * kWords + k] = x[k] ^ before;
+    }
+    __syncthreads();
+    const uint32_t total = s.lstart[kBinsP];
+    for (uint32_t b0 = 0; b0 < bins;) {
+      // bins [b0, b1): the whole tile, or as many as the stage holds
+      uint32_t b1 = bins;
+      const uint32_t p0 = s.lstart[b0];
+      if (total - p0 > kStage) {
+        b1 = b0 + 1;
+        while (b1 < bins && s.lstart[b1 + 1] - p0 <= kStage) ++b1;
+      }
+      const uint32_t np = s.lstart[b1] - p0;
+      // ---- prefix over the batches
+      for (uint32_t cw = b0 + warp * 8; cw < b1; cw += kWarps * 8) {  // eight bins a warp, four lanes each
+        const uint32_t c = cw + (lane >> 2);
+        constexpr int kEach = kBatches / 4;
+        const uint32_t g = t & 3u, cc = min(c, b1 - 1u);
+        uint32_t x[kEach], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+          x[i] = __popc(s.mask[g * kEach + i][cc]);
+          sum += x[i];
+        }
+        uint32_t run = sum;
+#pragma unroll
+        for (int d = 1; d < 4; d <<= 1) {
+          const uint32_t o = __shfl_up_sync(0xffffffffu, run, d, 4);
+          if (g >= static_cast<uint32_t>(d)) run += o;
+        }
+        run += s.lstart[cc] - p0 - sum;
+        if (c < b1) {
+#pragma unroll
+          for (int i = 0; i < kEach; ++i) {
+            s.pos[g * kEach + i][c] = static_cast<uint16_t>(run);
+            run += x[i];
+          }
+        }
+      }
+      __syncthreads();
+      // ---- expand
+#pragma unroll
+      for (int b = 0; b < kPerWarp; ++b) {
+        const uint32_t bat = warp * kPerWarp + b;
+        const uint32_t* m = s.mask[bat];
+        const uint16_t* ps = s.pos[bat];
+        const uint32_t l = max(lo[b], b0), h = min(hi[b], b1);
+        const uint32_t n = h > l ? h - l : 0u;
+        const uint32_t item0 = bat * 32;
+        const uint32_t full = __ballot_sync(0xffffffffu, n != 0u);
+        if ((full & (full + 1u)) == 0u) {
+          // Lane p of a step takes the batch's p-th pair: its owner is the
+          // last item that starts at or before it.  The starts that fall into
+          // the step's 32 pairs are one word, and the items are in lane order.
+          const uint32_t end = warp_incl_scan(n), st = end - n;
+          const uint32_t np_b = __shfl_sync(0xffffffffu, end, 31);
+          const uint32_t shift = l - st;            // bin of pair p of this item, less p
+          uint32_t at = n ? st : 0x80000000u;       // start relative to the step (never 0..31 if none)
+          uint32_t seen = 0xffffffffu;              // items that start before the step, less one
+          for (uint32_t p = lane; p < np_b + lane; p += 32, at -= 32) {
+            const uint32_t starts = __reduce_or_sync(0xffffffffu, bit_or_none(at));
+            const uint32_t src = seen + __popc(starts & le);
+            seen += __popc(starts);
+            const uint32_t c = p + __shfl_sync(0xffffffffu, shift, src);
+            if (p < np_b) s.stage[ps[c] + __popc(m[c] & low_bits(src))] = c * 65536u + (item0 + src);
+          }
+        } else {  // a window left items without bins between others: each lane walks its own
+          const uint32_t steps = __reduce_max_sync(0xffffffffu, n);
+          for (uint32_t j = 0; j < steps; ++j) {
+            const uint32_t c = l + j;
+            if (j < n) s.stage[ps[c] + __popc(m[c] & lt)] = c * 65536u + (item0 + lane);
+          }
+        }
+      }
+      __syncthreads();
+      // ---- flush
+      if constexpr (kLevel == 1) {
+#pragma unroll 2
+        for (uint32_t p = t; p < np; p += kThreads) {
+          const uint32_t e = s.stage[p];
+          a.segs[s.off[e >> 16] + p0 + p] = s.pay[e & 0xffffu];
+        }
+      } else {
+        const uint32_t row_tile = (r - pl.row0) * bins;  // the row's first tile in its view
+#pragma unroll 2
+        for (uint32_t p = t; p < np; p += kThreads) {
+          const uint32_t e = s.stage[p], c = e >> 16;
+          const uint2 q = s.pay[e & 0xffffu];
+          const uint32_t dst = s.off[c] + p0 + p;
+          a.keys[dst] = (static_cast<uint64_t>(row_tile + c) << 32) | q.x;
+          a.values[dst] = q.y;
+        }
+      }
+      __syncthreads();
+      b0 = b1;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- host side
+struct Form {
+  const void* fn;
+  size_t smem;
+};
+template <int kLevel>
+Form split_form(uint32_t bins) {
+  // an odd number of words keeps the lanes' consecutive bins in different banks
+  if (bins <= 32) return {reinterpret_cast<const void*>(&k_split<kLevel, 1>), sizeof(Smem<1>)};
+  if (bins <= 64) return {reinterpret_cast<const void*>(&k_split<kLevel, 2>), sizeof(Smem<2>)};
+  if (bins <= 96) return {reinterpret_cast<const void*>(&k_split<kLevel, 3>), sizeof(Smem<3>)};
+  if (bins <= 160) return {reinterpret_cast<const void*>(&k_split<kLevel, 5>), sizeof(Smem<5>)};
+  if (bins <= 224) return {reinterpret_cast<const void*>(&k_split<kLevel, 7>), sizeof(Smem<7>)};
+  return {reinterpret_cast<const void*>(&k_split<kLevel, 9>), sizeof(Smem<9>)};
+}
+
+cudaError_t launch_after(const void* fn, uint32_t grid, int threads, size_t smem, const SplitArgs& a, cudaStream_t s) {
+  SplitArgs args = a;
+  void* params[] = {(void*)&args};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
+cudaError_t launch_split(int level, const SplitArgs& a, uint32_t bins, uint32_t tiles, int ctas_per_sm, cudaStream_t s) {
+  const Form f = level == 1 ? split_form<1>(bins) : split_form<2>(bins);
+  const radix::Kernel k{f.fn, 0, kThreads, 0, f.smem, 4};
+  const uint32_t resident = radix::resident_ctas(k, ctas_per_sm);
+  if (resident == 0) return cudaErrorInvalidConfiguration;
+  return launch_after(f.fn, tiles < resident ? tiles : resident, kThreads, f.smem, a, s);
+}
+
+}  // namespace split
+
+cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s) {
+  if (a.ntiles1 == 0) return cudaSuccess;
+  return split::launch_after(reinterpret_cast<const void*>(&split::k_row_count), a.ntiles1, split::kCountThreads, 0, a,
+                             s);
+}
+cudaError_t launch_row_scan(const SplitArgs& a, cudaStream_t s) {
+  return split::launch_after(reinterpret_cast<const void*>(&split::k_row_scan), a.nrows, split::kCountThreads, 0, a, s);
+}
+cudaError_t launch_row_split(const SplitArgs& a, uint32_t max_rows, int ctas_per_sm, cudaStream_t s) {
+  if (a.ntiles1 == 0) return cudaSuccess;
+  return split::launch_split(1, a, max_rows, a.ntiles1, ctas_per_sm, s);
+}
+cudaError_t launch_col_count(const SplitArgs& a, uint32_t max_tiles, cudaStream_t s) {
+  if (max_tiles == 0) return cudaSuccess;
+  const uint32_t cap = 152u * 8u;
+  return split::launch_after(reinterpret_cast<const void*>(&split::k_col_count), max_tiles < cap ? max_tiles : cap,
+                             split::kCountThreads, 0, a, s);
+}
+cudaError_t launch_col_scan(const SplitArgs& a, cudaStream_t s) {
+  return split::launch_after(reinterpret_cast<const void*>(&split::k_col_scan), a.nrows, split::kScanThreads, 0, a, s);
+}
+cudaError_t launch_col_split(const SplitArgs& a, uint32_t max_cols, uint32_t max_tiles, int ctas_per_sm,
+                             cudaStream_t s) {
+  if (max_tiles == 0) return cudaSuccess;
+  return split::launch_split(2, a, max_cols, max_tiles, ctas_per_sm, s);
+}
+
+}  // namespace tdgs

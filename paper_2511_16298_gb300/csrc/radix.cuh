@@ -564,7 +564,7 @@ __device__ __forceinline__ void rank_keys(uint32_t valid, const Smem<K>& sm, Til
   // sets of the group first (independent ballot chains), then every lane
   // of a set reads the warp's counter and the set's highest lane writes it
   // back bumped
-  constexpr int kGroup = sizeof(K) == 8 ? 4 : 8;
+  constexpr int kGroup = sizeof(K) == 8 || kItems < 8 ? 4 : 8;
   static_assert(kItems % kGroup == 0, "items per thread: a multiple of the ranking group");
   uint16_t* my_wh = sm.wh + warp * kBins;
   const uint32_t lt = lanemask_lt();

@@ -30,15 +30,22 @@ const radix::Kernel& stream_kernel(bool wide, bool expand, uint32_t bits) {
 
 uint32_t stream_kernel_bits(uint32_t width) { return width <= 6 ? 6u : (width <= 8 ? 8u : 12u); }
 
-DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm) {
+DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets) {
   DepthPlan p{};
   const uint32_t nn = n ? n : 1;
   const uint32_t g = depth_sort_grid();
-  if (g && nn <= depth_sort_count_capacity(g)) {
+  if (g && nn <= depth_sort_count_capacity(g, 16)) {
     p.resident = true;
+    // the smallest tile that takes the keys with one CTA per SM, and no more
+    // CTAs than it fills
+    p.items = 16;
+    if (!offsets) {
+      while (p.items > 4 && nn <= depth_sort_count_capacity(g, p.items / 2)) p.items /= 2;
+    }
     p.bits = 9;
     p.passes = 4;  // at most; the kernel runs as many as the key range needs
-    p.grid = g;
+    const uint32_t tile = depth_sort_count_capacity(1, p.items);
+    p.grid = offsets ? g : (nn + tile - 1) / tile;
     p.result = 1;
     p.scratch_words = 0;  // its state lives in a buffer of its own (depth_sort_scratch_words)
     return p;

@@ -156,15 +156,34 @@ cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t n
 
 // ---- depth-first frame path over a table of views (one view = one frame)
 constexpr uint32_t kMaxViews = 256;
+// A batch of one view whose table travels in the kernel parameters: the
+// device arrays other than vtot and pbeg are then not read.
+struct OneView {
+  const float4* g;
+  FrameGeom geom;
+  uint32_t n, on;
+};
 struct ViewTable {             // device arrays
   const float4* const* g;      // [nv] records of each view
   const uint32_t* rec_begin;   // [nv+1] global index of each view's first record
   const uint32_t* tile_begin;  // [nv+1] global id of each view's first tile
   const FrameGeom* geom;       // [nv]
-  uint64_t* vtot;              // [nv] pair count per view (accumulated, zeroed beforehand)
+  uint64_t* vtot;              // [nv] pair count per view (accumulated; zero between frames)
   uint32_t* pbeg;              // [nv+1] first pair of each view in the sorted list
   uint32_t nv;
+  OneView one;
 };
+
+// A view of the table as the kernels need it.
+struct ViewOf {
+  const float4* g;
+  FrameGeom geom;
+  uint32_t rec0, nrec;  // first record (over all views), records
+};
+__device__ __forceinline__ ViewOf view_of(const ViewTable& vt, uint32_t v) {
+  if (vt.one.on) return ViewOf{vt.one.g, vt.one.geom, 0u, vt.one.n};
+  return ViewOf{vt.g[v], vt.geom[v], vt.rec_begin[v], vt.rec_begin[v + 1] - vt.rec_begin[v]};
+}
 
 // Largest v with begin[v] <= i (begin ascending, begin[0] = 0).
 __device__ __forceinline__ uint32_t find_view(const uint32_t* begin, uint32_t nv, uint32_t i) {
@@ -253,19 +272,22 @@ struct DepthPlan {
   bool onesweep;          // the onesweep passes over compressed 32-bit keys
   int bits;
   uint32_t passes, grid;  // passes: the most that run; grid 0: the device query failed
+  int items;              // resident: keys per thread (4, 8 or 16)
   uint32_t result;        // which of the three buffer pairs holds the sorted keys and indices
   size_t scratch_words;
 };
-DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm);
+// offsets: the single launch also scans the tile counts in depth order.
+DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets);
 // Stable sort of m (u32 key, u32 value) pairs on the low key_bits bits with
 // the per-pass 11-bit kernel (launch_depth_pass); result in pair passes & 1.
 DepthPlan plan_key32_sort(uint32_t m, uint32_t key_bits, int ctas_per_sm);
 cudaError_t launch_depth_pass(const DepthPlan& dp, uint32_t pass, const uint32_t* kin, const uint32_t* vin,
                               uint32_t* kout, uint32_t* vout, uint32_t n, uint32_t* scratch, uint32_t* bar,
                               uint32_t* err, cudaStream_t s);
-// Single-launch depth sort (depth_sort.cu).  Grid: one CTA per SM (0 if
-// the device query failed); it takes n <= depth_sort_count_capacity(grid)
-// keys (one tile of 8192 per CTA), with or without the count step.
+// Single-launch depth sort (depth_sort.cu).  Grid: at most one CTA per SM
+// (depth_sort_grid(); 0 if the device query failed); it takes
+// n <= depth_sort_count_capacity(grid, items) keys (one tile of 512 x items
+// per CTA; 16 items with the offsets), with or without the count step.
 // Results: v1 = record indices in depth order, offsets = the exclusive scan
 // of the tile counts in that order (the pair offsets in depth order); k1
 // receives the counts in depth order, (k2, v2) are intermediate.  range:
@@ -282,6 +304,8 @@ cudaError_t launch_depth_pass(const DepthPlan& dp, uint32_t pass, const uint32_t
 //    receives only counts of 1023 or more.
 //  * Without (launch_depth_sort): key0 = the count kernel's depth keys,
 //    counts its tile counts, range[2..3] its range.
+//  * With offsets null the launch stops at v1: counts is not read, k1 holds
+//    intermediate keys.
 struct DepthSortArgs {
   const uint32_t* key0;
   ViewTable vt;
@@ -297,10 +321,10 @@ struct DepthSortArgs {
   uint32_t* err;
 };
 uint32_t depth_sort_grid();
-uint32_t depth_sort_count_capacity(uint32_t grid);
+uint32_t depth_sort_count_capacity(uint32_t grid, int items);
 size_t depth_sort_scratch_words(uint32_t grid);
-cudaError_t launch_depth_sort(uint32_t grid, const DepthSortArgs& a, cudaStream_t s);
-cudaError_t launch_count_depth_sort(uint32_t grid, const DepthSortArgs& a, cudaStream_t s);
+cudaError_t launch_depth_sort(uint32_t grid, int items, const DepthSortArgs& a, cudaStream_t s);
+cudaError_t launch_count_depth_sort(uint32_t grid, int items, const DepthSortArgs& a, cudaStream_t s);
 // Stable pass over the packed stream on tile bits [shift, shift + width).
 // expand: write the final (local tile << 32 | depth bits) keys and local
 // indices; with rmin/rmax, record each global tile's first/last sorted
@@ -330,6 +354,49 @@ uint32_t stream_grid(bool wide, bool expand, uint32_t bits, uint32_t m, int ctas
 size_t stream_scratch_words(bool wide, bool expand, uint32_t bits, uint32_t grid);
 cudaError_t launch_stream_pass(const StreamPass& sp, uint32_t* scratch, uint32_t* bar,
                                uint32_t* err, cudaStream_t s);
+
+// Duplication and tile sort as two stable splits of intervals
+// (interval_split.cu): Gaussians in depth order to tile rows, a row's
+// segments to tile columns.  For views of at most kSplitMaxBins rows and
+// columns whose depth order is view after view (positions rec_begin[v] ..
+// rec_begin[v + 1] hold view v).
+constexpr uint32_t kSplitTile = 1024;     // items per tile of either level
+constexpr uint32_t kSplitMaxBins = 256;   // rows and columns of a view at most (4096 pixels)
+struct SplitArgs {
+  ViewTable vt;
+  const uint32_t* t1_begin;   // [nv+1] first level-1 tile of each view
+  const uint32_t* row_begin;  // [nv+1] first row (over all views) of each view
+  const uint32_t* c1_begin;   // [nv+1] first entry of c1 of each view
+  const uint32_t* sorder;     // record indices in depth order
+  uint32_t* rects;            // by depth position: columns and rows of the rectangle, a byte each
+  uint2* sdo;                 // by depth position: {depth bits, index in the view}
+  uint2* c1;                  // [view][row][level-1 tile]: {items, first position in the row's list}
+  uint2* row_tot;             // [nrows] {segments, pairs}
+  uint32_t* row_seg;          // [nrows+1] first segment of each row
+  uint32_t* row_tile;         // [nrows+1] first level-2 tile of each row
+  uint32_t* row_pair;         // [nrows] first pair of each row
+  uint32_t* info;             // {level-2 tiles, 1 if the pairs fit}
+  uint2* segs;                // {depth position, first column | last column << 8}
+  uint16_t* c2;               // [level-2 tile][pitch] items per column
+  uint32_t* b2;               // [level-2 tile][pitch] first output position per column
+  uint32_t pitch;             // columns of the widest view, rounded up to 8
+  uint2* ranges;
+  uint64_t* keys;
+  uint32_t* values;
+  uint64_t cap;               // pairs that segs, keys and values hold
+  const uint64_t* total;      // the pair count
+  uint32_t* ticket;           // a zero word, left zero
+  uint32_t ntiles1, nrows;
+  uint32_t* err;
+};
+cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s);
+cudaError_t launch_row_scan(const SplitArgs& a, cudaStream_t s);
+// max_rows, max_cols: of any view; max_tiles: a bound on the level-2 tiles.
+cudaError_t launch_row_split(const SplitArgs& a, uint32_t max_rows, int ctas_per_sm, cudaStream_t s);
+cudaError_t launch_col_count(const SplitArgs& a, uint32_t max_tiles, cudaStream_t s);
+cudaError_t launch_col_scan(const SplitArgs& a, cudaStream_t s);
+cudaError_t launch_col_split(const SplitArgs& a, uint32_t max_cols, uint32_t max_tiles, int ctas_per_sm,
+                             cudaStream_t s);
 
 // ---------------------------------------------------------------- tuning
 // Knobs picked by the autotuner (0 / -1 = built-in choice).

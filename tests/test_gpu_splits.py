@@ -1,0 +1,110 @@
+"""Frames whose pairs come from the interval splits (rows, then columns), at
+the sizes where the launches change form: 32-item batches, 1024-item tiles,
+tile rows and columns per 32-bit word, tiles with more pairs than are staged
+at once, the depth sort's tile sizes and the image size above which the tile
+passes take over.  Every output equals the CPU oracle's bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2511_16298_gb300 import synth
+from paper_2511_16298_gb300 import tdgs as T
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2511_16298_gb300 import build
+    build.build()
+    c = T.Context(0)
+    yield c
+    c.close()
+
+
+def same(ctx, oracle, fr):
+    ref = oracle.sort_frame(fr.gaussians, fr.width, fr.height)
+    assert ref["status"] == 0
+    k, v, r, m = ctx.sort_frame(T.records_to_tensor(fr.gaussians, DEV), fr.width, fr.height)
+    ctx.sync()
+    assert m == ref["m"]
+    assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
+    assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
+    assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 1023, 1024, 1025, 2048, 2049, 4097, 70_001])
+def test_item_counts(ctx, oracle, n):
+    same(ctx, oracle, synth.frame_random(n, n, 333, 209, depth_ties=0.3))
+
+
+@pytest.mark.parametrize("cols,rows", [(1, 1), (1, 70), (32, 33), (33, 32), (64, 65), (65, 64), (96, 97), (97, 96),
+                                       (160, 161), (161, 160), (224, 225), (225, 224), (256, 3), (3, 256),
+                                       (256, 256), (257, 2), (2, 257)])
+def test_grid_sizes(ctx, oracle, cols, rows):
+    """Rows and columns on both sides of each compiled width, 256 (the most
+    that the splits take) and 257."""
+    same(ctx, oracle, synth.frame_random(cols * 1000 + rows, 5000, 16 * cols - 7, 16 * rows - 3, max_sigma=90.0))
+
+
+def covering(n, width, height, seed, small=0.0):
+    """Gaussians over the whole image (a share of them a few pixels wide)."""
+    rng = np.random.default_rng(seed)
+    r = np.full(n, 4 * max(width, height))
+    r[rng.random(n) < small] = 5
+    return synth.Frame(width, height, synth.records(rng.uniform(0, width, n), rng.uniform(0, height, n),
+                                                    rng.uniform(0.5, 4.0, n).round(1), r), "covering")
+
+
+@pytest.mark.parametrize("n,width,height,small", [(1100, 4096, 48, 0.0), (1500, 640, 360, 0.5), (1030, 16, 16, 0.0),
+                                                  (700, 48, 4096, 0.3)])
+def test_windows_of_bins(ctx, oracle, n, width, height, small):
+    """Tiles with several times the pairs that are staged at once: windows
+    of whole rows or columns, in which some items have no bins."""
+    same(ctx, oracle, covering(n, width, height, n, small))
+
+
+@pytest.mark.parametrize("per_sm", [2048, 4096])
+def test_depth_sort_tile_sizes(ctx, oracle, per_sm):
+    """Frames that just fill, and just overflow, one depth-sort tile of 4 or 8
+    keys per thread on every SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (sms * per_sm, sms * per_sm + 1):
+        same(ctx, oracle, synth.frame_scene(n, n=n, width=640, height=360))
+
+
+def test_no_pairs_and_culled(ctx, oracle):
+    fr = synth.frame_random(3, 3000, 500, 300)
+    fr.gaussians["radius"] = 0
+    same(ctx, oracle, fr)
+    fr.gaussians["radius"][1234] = 9
+    same(ctx, oracle, fr)
+
+
+def test_async_one_view_capacity_then_exact(ctx, oracle):
+    """One reserved view: more pairs than the capacity are reported and leave
+    the context usable; within it, a tile digit width set after the
+    reservation does not change the reserved path."""
+    fr = synth.frame_small(2)
+    ref = oracle.sort_frame(fr.gaussians, fr.width, fr.height)
+    g = T.records_to_tensor(fr.gaussians, DEV)
+    views = [(g, fr.width, fr.height)]
+    ctx.reserve_views(views, ref["m"] - 1)
+    ctx.sort_views_async(views)
+    with pytest.raises(T.TdgsError) as e:
+        ctx.views_results(1)
+    assert e.value.status == T.CAPACITY
+    ctx.reserve_views(views, ref["m"])
+    ctx.apply_tuning({"tile_digit_bits": 8})
+    try:
+        for _ in range(2):
+            ctx.sort_views_async(views)
+            (k, v, r, m), = ctx.views_results(1)
+            assert m == ref["m"]
+            assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
+            assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
+            assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
+    finally:
+        ctx.apply_tuning({"tile_digit_bits": 0})
+    same(ctx, oracle, fr)
