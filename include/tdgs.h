@@ -133,7 +133,7 @@ tdgs_status tdgs_context_set_sort_variant(tdgs_context* ctx, int variant);
  *   TDGS_TUNE_SORT_VARIANT     pass kernel of tdgs_sort_pairs (as above)
  *   TDGS_TUNE_TILE_DIGIT_BITS  widest digit (4..12) of the frame's passes
  *                              over the tile bits (built-in: no such passes
- *                              for one view of at most 4096 x 4096 pixels,
+ *                              for views of at most 4096 x 4096 pixels,
  *                              whose pairs come from two interval splits;
  *                              8 otherwise)
  *   TDGS_TUNE_CTAS_PER_SM      CTAs per SM of the persistent radix grids

@@ -86,6 +86,7 @@ struct ViewBlob {
   uint32_t t1_begin[kMaxViews + 1];
   uint32_t row_begin[kMaxViews + 1];
   uint32_t c1_begin[kMaxViews + 1];
+  uint32_t n[512];  // records of each view, then zeros (the digit counts of a pass by view)
 };
 
 struct PendingTime {
@@ -710,6 +711,7 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
     h->tile_begin[v] = static_cast<uint32_t>(t_all);
     h->nt[v] = tdgs_num_tiles(w.f);
     h->vtot[v] = 0;
+    h->n[v] = w.n;
     n_all += w.n;
     t_all += h->nt[v];
     const uint32_t gx = static_cast<uint32_t>(h->geom[v].gx), gy = static_cast<uint32_t>(h->geom[v].gy);
@@ -725,6 +727,7 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
   }
   if (n_all > 0xffffffffull || t_all > 0xffffffffull)
     return fail(ctx, TDGS_ERR_OVERFLOW, "too many Gaussians or tiles in one batch");
+  std::memset(h->n + nv, 0, sizeof(h->n) - nv * sizeof(h->n[0]));
   h->rec_begin[nv] = static_cast<uint32_t>(n_all);
   h->tile_begin[nv] = static_cast<uint32_t>(t_all);
   h->t1_begin[nv] = static_cast<uint32_t>(t1);
@@ -758,11 +761,12 @@ ViewTable device_table(tdgs_context* ctx) {
   return vt;
 }
 
-// Whether the staged views' pairs come from the interval splits: one view,
-// images up to 4096 pixels a side; a tuned tile digit width asks for the
+// Whether the staged views' pairs come from the interval splits: images up to
+// 4096 pixels a side, and several views only up to the Gaussians that the
+// depth sort orders view after view; a tuned tile digit width asks for the
 // tile passes.
 bool splits(const tdgs_context* ctx) {
-  return ctx->nv == 1 && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
+  return (ctx->nv == 1 || ctx->n_all < (1u << 30)) && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
          ctx->tuning.tile_digit_bits == 0;
 }
 
@@ -771,8 +775,12 @@ uint32_t split_rows(const tdgs_context* ctx) { return ctx->h_views->row_begin[ct
 // Level-2 tiles of at most m segments: full ones, and one ragged one per row.
 uint64_t split_tiles(const tdgs_context* ctx, uint64_t m) { return m / kSplitTile + split_rows(ctx); }
 
+// Whether the depth sort orders a batch view after view.
+bool by_view(const tdgs_context* ctx) { return ctx->split && ctx->nv > 1; }
+
 DepthPlan depth_plan(const tdgs_context* ctx) {
-  return plan_depth_sort(ctx->n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm, !ctx->split);
+  return plan_depth_sort(ctx->n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm, !ctx->split,
+                         by_view(ctx));
 }
 
 struct Shape {
@@ -833,7 +841,7 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   }
   if (st == TDGS_OK && dp.onesweep) {
     grown = false;
-    st = ensure(ctx, ctx->f_dos, onesweep_scratch_words(n_all ? n_all : 1) * 4, s, &grown);
+    st = ensure(ctx, ctx->f_dos, onesweep_scratch_words(n_all ? n_all : 1, by_view(ctx)) * 4, s, &grown);
     if (st == TDGS_OK && (grown || ctx->dos_dirty)) {
       TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_dos.p, 0, onesweep_header_words() * 4, s));
       ctx->dos_dirty = false;
@@ -933,10 +941,11 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
     if (n_all) {
       uint32_t* dos = static_cast<uint32_t*>(ctx->f_dos.p);
       TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                  launch_depth_onesweep_hist(dk[0], n_all, ctx->d_range, dos, err_word(ctx), s));
+                  launch_depth_onesweep_hist(dk[0], n_all, ctx->d_range, by_view(ctx), dos, err_word(ctx), s));
       for (uint32_t p = 0; p < dpasses; ++p)
         TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                    launch_depth_onesweep_pass(p, dk, dv, n_all, ctx->d_range, dos, err_word(ctx), s));
+                    launch_depth_onesweep_pass(p, dk, dv, n_all, ctx->d_range, by_view(ctx) ? ctx->nv : 0u,
+                                               ctx->d_views->rec_begin, ctx->d_views->n, dos, err_word(ctx), s));
     }
   } else {
     for (uint32_t p = 0; p < dpasses; ++p) {

@@ -32,6 +32,8 @@
 //    half of the rows, and it waits for those rows only, not for a barrier.
 //  * One grid barrier ends each pass: the next pass reads what every CTA
 //    wrote.
+// A batch of views whose order is to be view after view takes one more pass
+// by view: the last depth pass writes each record's view in place of its key.
 // The value that travels with a key is the record index (22 bits) with the
 // Gaussian's tile count in the top 10 bits (1023: at least that many, the
 // count is read again at the end), made in pass 0.  The last pass writes
@@ -64,7 +66,8 @@ namespace depth {
 constexpr int kThreads = 512, kBits = 9;
 constexpr uint32_t kBins = 1u << kBits;
 constexpr uint32_t kWarps = kThreads / 32;
-constexpr uint32_t kMaxPasses = 4;  // 32 key bits in digits of at most 9
+constexpr uint32_t kMaxDepthPasses = 4;  // 32 key bits in digits of at most 9
+constexpr uint32_t kMaxPasses = kMaxDepthPasses + 1;  // and one by view
 constexpr uint32_t kMaxGrid = radix::kMaxGrid;  // chunks (CTAs) at most
 constexpr uint32_t kValueBits = 22; // record indices below 2^22 (N <= kMaxGrid * 8192)
 constexpr uint32_t kRecMask = (1u << kValueBits) - 1u;
@@ -91,7 +94,7 @@ constexpr uint32_t kFinalSlot = kSlots - 1;         // before the offsets
 constexpr uint32_t kHistWord = kSlots * kLine;      // [kMaxPasses][kBins] digit totals
 constexpr uint32_t kRawWord = kHistWord + kMaxPasses * kBins;  // fused count: [kBins] keys by low 9 bits, culled
 constexpr uint32_t kSumWord = kRawWord + kBins + kLine;          // [kMaxGrid] counts per output chunk
-constexpr uint32_t kRowWord = kSumWord + kMaxGrid;             // [kMaxPasses][G][kBins / 2] rows
+constexpr uint32_t kRowWord = kSumWord + kMaxGrid;             // [passes][G][kBins / 2] rows
 constexpr uint32_t kRowWords = kBins / 2;
 constexpr uint32_t kRowGroups = kThreads / (kBins / 8);        // rows read in parallel (8)
 constexpr uint32_t kRowBatch = 10;                             // rows per thread in flight
@@ -217,7 +220,7 @@ __device__ __forceinline__ void sum_rows(const uint32_t* __restrict__ rows, uint
 // Values come from vstage (items below nstaged) or vsrc + tb;
 // pass 0 (first) makes each value the record index with the tile count in
 // its top bits.  The last pass writes v1 (record index) and k1 (count) and
-// adds the counts it writes into the per-output-chunk sums csum (chunks of
+// (with kOffsets) adds the counts it writes into the per-output-chunk sums csum (chunks of
 // Sz positions; vstage is free by then and holds per-warp sums).  Returns
 // false if a destination fell outside [0, n).  Ends with a block barrier.
 template <bool kOffsets, int kItems>
@@ -229,7 +232,8 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
                                                  uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                  uint32_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                  const uint32_t* __restrict__ counts, uint32_t Sz, uint32_t G,
-                                                 uint32_t* __restrict__ csum) {
+                                                 uint32_t* __restrict__ csum,
+                                                 const uint32_t* s_begin = nullptr, uint32_t nv = 0) {
   using S = ShapeOf<kItems>;
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   bool ok = true;
@@ -267,7 +271,12 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
         const uint32_t key = static_cast<uint32_t>(x >> 32);
         const uint32_t dst = sm.off[(key >> sh) & mask] + xp;
         if (dst < n) {
-          if (kOffsets || !last) kout[dst] = key;
+          if (kOffsets || !last) {
+            uint32_t out = key;
+            if constexpr (!kOffsets)
+              if (nv) out = find_view(s_begin, nv, static_cast<uint32_t>(x));
+            kout[dst] = out;
+          }
           vout[dst] = static_cast<uint32_t>(x);
         } else {
           ok = false;
@@ -473,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   // the row sums of the groups share the exchange buffers (not live then)
   uint32_t* s_part = sm.xk;
   static_assert(S::kXkBytes + S::kXvBytes >= kRowGroups * kBins * 4, "row-sum partials fit the exchange");
-  __shared__ uint32_t s_hx[kMaxPasses - 1][kBins];  // pass 0: this chunk's counts of the later digits
+  __shared__ uint32_t s_hx[kMaxDepthPasses - 1][kBins];  // pass 0: this chunk's counts of the later digits
   __shared__ uint2 s_warp2[kWarps];
   __shared__ unsigned long long s_sum[kWarps + 1];
   __shared__ unsigned long long s_base;
@@ -487,7 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   {
     uint4* z = reinterpret_cast<uint4*>(sm.wh);
     for (uint32_t i = t; i < S::kWhBytes / 16; i += kThreads) z[i] = make_uint4(0, 0, 0, 0);
-    for (uint32_t i = t; i < (kMaxPasses - 1) * kBins; i += kThreads) (&s_hx[0][0])[i] = 0u;
+    for (uint32_t i = t; i < (kMaxDepthPasses - 1) * kBins; i += kThreads) (&s_hx[0][0])[i] = 0u;
   }
   uint32_t* hist = scratch + kHistWord;
   uint32_t* csum = scratch + kSumWord;
@@ -496,12 +505,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   radix::TileRegs<uint32_t, false, kItems> R;
   __shared__ uint32_t s_h0[kCount ? kBins : 1];  // fused count: pass 0's digit totals
   uint32_t lo, hi;
+  // several views in view order: one more pass, by view
+  __shared__ uint32_t s_begin[kMaxViews + 1];
+  const uint32_t by_view = !kOffsets && A.vt.nv > 1 ? A.vt.nv : 0u;
+  if constexpr (!kCount && !kOffsets)
+    if (by_view)
+      for (uint32_t v = t; v <= by_view; v += kThreads) s_begin[v] = A.vt.rec_begin[v];
   if constexpr (kCount) {
     // ---- the tile count step (Sec. II-A): per record its tile count and
     // depth key (raw depth bits; all ones without pairs), kept in R.k and,
     // for the counts, in the staging buffer; per view its pair total; the
     // smallest / largest key with pairs; the keys' low 9 bits counted
-    __shared__ uint32_t s_begin[kMaxViews + 1];
     __shared__ const float4* s_g[kMaxViews];
     __shared__ FrameGeom s_geom[kMaxViews];
     __shared__ unsigned long long s_tot[kMaxViews];
@@ -655,15 +669,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   __syncthreads();
   const uint32_t g = t / (kBins / 8), q = t % (kBins / 8);  // row group, column of 8 bins
   const bool low_half = c < G / 2;
-  for (uint32_t p = 0; p < passes; ++p) {
-    const bool last = p + 1 == passes;
+  const uint32_t all_passes = passes + (by_view ? 1u : 0u);
+  for (uint32_t p = 0; p < all_passes; ++p) {
+    const bool last = p + 1 == all_passes;
+    const bool view_pass = p == passes, to_view = by_view && p + 1 == passes;
     // pass p reads pair (p - 1) and writes pair p; the last pass writes (k1, v1)
-    const bool to_one = ((passes - 1 - p) & 1u) == 0;
+    const bool to_one = ((all_passes - 1 - p) & 1u) == 0;
     const uint32_t* kin = p == 0 ? key0 : (to_one ? k2 : k1);
     const uint32_t* vin = to_one ? v2 : v1;
     uint32_t* kout = to_one ? k1 : k2;
     uint32_t* vout = to_one ? v1 : v2;
-    a.shift = p * width;
+    a.shift = view_pass ? 0u : p * width;
+    a.mask = view_pass ? kBins - 1u : mask;  // (at most 256 views)
     const uint32_t* vsrc = p == 0 ? counts : vin;
     const bool counted = kCount && p == 0;  // keys in registers, values (the counts) already staged
     const bool unstaged = counted || (!kOffsets && p == 0);  // no values to copy in
@@ -696,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
         }
       }
 #pragma unroll
-      for (int j = 0; j < kItems; ++j) R.d[j] = (R.k[j] >> a.shift) & mask;
+      for (int j = 0; j < kItems; ++j) R.d[j] = (R.k[j] >> a.shift) & a.mask;
       radix::rank_keys<false, S, uint32_t, false, kBits, kItems>(valid, sm, R);
     }
     // publish this chunk's digit counts (lstart) as its row (count + 1)
@@ -729,7 +746,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     // output base per digit: keys of smaller digits + this digit's keys in
     // the chunks before this one
     {
-      const uint32_t tot = (kCount && p == 0) ? s_h0[t] : __ldcg(hist + p * kBins + t);
+      uint32_t tot;
+      if (view_pass)
+        tot = t < by_view ? s_begin[t + 1] - s_begin[t] : 0u;
+      else
+        tot = (kCount && p == 0) ? s_h0[t] : __ldcg(hist + p * kBins + t);
       const uint32_t own = sm.lstart[t];
       uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       sum_rows(rows + static_cast<size_t>(p) * G * kRowWords, low_half ? 0u : c + 1, low_half ? c : G, g, q,
@@ -761,8 +782,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     uint32_t hk[kItems];  // exchanged with each value: the key, in the last pass its digit
 #pragma unroll
     for (int j = 0; j < kItems; ++j) hk[j] = last ? R.d[j] : R.k[j];
-    ok &= exchange_scatter<kOffsets, kItems>(sm, vstage, hk, R.r, valid, beg, nstaged, vsrc, p == 0, last, a.shift, mask, n, kout,
-                           vout, k1, v1, counts, Sz, G, csum);
+    ok &= exchange_scatter<kOffsets, kItems>(sm, vstage, hk, R.r, valid, beg, nstaged, vsrc, p == 0, last, a.shift, a.mask, n, kout,
+                           vout, k1, v1, counts, Sz, G, csum, s_begin, to_view ? by_view : 0u);
     arrive_and_wait(scratch + (last ? kFinalSlot : 1 + p) * kLine, G, err);
   }
   if (!ok) latch_error(err, TDGS_ERR_CAPACITY, kSiteRadixRange);
@@ -779,7 +800,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   // Reset for the next launch (every reader of these is past the final
   // barrier): this chunk's rows; CTA 0 the totals, the histogram of the
   // count step, the key range and the mid-launch counters.
-  for (uint32_t i = t; i < passes * (kRowWords / 4); i += kThreads) {
+  for (uint32_t i = t; i < all_passes * (kRowWords / 4); i += kThreads) {
     const uint32_t pp = i / (kRowWords / 4), w = i % (kRowWords / 4);
     reinterpret_cast<uint4*>(rows + (static_cast<size_t>(pp) * G + c) * kRowWords)[w] = make_uint4(0, 0, 0, 0);
   }
@@ -793,7 +814,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
         range[1] = 0u;
       }
     }
-    if (t < passes) scratch[t * kLine] = 0u;  // slots 0 .. passes-1
+    if (t < all_passes) scratch[t * kLine] = 0u;  // slots 0 .. all_passes-1
   }
 }
 

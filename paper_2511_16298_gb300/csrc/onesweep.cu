@@ -135,6 +135,7 @@ struct HistArgs {
   uint32_t* done;      // block counter, zero on entry, left zero
   uint32_t* tickets;   // [kMaxPasses] tile tickets, cleared here
   uint32_t* status0;   // [ntiles][kBins] look-back status of pass 0, cleared here
+  uint32_t* status_view;  // the same of a last pass by view, or null
   uint32_t* range;     // depth keys: the key range (range[2..3]); the pass count goes to range[4]
   uint32_t* err;
 };
@@ -155,6 +156,12 @@ struct PassArgs {
   const uint32_t* range;
   uint32_t* dk[3];
   uint32_t* dv[3];
+  // a batch to be ordered view after view: its views (0: none) and their
+  // first records; the last depth pass writes each record's view as its key,
+  // and one more pass (view_pass) sorts by it from buffer 1 to buffer 2
+  uint32_t nv;
+  const uint32_t* rec_begin;
+  uint32_t view_pass;
   uint32_t* err;
 };
 
@@ -187,6 +194,10 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMod
     for (size_t i = static_cast<size_t>(blockIdx.x) * kHistThreads + t; i < nz;
          i += static_cast<size_t>(gridDim.x) * kHistThreads)
       z[i] = make_uint4(0, 0, 0, 0);
+    if (uint4* zv = reinterpret_cast<uint4*>(a.status_view))
+      for (size_t i = static_cast<size_t>(blockIdx.x) * kHistThreads + t; i < nz;
+           i += static_cast<size_t>(gridDim.x) * kHistThreads)
+        zv[i] = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
   const uint32_t m = a.m;
@@ -338,6 +349,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t s_tile[2];
   __shared__ uint32_t s_warp[kWarps];
+  __shared__ uint32_t s_begin[kMode == kDigitDepth ? kMaxViews + 1 : 1];
+  bool to_view = false;  // the last depth pass of a batch in view order
 
   Digit dg = a.dg, dgn = a.dgn;
   uint32_t* hist_next = a.hist_next;
@@ -347,16 +360,24 @@ __global__ void __launch_bounds__(kThreads, 2)
     // every CTA (scan CTAs included); the buffers alternate so that the
     // last pass that runs writes buffer 1.
     const DepthDigits dd = depth_digits(a.range);
-    if (a.pass >= dd.passes) return;
-    dg = Digit{kDigitDepth, a.pass * dd.width, 0u, dd.mask, dd.lo, dd.cull};
-    dgn = dg;
-    dgn.msh += dd.width;
-    if (a.pass + 1 >= dd.passes) {
-      hist_next = nullptr;
-      status_next = nullptr;
+    uint32_t in = 1u, out = 2u;
+    if (a.view_pass) {
+      dg = Digit{kDigitDepth, 0u, 0u, kBins - 1u, 0u, 0u};  // keys are views
+    } else {
+      if (a.pass >= dd.passes) return;
+      dg = Digit{kDigitDepth, a.pass * dd.width, 0u, dd.mask, dd.lo, dd.cull};
+      dgn = dg;
+      dgn.msh += dd.width;
+      if (a.pass + 1 >= dd.passes) {
+        hist_next = nullptr;
+        status_next = nullptr;
+        to_view = a.nv != 0;
+      }
+      out = ((dd.passes - 1 - a.pass) & 1u) ? 2u : 1u;
+      in = a.pass == 0 ? 0u : (((dd.passes - a.pass) & 1u) ? 2u : 1u);
     }
-    const uint32_t out = ((dd.passes - 1 - a.pass) & 1u) ? 2u : 1u;
-    const uint32_t in = a.pass == 0 ? 0u : (((dd.passes - a.pass) & 1u) ? 2u : 1u);
+    if (to_view)
+      for (uint32_t v = threadIdx.x; v <= a.nv; v += kThreads) s_begin[v] = __ldg(a.rec_begin + v);
     kin = a.dk[in];
     vin = a.dv[in];
     kout = a.dk[out];
@@ -521,7 +542,10 @@ __global__ void __launch_bounds__(kThreads, 2)
           const K key = pb.k[p];
           const uint32_t dst = off[slot<kSwz>(digit_m<kMode>(key, dg))] + p;
           if (dst < m) {
-            kout[dst] = key;
+            K out = key;
+            if constexpr (kMode == kDigitDepth)
+              if (to_view) out = find_view(s_begin, a.nv, pb.v[p]);
+            kout[dst] = out;
             vout[dst] = pb.v[p];
           } else {
             ok = false;
@@ -599,6 +623,10 @@ void scratch_layout(onesweep::HistArgs& a, uint32_t* scratch) {
   a.done = scratch + 2 * kMaxPasses * kBins;
   a.tickets = a.done + 4;
   a.status0 = scratch + onesweep_header_words();
+}
+// Status rows of a pass by view, after those of the two digit passes.
+uint32_t* view_status(uint32_t* scratch, uint32_t ntiles) {
+  return scratch + onesweep_header_words() + 2 * static_cast<size_t>(ntiles) * onesweep::kBins;
 }
 void pass_layout(onesweep::PassArgs& a, uint32_t pass, bool has_next, uint32_t* scratch) {
   using namespace onesweep;
@@ -692,9 +720,9 @@ bool onesweep_eligible(uint32_t m, const void* keys, const void* values, const v
   return m > 0 && m < onesweep::kMaxPairs && a16(keys) && a16(values) && a16(keys_alt) && a16(values_alt);
 }
 
-size_t onesweep_scratch_words(uint32_t m) {
+size_t onesweep_scratch_words(uint32_t m, bool by_view) {
   const size_t ntiles = (static_cast<size_t>(m) + onesweep::kTileKeys - 1) / onesweep::kTileKeys;
-  return onesweep_header_words() + 2 * ntiles * onesweep::kBins;
+  return onesweep_header_words() + (by_view ? 3 : 2) * ntiles * onesweep::kBins;
 }
 
 size_t onesweep_header_words() {
@@ -740,8 +768,8 @@ cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint
   return launch_pass(fn, false, kin, vin, kout, vout, a, s);
 }
 
-cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, uint32_t* scratch,
-                                       uint32_t* err, cudaStream_t s) {
+cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, bool by_view,
+                                       uint32_t* scratch, uint32_t* err, cudaStream_t s) {
   using namespace onesweep;
   HistArgs a{};
   a.m = n;
@@ -749,6 +777,7 @@ cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_
   a.ntiles = (n + kTileKeys - 1) / kTileKeys;
   a.range = range;
   scratch_layout(a, scratch);
+  if (by_view) a.status_view = view_status(scratch, a.ntiles);
   a.err = err;
   const uint32_t grid = hist_grid(n);
   if (grid == 0) return cudaErrorInvalidDevice;
@@ -757,15 +786,24 @@ cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_
 }
 
 cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uint32_t* const dv[3], uint32_t n,
-                                       const uint32_t* range, uint32_t* scratch, uint32_t* err, cudaStream_t s) {
+                                       const uint32_t* range, uint32_t nv, const uint32_t* rec_begin,
+                                       const uint32_t* view_counts, uint32_t* scratch, uint32_t* err,
+                                       cudaStream_t s) {
   using namespace onesweep;
-  if (pass >= kDepthOnesweepPasses) return cudaErrorInvalidValue;
+  if (pass > kDepthOnesweepPasses || (pass == kDepthOnesweepPasses && !nv)) return cudaErrorInvalidValue;
   PassArgs a{};
   a.m = n;
   a.ntiles = (n + kTileKeys - 1) / kTileKeys;
+  a.nv = nv;
+  a.rec_begin = rec_begin;
   // the device drops the next pass's counts and status when this pass is
   // the last that the key range needs
   pass_layout(a, pass, pass + 1 < kDepthOnesweepPasses, scratch);
+  if (pass == kDepthOnesweepPasses) {  // by view: the digit counts are the views' sizes
+    a.view_pass = 1u;
+    a.hist = view_counts;
+    a.status = view_status(scratch, a.ntiles);
+  }
   a.pass = pass;
   a.range = range;
   for (int i = 0; i < 3; ++i) {

@@ -30,7 +30,7 @@ const radix::Kernel& stream_kernel(bool wide, bool expand, uint32_t bits) {
 
 uint32_t stream_kernel_bits(uint32_t width) { return width <= 6 ? 6u : (width <= 8 ? 8u : 12u); }
 
-DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets) {
+DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets, bool by_view) {
   DepthPlan p{};
   const uint32_t nn = n ? n : 1;
   const uint32_t g = depth_sort_grid();
@@ -54,9 +54,10 @@ DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offs
   if (g && nn < (1u << 30)) {
     p.onesweep = true;
     p.bits = 9;
-    p.passes = kDepthOnesweepPasses;  // launches; the device runs as many as the key range needs
+    // launches: the device runs as many as the key range needs, and the one by view
+    p.passes = kDepthOnesweepPasses + (by_view ? 1 : 0);
     p.grid = g;
-    p.result = 1;
+    p.result = by_view ? 2 : 1;
     p.scratch_words = 0;  // its scratch is a buffer of its own (onesweep_scratch_words)
     return p;
   }

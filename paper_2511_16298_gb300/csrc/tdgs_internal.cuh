@@ -276,8 +276,9 @@ struct DepthPlan {
   uint32_t result;        // which of the three buffer pairs holds the sorted keys and indices
   size_t scratch_words;
 };
-// offsets: the single launch also scans the tile counts in depth order.
-DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets);
+// offsets: the single launch also scans the tile counts in depth order;
+// by_view: several views, ordered view after view (not with offsets).
+DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offsets, bool by_view);
 // Stable sort of m (u32 key, u32 value) pairs on the low key_bits bits with
 // the per-pass 11-bit kernel (launch_depth_pass); result in pair passes & 1.
 DepthPlan plan_key32_sort(uint32_t m, uint32_t key_bits, int ctas_per_sm);
@@ -305,7 +306,8 @@ cudaError_t launch_depth_pass(const DepthPlan& dp, uint32_t pass, const uint32_t
 //  * Without (launch_depth_sort): key0 = the count kernel's depth keys,
 //    counts its tile counts, range[2..3] its range.
 //  * With offsets null the launch stops at v1: counts is not read, k1 holds
-//    intermediate keys.
+//    intermediate keys, and several views are ordered view after view (by
+//    depth inside each).
 struct DepthSortArgs {
   const uint32_t* key0;
   ViewTable vt;
@@ -451,7 +453,7 @@ cudaError_t launch_radix_pass(const SortPlan& plan, uint32_t pass, const uint64_
 // them zero).  Passes ping-pong between (keys, values) and the alternates.
 bool onesweep_eligible(uint32_t m, const void* keys, const void* values, const void* keys_alt,
                        const void* values_alt);
-size_t onesweep_scratch_words(uint32_t m);
+size_t onesweep_scratch_words(uint32_t m, bool by_view = false);
 size_t onesweep_header_words();
 uint32_t onesweep_tile_keys();
 cudaError_t launch_onesweep_hist(const SortPlan& plan, const uint64_t* keys, uint32_t m, uint32_t* scratch,
@@ -468,9 +470,15 @@ cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint
 // (dk[2], dv[2] hold intermediate passes).  Scratch as above for m = n,
 // separate from any other sort's while both may be in use.
 constexpr uint32_t kDepthOnesweepPasses = 4;  // 32 bits in 9-bit digits
-cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, uint32_t* scratch,
-                                       uint32_t* err, cudaStream_t s);
+// To order a batch view after view (nv > 0; 0 otherwise): pass
+// kDepthOnesweepPasses sorts by view at the end (rec_begin: [nv+1] first
+// record of each view; view_counts: 512 words, the views' records and zeros),
+// the scratch is sized with by_view, and the result is in dk[2], dv[2].
+cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, bool by_view,
+                                       uint32_t* scratch, uint32_t* err, cudaStream_t s);
 cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uint32_t* const dv[3], uint32_t n,
-                                       const uint32_t* range, uint32_t* scratch, uint32_t* err, cudaStream_t s);
+                                       const uint32_t* range, uint32_t nv, const uint32_t* rec_begin,
+                                       const uint32_t* view_counts, uint32_t* scratch, uint32_t* err,
+                                       cudaStream_t s);
 
 }  // namespace tdgs

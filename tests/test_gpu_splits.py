@@ -108,3 +108,34 @@ def test_async_one_view_capacity_then_exact(ctx, oracle):
     finally:
         ctx.apply_tuning({"tile_digit_bits": 0})
     same(ctx, oracle, fr)
+
+
+def depths(kind, n, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "equal":
+        return np.full(n, 2.5)
+    if kind == "narrow":
+        return rng.uniform(1.0, 1.0001, n)
+    return np.exp(rng.uniform(np.log(1e-37), np.log(1e37), n))
+
+
+@pytest.mark.parametrize("kind", ["equal", "narrow", "wide"])
+@pytest.mark.parametrize("sizes", [(700, 0, 1, 2500), (1030, 5000, 40_000), (650_000, 3, 700_000)])
+def test_batches_in_view_order(ctx, oracle, kind, sizes):
+    """Batches whose depth keys need one to four digit passes, then the pass
+    by view: the single launch at two tile sizes and the onesweep passes,
+    with empty and tiny views among the others."""
+    frames = []
+    for i, n in enumerate(sizes):
+        f = synth.frame_random(40 + i, n, 300 + 50 * i, 200, max_sigma=8.0) if n else synth.Frame(
+            64, 64, synth.records([], [], [], []), "empty")
+        if n:
+            f.gaussians["depth"] = depths(kind, n, i).astype(np.float32)
+        frames.append(f)
+    res = ctx.sort_views([(T.records_to_tensor(f.gaussians, DEV), f.width, f.height) for f in frames])
+    for f, (k, v, r, m) in zip(frames, res):
+        ref = oracle.sort_frame(f.gaussians, f.width, f.height)
+        assert ref["status"] == 0 and m == ref["m"]
+        assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
+        assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
