@@ -1,15 +1,14 @@
 // Rendering (Sec. II-A "Rendering"; Sec. IV-C "Efficient Tile-Based
 // Rendering"): one thread block per 16x16 tile blends the tile's sorted
-// Gaussians front to back into every pixel.  Each thread owns kPix pixels
-// of one column (rows t / 16 + kRowStep * k) and the three colour channels
-// are unrolled.  The paper gives each thread four pixels so one Gaussian
-// fetch serves four SIMD lanes; on this GPU one pixel per thread (256
-// threads per tile) measured fastest -- 0.44 / 0.36 / 0.34 ms for 4 / 2 / 1
-// pixels per thread on the 1280x720 frame of the 500k scene -- because
-// tiles with many Gaussians set the kernel's end and more threads per tile
-// finish them sooner; kPix stays a compile-time choice.
+// Gaussians front to back into every pixel, one pixel per thread, with the
+// three colour channels unrolled.  The paper gives each thread four pixels so
+// one Gaussian fetch serves four SIMD lanes; on this GPU one pixel per thread
+// (256 threads per tile) measured fastest -- 0.44 / 0.36 / 0.34 ms for 4 / 2 /
+// 1 pixels per thread on the 1280x720 frame of the 500k scene -- because tiles
+// with many Gaussians set the kernel's end and more threads per tile finish
+// them sooner.
 //
-// Further measures on that frame (0.32 -> 0.21 ms together):
+// Further measures:
 //  * tiles run heaviest first when they take more than one wave of
 //    resident blocks.  A one-block kernel buckets the tiles by their
 //    Gaussian count (64 buckets, descending) and block b renders the b-th
@@ -25,17 +24,21 @@
 //    pixels per thread measured 243-265 us).  A finished pixel keeps
 //    testing its flag each step: letting it run on with T = 0 instead made
 //    whole finished warps do every step's arithmetic (361 against 241 us).
-//  * row culling per warp: a Gaussian reaches a pixel only inside the
-//    ellipse where power >= cut, so when it is staged, its thread marks
-//    the warps (row pairs of the tile) the ellipse can reach, with a
-//    margin; each warp then blends only the list of staged Gaussians that
-//    reach it, kept in front-to-back order by one ballot per 32.  What a
-//    warp skips is what its pixels' own cut test would have skipped, so
-//    the image is unchanged (a probe: 220 -> 198 us; here the kernel
-//    takes 39 registers, 6 blocks per SM, and a render call 0.234 ->
-//    0.217 ms, 0.208 ms with the quarter-pixel margin of warp_mask
-//    instead of one pixel).  Asking for 8 blocks per SM (32 registers)
-//    spills and loses most of the gain.
+//  * culling per warp: a Gaussian reaches a pixel only inside the ellipse
+//    where power >= cut, so when it is staged, its thread marks the warps the
+//    ellipse can reach, with a margin; each warp then blends only the list of
+//    staged Gaussians that reach it, kept in front-to-back order by one ballot
+//    per 32.  What a warp skips is what its pixels' own cut test would have
+//    skipped, so the image is unchanged.  A warp's pixels are 8 x 4: an
+//    ellipse of w x h pixels meets (w + 8)(h + 4) / 32 warps on average,
+//    against (w + 16)(h + 2) / 32 for rows of 16 x 2.  With the list holding
+//    byte offsets, the colour one 16-byte word and stopped warps leaving the
+//    batch, a render call went 266 -> 222 us (500k Gaussians, 1280x720), 135 ->
+//    112 (300k, 640x360) and 517 -> 441 (700k, 3840x2160).  The bound of 6
+//    blocks per SM holds the kernel at 40 registers (64 without it: 242, 122
+//    and 524 us); 8 blocks spill and measure the same.
+//  * the order kernel keeps its tiles' counts in registers, and the blend is
+//    launched while it runs (programmatic dependent launch).
 //
 // Per pixel (sample point = the pixel's integer coordinate), in float32
 // with CUDA's fast exponential and multiply-adds (the result is compared
@@ -53,9 +56,7 @@ namespace tdgs {
 
 namespace {
 
-constexpr int kPix = 1;                        // pixels per thread
-constexpr int kRenderThreads = 256 / kPix;      // one 16x16 tile per block
-constexpr int kRowStep = kRenderThreads / 16;   // rows between a thread's pixels
+constexpr int kRenderThreads = 256;             // one 16x16 tile per block, one pixel per thread
 constexpr int kOrderThreads = 1024;             // the tile-order kernel's one block
 constexpr uint32_t kOrderBuckets = 64;          // Gaussian-count buckets, heaviest first
 static_assert(kOrderBuckets == 64, "the bucket scan takes two counts per lane of one warp");
@@ -65,20 +66,31 @@ static_assert(kRenderWarps <= 8, "one bit per warp in an 8-bit mask");
 
 __device__ __forceinline__ uint32_t tile_len(uint2 r) { return r.y > r.x ? r.y - r.x : 0u; }
 
-// Warps of the tile a staged Gaussian can reach (bit w: warp w, whose
-// pixels sit on rows 2w, 2w+1 (+ kRowStep k) of the tile).  A pixel passes
-// the cut test only inside the ellipse d^T Q d <= K, K = -2 cut, where
-// Q = [[a, b], [b, c]] is the conic; its squared half-extents are
+// Pixels of a warp: 8 x 4, two warps across the tile and four down.
+constexpr int kWarpW = 8, kWarpH = 4;
+static_assert(kWarpW * kWarpH == 32 && 2 * kWarpW == 16 && 4 * kWarpH == 16, "eight warps cover the tile");
+
+// Warps of the tile a staged Gaussian can reach (bit w: warp w, whose pixels
+// are columns 8 (w & 1) .. + 7 and rows 4 (w >> 1) .. + 3 of the tile).  A
+// pixel passes the cut test only inside the ellipse d^T Q d <= K, K = -2 cut,
+// where Q = [[a, b], [b, c]] is the conic; its squared half-extents are
 // K a / det in y and K c / det in x (det = ac - b^2).  A warp is left out
-// when all its rows lie farther from the mean than 1.01 half-extents plus
-// a quarter pixel (tested on squares), and every warp when the columns of
-// the tile do.  det comes from one fused multiply-add (relative error
-// below 6e-5 when det > 1e-3 ac, inside the 1 %); with |cut| <= ln 255 and
-// the terms of the exponent below sqrt(ac / det) K, float rounding moves
-// the cut boundary by about 1e-3 pixel at most, inside the quarter pixel.
-// Flatter conics, Q not positive definite, or anything not finite reach
-// every warp.  K < 0: no pixel passes the cut test (no warp).
-__device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, float cut, float tx0, float ty0) {
+// when all its rows, or all its columns, lie farther from the mean than 1.01
+// half-extents plus a quarter pixel (tested on squares).  det comes from one
+// fused multiply-add (relative error below 6e-5 when det > 1e-3 ac, inside
+// the 1 %); with |cut| <= ln 255 and the terms of the exponent below
+// sqrt(ac / det) K, float rounding moves the cut boundary by about 1e-3 pixel
+// at most, inside the quarter pixel.  With `ellipse`, a warp is also left out
+// when the ellipse d^T Q d <= 1.0201 K misses its rectangle grown by a quarter
+// pixel: the least d^T Q d over the rectangle lies on the edges that face the
+// mean, at the edge's own minimum or its nearer corner.  That costs the
+// staging thread 110 instructions, so only tiles of more than one batch take
+// it (render of 700k Gaussians: 400x300 88 -> 84 us, 20k at 320x180 29 -> 27,
+// but 4K with 86 Gaussians a tile 455 -> 467).  Flatter conics, Q not positive
+// definite, or anything not finite reach every warp.  K < 0: no pixel passes
+// the cut test (no warp).
+__device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, float cut, float tx0, float ty0,
+                                              bool ellipse) {
   const float K = -2.0f * cut;
   if (K < 0.0f) return 0u;
   const uint32_t all = (1u << kRenderWarps) - 1u;
@@ -88,32 +100,57 @@ __device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, floa
   const float hy2 = __fdividef(K * c.x, det) * 1.0201f;
   const float hx2 = __fdividef(K * c.z, det) * 1.0201f;
   if (!(hy2 < 1e30f && hx2 < 1e30f)) return all;
-  const float ex = fmaxf(fmaxf(tx0 - mx, mx - (tx0 + 15.0f)) - 0.25f, 0.0f);
-  if (ex * ex > hx2) return 0u;
-  const float yr = my - ty0;  // the mean's row inside the tile
-  uint32_t m = 0;
+  const float xr = mx - tx0, yr = my - ty0;  // the mean inside the tile
+  uint32_t columns = 0, m = 0;
 #pragma unroll
-  for (int w = 0; w < kRenderWarps; ++w)
+  for (int h = 0; h < 2; ++h) {
+    const float c0 = static_cast<float>(kWarpW * h);
+    const float ex = fmaxf(fmaxf(c0 - xr, xr - (c0 + (kWarpW - 1.0f))) - 0.25f, 0.0f);
+    if (ex * ex <= hx2) columns |= 1u << h;
+  }
 #pragma unroll
-    for (int k = 0; k < kPix; ++k) {
-      const float r0 = static_cast<float>(2 * w + kRowStep * k);
-      const float ey = fmaxf(fmaxf(r0 - yr, yr - (r0 + 1.0f)) - 0.25f, 0.0f);
-      if (ey * ey <= hy2) m |= 1u << w;
-    }
+  for (int q = 0; q < 4; ++q) {
+    const float r0 = static_cast<float>(kWarpH * q);
+    const float ey = fmaxf(fmaxf(r0 - yr, yr - (r0 + (kWarpH - 1.0f))) - 0.25f, 0.0f);
+    if (ey * ey <= hy2) m |= columns << (2 * q);
+  }
+  if (!ellipse) return m;
+  const float bc = __fdividef(-c.y, c.z), ba = __fdividef(-c.y, c.x), K2 = K * 1.0201f;
+#pragma unroll
+  for (int w = 0; w < kRenderWarps; ++w) {
+    const float x0 = static_cast<float>(kWarpW * (w & 1)) - 0.25f - xr, x1 = x0 + (kWarpW - 1.0f) + 0.5f;
+    const float y0 = static_cast<float>(kWarpH * (w >> 1)) - 0.25f - yr, y1 = y0 + (kWarpH - 1.0f) + 0.5f;
+    const float xe = fminf(fmaxf(0.0f, x0), x1), ye = fminf(fmaxf(0.0f, y0), y1);
+    const float ys = fminf(fmaxf(bc * xe, y0), y1), xs = fminf(fmaxf(ba * ye, x0), x1);
+    const float q1 = fmaf(xe, fmaf(c.x, xe, 2.0f * c.y * ys), c.z * ys * ys);
+    const float q2 = fmaf(xs, fmaf(c.x, xs, 2.0f * c.y * ye), c.z * ye * ye);
+    if (fminf(q1, q2) > K2) m &= ~(1u << w);
+  }
   return m;
 }
 
 // order[0 .. tiles) = every tile once, by descending bucket of its
-// Gaussian count: bucket = (max - len) * 63 / max (0 when every tile is
-// empty).  Positions come from the exclusive bucket scan, so they are a
+// Gaussian count: bucket = (max - len) * 63 / max in float (0 when every tile
+// is empty).  Positions come from the exclusive bucket scan, so they are a
 // permutation of 0 .. tiles-1.
 __global__ void __launch_bounds__(kOrderThreads)
     k_render_order(const uint2* __restrict__ ranges, uint32_t tiles, uint32_t* __restrict__ order) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (k_render waits for this launch's end)
   __shared__ uint32_t s_max[kOrderThreads / 32];
   __shared__ uint32_t s_cnt[kOrderBuckets];
   const uint32_t t = threadIdx.x;
+  // the first tiles of each thread stay in registers; images above 8192
+  // tiles read the rest again
+  constexpr uint32_t kHeld = 8;
+  uint32_t held[kHeld];
   uint32_t mx = 0;
-  for (uint32_t i = t; i < tiles; i += kOrderThreads) mx = max(mx, tile_len(ranges[i]));
+#pragma unroll
+  for (uint32_t k = 0; k < kHeld; ++k) {
+    const uint32_t i = t + k * kOrderThreads;
+    held[k] = i < tiles ? tile_len(ranges[i]) : 0u;
+    mx = max(mx, held[k]);
+  }
+  for (uint32_t i = t + kHeld * kOrderThreads; i < tiles; i += kOrderThreads) mx = max(mx, tile_len(ranges[i]));
   mx = __reduce_max_sync(0xffffffffu, mx);
   if ((t & 31) == 0) s_max[t >> 5] = mx;
   if (t < kOrderBuckets) s_cnt[t] = 0;
@@ -121,10 +158,15 @@ __global__ void __launch_bounds__(kOrderThreads)
   mx = 0;
 #pragma unroll
   for (int w = 0; w < kOrderThreads / 32; ++w) mx = max(mx, s_max[w]);
-  auto bucket = [mx](uint32_t len) -> uint32_t {
-    return mx ? static_cast<uint32_t>(static_cast<uint64_t>(mx - len) * (kOrderBuckets - 1) / mx) : 0u;
+  const float scale = mx ? static_cast<float>(kOrderBuckets - 1) / static_cast<float>(mx) : 0.0f;
+  auto bucket = [mx, scale](uint32_t len) -> uint32_t {
+    return min(static_cast<uint32_t>(static_cast<float>(mx - len) * scale), kOrderBuckets - 1);
   };
-  for (uint32_t i = t; i < tiles; i += kOrderThreads) atomicAdd(&s_cnt[bucket(tile_len(ranges[i]))], 1u);
+#pragma unroll
+  for (uint32_t k = 0; k < kHeld; ++k)
+    if (t + k * kOrderThreads < tiles) atomicAdd(&s_cnt[bucket(held[k])], 1u);
+  for (uint32_t i = t + kHeld * kOrderThreads; i < tiles; i += kOrderThreads)
+    atomicAdd(&s_cnt[bucket(tile_len(ranges[i]))], 1u);
   __syncthreads();
   if (t < 32) {  // exclusive scan of the 64 bucket counts: two per lane
     const uint32_t c0 = s_cnt[2 * t], c1 = s_cnt[2 * t + 1];
@@ -139,45 +181,41 @@ __global__ void __launch_bounds__(kOrderThreads)
     s_cnt[2 * t + 1] = excl + c0;
   }
   __syncthreads();
-  for (uint32_t i = t; i < tiles; i += kOrderThreads)
+#pragma unroll
+  for (uint32_t k = 0; k < kHeld; ++k)
+    if (t + k * kOrderThreads < tiles) order[atomicAdd(&s_cnt[bucket(held[k])], 1u)] = t + k * kOrderThreads;
+  for (uint32_t i = t + kHeld * kOrderThreads; i < tiles; i += kOrderThreads)
     order[atomicAdd(&s_cnt[bucket(tile_len(ranges[i]))], 1u)] = i;
 }
 
 
-__global__ void __launch_bounds__(kRenderThreads)
+__global__ void __launch_bounds__(kRenderThreads, 6)
     k_render(const float4* __restrict__ rec, const float4* __restrict__ conic, const float* __restrict__ rgb,
              const uint32_t* __restrict__ values, const uint2* __restrict__ ranges,
              const uint32_t* __restrict__ order, uint32_t gx, uint32_t width,
              uint32_t height, float3 bg, uint32_t n, float* __restrict__ image, uint32_t* err) {
   // staged Gaussians, two 16-byte loads per step: (x, y, cut, -c/2) and
-  // (-a/2, -b, opacity, -); cut = the exponent below which alpha < 1/255
+  // (-a/2, -b, opacity, -); cut = the exponent below which alpha < 1/255; a
+  // third one, the colour, for the pixels that blend it
   __shared__ float4 s_g0[kRenderThreads];
   __shared__ float4 s_g1[kRenderThreads];
-  __shared__ float s_rgb[kRenderThreads][3];
+  __shared__ float4 s_rgb[kRenderThreads];
   __shared__ uint8_t s_mask[kRenderThreads];                 // warps each staged Gaussian reaches
-  __shared__ uint8_t s_list[kRenderWarps][kRenderThreads];  // per warp: staged Gaussians to blend
+  __shared__ uint16_t s_list[kRenderWarps][kRenderThreads];  // per warp: staged Gaussians to blend, as byte offsets
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tile = order ? order[blockIdx.x] : blockIdx.x, t = threadIdx.x;
-  const uint32_t px = (tile % gx) * 16 + (t & 15);
-  const uint32_t py0 = (tile / gx) * 16 + (t >> 4);
-  const float fx = __uint2float_rn(px);
   const uint32_t warp = t >> 5, lane = t & 31;
-  float fy[kPix], T[kPix], C[kPix][3];
-  bool done[kPix];
-#pragma unroll
-  for (int k = 0; k < kPix; ++k) {
-    const uint32_t py = py0 + kRowStep * k;
-    fy[k] = __uint2float_rn(py);
-    T[k] = 1.0f;
-    C[k][0] = C[k][1] = C[k][2] = 0.0f;
-    done[k] = !(px < width && py < height);
-  }
+  const uint32_t tx = (tile % gx) * 16, ty = (tile / gx) * 16;
+  const uint32_t px = tx + (warp & 1) * kWarpW + (lane % kWarpW);
+  const uint32_t py = ty + (warp >> 1) * kWarpH + lane / kWarpW;
+  const float fx = __uint2float_rn(px), fy = __uint2float_rn(py);
+  float T = 1.0f, C[3] = {0.0f, 0.0f, 0.0f};
+  bool done = !(px < width && py < height);
   const uint2 r = ranges[tile];
   bool bad = false;
+  const bool ellipse = tile_len(r) > kRenderThreads;
   for (uint32_t b = r.x; b < r.y; b += kRenderThreads) {
-    bool mine_done = true;
-#pragma unroll
-    for (int k = 0; k < kPix; ++k) mine_done = mine_done && done[k];
-    if (__syncthreads_count(mine_done) == kRenderThreads) break;
+    if (__syncthreads_count(done) == kRenderThreads) break;
     const uint32_t idx = b + t;
     if (idx < r.y) {
       uint32_t g = values[idx];
@@ -186,7 +224,7 @@ __global__ void __launch_bounds__(kRenderThreads)
         s_g0[t] = make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
         s_g1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
         s_mask[t] = 0;
-        s_rgb[t][0] = s_rgb[t][1] = s_rgb[t][2] = 0.f;
+        s_rgb[t] = make_float4(0.f, 0.f, 0.f, 0.f);
       } else {
         const float4 q = __ldg(rec + g);
         const float4 c = __ldg(conic + g);
@@ -195,62 +233,59 @@ __global__ void __launch_bounds__(kRenderThreads)
         const float cut = c.w > 0.0f ? -__logf(255.0f * c.w) : __int_as_float(0x7f800000);
         s_g0[t] = make_float4(q.x, q.y, cut, -0.5f * c.z);
         s_g1[t] = make_float4(-0.5f * c.x, -c.y, c.w, 0.f);
-        s_mask[t] = static_cast<uint8_t>(
-            warp_mask(q.x, q.y, c, cut, __uint2float_rn((tile % gx) * 16), __uint2float_rn((tile / gx) * 16)));
-        s_rgb[t][0] = __ldg(rgb + 3 * static_cast<size_t>(g));
-        s_rgb[t][1] = __ldg(rgb + 3 * static_cast<size_t>(g) + 1);
-        s_rgb[t][2] = __ldg(rgb + 3 * static_cast<size_t>(g) + 2);
+        s_mask[t] = static_cast<uint8_t>(warp_mask(q.x, q.y, c, cut, __uint2float_rn(tx), __uint2float_rn(ty),
+                                                 ellipse));
+        s_rgb[t] = make_float4(__ldg(rgb + 3 * static_cast<size_t>(g)), __ldg(rgb + 3 * static_cast<size_t>(g) + 1),
+                               __ldg(rgb + 3 * static_cast<size_t>(g) + 2), 0.f);
       }
     }
     __syncthreads();
+    if (__all_sync(0xffffffffu, done)) continue;  // this warp's pixels have stopped
     const uint32_t cnt = min(static_cast<uint32_t>(kRenderThreads), r.y - b);
-    // this warp's list of the staged Gaussians that can reach its rows
+    // this warp's list of the staged Gaussians that can reach its pixels
     uint32_t nw = 0;
 #pragma unroll
     for (uint32_t k = 0; k < kRenderThreads / 32; ++k) {
       const uint32_t e = k * 32 + lane;
       const bool hit = e < cnt && ((s_mask[e] >> warp) & 1u);
       const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-      if (hit) s_list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = static_cast<uint8_t>(e);
+      if (hit) s_list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = static_cast<uint16_t>(e * sizeof(float4));
       nw += __popc(bal);
     }
     __syncwarp();
+    const char* g0p = reinterpret_cast<const char*>(s_g0);
+    const char* g1p = reinterpret_cast<const char*>(s_g1);
+    const char* cp = reinterpret_cast<const char*>(s_rgb);
 #pragma unroll 8
     for (uint32_t jj = 0; jj < nw; ++jj) {
-      const uint32_t j = s_list[warp][jj];
-      const float4 g0 = s_g0[j];
-      const float4 g1 = s_g1[j];
-      const float dx = g0.x - fx;
-#pragma unroll
-      for (int k = 0; k < kPix; ++k) {
-        if (done[k]) continue;
-        const float dy = g0.y - fy[k];
-        const float power = fmaf(dx, fmaf(g1.x, dx, g1.y * dy), g0.w * dy * dy);
-        if (power > 0.0f || power < g0.z) continue;
-        const float alpha = fminf(0.99f, g1.z * __expf(power));
-        if (alpha < 1.0f / 255.0f) continue;
-        const float test_t = T[k] * (1.0f - alpha);
-        if (test_t < 0.0001f) {
-          done[k] = true;
-          continue;
-        }
-        const float w = alpha * T[k];
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) C[k][ch] += s_rgb[j][ch] * w;
-        T[k] = test_t;
+      const uint32_t at = s_list[warp][jj];
+      const float4 g0 = *reinterpret_cast<const float4*>(g0p + at);
+      const float4 g1 = *reinterpret_cast<const float4*>(g1p + at);
+      if (done) continue;
+      const float dx = g0.x - fx, dy = g0.y - fy;
+      const float power = fmaf(dx, fmaf(g1.x, dx, g1.y * dy), g0.w * dy * dy);
+      if (power > 0.0f || power < g0.z) continue;
+      const float alpha = fminf(0.99f, g1.z * __expf(power));
+      if (alpha < 1.0f / 255.0f) continue;
+      const float test_t = T * (1.0f - alpha);
+      if (test_t < 0.0001f) {
+        done = true;
+        continue;
       }
+      const float w = alpha * T;
+      const float4 col = *reinterpret_cast<const float4*>(cp + at);
+      C[0] += col.x * w;
+      C[1] += col.y * w;
+      C[2] += col.z * w;
+      T = test_t;
     }
   }
-  if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) latch_error(err, TDGS_ERR_INVALID_ARGUMENT, kSiteRender);
-#pragma unroll
-  for (int k = 0; k < kPix; ++k) {
-    const uint32_t py = py0 + kRowStep * k;
-    if (px < width && py < height) {
-      float* o = image + 3 * (static_cast<size_t>(py) * width + px);
-      o[0] = C[k][0] + T[k] * bg.x;
-      o[1] = C[k][1] + T[k] * bg.y;
-      o[2] = C[k][2] + T[k] * bg.z;
-    }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) latch_error(err, TDGS_ERR_INVALID_ARGUMENT, kSiteRender);
+  if (px < width && py < height) {
+    float* o = image + 3 * (static_cast<size_t>(py) * width + px);
+    o[0] = C[0] + T * bg.x;
+    o[1] = C[1] + T * bg.y;
+    o[2] = C[2] + T * bg.z;
   }
 }
 
@@ -268,9 +303,18 @@ cudaError_t launch_render_ordered(const float4* rec, const float4* conic, const 
   const uint32_t gx = (width + 15) / 16, gy = (height + 15) / 16;
   const uint32_t tiles = gx * gy;
   if (tiles == 0) return cudaSuccess;
-  k_render<<<tiles, kRenderThreads, 0, s>>>(rec, conic, rgb, values, ranges, order, gx, width, height,
-                                            make_float3(bg[0], bg[1], bg[2]), n, image, err);
-  return cudaGetLastError();
+  // the blend may be set up while the order kernel still runs (it waits for its end)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tiles);
+  cfg.blockDim = dim3(kRenderThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = order ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_render, rec, conic, rgb, values, ranges, order, gx, width, height,
+                            make_float3(bg[0], bg[1], bg[2]), n, image, err);
 }
 
 cudaError_t launch_render(const float4* rec, const float4* conic, const float* rgb, const uint32_t* values,
