@@ -64,14 +64,14 @@ enum KernelId {
   kKCount, kKScan, kKDuplicate, kKRanges, kKRadixPass,
   kKFrameCount, kKDepthSort, kKFrameScan, kKDupDepth, kKTilePass, kKTileExpand, kKPreprocess, kKBitonic, kKRender, kKPreCount, kKNormRange, kKNormDup, kKNormPass,
   kKNormRanges, kKRenderOrder, kKSortHist, kKOnesweep, kKCountDepth,
-  kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
+  kKNormKeys, kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
 };
 const char* const kKernelNames[kKNum] = {
     "count_tiles",  "scan",       "duplicate_keys",     "tile_ranges",    "radix_pass",
     "frame_count",  "depth_sort", "scan_by_depth", "duplicate_by_depth", "tile_sort_pass",
     "tile_expand_pass", "preprocess", "bitonic_sort", "render", "preprocess_count", "norm_range",
     "norm_duplicate", "norm_sort_pass", "norm_ranges", "render_order", "sort_histogram", "onesweep_pass",
-    "count_depth_sort", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
+    "count_depth_sort", "norm_keys", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
 
 // View table as stored in device memory (SoA, fixed maximum size).
 struct ViewBlob {
@@ -143,6 +143,7 @@ struct tdgs_context {
   ViewBlob* h_views = nullptr;  // pinned staging of the table
   uint32_t nv = 0, n_all = 0, t_all = 0;
   uint32_t max_gx = 0, max_gy = 0;  // over the staged views
+  bool norm = false;            // the frame with the 32-bit normalised key (by interval splits)
   bool split = false;           // pairs by interval splits (else packed elements and tile passes)
   uint64_t capacity = 0;        // pair capacity reserved for the asynchronous path
   bool reserved = false;
@@ -852,7 +853,7 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
 
 // Buffers that depend on the pair count (or capacity) m.
 tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
-  tdgs_status st = ensure(ctx, ctx->f_keys, m * 8 + 16, s);
+  tdgs_status st = ctx->norm ? ensure(ctx, ctx->n_keys[0], m * 4 + 16, s) : ensure(ctx, ctx->f_keys, m * 8 + 16, s);
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_values, m * 4 + 16, s);
   if (ctx->split) {
     // every segment has a pair: at most m segments
@@ -904,11 +905,12 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   da.v2 = dv[2];
   da.counts = counts;
   da.offsets = ctx->split ? nullptr : static_cast<uint32_t*>(ctx->f_soff.p);  // the interval splits take none
-  da.range = ctx->d_range;
+  uint32_t* range = ctx->norm ? static_cast<uint32_t*>(ctx->n_norm.p) : ctx->d_range;  // of the keys that are sorted
+  da.range = range;
   da.n = n_all;
   da.scratch = static_cast<uint32_t*>(ctx->f_dsort.p);
   da.err = err_word(ctx);
-  ctx->early_fused = dp.resident && n_all > 0 && !ctx->proj_on;
+  ctx->early_fused = dp.resident && n_all > 0 && !ctx->proj_on && !ctx->norm;
   if (ctx->early_fused) {
     // one launch: counts, M (also to the mapped host status, tagged with a
     // fresh seq), the depth sort and the offsets
@@ -932,6 +934,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
     // kernel wrote them to the mapped host status (h_early)
     TDGS_CUDA(ctx, cudaEventRecord(ctx->ev_count, s));
   }
+  if (ctx->norm) TDGS_TRACED(ctx, kKNormKeys, n_all, s, launch_norm_keys(dk[0], n_all, ctx->d_range, range, s));
   const uint32_t dpasses = dp.passes;
   uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
   if (dp.resident) {  // one launch: the sort (pass count from the depth range) and the offsets
@@ -941,10 +944,10 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
     if (n_all) {
       uint32_t* dos = static_cast<uint32_t*>(ctx->f_dos.p);
       TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                  launch_depth_onesweep_hist(dk[0], n_all, ctx->d_range, by_view(ctx), dos, err_word(ctx), s));
+                  launch_depth_onesweep_hist(dk[0], n_all, range, by_view(ctx), dos, err_word(ctx), s));
       for (uint32_t p = 0; p < dpasses; ++p)
         TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                    launch_depth_onesweep_pass(p, dk, dv, n_all, ctx->d_range, by_view(ctx) ? ctx->nv : 0u,
+                    launch_depth_onesweep_pass(p, dk, dv, n_all, range, by_view(ctx) ? ctx->nv : 0u,
                                                ctx->d_views->rec_begin, ctx->d_views->n, dos, err_word(ctx), s));
     }
   } else {
@@ -992,6 +995,10 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.ranges = static_cast<uint2*>(ctx->f_ranges.p);
   a.keys = static_cast<uint64_t*>(ctx->f_keys.p);
   a.values = static_cast<uint32_t*>(ctx->f_values.p);
+  if (ctx->norm) {
+    a.keys32 = static_cast<uint32_t*>(ctx->n_keys[0].p);
+    a.norm = ctx->d_range + 2;
+  }
   a.cap = m;
   a.total = &ctx->d_status->total;
   a.ticket = ctx->d_tickets;
@@ -1078,7 +1085,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
 // sort and the scan run; the back half is then enqueued with the exact M
 // before the GPU runs out of work.
 tdgs_status sort_views_exact(tdgs_context* ctx, cudaStream_t s, uint32_t* m_out) {
-  ctx->split = splits(ctx);
+  ctx->split = ctx->norm || splits(ctx);
   tdgs_status st = ensure_record_buffers(ctx, s);
   if (st != TDGS_OK) return st;
   st = run_front(ctx, s, true);
@@ -1326,10 +1333,29 @@ tdgs_status tdgs_sort_frame_normalized(tdgs_context* ctx, const tdgs_gaussian2d*
   if (!aligned(g, 16)) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "misaligned pointer");
   DeviceGuard dg(ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  tdgs_status st = ensure(ctx, ctx->n_norm, 32, s);
+  if (st != TDGS_OK) return st;
+  if ((f.width + 15) / 16 <= kSplitMaxBins && (f.height + 15) / 16 <= kSplitMaxBins) {
+    // the fused frame with normalised depths for keys; its order is that of
+    // the steps below: equal keys keep the Gaussians' index order
+    tdgs_view view{g, n, f};
+    st = stage_views(ctx, &view, 1);
+    if (st != TDGS_OK) return st;
+    ctx->reserved = false;
+    ctx->norm = true;
+    uint32_t m = 0;
+    st = sort_views_exact(ctx, s, &m);
+    ctx->norm = false;
+    if (st != TDGS_OK) return st;
+    *sorted_keys = static_cast<const uint32_t*>(ctx->n_keys[0].p);
+    *sorted_values = static_cast<const uint32_t*>(ctx->f_values.p);
+    *ranges = static_cast<const tdgs_range*>(ctx->f_ranges.p);
+    *m_out = m;
+    return TDGS_OK;
+  }
   const size_t n4 = static_cast<size_t>(n) * 4 + 16;
-  tdgs_status st = ensure(ctx, ctx->n_counts, n4, s);
+  st = ensure(ctx, ctx->n_counts, n4, s);
   if (st == TDGS_OK) st = ensure(ctx, ctx->n_offs, n4, s);
-  if (st == TDGS_OK) st = ensure(ctx, ctx->n_norm, 16, s);
   if (st == TDGS_OK) st = ensure(ctx, ctx->n_ranges, T * 8 + 16, s);
   if (st != TDGS_OK) return st;
   uint32_t* counts = static_cast<uint32_t*>(ctx->n_counts.p);

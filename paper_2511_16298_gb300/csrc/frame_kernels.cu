@@ -205,9 +205,7 @@ cudaError_t launch_scan(const uint32_t* counts, const float4* recs, const uint32
 // local index (row-major within the Gaussian's tile rectangle).  Every
 // store is a fully coalesced 256-byte (keys) / 128-byte (values) run.
 // kNorm: the paper's 32-bit key (Sec. IV-B), tile << 10 | q with q the
-// depth normalised to 2^10 over the visible range norm[0..1] (float bits):
-// scale = 1024 / (dmax - dmin) (0 if equal), q = min(1023, floor((depth -
-// dmin) * scale)), in float32 in this order.
+// depth normalised to 2^10 over the visible range norm[0..1] (float bits).
 template <bool kNorm>
 __global__ void __launch_bounds__(256)
     k_duplicate(const float4* __restrict__ g, const uint32_t* __restrict__ offsets, uint32_t n,
@@ -216,8 +214,7 @@ __global__ void __launch_bounds__(256)
   float dmin = 0.0f, scale = 0.0f;
   if constexpr (kNorm) {
     dmin = __uint_as_float(norm[0]);
-    const float dmax = __uint_as_float(norm[1]);
-    scale = dmax > dmin ? __fdiv_rn(1024.0f, __fsub_rn(dmax, dmin)) : 0.0f;
+    scale = norm_scale(dmin, __uint_as_float(norm[1]));
   }
   const uint32_t lane = lane_id();
   const uint32_t warps_total = (gridDim.x * blockDim.x) >> 5;
@@ -236,10 +233,7 @@ __global__ void __launch_bounds__(256)
       q.count = 0;
     }
     uint32_t depth_bits = i < n ? __float_as_uint(__ldg(&g[i].z)) : 0u;
-    if constexpr (kNorm) {
-      const float f = floorf(__fmul_rn(__fsub_rn(__uint_as_float(depth_bits), dmin), scale));
-      depth_bits = f >= 1023.0f ? 1023u : static_cast<uint32_t>(f);
-    }
+    if constexpr (kNorm) depth_bits = norm_depth(__uint_as_float(depth_bits), dmin, scale);
     uint64_t end = start + q.count;
     // warp range [begin, end_max)
     uint64_t end_max = end;
@@ -334,6 +328,32 @@ cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t 
   const uint32_t blocks = (n + 255) / 256;
   const uint32_t grid = blocks < 152u * 8u ? blocks : 152u * 8u;
   k_norm_range<<<grid, 256, 0, s>>>(g, counts, n, norm);
+  return cudaGetLastError();
+}
+
+// Four keys per thread.  The normalised depths are 0 .. 1023 whatever the
+// frame, so their range is constant.
+__global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, uint32_t n,
+                                                   const uint32_t* __restrict__ range, uint32_t* __restrict__ out) {
+  const float dmin = __uint_as_float(__ldcg(range + 2));
+  const float scale = norm_scale(dmin, __uint_as_float(__ldcg(range + 3)));
+  const uint32_t first = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+#pragma unroll
+  for (uint32_t u = 0; u < 4; ++u) {
+    if (first + u < n) {
+      const uint32_t k = keys[first + u];
+      if (k != 0xffffffffu) keys[first + u] = norm_depth(__uint_as_float(k), dmin, scale);
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    out[2] = 0u;
+    out[3] = 1023u;
+  }
+}
+
+cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  k_norm_keys<<<(n + 1023) / 1024, 256, 0, s>>>(keys, n, range, out);
   return cudaGetLastError();
 }
 

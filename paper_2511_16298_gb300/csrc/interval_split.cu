@@ -142,6 +142,11 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
   __syncthreads();
   constexpr int kPer = kTile / kCountThreads;
   const uint32_t first = tl * kTile;
+  float dmin = 0.0f, scale = 0.0f;
+  if (a.keys32) {
+    dmin = __uint_as_float(__ldcg(a.norm));
+    scale = norm_scale(dmin, __uint_as_float(__ldcg(a.norm + 1)));
+  }
   uint32_t gi[kPer];
   float4 rec[kPer];
 #pragma unroll
@@ -168,7 +173,9 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
       atomicAdd(&s_d[q.y1][1], -w);
     }
     a.rects[rec0 + p] = pack;
-    a.sdo[rec0 + p] = make_uint2(__float_as_uint(rec[u].z), gi[u]);
+    // the low part of the pairs' keys: depth bits, or the normalised depth
+    const uint32_t low = a.keys32 ? norm_depth(rec[u].z, dmin, scale) : __float_as_uint(rec[u].z);
+    a.sdo[rec0 + p] = make_uint2(low, gi[u]);
   }
   __syncthreads();
   uint32_t c = static_cast<uint32_t>(s_d[t][0]), w = static_cast<uint32_t>(s_d[t][1]);
@@ -587,6 +594,16 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
         }
       } else {
         const uint32_t row_tile = (r - pl.row0) * bins;  // the row's first tile in its view
+        if (a.keys32) {
+#pragma unroll 2
+          for (uint32_t p = t; p < np; p += kThreads) {
+            const uint32_t e = s.stage[p], c = e >> 16;
+            const uint2 q = s.pay[e & 0xffffu];
+            const uint32_t dst = s.off[c] + p0 + p;
+            a.keys32[dst] = ((row_tile + c) << 10) | q.x;
+            a.values[dst] = q.y;
+          }
+        } else {
 #pragma unroll 2
         for (uint32_t p = t; p < np; p += kThreads) {
           const uint32_t e = s.stage[p], c = e >> 16;
@@ -594,6 +611,7 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
           const uint32_t dst = s.off[c] + p0 + p;
           a.keys[dst] = (static_cast<uint64_t>(row_tile + c) << 32) | q.x;
           a.values[dst] = q.y;
+        }
         }
       }
       __syncthreads();

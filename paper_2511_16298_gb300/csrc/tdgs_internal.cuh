@@ -82,6 +82,17 @@ __device__ __forceinline__ TileRect tile_rect(const float4 rec, const FrameGeom&
   return tile_rect(rec.x, rec.y, rec.z, __float_as_int(rec.w), fg);
 }
 
+// The paper's 10-bit normalised depth (Sec. IV-B) over the visible depths
+// [dmin, dmax]: scale = 1024 / (dmax - dmin) (0 if equal), q = min(1023,
+// floor((depth - dmin) * scale)), in float32 in this order.
+__device__ __forceinline__ float norm_scale(float dmin, float dmax) {
+  return dmax > dmin ? __fdiv_rn(1024.0f, __fsub_rn(dmax, dmin)) : 0.0f;
+}
+__device__ __forceinline__ uint32_t norm_depth(float depth, float dmin, float scale) {
+  const float f = floorf(__fmul_rn(__fsub_rn(depth, dmin), scale));
+  return f >= 1023.0f ? 1023u : static_cast<uint32_t>(f);
+}
+
 // ------------------------------------------------------------ device sync
 // The first non-zero code wins; later errors are dropped.  err[1] records
 // which site latched it (kSite* below), for the host's error message.
@@ -151,6 +162,11 @@ cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t 
 cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint32_t n, FrameGeom fg,
                                   uint32_t* keys, uint32_t* values, uint32_t cap, const uint32_t* norm,
                                   uint32_t* err, cudaStream_t s);
+// Frames whose pairs come from the interval splits sort by the normalised
+// depth instead of duplicating: keys (the count kernel's depth bits, all ones
+// without pairs) become normalised depths over range[2..3], and out[2..3]
+// receives their own range for the depth sort.
+cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, cudaStream_t s);
 cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t num_tiles, uint2* ranges,
                                     uint32_t* err, cudaStream_t s);
 
@@ -385,6 +401,8 @@ struct SplitArgs {
   uint2* ranges;
   uint64_t* keys;
   uint32_t* values;
+  uint32_t* keys32;           // not null: the 32-bit normalised keys, in place of keys
+  const uint32_t* norm;       // with keys32: smallest and largest visible depth (float bits)
   uint64_t cap;               // pairs that segs, keys and values hold
   const uint64_t* total;      // the pair count
   uint32_t* ticket;           // a zero word, left zero

@@ -139,3 +139,19 @@ def test_batches_in_view_order(ctx, oracle, kind, sizes):
         assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
         assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
         assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
+
+
+@pytest.mark.parametrize("n,width,height", [(1, 16, 16), (2049, 4096, 50), (2049, 4112, 50), (50_000, 700, 500),
+                                            (1_300_000, 320, 200)])
+def test_normalized_key(ctx, oracle, n, width, height):
+    """The 32-bit normalised key through the splits (the single-launch and the
+    onesweep depth sort) and, above 4096 pixels, through the five steps."""
+    fr = synth.frame_random(n % 97, n, width, height, max_sigma=6.0 if n > 100_000 else 64.0, depth_ties=0.2)
+    st, ek, ev, er = oracle.sort_frame_normalized(fr.gaussians, width, height)
+    assert st == 0
+    k, v, r, m = ctx.sort_frame_normalized(T.records_to_tensor(fr.gaussians, DEV), width, height)
+    ctx.sync()
+    assert m == len(ek)
+    assert np.array_equal(k.cpu().numpy().view(np.uint32), ek)
+    assert np.array_equal(v.cpu().numpy().view(np.uint32), ev)
+    assert np.array_equal(r.cpu().numpy().view(np.uint32), er)
