@@ -131,7 +131,7 @@ struct tdgs_context {
   Buffer b_keys, b_vals;   // padded scratch of tdgs_sort_pairs_bitonic
   Buffer n_counts, n_offs, n_norm, n_keys[2], n_vals[2], n_ranges;  // tdgs_sort_frame_normalized
   Buffer f_counts, f_dkey[3], f_dval[3], f_soff, f_sdo, f_rminmax, f_stream[2], f_keys, f_values, f_ranges;
-  Buffer f_rects, f_c1, f_rows, f_segs, f_c2, f_b2;  // interval splits
+  Buffer f_rects, f_c1, f_rows, f_segs, f_cols, f_c2, f_b2;  // interval splits
   // depth-key range: accumulators [0..1], result [2..3], passes of the last
   // resident depth sort [4]
   uint32_t* d_range = nullptr;
@@ -557,7 +557,7 @@ void tdgs_context_destroy(tdgs_context* ctx) {
                     &ctx->n_vals[0],    &ctx->n_vals[1],    &ctx->n_ranges,
                     &ctx->f_rminmax,    &ctx->f_stream[0],   &ctx->f_stream[1],  &ctx->f_keys,
                     &ctx->f_values,     &ctx->f_ranges,     &ctx->r_order,
-                    &ctx->f_rects,      &ctx->f_c1,         &ctx->f_rows,       &ctx->f_segs,       &ctx->f_c2,
+                    &ctx->f_rects,      &ctx->f_c1,         &ctx->f_rows,       &ctx->f_segs,       &ctx->f_cols,       &ctx->f_c2,
                     &ctx->f_b2};
   if (ctx->d_views) cudaFree(ctx->d_views);
   if (ctx->h_views) cudaFreeHost(ctx->h_views);
@@ -859,6 +859,7 @@ tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
     // every segment has a pair: at most m segments
     const size_t entries = static_cast<size_t>(split_tiles(ctx, m)) * split_pitch(ctx);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_segs, m * 8 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_cols, m * 2 + 16, s);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_c2, entries * 2 + 16, s);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_b2, entries * 4 + 16, s);
     return st;
@@ -989,6 +990,7 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.row_pair = a.row_tile + a.nrows + 1;
   a.info = a.row_pair + a.nrows;
   a.segs = static_cast<uint2*>(ctx->f_segs.p);
+  a.cols = static_cast<uint16_t*>(ctx->f_cols.p);
   a.c2 = static_cast<uint16_t*>(ctx->f_c2.p);
   a.b2 = static_cast<uint32_t*>(ctx->f_b2.p);
   a.pitch = split_pitch(ctx);

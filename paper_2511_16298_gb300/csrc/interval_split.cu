@@ -5,7 +5,7 @@
 // tile columns, so the pairs need no sort of their own:
 //   level 1  items = Gaussians in depth order, bins = tile rows: every
 //            Gaussian goes, in order, to the list of each row it covers, as a
-//            segment {depth position, its columns};
+//            segment {depth bits, index} and its columns;
 //   level 2  items = a row's segments in order, bins = tile columns: every
 //            segment goes to the list of each column it covers, as the final
 //            (tile << 32 | depth bits, index) pair.
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const uint32_t p = beg + u * kCountThreads + t;
-      x[u] = p < end ? __ldg(&a.segs[p].y) : 0xffffffffu;
+      x[u] = p < end ? __ldg(a.cols + p) : 0xffffffffu;
     }
     for (uint32_t b = t; b <= kMaxBins; b += kCountThreads) s_d[b] = 0;
     __syncthreads();
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
     for (int u = 0; u < kPer; ++u) {
       if (x[u] != 0xffffffffu) {
         atomicAdd(&s_d[x[u] & 0xffu], 1);
-        atomicAdd(&s_d[((x[u] >> 8) & 0xffu) + 1u], -1);
+        atomicAdd(&s_d[(x[u] >> 8) + 1u], -1);
       }
     }
     __syncthreads();
@@ -402,6 +402,7 @@ struct Smem {
   uint32_t lstart[kBinsP + 1];
   uint32_t off[kBinsP];
   uint16_t pos[kBatches][kPitch];
+  uint16_t cols[kTile];  // level 1: the items' columns
 };
 
 template <int kLevel, int kWords>
@@ -446,12 +447,13 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
           lo[b] = (q >> 16) & 0xffu;
           hi[b] = (q >> 24) + 1u;
           if (hi[b] <= lo[b]) lo[b] = hi[b] = 0u;
-          s.pay[i] = make_uint2(beg + i, q & 0xffffu);
+          s.pay[i] = __ldg(a.sdo + beg + i);
+          s.cols[i] = static_cast<uint16_t>(q);
         } else {
-          const uint2 q = __ldg(a.segs + beg + i);
-          lo[b] = q.y & 0xffu;
-          hi[b] = (q.y >> 8) + 1u;
-          s.pay[i] = __ldg(a.sdo + q.x);
+          const uint32_t q = __ldg(a.cols + beg + i);
+          lo[b] = q & 0xffu;
+          hi[b] = (q >> 8) + 1u;
+          s.pay[i] = __ldg(a.segs + beg + i);
         }
       }
     }
@@ -589,8 +591,9 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
       if constexpr (kLevel == 1) {
 #pragma unroll 2
         for (uint32_t p = t; p < np; p += kThreads) {
-          const uint32_t e = s.stage[p];
-          a.segs[s.off[e >> 16] + p0 + p] = s.pay[e & 0xffffu];
+          const uint32_t e = s.stage[p], i = e & 0xffffu, dst = s.off[e >> 16] + p0 + p;
+          a.segs[dst] = s.pay[i];
+          a.cols[dst] = s.cols[i];
         }
       } else {
         const uint32_t row_tile = (r - pl.row0) * bins;  // the row's first tile in its view

@@ -394,7 +394,8 @@ struct SplitArgs {
   uint32_t* row_tile;         // [nrows+1] first level-2 tile of each row
   uint32_t* row_pair;         // [nrows] first pair of each row
   uint32_t* info;             // {level-2 tiles, 1 if the pairs fit}
-  uint2* segs;                // {depth position, first column | last column << 8}
+  uint2* segs;                // {depth bits, index in the view}
+  uint16_t* cols;             // by segment: first column | last column << 8
   uint16_t* c2;               // [level-2 tile][pitch] items per column
   uint32_t* b2;               // [level-2 tile][pitch] first output position per column
   uint32_t pitch;             // columns of the widest view, rounded up to 8
