@@ -11,6 +11,7 @@ namespace tdgs {
 __global__ void __launch_bounds__(256) k_count_tiles(const float4* __restrict__ g, uint32_t n,
                                                      FrameGeom fg, uint32_t* __restrict__ counts,
                                                      uint32_t* err) {
+  begin_launch();
   bool bad = false;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const TileRect q = tile_rect(__ldg(g + i), fg);
@@ -25,8 +26,7 @@ cudaError_t launch_count_tiles(const float4* g, uint32_t n, FrameGeom fg, uint32
   if (n == 0) return cudaSuccess;
   const uint32_t blocks = (n + 255) / 256;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
-  k_count_tiles<<<grid, 256, 0, s>>>(g, n, fg, counts, err);
-  return cudaGetLastError();
+  return launch_after(k_count_tiles, grid, 256, 0, s, g, n, fg, counts, err);
 }
 
 // --------------------------------------------------------- exclusive scan
@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kScanThreads)
   __shared__ uint64_t s_warp[kScanThreads / 32];
   __shared__ uint64_t s_excl;
   __shared__ uint32_t s_tile;
+  begin_launch();
   const uint32_t t = threadIdx.x;
   const uint32_t lane = lane_id();
   const uint32_t warp = t >> 5;
@@ -184,16 +185,9 @@ cudaError_t launch_scan(const uint32_t* counts, const float4* recs, const uint32
                         uint32_t* total32, uint32_t* err, cudaStream_t s) {
   const uint32_t tiles = (n + kScanTileItems - 1) / kScanTileItems;
   if (tiles == 0) return cudaSuccess;
-  if (recs)
-    k_scan<1><<<tiles, kScanThreads, 0, s>>>(counts, recs, gather, fg, n, offsets, status, ticket,
-                                             ticket_base, total64, total32, err);
-  else if (gather)
-    k_scan<2><<<tiles, kScanThreads, 0, s>>>(counts, recs, gather, fg, n, offsets, status, ticket,
-                                             ticket_base, total64, total32, err);
-  else
-    k_scan<0><<<tiles, kScanThreads, 0, s>>>(counts, recs, gather, fg, n, offsets, status, ticket,
-                                             ticket_base, total64, total32, err);
-  return cudaGetLastError();
+  const auto fn = recs ? k_scan<1> : gather ? k_scan<2> : k_scan<0>;
+  return launch_after(fn, tiles, kScanThreads, 0, s, counts, recs, gather, fg, n, offsets, status, ticket, ticket_base,
+                      total64, total32, err);
 }
 
 // ------------------------------------------------------------- duplicate
@@ -211,6 +205,7 @@ __global__ void __launch_bounds__(256)
     k_duplicate(const float4* __restrict__ g, const uint32_t* __restrict__ offsets, uint32_t n,
                 FrameGeom fg, void* __restrict__ keys_raw, uint32_t* __restrict__ values,
                 uint32_t cap, const uint32_t* __restrict__ norm, uint32_t* err) {
+  begin_launch();
   float dmin = 0.0f, scale = 0.0f;
   if constexpr (kNorm) {
     dmin = __uint_as_float(norm[0]);
@@ -287,8 +282,7 @@ cudaError_t launch_duplicate(const float4* g, const uint32_t* offsets, uint32_t 
   const uint32_t warps = (n + 31) / 32;
   const uint32_t blocks = (warps + 7) / 8;
   const uint32_t grid = blocks < 152u * 32u ? blocks : 152u * 32u;
-  k_duplicate<false><<<grid, 256, 0, s>>>(g, offsets, n, fg, keys, values, cap, nullptr, err);
-  return cudaGetLastError();
+  return launch_after(k_duplicate<false>, grid, 256, 0, s, g, offsets, n, fg, keys, values, cap, nullptr, err);
 }
 
 cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint32_t n, FrameGeom fg,
@@ -298,8 +292,7 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
   const uint32_t warps = (n + 31) / 32;
   const uint32_t blocks = (warps + 7) / 8;
   const uint32_t grid = blocks < 152u * 32u ? blocks : 152u * 32u;
-  k_duplicate<true><<<grid, 256, 0, s>>>(g, offsets, n, fg, keys, values, cap, norm, err);
-  return cudaGetLastError();
+  return launch_after(k_duplicate<true>, grid, 256, 0, s, g, offsets, n, fg, keys, values, cap, norm, err);
 }
 
 // Smallest and largest depth (float bits; positive finite depths order as
@@ -335,6 +328,7 @@ cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t 
 // frame, so their range is constant.
 __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, uint32_t n,
                                                    const uint32_t* __restrict__ range, uint32_t* __restrict__ out) {
+  begin_launch();
   const float dmin = __uint_as_float(__ldcg(range + 2));
   const float scale = norm_scale(dmin, __uint_as_float(__ldcg(range + 3)));
   const uint32_t first = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
@@ -353,8 +347,7 @@ __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, 
 
 cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  k_norm_keys<<<(n + 1023) / 1024, 256, 0, s>>>(keys, n, range, out);
-  return cudaGetLastError();
+  return launch_after(k_norm_keys, (n + 1023) / 1024, 256, 0, s, keys, n, range, out);
 }
 
 // ---------------------------------------------------------- tile ranges
@@ -367,6 +360,7 @@ template <typename K, int kShift>
 __global__ void __launch_bounds__(256) k_tile_ranges(const K* __restrict__ keys, uint32_t m,
                                                      uint32_t num_tiles, uint2* ranges,
                                                      uint32_t* err) {
+  begin_launch();
   bool bad = false;
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
     const uint64_t t = static_cast<uint64_t>(__ldg(keys + k)) >> kShift;
@@ -387,8 +381,7 @@ cudaError_t launch_tile_ranges(const uint64_t* keys, uint32_t m, uint32_t num_ti
   if (m == 0) return cudaSuccess;
   const uint32_t blocks = (m + 255) / 256;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
-  k_tile_ranges<uint64_t, 32><<<grid, 256, 0, s>>>(keys, m, num_tiles, ranges, err);
-  return cudaGetLastError();
+  return launch_after(k_tile_ranges<uint64_t, 32>, grid, 256, 0, s, keys, m, num_tiles, ranges, err);
 }
 
 cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t num_tiles, uint2* ranges,
@@ -396,8 +389,7 @@ cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t n
   if (m == 0) return cudaSuccess;
   const uint32_t blocks = (m + 255) / 256;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
-  k_tile_ranges<uint32_t, 10><<<grid, 256, 0, s>>>(keys, m, num_tiles, ranges, err);
-  return cudaGetLastError();
+  return launch_after(k_tile_ranges<uint32_t, 10>, grid, 256, 0, s, keys, m, num_tiles, ranges, err);
 }
 
 }  // namespace tdgs

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(256)
   __shared__ uint32_t s_lo, s_hi;
   __shared__ CameraDev s_cam[kProject ? kMaxViews : 1];
   __shared__ float2 s_lim[kProject ? kMaxViews : 1];
+  begin_launch();
   for (uint32_t v = threadIdx.x; v < vt.nv; v += blockDim.x) {
     const ViewOf w = view_of(vt, v);
     s_begin[v] = w.rec0;
@@ -184,13 +185,8 @@ cudaError_t launch_views_count(const ViewTable& vt, uint32_t n_all, uint32_t* co
   const uint32_t per_block = 256u * (proj ? 2u : static_cast<uint32_t>(kCountUnroll));
   const uint32_t blocks = (n_all + per_block - 1) / per_block;
   const uint32_t grid = blocks < 1u ? 1u : (blocks < 152u * 8u ? blocks : 152u * 8u);
-  if (proj)
-    k_views_count<true><<<grid, 256, 0, s>>>(vt, n_all, counts, dkey, dval, err, ticket, total, range,
-                                             static_cast<uint32_t*>(host_status), *proj);
-  else
-    k_views_count<false><<<grid, 256, 0, s>>>(vt, n_all, counts, dkey, dval, err, ticket, total, range,
-                                              static_cast<uint32_t*>(host_status), Proj3D{});
-  return cudaGetLastError();
+  return launch_after(proj ? k_views_count<true> : k_views_count<false>, grid, 256, 0, s, vt, n_all, counts, dkey, dval,
+                      err, ticket, total, range, static_cast<uint32_t*>(host_status), proj ? *proj : Proj3D{});
 }
 
 // Duplicate in depth order: depth position j is record sorder[j]; its

@@ -45,15 +45,6 @@ static_assert(kTile == kSplitTile, "the host sizes the tile tables");
 static_assert(kMaxBins == 256, "bins and columns are packed in bytes");
 static_assert(kTile <= kStage, "one bin of a tile fits the stage");
 
-// Every launch here may start while the one before it on the stream still
-// runs (programmatic dependent launch): its blocks wait for that launch's
-// end, and all of its writes, before they touch memory.  Every block waits,
-// so a launch's end implies the end of all launches before it.
-__device__ __forceinline__ void begin_launch() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Largest i < n with begin[i] <= x (begin ascending, begin[0] <= x), by the
 // whole warp: 32 probes at a time.
 __device__ __forceinline__ uint32_t warp_find(const uint32_t* __restrict__ begin, uint32_t n, uint32_t x) {
@@ -624,72 +615,51 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
 }
 
 // ---------------------------------------------------------------- host side
-struct Form {
-  const void* fn;
-  size_t smem;
-};
-template <int kLevel>
-Form split_form(uint32_t bins) {
-  // an odd number of words keeps the lanes' consecutive bins in different banks
-  if (bins <= 32) return {reinterpret_cast<const void*>(&k_split<kLevel, 1>), sizeof(Smem<1>)};
-  if (bins <= 64) return {reinterpret_cast<const void*>(&k_split<kLevel, 2>), sizeof(Smem<2>)};
-  if (bins <= 96) return {reinterpret_cast<const void*>(&k_split<kLevel, 3>), sizeof(Smem<3>)};
-  if (bins <= 160) return {reinterpret_cast<const void*>(&k_split<kLevel, 5>), sizeof(Smem<5>)};
-  if (bins <= 224) return {reinterpret_cast<const void*>(&k_split<kLevel, 7>), sizeof(Smem<7>)};
-  return {reinterpret_cast<const void*>(&k_split<kLevel, 9>), sizeof(Smem<9>)};
-}
-
-cudaError_t launch_after(const void* fn, uint32_t grid, int threads, size_t smem, const SplitArgs& a, cudaStream_t s) {
-  SplitArgs args = a;
-  void* params[] = {(void*)&args};
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelExC(&cfg, fn, params);
-}
-
-cudaError_t launch_split(int level, const SplitArgs& a, uint32_t bins, uint32_t tiles, int ctas_per_sm, cudaStream_t s) {
-  const Form f = level == 1 ? split_form<1>(bins) : split_form<2>(bins);
-  const radix::Kernel k{f.fn, 0, kThreads, 0, f.smem, 4};
+template <int kLevel, int kWords>
+cudaError_t launch_split_form(const SplitArgs& a, uint32_t tiles, int ctas_per_sm, cudaStream_t s) {
+  const size_t smem = sizeof(Smem<kWords>);
+  const radix::Kernel k{reinterpret_cast<const void*>(&k_split<kLevel, kWords>), 0, kThreads, 0, smem, 4};
   const uint32_t resident = radix::resident_ctas(k, ctas_per_sm);
   if (resident == 0) return cudaErrorInvalidConfiguration;
-  return launch_after(f.fn, tiles < resident ? tiles : resident, kThreads, f.smem, a, s);
+  return launch_after(k_split<kLevel, kWords>, tiles < resident ? tiles : resident, kThreads, smem, s, a);
+}
+
+template <int kLevel>
+cudaError_t launch_split(const SplitArgs& a, uint32_t bins, uint32_t tiles, int ctas_per_sm, cudaStream_t s) {
+  // an odd number of words keeps the lanes' consecutive bins in different banks
+  if (bins <= 32) return launch_split_form<kLevel, 1>(a, tiles, ctas_per_sm, s);
+  if (bins <= 64) return launch_split_form<kLevel, 2>(a, tiles, ctas_per_sm, s);
+  if (bins <= 96) return launch_split_form<kLevel, 3>(a, tiles, ctas_per_sm, s);
+  if (bins <= 160) return launch_split_form<kLevel, 5>(a, tiles, ctas_per_sm, s);
+  if (bins <= 224) return launch_split_form<kLevel, 7>(a, tiles, ctas_per_sm, s);
+  return launch_split_form<kLevel, 9>(a, tiles, ctas_per_sm, s);
 }
 
 }  // namespace split
 
 cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s) {
   if (a.ntiles1 == 0) return cudaSuccess;
-  return split::launch_after(reinterpret_cast<const void*>(&split::k_row_count), a.ntiles1, split::kCountThreads, 0, a,
-                             s);
+  return launch_after(split::k_row_count, a.ntiles1, split::kCountThreads, 0, s, a);
 }
 cudaError_t launch_row_scan(const SplitArgs& a, cudaStream_t s) {
-  return split::launch_after(reinterpret_cast<const void*>(&split::k_row_scan), a.nrows, split::kCountThreads, 0, a, s);
+  return launch_after(split::k_row_scan, a.nrows, split::kCountThreads, 0, s, a);
 }
 cudaError_t launch_row_split(const SplitArgs& a, uint32_t max_rows, int ctas_per_sm, cudaStream_t s) {
   if (a.ntiles1 == 0) return cudaSuccess;
-  return split::launch_split(1, a, max_rows, a.ntiles1, ctas_per_sm, s);
+  return split::launch_split<1>(a, max_rows, a.ntiles1, ctas_per_sm, s);
 }
 cudaError_t launch_col_count(const SplitArgs& a, uint32_t max_tiles, cudaStream_t s) {
   if (max_tiles == 0) return cudaSuccess;
   const uint32_t cap = 152u * 8u;
-  return split::launch_after(reinterpret_cast<const void*>(&split::k_col_count), max_tiles < cap ? max_tiles : cap,
-                             split::kCountThreads, 0, a, s);
+  return launch_after(split::k_col_count, max_tiles < cap ? max_tiles : cap, split::kCountThreads, 0, s, a);
 }
 cudaError_t launch_col_scan(const SplitArgs& a, cudaStream_t s) {
-  return split::launch_after(reinterpret_cast<const void*>(&split::k_col_scan), a.nrows, split::kScanThreads, 0, a, s);
+  return launch_after(split::k_col_scan, a.nrows, split::kScanThreads, 0, s, a);
 }
 cudaError_t launch_col_split(const SplitArgs& a, uint32_t max_cols, uint32_t max_tiles, int ctas_per_sm,
                              cudaStream_t s) {
   if (max_tiles == 0) return cudaSuccess;
-  return split::launch_split(2, a, max_cols, max_tiles, ctas_per_sm, s);
+  return split::launch_split<2>(a, max_cols, max_tiles, ctas_per_sm, s);
 }
 
 }  // namespace tdgs

@@ -9,14 +9,14 @@
 //                    pass's digit starts.  It also clears the first pass's
 //                    status words, the later passes' counters and the tile
 //                    tickets.
-//   k_onesweep_pass  one cooperative launch per digit.  Compute CTAs take
+//   k_onesweep_pass  one launch per digit.  Compute CTAs take
 //                    tiles of 4096 pairs in ticket order; a tile arrives in
 //                    shared memory by bulk copies (double buffered: the
 //                    next tile is in flight while this one is ranked), is
 //                    ranked stably with one ballot per digit bit, publishes
 //                    its per-digit counts at once, counts the next pass's
 //                    digits and is exchanged into digit order in place.
-//                    The last CTAs of the grid are scan CTAs that turn the
+//                    The first CTAs of the grid are scan CTAs that turn the
 //                    published counts into per-tile prefixes; a compute CTA
 //                    takes tile k's prefix one iteration after publishing
 //                    it (while it ranked the next tile) and writes tile k
@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMod
   __shared__ uint32_t h[kBins];
   __shared__ uint32_t s_warp[kHistThreads / 32];
   __shared__ bool s_last;
+  begin_launch();
   const uint32_t t = threadIdx.x;
   for (uint32_t i = t; i < kBins; i += kHistThreads) h[i] = 0;
   // housekeeping for the passes: tile tickets, later passes' counters,
@@ -332,8 +333,11 @@ __device__ __forceinline__ void rank_in_warps(const TileBuf<KeyOf<kMode>>& tb, u
 // that tile.  The prefix is needed a whole ranking phase after the counts
 // went out, so the scan has (nearly always) produced it.  Ranking never
 // waits for another CTA, so every tile with a ticket publishes its counts
-// and the scan always completes.  Launched cooperatively: the scan CTAs
-// must run alongside every other CTA.  While ranking, the CTA also counts
+// and the scan always completes.  The grid has no more CTAs than are resident
+// at once, and the scan CTAs come first in it: they run alongside whichever
+// others do, and a CTA that is not resident yet holds no ticket.  (A
+// cooperative launch would start only after the launch before it has ended.)
+// While ranking, the CTA also counts
 // the next pass's digits; the counts reach hist_next when it finishes.
 template <int kMode, int kModeN>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -352,6 +356,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ uint32_t s_begin[kMode == kDigitDepth ? kMaxViews + 1 : 1];
   bool to_view = false;  // the last depth pass of a batch in view order
 
+  begin_launch();
   Digit dg = a.dg, dgn = a.dgn;
   uint32_t* hist_next = a.hist_next;
   uint32_t* status_next = a.status_next;
@@ -387,8 +392,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   const uint32_t m = a.m, ntiles = a.ntiles;
-  if (blockIdx.x >= gridDim.x - kScanCtas) {  // a scan CTA
-    scan_tiles<kBins>(a.status, ntiles, blockIdx.x - (gridDim.x - kScanCtas), a.err, reinterpret_cast<uint32_t*>(smem));
+  if (blockIdx.x < kScanCtas) {
+    scan_tiles<kBins>(a.status, ntiles, blockIdx.x, a.err, reinterpret_cast<uint32_t*>(smem));
     return;
   }
   uint16_t* my_wh = wh + warp * kBins;
@@ -655,29 +660,21 @@ uint32_t hist_grid(uint32_t m) {
   return grid ? grid : 1;
 }
 
-// One cooperative launch of a pass: CTAs that take tiles while they last,
-// plus the scan CTAs (all resident).
-cudaError_t launch_pass(const void* fn, bool depth, const void* kin, const uint32_t* vin, void* kout, uint32_t* vout,
-                        onesweep::PassArgs& a, cudaStream_t s) {
+// One launch of a pass: the scan CTAs, and CTAs that take tiles while they
+// last (all resident).
+template <typename K, typename Fn>
+cudaError_t launch_pass(Fn fn, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, onesweep::PassArgs& a,
+                        cudaStream_t s) {
   using namespace onesweep;
+  constexpr bool depth = sizeof(K) == 4;
   const uint32_t resident = pass_grid(depth);
   if (resident < 2 * kScanCtas) return cudaErrorInvalidConfiguration;
   const uint32_t grid = (a.ntiles < resident - kScanCtas ? a.ntiles : resident - kScanCtas) + kScanCtas;
-  void* args[] = {(void*)&kin, (void*)&vin, (void*)&kout, (void*)&vout, (void*)&a};
   const size_t smem = pass_smem(depth);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+  if (cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(smem)) != cudaSuccess)
     return cudaErrorInvalidConfiguration;
-  return cudaLaunchKernelExC(&cfg, fn, args);
+  return launch_after(fn, grid, kThreads, smem, s, kin, vin, kout, vout, a);
 }
 
 onesweep::Digit make_digit(uint32_t shift, uint32_t mask, bool drop31) {
@@ -702,14 +699,15 @@ onesweep::Digit make_digit(uint32_t shift, uint32_t mask, bool drop31) {
 }
 
 // The pass kernel for a digit form and the next pass's digit form.
+using PassFn = void (*)(const uint64_t*, const uint32_t*, uint64_t*, uint32_t*, onesweep::PassArgs);
 template <int kMode>
-const void* pass_kernel(uint32_t next) {
+PassFn pass_kernel(uint32_t next) {
   using namespace onesweep;
   switch (next) {
-    case kDigitLo: return reinterpret_cast<const void*>(&k_onesweep_pass<kMode, kDigitLo>);
-    case kDigitHi: return reinterpret_cast<const void*>(&k_onesweep_pass<kMode, kDigitHi>);
-    case kDigitSpan: return reinterpret_cast<const void*>(&k_onesweep_pass<kMode, kDigitSpan>);
-    default: return reinterpret_cast<const void*>(&k_onesweep_pass<kMode, kDigitNone>);
+    case kDigitLo: return &k_onesweep_pass<kMode, kDigitLo>;
+    case kDigitHi: return &k_onesweep_pass<kMode, kDigitHi>;
+    case kDigitSpan: return &k_onesweep_pass<kMode, kDigitSpan>;
+    default: return &k_onesweep_pass<kMode, kDigitNone>;
   }
 }
 }  // namespace
@@ -745,8 +743,7 @@ cudaError_t launch_onesweep_hist(const SortPlan& plan, const uint64_t* keys, uin
   a.err = err;
   const uint32_t grid = hist_grid(m);
   if (grid == 0) return cudaErrorInvalidDevice;
-  k_onesweep_hist<kDigitLo><<<grid, kHistThreads, 0, s>>>(keys, a);
-  return cudaGetLastError();
+  return launch_after(k_onesweep_hist<kDigitLo>, grid, kHistThreads, 0, s, keys, a);
 }
 
 cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint64_t* kin, const uint32_t* vin,
@@ -762,10 +759,10 @@ cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint
   pass_layout(a, pass, has_next, scratch);
   a.err = err;
   const uint32_t next = has_next ? a.dgn.mode : static_cast<uint32_t>(kDigitNone);
-  const void* fn = a.dg.mode == kDigitLo   ? pass_kernel<kDigitLo>(next)
-                   : a.dg.mode == kDigitHi ? pass_kernel<kDigitHi>(next)
-                                           : pass_kernel<kDigitSpan>(next);
-  return launch_pass(fn, false, kin, vin, kout, vout, a, s);
+  const PassFn fn = a.dg.mode == kDigitLo   ? pass_kernel<kDigitLo>(next)
+                    : a.dg.mode == kDigitHi ? pass_kernel<kDigitHi>(next)
+                                            : pass_kernel<kDigitSpan>(next);
+  return launch_pass<uint64_t>(fn, kin, vin, kout, vout, a, s);
 }
 
 cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, bool by_view,
@@ -781,8 +778,7 @@ cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_
   a.err = err;
   const uint32_t grid = hist_grid(n);
   if (grid == 0) return cudaErrorInvalidDevice;
-  k_onesweep_hist<kDigitDepth><<<grid, kHistThreads, 0, s>>>(keys, a);
-  return cudaGetLastError();
+  return launch_after(k_onesweep_hist<kDigitDepth>, grid, kHistThreads, 0, s, keys, a);
 }
 
 cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uint32_t* const dv[3], uint32_t n,
@@ -811,7 +807,7 @@ cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uin
     a.dv[i] = dv[i];
   }
   a.err = err;
-  return launch_pass(depth_pass_kernel(), true, nullptr, nullptr, nullptr, nullptr, a, s);
+  return launch_pass<uint32_t>(k_onesweep_pass<kDigitDepth, kDigitDepth>, nullptr, nullptr, nullptr, nullptr, a, s);
 }
 
 }  // namespace tdgs

@@ -96,7 +96,7 @@ __device__ __forceinline__ uint32_t cta_excl_scan(uint32_t v, uint32_t* s_warp) 
   return r;
 }
 
-// The scan CTAs: the last scan_ctas<kBins>() CTAs of the grid take no tiles; scan
+// The scan CTAs: the first scan_ctas<kBins>() CTAs of the grid take no tiles; scan
 // CTA c owns digits [64 c, 64 c + 64).  Lane l of every warp owns digit
 // pair 64 c + 2 l, +1; warp w reads rows (tiles) k + 8 w .. k + 8 w + 7 of
 // it, so one round reads 64 rows per pair at once (one L2 round trip).

@@ -13,6 +13,7 @@ namespace {
 __global__ void __launch_bounds__(256)
     k_preprocess(const float4* __restrict__ g, const float4* __restrict__ cov, uint32_t n, CameraDev cam,
                  float4* __restrict__ rec, float4* __restrict__ conic) {
+  begin_launch();
   const float2 lim = proj::slope_limits(cam);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float4 p = __ldg(g + i);
@@ -32,8 +33,7 @@ cudaError_t launch_preprocess(const float4* g, const float4* cov, uint32_t n, co
   if (n == 0) return cudaSuccess;
   const uint32_t blocks = (n + 255) / 256;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
-  k_preprocess<<<grid, 256, 0, s>>>(g, cov, n, cam, rec, conic);
-  return cudaGetLastError();
+  return launch_after(k_preprocess, grid, 256, 0, s, g, cov, n, cam, rec, conic);
 }
 
 }  // namespace tdgs

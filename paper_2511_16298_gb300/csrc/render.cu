@@ -37,8 +37,7 @@
 //    112 (300k, 640x360) and 517 -> 441 (700k, 3840x2160).  The bound of 6
 //    blocks per SM holds the kernel at 40 registers (64 without it: 242, 122
 //    and 524 us); 8 blocks spill and measure the same.
-//  * the order kernel keeps its tiles' counts in registers, and the blend is
-//    launched while it runs (programmatic dependent launch).
+//  * the order kernel keeps its tiles' counts in registers.
 //
 // Per pixel (sample point = the pixel's integer coordinate), in float32
 // with CUDA's fast exponential and multiply-adds (the result is compared
@@ -135,7 +134,7 @@ __device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, floa
 // permutation of 0 .. tiles-1.
 __global__ void __launch_bounds__(kOrderThreads)
     k_render_order(const uint2* __restrict__ ranges, uint32_t tiles, uint32_t* __restrict__ order) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (k_render waits for this launch's end)
+  begin_launch();
   __shared__ uint32_t s_max[kOrderThreads / 32];
   __shared__ uint32_t s_cnt[kOrderBuckets];
   const uint32_t t = threadIdx.x;
@@ -202,7 +201,7 @@ __global__ void __launch_bounds__(kRenderThreads, 6)
   __shared__ float4 s_rgb[kRenderThreads];
   __shared__ uint8_t s_mask[kRenderThreads];                 // warps each staged Gaussian reaches
   __shared__ uint16_t s_list[kRenderWarps][kRenderThreads];  // per warp: staged Gaussians to blend, as byte offsets
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  begin_launch();
   const uint32_t tile = order ? order[blockIdx.x] : blockIdx.x, t = threadIdx.x;
   const uint32_t warp = t >> 5, lane = t & 31;
   const uint32_t tx = (tile % gx) * 16, ty = (tile / gx) * 16;
@@ -293,8 +292,7 @@ __global__ void __launch_bounds__(kRenderThreads, 6)
 
 cudaError_t launch_render_order(const uint2* ranges, uint32_t tiles, uint32_t* order, cudaStream_t s) {
   if (tiles == 0) return cudaSuccess;
-  k_render_order<<<1, kOrderThreads, 0, s>>>(ranges, tiles, order);
-  return cudaGetLastError();
+  return launch_after(k_render_order, 1, kOrderThreads, 0, s, ranges, tiles, order);
 }
 
 cudaError_t launch_render_ordered(const float4* rec, const float4* conic, const float* rgb, const uint32_t* values,
@@ -303,18 +301,8 @@ cudaError_t launch_render_ordered(const float4* rec, const float4* conic, const 
   const uint32_t gx = (width + 15) / 16, gy = (height + 15) / 16;
   const uint32_t tiles = gx * gy;
   if (tiles == 0) return cudaSuccess;
-  // the blend may be set up while the order kernel still runs (it waits for its end)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tiles);
-  cfg.blockDim = dim3(kRenderThreads);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = order ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_render, rec, conic, rgb, values, ranges, order, gx, width, height,
-                            make_float3(bg[0], bg[1], bg[2]), n, image, err);
+  return launch_after(k_render, tiles, kRenderThreads, 0, s, rec, conic, rgb, values, ranges, order, gx, width, height,
+                      make_float3(bg[0], bg[1], bg[2]), n, image, err);
 }
 
 cudaError_t launch_render(const float4* rec, const float4* conic, const float* rgb, const uint32_t* values,
