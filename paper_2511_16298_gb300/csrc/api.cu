@@ -115,6 +115,7 @@ struct tdgs_context {
   Buffer os_scratch;  // onesweep sort: histograms, digit starts, tickets, look-back status
   Buffer f_dsort;     // single-launch depth sort: barrier counters, totals, rows (kept zero between launches)
   Buffer f_dos;       // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
+  Buffer f_raw;       // its first pass's digit counts (zero between frames)
   // State that kernels keep between launches, to be cleared before its next
   // use after an error was latched on the device (a bounded wait may have
   // given up mid-launch): the depth sort's buffers, the onesweep header, the
@@ -549,7 +550,7 @@ void tdgs_context_destroy(tdgs_context* ctx) {
   DeviceGuard g(ctx->device);
   drain_timings(ctx);
   for (cudaEvent_t e : ctx->free_events) cudaEventDestroy(e);
-  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort, &ctx->f_dos, &ctx->f_counts, &ctx->f_dkey[0],
+  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort, &ctx->f_dos, &ctx->f_raw, &ctx->f_counts, &ctx->f_dkey[0],
                     &ctx->f_dkey[1],    &ctx->f_dkey[2],     &ctx->f_dval[0],    &ctx->f_dval[1],
                     &ctx->f_dval[2],    &ctx->f_soff,       &ctx->f_sdo,        &ctx->f_rec3,
                     &ctx->f_conic,      &ctx->d_cams,       &ctx->diag,       &ctx->b_keys,       &ctx->b_vals,       &ctx->n_counts,
@@ -843,8 +844,9 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   if (st == TDGS_OK && dp.onesweep) {
     grown = false;
     st = ensure(ctx, ctx->f_dos, onesweep_scratch_words(n_all ? n_all : 1, by_view(ctx)) * 4, s, &grown);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_raw, (kRawBins + 1) * 4, s, &grown);
     if (st == TDGS_OK && (grown || ctx->dos_dirty)) {
-      TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_dos.p, 0, onesweep_header_words() * 4, s));
+      TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_raw.p, 0, (kRawBins + 1) * 4, s));
       ctx->dos_dirty = false;
     }
   }
@@ -925,30 +927,35 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
     if (early_total) TDGS_CUDA(ctx, cudaEventRecord(ctx->ev_count, s));
     return TDGS_OK;
   }
+  uint32_t* raw = static_cast<uint32_t*>(ctx->f_raw.p);
+  DepthPrep prep{};
+  if (dp.onesweep) {
+    prep = depth_onesweep_prep(n_all, by_view(ctx), static_cast<uint32_t*>(ctx->f_dos.p), raw);
+    if (ctx->norm) prep.raw = nullptr;  // the normalised keys are counted later
+  }
   // launched even for zero Gaussians: it writes the view starts and M = 0
   TDGS_TRACED(ctx, ctx->proj_on ? kKPreCount : kKFrameCount, n_all ? n_all : 1, s,
-              launch_views_count(vt, n_all, counts, dk[0], dv[0], err_word(ctx), ctx->d_tickets + 1,
+              launch_views_count(vt, n_all, ctx->split ? nullptr : counts, dk[0],
+                                 dp.resident || dp.onesweep ? nullptr : dv[0], err_word(ctx), ctx->d_tickets + 1,
                                  &ctx->d_status->total, ctx->d_range, early_total ? ctx->d_early : nullptr, s,
-                                 ctx->proj_on ? &ctx->proj : nullptr));
+                                 prep, ctx->proj_on ? &ctx->proj : nullptr));
   if (early_total) {
     // M (and any latched error) as soon as the count kernel is done: the
     // kernel wrote them to the mapped host status (h_early)
     TDGS_CUDA(ctx, cudaEventRecord(ctx->ev_count, s));
   }
-  if (ctx->norm) TDGS_TRACED(ctx, kKNormKeys, n_all, s, launch_norm_keys(dk[0], n_all, ctx->d_range, range, s));
+  if (ctx->norm) TDGS_TRACED(ctx, kKNormKeys, n_all, s, launch_norm_keys(dk[0], n_all, ctx->d_range, range, dp.onesweep ? raw : nullptr, s));
   const uint32_t dpasses = dp.passes;
   uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
   if (dp.resident) {  // one launch: the sort (pass count from the depth range) and the offsets
     da.key0 = dk[0];
     TDGS_TRACED(ctx, kKDepthSort, n_all, s, launch_depth_sort(dp.grid, dp.items, da, s));
-  } else if (dp.onesweep) {  // histogram, then the passes the key range needs (result in pair 1)
+  } else if (dp.onesweep) {  // the passes that the key range needs, and the one by view
     if (n_all) {
       uint32_t* dos = static_cast<uint32_t*>(ctx->f_dos.p);
-      TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                  launch_depth_onesweep_hist(dk[0], n_all, range, by_view(ctx), dos, err_word(ctx), s));
       for (uint32_t p = 0; p < dpasses; ++p)
         TDGS_TRACED(ctx, kKDepthSort, n_all, s,
-                    launch_depth_onesweep_pass(p, dk, dv, n_all, range, by_view(ctx) ? ctx->nv : 0u,
+                    launch_depth_onesweep_pass(p, dk, dv, n_all, range, raw, by_view(ctx) ? ctx->nv : 0u,
                                                ctx->d_views->rec_begin, ctx->d_views->n, dos, err_word(ctx), s));
     }
   } else {
@@ -1143,11 +1150,10 @@ tdgs_status sort_views_exact(tdgs_context* ctx, cudaStream_t s, uint32_t* m_out)
 
 // Per-view results, read after the work on `s` is complete.
 tdgs_status fill_results(tdgs_context* ctx, tdgs_view_result* results, uint32_t nv, cudaStream_t s) {
-  tdgs_status st = read_and_clear_error(ctx, s);
-  if (st != TDGS_OK) return st;
   TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->h_views->pbeg, ctx->d_views->pbeg, sizeof(uint32_t) * (nv + 1),
                                  cudaMemcpyDeviceToHost, s));
-  TDGS_CUDA(ctx, cudaStreamSynchronize(s));
+  tdgs_status st = read_and_clear_error(ctx, s);  // waits for both copies
+  if (st != TDGS_OK) return st;
   const uint64_t* k = static_cast<const uint64_t*>(ctx->f_keys.p);
   const uint32_t* v = static_cast<const uint32_t*>(ctx->f_values.p);
   const tdgs_range* r = static_cast<const tdgs_range*>(ctx->f_ranges.p);

@@ -327,8 +327,12 @@ cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t 
 // Four keys per thread.  The normalised depths are 0 .. 1023 whatever the
 // frame, so their range is constant.
 __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, uint32_t n,
-                                                   const uint32_t* __restrict__ range, uint32_t* __restrict__ out) {
+                                                   const uint32_t* __restrict__ range, uint32_t* __restrict__ out,
+                                                   uint32_t* __restrict__ raw) {
+  __shared__ uint32_t s_raw[kRawBins + 1];
   begin_launch();
+  for (uint32_t i = threadIdx.x; i <= kRawBins; i += blockDim.x) s_raw[i] = 0;
+  __syncthreads();
   const float dmin = __uint_as_float(__ldcg(range + 2));
   const float scale = norm_scale(dmin, __uint_as_float(__ldcg(range + 3)));
   const uint32_t first = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
@@ -336,8 +340,15 @@ __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, 
   for (uint32_t u = 0; u < 4; ++u) {
     if (first + u < n) {
       const uint32_t k = keys[first + u];
-      if (k != 0xffffffffu) keys[first + u] = norm_depth(__uint_as_float(k), dmin, scale);
+      const uint32_t q = k != 0xffffffffu ? norm_depth(__uint_as_float(k), dmin, scale) : k;
+      if (k != 0xffffffffu) keys[first + u] = q;
+      if (raw) atomicAdd(&s_raw[k != 0xffffffffu ? q & (kRawBins - 1) : kRawBins], 1u);
     }
+  }
+  if (raw) {
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i <= kRawBins; i += blockDim.x)
+      if (s_raw[i]) atomicAdd(raw + i, s_raw[i]);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     out[2] = 0u;
@@ -345,9 +356,10 @@ __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, 
   }
 }
 
-cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, cudaStream_t s) {
+cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, uint32_t* raw,
+                             cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  return launch_after(k_norm_keys, (n + 1023) / 1024, 256, 0, s, keys, n, range, out);
+  return launch_after(k_norm_keys, (n + 1023) / 1024, 256, 0, s, keys, n, range, out, raw);
 }
 
 // ---------------------------------------------------------- tile ranges

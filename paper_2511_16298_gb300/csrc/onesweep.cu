@@ -135,8 +135,6 @@ struct HistArgs {
   uint32_t* done;      // block counter, zero on entry, left zero
   uint32_t* tickets;   // [kMaxPasses] tile tickets, cleared here
   uint32_t* status0;   // [ntiles][kBins] look-back status of pass 0, cleared here
-  uint32_t* status_view;  // the same of a last pass by view, or null
-  uint32_t* range;     // depth keys: the key range (range[2..3]); the pass count goes to range[4]
   uint32_t* err;
 };
 
@@ -153,7 +151,8 @@ struct PassArgs {
   // depth keys: the pass number, the key range and the three key and value
   // buffers (0: input; the last pass that runs writes buffer 1)
   uint32_t pass;
-  const uint32_t* range;
+  uint32_t* range;  // (pass 0 writes the pass count to range[4])
+  uint32_t* raw;    // [kRawBins + 1] the keys' low 9 bits counted, culled keys; cleared by pass 1
   uint32_t* dk[3];
   uint32_t* dv[3];
   // a batch to be ordered view after view: its views (0: none) and their
@@ -174,9 +173,7 @@ struct PassArgs {
 // into L2 while it counts.  Few blocks (4 per SM) keep the final global
 // atomics on the counters few.
 constexpr int kHistThreads = 512;
-template <int kMode>
-__global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMode>* __restrict__ keys, HistArgs a) {
-  using K = KeyOf<kMode>;
+__global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const uint64_t* __restrict__ keys, HistArgs a) {
   __shared__ uint32_t h[kBins];
   __shared__ uint32_t s_warp[kHistThreads / 32];
   __shared__ bool s_last;
@@ -195,19 +192,10 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMod
     for (size_t i = static_cast<size_t>(blockIdx.x) * kHistThreads + t; i < nz;
          i += static_cast<size_t>(gridDim.x) * kHistThreads)
       z[i] = make_uint4(0, 0, 0, 0);
-    if (uint4* zv = reinterpret_cast<uint4*>(a.status_view))
-      for (size_t i = static_cast<size_t>(blockIdx.x) * kHistThreads + t; i < nz;
-           i += static_cast<size_t>(gridDim.x) * kHistThreads)
-        zv[i] = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
   const uint32_t m = a.m;
-  Digit dg0 = a.dg[0];  // 64-bit keys: the first digit is bits [0, width) of the low word
-  if constexpr (kMode == kDigitDepth) {
-    const DepthDigits dd = depth_digits(a.range);
-    dg0 = Digit{kDigitDepth, 0u, 0u, dd.mask, dd.lo, dd.cull};
-    if (blockIdx.x == 0 && t == 0) a.range[4] = dd.passes;  // for the host's diagnostics
-  }
+  const Digit dg0 = a.dg[0];  // the first digit is bits [0, width) of the low word
   const bool vec = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
   constexpr uint32_t kStep = 8 * kHistThreads;  // keys per block and step: 8 consecutive per thread
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kStep;
@@ -216,35 +204,24 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMod
     if (t == 0 && base + stride < m)  // the next step's keys into L2 while this step counts
       radix::prefetch_l2(keys + base + stride, (min(static_cast<uint64_t>(kStep), m - (base + stride))) * 8);
     const uint64_t i0 = base + 8 * t;
-    K k[8];
+    uint64_t k[8];
     if (vec && i0 + 8 <= m) {
-      if constexpr (sizeof(K) == 8) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint4 w = __ldcs(reinterpret_cast<const uint4*>(keys + i0) + u);
-          k[2 * u] = (static_cast<uint64_t>(w.y) << 32) | w.x;
-          k[2 * u + 1] = (static_cast<uint64_t>(w.w) << 32) | w.z;
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const uint4 w = __ldcs(reinterpret_cast<const uint4*>(keys + i0) + u);
-          k[4 * u] = w.x;
-          k[4 * u + 1] = w.y;
-          k[4 * u + 2] = w.z;
-          k[4 * u + 3] = w.w;
-        }
+      for (int u = 0; u < 4; ++u) {
+        const uint4 w = __ldcs(reinterpret_cast<const uint4*>(keys + i0) + u);
+        k[2 * u] = (static_cast<uint64_t>(w.y) << 32) | w.x;
+        k[2 * u + 1] = (static_cast<uint64_t>(w.w) << 32) | w.z;
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) k[j] = i0 + j < m ? keys[i0 + j] : K(0);
+      for (int j = 0; j < 8; ++j) k[j] = i0 + j < m ? keys[i0 + j] : 0ull;
     }
     uint32_t run_d = 0, run_n = 0;  // runs of equal digits: one atomic each
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       if (i0 + j < m) {
-        if constexpr (kMode != kDigitDepth) bad |= (k[j] & a.bad_mask) != 0;
-        const uint32_t d = digit_m<kMode>(k[j], dg0);
+        bad |= (k[j] & a.bad_mask) != 0;
+        const uint32_t d = digit_m<kDigitLo>(k[j], dg0);
         if (run_n && d != run_d) {
           atomicAdd(&h[run_d], run_n);
           run_n = 0;
@@ -274,15 +251,15 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const KeyOf<kMod
 }
 
 // One tile's keys and values (first `nbulk` pairs, a multiple of 4) by bulk
-// copies completing on `bar`.
+// copies completing on `bar`; keys only if `iota` (the values are positions).
 template <typename K>
 __device__ __forceinline__ void load_tile(TileBuf<K>* b, uint64_t* bar, const K* kin, const uint32_t* vin,
-                                          uint32_t first, uint32_t nbulk) {
-  const uint32_t kb = nbulk * static_cast<uint32_t>(sizeof(K)), vb = nbulk * 4;
+                                          uint32_t first, uint32_t nbulk, bool iota) {
+  const uint32_t kb = nbulk * static_cast<uint32_t>(sizeof(K)), vb = iota ? 0u : nbulk * 4;
   mbar_arrive(bar, kb + vb);
   if (nbulk) {
     bulk_g2s(b->k, kin + first, kb, bar);
-    bulk_g2s(b->v, vin + first, vb, bar);
+    if (!iota) bulk_g2s(b->v, vin + first, vb, bar);
   }
 }
 
@@ -355,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ uint32_t s_warp[kWarps];
   __shared__ uint32_t s_begin[kMode == kDigitDepth ? kMaxViews + 1 : 1];
   bool to_view = false;  // the last depth pass of a batch in view order
+  bool iota = false;     // the first depth pass: values are the records' positions
 
   begin_launch();
   Digit dg = a.dg, dgn = a.dgn;
@@ -369,7 +347,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (a.view_pass) {
       dg = Digit{kDigitDepth, 0u, 0u, kBins - 1u, 0u, 0u};  // keys are views
     } else {
+      if (blockIdx.x == 0) {
+        if (a.pass == 0 && threadIdx.x == 0) a.range[4] = dd.passes;  // for the host's diagnostics
+        if (a.pass == 1)  // read by the pass before
+          for (uint32_t i = threadIdx.x; i <= kRawBins; i += kThreads) a.raw[i] = 0u;
+      }
       if (a.pass >= dd.passes) return;
+      iota = a.pass == 0;
       dg = Digit{kDigitDepth, a.pass * dd.width, 0u, dd.mask, dd.lo, dd.cull};
       dgn = dg;
       dgn.msh += dd.width;
@@ -406,7 +390,22 @@ __global__ void __launch_bounds__(kThreads, 2)
     hn[2 * t + 1] = 0;
   }
   uint32_t g0, g1;  // this pass's first output position of digits 2t and 2t+1
-  if (a.gstart) {
+  if (kMode == kDigitDepth && iota) {
+    // the first digit's counts: of (key - lo) & mask, a rotation of the keys'
+    // low 9 bits (mask has at most 9); the culled keys' digit is cull & mask
+    lstart[2 * t] = lstart[2 * t + 1] = 0u;
+    __syncthreads();
+    for (uint32_t i = t; i < kRawBins; i += kThreads)
+      if (const uint32_t c = __ldcg(a.raw + i)) atomicAdd(&lstart[(i - dg.lo) & dg.mask], c);
+    if (t == 0) {
+      const uint32_t c = __ldcg(a.raw + kRawBins);
+      if (c) atomicAdd(&lstart[dg.cull & dg.mask], c);
+    }
+    __syncthreads();
+    const uint32_t h0 = lstart[2 * t], h1 = lstart[2 * t + 1];
+    g0 = cta_excl_scan(h0 + h1, s_warp);
+    g1 = g0 + h0;
+  } else if (a.gstart) {
     g0 = __ldg(a.gstart + 2 * t);
     g1 = __ldg(a.gstart + 2 * t + 1);
   } else {
@@ -426,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     const uint32_t first = atomicAdd(a.ticket, 1u);
     s_tile[1] = first;
-    if (first < ntiles) load_tile(&buf[0], &mbar[0], kin, vin, first * kTileKeys, bulk_items(first));
+    if (first < ntiles) load_tile(&buf[0], &mbar[0], kin, vin, first * kTileKeys, bulk_items(first), iota);
   }
   __syncthreads();
   uint32_t cur = s_tile[1];
@@ -465,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t nb = valid & ~3u;
         if (t < valid - nb) {
           tb.k[nb + t] = kin[first + nb + t];
-          tb.v[nb + t] = vin[first + nb + t];
+          if (!iota) tb.v[nb + t] = vin[first + nb + t];
         }
         __syncthreads();
       }
@@ -475,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       if (t == 0 && nxt < ntiles) {
         const uint32_t nf = nxt * kTileKeys, nv = min(kTileKeys, m - nf);
         radix::prefetch_l2(kin + nf, static_cast<uint64_t>(nv) * 8);
-        radix::prefetch_l2(vin + nf, static_cast<uint64_t>(nv) * 4);
+        if (!iota) radix::prefetch_l2(vin + nf, static_cast<uint64_t>(nv) * 4);
       }
       __syncthreads();
       // ---- per-digit counts (column t holds digits 2t and 2t+1), prefixes over warps
@@ -507,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t idx = wbase + j * 32 + lane;
         if (idx < valid) {
           kr[j] = tb.k[idx];
-          vr[j] = tb.v[idx];
+          vr[j] = iota ? first + idx : tb.v[idx];
           const uint32_t dd = digit_m<kMode>(kr[j], dg);
           const uint32_t sd = slot<kSwz>(dd);
           r[j] += lstart[sd] + my_wh[sd];
@@ -562,7 +561,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();  // buf[b ^ 1] is free; the next tile's number is visible
     if (t == 0 && nxt < ntiles) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      load_tile(&buf[b ^ 1u], &mbar[b ^ 1u], kin, vin, nxt * kTileKeys, bulk_items(nxt));
+      load_tile(&buf[b ^ 1u], &mbar[b ^ 1u], kin, vin, nxt * kTileKeys, bulk_items(nxt), iota);
     }
     have_prev = have_cur;
     if (have_cur) {
@@ -743,7 +742,7 @@ cudaError_t launch_onesweep_hist(const SortPlan& plan, const uint64_t* keys, uin
   a.err = err;
   const uint32_t grid = hist_grid(m);
   if (grid == 0) return cudaErrorInvalidDevice;
-  return launch_after(k_onesweep_hist<kDigitLo>, grid, kHistThreads, 0, s, keys, a);
+  return launch_after(k_onesweep_hist, grid, kHistThreads, 0, s, keys, a);
 }
 
 cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint64_t* kin, const uint32_t* vin,
@@ -765,24 +764,21 @@ cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint
   return launch_pass<uint64_t>(fn, kin, vin, kout, vout, a, s);
 }
 
-cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, bool by_view,
-                                       uint32_t* scratch, uint32_t* err, cudaStream_t s) {
+DepthPrep depth_onesweep_prep(uint32_t n, bool by_view, uint32_t* scratch, uint32_t* raw) {
   using namespace onesweep;
-  HistArgs a{};
-  a.m = n;
-  a.passes = 1;
-  a.ntiles = (n + kTileKeys - 1) / kTileKeys;
-  a.range = range;
-  scratch_layout(a, scratch);
-  if (by_view) a.status_view = view_status(scratch, a.ntiles);
-  a.err = err;
-  const uint32_t grid = hist_grid(n);
-  if (grid == 0) return cudaErrorInvalidDevice;
-  return launch_after(k_onesweep_hist<kDigitDepth>, grid, kHistThreads, 0, s, keys, a);
+  const uint32_t ntiles = (n + kTileKeys - 1) / kTileKeys;
+  DepthPrep p{};
+  p.raw = raw;
+  p.header = scratch;
+  p.header_words = static_cast<uint32_t>(onesweep_header_words());
+  p.status0 = scratch + onesweep_header_words();
+  p.status_view = by_view ? view_status(scratch, ntiles) : nullptr;
+  p.status_quads = static_cast<size_t>(ntiles) * kBins / 4;
+  return p;
 }
 
 cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uint32_t* const dv[3], uint32_t n,
-                                       const uint32_t* range, uint32_t nv, const uint32_t* rec_begin,
+                                       uint32_t* range, uint32_t* raw, uint32_t nv, const uint32_t* rec_begin,
                                        const uint32_t* view_counts, uint32_t* scratch, uint32_t* err,
                                        cudaStream_t s) {
   using namespace onesweep;
@@ -802,6 +798,7 @@ cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uin
   }
   a.pass = pass;
   a.range = range;
+  a.raw = raw;
   for (int i = 0; i < 3; ++i) {
     a.dk[i] = dk[i];
     a.dv[i] = dv[i];

@@ -193,7 +193,9 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
 // depth instead of duplicating: keys (the count kernel's depth bits, all ones
 // without pairs) become normalised depths over range[2..3], and out[2..3]
 // receives their own range for the depth sort.
-cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, cudaStream_t s);
+// raw: as DepthPrep's, of the new keys, or null.
+cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, uint32_t* raw,
+                             cudaStream_t s);
 cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t num_tiles, uint2* ranges,
                                     uint32_t* err, cudaStream_t s);
 
@@ -284,13 +286,26 @@ struct Proj3D {
   CameraDev cam0;         // cams[0], passed by value (kernel parameter space) for one view
 };
 
+// What the count kernel prepares for the onesweep depth sort (all null: the
+// depth sort is another): its counters and status words cleared, and the
+// keys' low 9 bits counted into raw (zero on entry; raw[512]: culled keys).
+constexpr uint32_t kRawBins = 512;
+struct DepthPrep {
+  uint32_t* raw;
+  uint32_t* header;
+  uint32_t header_words;
+  uint32_t* status0;
+  uint32_t* status_view;
+  size_t status_quads;  // 16-byte words of each
+};
+
 // host_status (optional): device address of mapped pinned memory that
 // also receives {uint64 pair count, uint32 error, uint32 site} from the
 // last block (the host reads it after an event on the kernel, no copy).
 cudaError_t launch_views_count(const ViewTable& vt, uint32_t n_all, uint32_t* counts,
                                uint32_t* dkey, uint32_t* dval, uint32_t* err, uint32_t* ticket,
                                uint64_t* total, uint32_t* range, void* host_status, cudaStream_t s,
-                               const Proj3D* proj = nullptr);
+                               const DepthPrep& prep, const Proj3D* proj = nullptr);
 // sdo: receives {depth key, record index} per depth position (read by the
 // expanding tile pass with one 8-byte load per pair).
 cudaError_t launch_views_dup(const ViewTable& vt, const uint32_t* sorder, const uint32_t* soff,
@@ -520,10 +535,9 @@ constexpr uint32_t kDepthOnesweepPasses = 4;  // 32 bits in 9-bit digits
 // kDepthOnesweepPasses sorts by view at the end (rec_begin: [nv+1] first
 // record of each view; view_counts: 512 words, the views' records and zeros),
 // the scratch is sized with by_view, and the result is in dk[2], dv[2].
-cudaError_t launch_depth_onesweep_hist(const uint32_t* keys, uint32_t n, uint32_t* range, bool by_view,
-                                       uint32_t* scratch, uint32_t* err, cudaStream_t s);
+DepthPrep depth_onesweep_prep(uint32_t n, bool by_view, uint32_t* scratch, uint32_t* raw);
 cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uint32_t* const dv[3], uint32_t n,
-                                       const uint32_t* range, uint32_t nv, const uint32_t* rec_begin,
+                                       uint32_t* range, uint32_t* raw, uint32_t nv, const uint32_t* rec_begin,
                                        const uint32_t* view_counts, uint32_t* scratch, uint32_t* err,
                                        cudaStream_t s);
 
