@@ -485,15 +485,16 @@ class Context:
         return arr
 
     def _results(self, res, n, copy):
-        out = []
-        for i in range(n):
-            r = res[i]
-            k = _view(r.keys or 0, r.m, torch.int64, self.device)
-            v = _view(r.values or 0, r.m, torch.int32, self.device)
-            rg = _view(r.ranges or 0, 2 * r.num_tiles, torch.int32, self.device).view(r.num_tiles, 2)
-            if copy:
-                k, v, rg = k.clone(), v.clone(), rg.clone()
-            out.append((k, v, rg, int(r.m)))
+        # the views' lists lie one after the other in the context's buffers:
+        # one tensor over each buffer, split (a batch of 16 views made 48
+        # tensors one by one in a fifth of its time)
+        m, tiles = [res[i].m for i in range(n)], [res[i].num_tiles for i in range(n)]
+        k = _view(res[0].keys or 0, sum(m), torch.int64, self.device).split(m)
+        v = _view(res[0].values or 0, sum(m), torch.int32, self.device).split(m)
+        rg = _view(res[0].ranges or 0, 2 * sum(tiles), torch.int32, self.device).view(-1, 2).split(tiles)
+        out = list(zip(k, v, rg, m))
+        if copy:
+            out = [(a.clone(), b.clone(), c.clone(), d) for a, b, c, d in out]
         return out
 
     def sort_views(self, views, copy: bool = False):
