@@ -64,14 +64,14 @@ enum KernelId {
   kKCount, kKScan, kKDuplicate, kKRanges, kKRadixPass,
   kKFrameCount, kKDepthSort, kKFrameScan, kKDupDepth, kKTilePass, kKTileExpand, kKPreprocess, kKBitonic, kKRender, kKPreCount, kKNormRange, kKNormDup, kKNormPass,
   kKNormRanges, kKRenderOrder, kKSortHist, kKOnesweep, kKCountDepth,
-  kKNormKeys, kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
+  kKNormKeys, kKSmallSplit, kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
 };
 const char* const kKernelNames[kKNum] = {
     "count_tiles",  "scan",       "duplicate_keys",     "tile_ranges",    "radix_pass",
     "frame_count",  "depth_sort", "scan_by_depth", "duplicate_by_depth", "tile_sort_pass",
     "tile_expand_pass", "preprocess", "bitonic_sort", "render", "preprocess_count", "norm_range",
     "norm_duplicate", "norm_sort_pass", "norm_ranges", "render_order", "sort_histogram", "onesweep_pass",
-    "count_depth_sort", "norm_keys", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
+    "count_depth_sort", "norm_keys", "small_split", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
 
 // View table as stored in device memory (SoA, fixed maximum size).
 struct ViewBlob {
@@ -772,6 +772,10 @@ bool splits(const tdgs_context* ctx) {
          ctx->tuning.tile_digit_bits == 0;
 }
 
+// A view of at most kSplitSmall Gaussians and kSmallTiles tiles of segments
+// takes one launch for all of it.
+constexpr uint32_t kSmallTiles = 1024;
+
 uint32_t split_pitch(const tdgs_context* ctx) { return (ctx->max_gx + 7u) & ~7u; }
 uint32_t split_rows(const tdgs_context* ctx) { return ctx->h_views->row_begin[ctx->nv]; }
 // Level-2 tiles of at most m segments: full ones, and one ragged one per row.
@@ -1011,10 +1015,15 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.cap = m;
   a.total = &ctx->d_status->total;
   a.ticket = ctx->d_tickets;
+  a.bar = ctx->d_tickets + 2;
   a.ntiles1 = ctx->h_views->t1_begin[ctx->nv];
   a.err = err_word(ctx);
   const uint32_t tiles2 = static_cast<uint32_t>(split_tiles(ctx, m));
   const int cps = ctx->tuning.ctas_per_sm;
+  if (ctx->nv == 1 && n_all > 0 && n_all <= kSplitSmall && tiles2 <= kSmallTiles) {
+    TDGS_TRACED(ctx, kKSmallSplit, m, s, launch_small_split(a, std::max(ctx->max_gx, ctx->max_gy), tiles2, s));
+    return TDGS_OK;
+  }
   TDGS_TRACED(ctx, kKRowCount, n_all, s, launch_row_count(a, s));
   TDGS_TRACED(ctx, kKRowScan, a.nrows, s, launch_row_scan(a, s));
   TDGS_TRACED(ctx, kKRowSplit, n_all, s, launch_row_split(a, ctx->max_gy, cps, s));

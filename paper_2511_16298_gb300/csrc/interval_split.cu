@@ -395,6 +395,149 @@ struct Smem {
   uint16_t pos[kBatches][kPitch];
   uint16_t cols[kTile];  // level 1: the items' columns
 };
+static_assert(sizeof(Smem<9>) < 220 * 1024, "one CTA fits an SM");
+
+// The steps after the load, for one tile whose counts and positions are in
+// s.lstart and s.off.  row_tile: level 2, the row's first tile in its view.
+// Starts and ends with a block barrier.
+template <int kLevel, int kWords>
+__device__ __forceinline__ void split_tile(Smem<kWords>& s, const SplitArgs& a, const uint32_t (&lo)[kPerWarp],
+                                           const uint32_t (&hi)[kPerWarp], uint32_t bins, uint32_t row_tile) {
+  constexpr int kBinsP = Smem<kWords>::kBinsP;
+  const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
+  // ---- masks
+#pragma unroll
+  for (int b = 0; b < kPerWarp; ++b) {
+    uint32_t* m = s.mask[warp * kPerWarp + b];
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) m[k * 32 + lane] = 0u;
+    __syncwarp();
+    if (hi[b] > lo[b]) {
+      atomicXor(m + lo[b], 1u << lane);
+      if (hi[b] < bins) atomicXor(m + hi[b], 1u << lane);
+    }
+    __syncwarp();
+    uint32_t x[kWords], own = 0;  // inclusive over this lane's bins, then over the lanes before
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) {
+      own ^= m[lane * kWords + k];
+      x[k] = own;
+    }
+    uint32_t before = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xffffffffu, before, d);
+      if (lane >= static_cast<uint32_t>(d)) before ^= o;
+    }
+    before ^= own;
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) m[lane * kWords + k] = x[k] ^ before;
+  }
+  __syncthreads();
+  const uint32_t total = s.lstart[kBinsP];
+  for (uint32_t b0 = 0; b0 < bins;) {
+    // bins [b0, b1): the whole tile, or as many as the stage holds
+    uint32_t b1 = bins;
+    const uint32_t p0 = s.lstart[b0];
+    if (total - p0 > kStage) {
+      b1 = b0 + 1;
+      while (b1 < bins && s.lstart[b1 + 1] - p0 <= kStage) ++b1;
+    }
+    const uint32_t np = s.lstart[b1] - p0;
+    // ---- prefix over the batches
+    for (uint32_t cw = b0 + warp * 8; cw < b1; cw += kWarps * 8) {  // eight bins a warp, four lanes each
+      const uint32_t c = cw + (lane >> 2);
+      constexpr int kEach = kBatches / 4;
+      const uint32_t g = t & 3u, cc = min(c, b1 - 1u);
+      uint32_t x[kEach], sum = 0;
+#pragma unroll
+      for (int i = 0; i < kEach; ++i) {
+        x[i] = __popc(s.mask[g * kEach + i][cc]);
+        sum += x[i];
+      }
+      uint32_t run = sum;
+#pragma unroll
+      for (int d = 1; d < 4; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, run, d, 4);
+        if (g >= static_cast<uint32_t>(d)) run += o;
+      }
+      run += s.lstart[cc] - p0 - sum;
+      if (c < b1) {
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+          s.pos[g * kEach + i][c] = static_cast<uint16_t>(run);
+          run += x[i];
+        }
+      }
+    }
+    __syncthreads();
+    // ---- expand
+#pragma unroll
+    for (int b = 0; b < kPerWarp; ++b) {
+      const uint32_t bat = warp * kPerWarp + b;
+      const uint32_t* m = s.mask[bat];
+      const uint16_t* ps = s.pos[bat];
+      const uint32_t l = max(lo[b], b0), h = min(hi[b], b1);
+      const uint32_t n = h > l ? h - l : 0u;
+      const uint32_t item0 = bat * 32;
+      const uint32_t full = __ballot_sync(0xffffffffu, n != 0u);
+      if ((full & (full + 1u)) == 0u) {
+        // Lane p of a step takes the batch's p-th pair: its owner is the
+        // last item that starts at or before it.  The starts that fall into
+        // the step's 32 pairs are one word, and the items are in lane order.
+        const uint32_t end = warp_incl_scan(n), st = end - n;
+        const uint32_t np_b = __shfl_sync(0xffffffffu, end, 31);
+        const uint32_t shift = l - st;            // bin of pair p of this item, less p
+        uint32_t at = n ? st : 0x80000000u;       // start relative to the step (never 0..31 if none)
+        uint32_t seen = 0xffffffffu;              // items that start before the step, less one
+        for (uint32_t p = lane; p < np_b + lane; p += 32, at -= 32) {
+          const uint32_t starts = __reduce_or_sync(0xffffffffu, bit_or_none(at));
+          const uint32_t src = seen + __popc(starts & le);
+          seen += __popc(starts);
+          const uint32_t c = p + __shfl_sync(0xffffffffu, shift, src);
+          if (p < np_b) s.stage[ps[c] + __popc(m[c] & low_bits(src))] = c * 65536u + (item0 + src);
+        }
+      } else {  // a window left items without bins between others: each lane walks its own
+        const uint32_t steps = __reduce_max_sync(0xffffffffu, n);
+        for (uint32_t j = 0; j < steps; ++j) {
+          const uint32_t c = l + j;
+          if (j < n) s.stage[ps[c] + __popc(m[c] & lt)] = c * 65536u + (item0 + lane);
+        }
+      }
+    }
+    __syncthreads();
+    // ---- flush
+    if constexpr (kLevel == 1) {
+#pragma unroll 2
+      for (uint32_t p = t; p < np; p += kThreads) {
+        const uint32_t e = s.stage[p], i = e & 0xffffu, dst = s.off[e >> 16] + p0 + p;
+        a.segs[dst] = s.pay[i];
+        a.cols[dst] = s.cols[i];
+      }
+    } else if (a.keys32) {
+#pragma unroll 2
+      for (uint32_t p = t; p < np; p += kThreads) {
+        const uint32_t e = s.stage[p], c = e >> 16;
+        const uint2 q = s.pay[e & 0xffffu];
+        const uint32_t dst = s.off[c] + p0 + p;
+        a.keys32[dst] = ((row_tile + c) << 10) | q.x;
+        a.values[dst] = q.y;
+      }
+    } else {
+#pragma unroll 2
+      for (uint32_t p = t; p < np; p += kThreads) {
+        const uint32_t e = s.stage[p], c = e >> 16;
+        const uint2 q = s.pay[e & 0xffffu];
+        const uint32_t dst = s.off[c] + p0 + p;
+        a.keys[dst] = (static_cast<uint64_t>(row_tile + c) << 32) | q.x;
+        a.values[dst] = q.y;
+      }
+    }
+    __syncthreads();
+    b0 = b1;
+  }
+}
 
 template <int kLevel, int kWords>
 __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArgs a) {
@@ -404,7 +547,6 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
   S& s = *reinterpret_cast<S*>(smem);
   begin_launch();
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
-  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
   if (__ldg(a.info + 1) == 0u) return;
   const uint32_t ntiles = kLevel == 1 ? a.ntiles1 : __ldg(a.info);
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -477,144 +619,248 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
       }
       if (lane == 31) s.lstart[kBinsP] = run;  // (all pairs; every bin past the last starts here too)
     }
-    // ---- masks
-#pragma unroll
-    for (int b = 0; b < kPerWarp; ++b) {
-      uint32_t* m = s.mask[warp * kPerWarp + b];
-#pragma unroll
-      for (int k = 0; k < kWords; ++k) m[k * 32 + lane] = 0u;
-      __syncwarp();
-      if (hi[b] > lo[b]) {
-        atomicXor(m + lo[b], 1u << lane);
-        if (hi[b] < bins) atomicXor(m + hi[b], 1u << lane);
+    split_tile<kLevel, kWords>(s, a, lo, hi, bins, kLevel == 2 ? (r - pl.row0) * bins : 0u);
+  }
+}
+
+// ------------------------------------------------------------- small frames
+// All of it for one small view in one cooperative launch: count, row split,
+// column split, with a grid barrier between them.  The scans and the column
+// counts need no phase of their own: every block sums the few tiles' counts of
+// all rows for level 1, and counts all segments of its tile's row for level 2
+// (at most kSplitSmall of them: the sums are kept in 16 bits).
+// What an earlier phase wrote is read through L2 (__ldcg).  A barrier that
+// times out ends the block: the counts that size the staging are then not to
+// be trusted.
+__device__ __forceinline__ bool small_barrier(uint32_t* bar, uint32_t* err) {
+  __shared__ bool s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bool ok = true;
+    const uint32_t gen = radix::ld_acquire32(bar + 1);
+    if (radix::atom_add_acq_rel32(bar, 1u) == gridDim.x - 1) {
+      bar[0] = 0u;  // ordered before the release below
+      radix::st_release32(bar + 1, gen + 1);
+    } else {
+      uint32_t spins = 0;
+      while (radix::ld_acquire32(bar + 1) == gen) {
+        if (++spins > kSpinLimit) {
+          latch_error(err, TDGS_ERR_TIMEOUT, kSiteBarrier);
+          ok = false;
+          break;
+        }
+        __nanosleep(20);
       }
-      __syncwarp();
-      uint32_t x[kWords], own = 0;  // inclusive over this lane's bins, then over the lanes before
+    }
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok;
+}
+
+template <int kWords>
+__global__ void __launch_bounds__(kThreads, 1) k_small(SplitArgs a) {
+  using S = Smem<kWords>;
+  constexpr int kBinsP = S::kBinsP;
+  extern __shared__ __align__(16) unsigned char smem[];
+  S& s = *reinterpret_cast<S*>(smem);
+  __shared__ uint32_t s_seg[kMaxBins + 1], s_tile[kMaxBins + 1], s_pair[kMaxBins];  // of each row: the first
+  __shared__ unsigned long long s_w[kWarps][2];
+  __shared__ uint32_t s_w32[kWarps][2];
+  int(*s_d)[2] = reinterpret_cast<int(*)[2]>(s.stage);  // differences of a count phase
+  static_assert(sizeof(s.stage) >= (kMaxBins + 1) * sizeof(int[2]), "the differences fit the stage");
+  static_assert(kThreads >= kMaxBins, "one bin per thread");
+  const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+  const FrameGeom fg = a.vt.one.geom;
+  const uint32_t n = a.vt.one.n, nt = a.ntiles1;
+  const uint32_t gx = static_cast<uint32_t>(fg.gx), gy = static_cast<uint32_t>(fg.gy);
+  const float4* __restrict__ g = a.vt.one.g;
+  constexpr int kPer = kTile / kThreads;
+  // ---- rectangles in depth order and the rows' counts
+  float dmin = 0.0f, scale = 0.0f;
+  if (a.keys32) {
+    dmin = __uint_as_float(__ldcg(a.norm));
+    scale = norm_scale(dmin, __uint_as_float(__ldcg(a.norm + 1)));
+  }
+  for (uint32_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+    if (t <= kMaxBins) s_d[t][0] = s_d[t][1] = 0;
+    __syncthreads();
 #pragma unroll
-      for (int k = 0; k < kWords; ++k) {
-        own ^= m[lane * kWords + k];
-        x[k] = own;
+    for (int u = 0; u < kPer; ++u) {
+      const uint32_t p = tile * kTile + u * kThreads + t;
+      if (p >= n) continue;
+      const uint32_t gi = __ldg(a.sorder + p);
+      const float4 rec = gi < n ? __ldg(g + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const TileRect q = tile_rect(rec, fg);
+      uint32_t pack = kEmptyRect;
+      if (q.count) {
+        const int w = q.x1 - q.x0;
+        pack = static_cast<uint32_t>(q.x0) | (static_cast<uint32_t>(q.x1 - 1) << 8) |
+               (static_cast<uint32_t>(q.y0) << 16) | (static_cast<uint32_t>(q.y1 - 1) << 24);
+        atomicAdd(&s_d[q.y0][0], 1);
+        atomicAdd(&s_d[q.y0][1], w);
+        atomicAdd(&s_d[q.y1][0], -1);
+        atomicAdd(&s_d[q.y1][1], -w);
       }
-      uint32_t before = own;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xffffffffu, before, d);
-        if (lane >= static_cast<uint32_t>(d)) before ^= o;
-      }
-      before ^= own;
-#pragma unroll
-      for (int k = 0; k < kWords; ++k) m[lane * kWords + k] = x[k] ^ before;
+      a.rects[p] = pack;
+      a.sdo[p] = make_uint2(a.keys32 ? norm_depth(rec.z, dmin, scale) : __float_as_uint(rec.z), gi);
     }
     __syncthreads();
-    const uint32_t total = s.lstart[kBinsP];
-    for (uint32_t b0 = 0; b0 < bins;) {
-      // bins [b0, b1): the whole tile, or as many as the stage holds
-      uint32_t b1 = bins;
-      const uint32_t p0 = s.lstart[b0];
-      if (total - p0 > kStage) {
-        b1 = b0 + 1;
-        while (b1 < bins && s.lstart[b1 + 1] - p0 <= kStage) ++b1;
+    unsigned long long c = t < kMaxBins ? static_cast<uint32_t>(s_d[t][0]) : 0u;
+    unsigned long long w = t < kMaxBins ? static_cast<uint32_t>(s_d[t][1]) : 0u;
+    block_incl_scan2<kWarps>(c, w, s_w);  // (differences modulo 2^32)
+    if (t < gy) a.c1[t * nt + tile] = make_uint2(static_cast<uint32_t>(c), static_cast<uint32_t>(w));
+    __syncthreads();
+  }
+  if (!small_barrier(a.bar, a.err)) return;
+  // ---- the rows' segments: every block finds all rows' starts, and its
+  // tile's positions in them
+  const uint64_t m = __ldcg(a.total);
+  uint32_t tile = blockIdx.x;
+  do {
+    uint32_t cnt = 0, before = 0, segs = 0, pairs = 0;
+    if (t < gy) {
+      for (uint32_t k = 0; k < nt; ++k) {
+        const uint2 x = __ldcg(a.c1 + t * nt + k);
+        segs += x.x;
+        pairs += x.y;
+        if (k < tile) before += x.x;
+        if (k == tile) cnt = x.x;
       }
-      const uint32_t np = s.lstart[b1] - p0;
-      // ---- prefix over the batches
-      for (uint32_t cw = b0 + warp * 8; cw < b1; cw += kWarps * 8) {  // eight bins a warp, four lanes each
-        const uint32_t c = cw + (lane >> 2);
-        constexpr int kEach = kBatches / 4;
-        const uint32_t g = t & 3u, cc = min(c, b1 - 1u);
-        uint32_t x[kEach], sum = 0;
-#pragma unroll
-        for (int i = 0; i < kEach; ++i) {
-          x[i] = __popc(s.mask[g * kEach + i][cc]);
-          sum += x[i];
-        }
-        uint32_t run = sum;
-#pragma unroll
-        for (int d = 1; d < 4; d <<= 1) {
-          const uint32_t o = __shfl_up_sync(0xffffffffu, run, d, 4);
-          if (g >= static_cast<uint32_t>(d)) run += o;
-        }
-        run += s.lstart[cc] - p0 - sum;
-        if (c < b1) {
-#pragma unroll
-          for (int i = 0; i < kEach; ++i) {
-            s.pos[g * kEach + i][c] = static_cast<uint16_t>(run);
-            run += x[i];
-          }
-        }
-      }
-      __syncthreads();
-      // ---- expand
+    }
+    const uint32_t nt2 = (segs + kTile - 1) / kTile;
+    // two sums a word: {level-2 tiles, segments}, {items of this tile, pairs}
+    const unsigned long long own0 = (static_cast<unsigned long long>(nt2) << 32) | segs;
+    const unsigned long long own1 = (static_cast<unsigned long long>(cnt) << 40) | pairs;
+    unsigned long long in0 = own0, in1 = own1;
+    block_incl_scan2<kWarps>(in0, in1, s_w);
+    const unsigned long long ex0 = in0 - own0, ex1 = in1 - own1;
+    const uint32_t lstart = static_cast<uint32_t>(ex1 >> 40);
+    if (t <= gy) {
+      s_seg[t] = static_cast<uint32_t>(ex0);
+      s_tile[t] = static_cast<uint32_t>(ex0 >> 32);
+      if (t < gy) s_pair[t] = static_cast<uint32_t>(ex1);
+    }
+    if (t < kBinsP) {
+      s.lstart[t] = lstart;
+      s.off[t] = static_cast<uint32_t>(ex0) + before - lstart;
+    }
+    if (t == kThreads - 1) s.lstart[kBinsP] = static_cast<uint32_t>(in1 >> 40);
+    const unsigned long long sum = in1 & ((1ull << 40) - 1);  // (the last thread's: all pairs)
+    if (__syncthreads_or(t == kThreads - 1 && (sum != m || m > a.cap))) {
+      if (t == 0 && blockIdx.x == 0)
+        latch_error(a.err, m > 0xffffffffull ? TDGS_ERR_OVERFLOW : TDGS_ERR_CAPACITY, kSiteViewsDup);
+      return;  // in every block: all see the same sums
+    }
+    if (tile < nt) {
+      uint32_t lo[kPerWarp], hi[kPerWarp];
 #pragma unroll
       for (int b = 0; b < kPerWarp; ++b) {
-        const uint32_t bat = warp * kPerWarp + b;
-        const uint32_t* m = s.mask[bat];
-        const uint16_t* ps = s.pos[bat];
-        const uint32_t l = max(lo[b], b0), h = min(hi[b], b1);
-        const uint32_t n = h > l ? h - l : 0u;
-        const uint32_t item0 = bat * 32;
-        const uint32_t full = __ballot_sync(0xffffffffu, n != 0u);
-        if ((full & (full + 1u)) == 0u) {
-          // Lane p of a step takes the batch's p-th pair: its owner is the
-          // last item that starts at or before it.  The starts that fall into
-          // the step's 32 pairs are one word, and the items are in lane order.
-          const uint32_t end = warp_incl_scan(n), st = end - n;
-          const uint32_t np_b = __shfl_sync(0xffffffffu, end, 31);
-          const uint32_t shift = l - st;            // bin of pair p of this item, less p
-          uint32_t at = n ? st : 0x80000000u;       // start relative to the step (never 0..31 if none)
-          uint32_t seen = 0xffffffffu;              // items that start before the step, less one
-          for (uint32_t p = lane; p < np_b + lane; p += 32, at -= 32) {
-            const uint32_t starts = __reduce_or_sync(0xffffffffu, bit_or_none(at));
-            const uint32_t src = seen + __popc(starts & le);
-            seen += __popc(starts);
-            const uint32_t c = p + __shfl_sync(0xffffffffu, shift, src);
-            if (p < np_b) s.stage[ps[c] + __popc(m[c] & low_bits(src))] = c * 65536u + (item0 + src);
-          }
-        } else {  // a window left items without bins between others: each lane walks its own
-          const uint32_t steps = __reduce_max_sync(0xffffffffu, n);
-          for (uint32_t j = 0; j < steps; ++j) {
-            const uint32_t c = l + j;
-            if (j < n) s.stage[ps[c] + __popc(m[c] & lt)] = c * 65536u + (item0 + lane);
-          }
+        const uint32_t i = (warp * kPerWarp + b) * 32 + lane, p = tile * kTile + i;
+        lo[b] = hi[b] = 0u;
+        if (p < n) {
+          const uint32_t q = __ldcg(a.rects + p);
+          lo[b] = (q >> 16) & 0xffu;
+          hi[b] = (q >> 24) + 1u;
+          if (hi[b] <= lo[b]) lo[b] = hi[b] = 0u;
+          s.pay[i] = __ldcg(a.sdo + p);
+          s.cols[i] = static_cast<uint16_t>(q);
         }
       }
-      __syncthreads();
-      // ---- flush
-      if constexpr (kLevel == 1) {
-#pragma unroll 2
-        for (uint32_t p = t; p < np; p += kThreads) {
-          const uint32_t e = s.stage[p], i = e & 0xffffu, dst = s.off[e >> 16] + p0 + p;
-          a.segs[dst] = s.pay[i];
-          a.cols[dst] = s.cols[i];
-        }
-      } else {
-        const uint32_t row_tile = (r - pl.row0) * bins;  // the row's first tile in its view
-        if (a.keys32) {
-#pragma unroll 2
-          for (uint32_t p = t; p < np; p += kThreads) {
-            const uint32_t e = s.stage[p], c = e >> 16;
-            const uint2 q = s.pay[e & 0xffffu];
-            const uint32_t dst = s.off[c] + p0 + p;
-            a.keys32[dst] = ((row_tile + c) << 10) | q.x;
-            a.values[dst] = q.y;
-          }
-        } else {
-#pragma unroll 2
-        for (uint32_t p = t; p < np; p += kThreads) {
-          const uint32_t e = s.stage[p], c = e >> 16;
-          const uint2 q = s.pay[e & 0xffffu];
-          const uint32_t dst = s.off[c] + p0 + p;
-          a.keys[dst] = (static_cast<uint64_t>(row_tile + c) << 32) | q.x;
-          a.values[dst] = q.y;
-        }
-        }
-      }
-      __syncthreads();
-      b0 = b1;
+      split_tile<1, kWords>(s, a, lo, hi, gy, 0u);
     }
+    tile += gridDim.x;
+  } while (tile < nt);
+  if (!small_barrier(a.bar, a.err)) return;
+  const uint32_t ntiles2 = s_tile[gy];
+  auto row_of = [&](uint32_t x) {  // the last row that starts at or before tile x
+    uint32_t lo = 0, len = gy;
+    while (len > 1) {
+      const uint32_t half = len >> 1;
+      if (s_tile[lo + half] <= x) {
+        lo += half;
+        len -= half;
+      } else {
+        len = half;
+      }
+    }
+    return lo;
+  };
+  // ---- the ranges of rows without tiles, then the pairs: a tile's positions
+  // from the columns of all its row's segments
+  for (uint32_t r = blockIdx.x; r < gy; r += gridDim.x)
+    if (s_tile[r] == s_tile[r + 1] && t < gx) a.ranges[r * gx + t] = make_uint2(0u, 0u);
+  for (uint32_t x = blockIdx.x; x < ntiles2; x += gridDim.x) {
+    const uint32_t r = row_of(x), k0 = x - s_tile[r];
+    const uint32_t beg = s_seg[r] + k0 * kTile, cnt_items = min(kTile, s_seg[r + 1] - beg);
+    uint32_t lo[kPerWarp], hi[kPerWarp];
+#pragma unroll
+    for (int b = 0; b < kPerWarp; ++b) {
+      const uint32_t i = (warp * kPerWarp + b) * 32 + lane;
+      lo[b] = hi[b] = 0u;
+      if (i < cnt_items) {
+        const uint32_t q = __ldcg(a.cols + beg + i);
+        lo[b] = q & 0xffu;
+        hi[b] = (q >> 8) + 1u;
+        s.pay[i] = __ldcg(a.segs + beg + i);
+      }
+    }
+    // per column, as differences: [0] segments in the row (low half) and in
+    // its tiles before this one (high half), [1] in this tile
+    if (t <= kMaxBins) s_d[t][0] = s_d[t][1] = 0;
+    __syncthreads();
+    for (uint32_t p = s_seg[r] + t; p < s_seg[r + 1]; p += kThreads) {
+      const uint32_t q = __ldcg(a.cols + p), c0 = q & 0xffu, c1 = (q >> 8) + 1u;
+      const int one = p < beg ? 0x10001 : 1;
+      atomicAdd(&s_d[c0][0], one);
+      atomicAdd(&s_d[c1][0], -one);
+      if (p - beg < cnt_items) {
+        atomicAdd(&s_d[c0][1], 1);
+        atomicAdd(&s_d[c1][1], -1);
+      }
+    }
+    __syncthreads();
+    uint32_t both = t < kMaxBins ? static_cast<uint32_t>(s_d[t][0]) : 0u;
+    uint32_t cnt = t < kMaxBins ? static_cast<uint32_t>(s_d[t][1]) : 0u;
+    block_incl_scan2<kWarps>(both, cnt, s_w32);
+    const uint32_t total = t < gx ? both & 0xffffu : 0u, before = both >> 16;
+    if (t >= gx) cnt = 0u;
+    unsigned long long in0 = total, in1 = cnt;
+    block_incl_scan2<kWarps>(in0, in1, s_w);
+    const uint32_t start = s_pair[r] + static_cast<uint32_t>(in0) - total, lstart = static_cast<uint32_t>(in1) - cnt;
+    if (t < kBinsP) {
+      s.lstart[t] = lstart;
+      s.off[t] = start + before - lstart;
+    }
+    if (t == kThreads - 1) s.lstart[kBinsP] = static_cast<uint32_t>(in1);
+    if (k0 == 0 && t < gx) a.ranges[r * gx + t] = total ? make_uint2(start, start + total) : make_uint2(0u, 0u);
+    __syncthreads();
+    split_tile<2, kWords>(s, a, lo, hi, gx, r * gx);
   }
 }
 
 // ---------------------------------------------------------------- host side
+template <int kWords>
+cudaError_t launch_small_form(const SplitArgs& a, uint32_t tiles, cudaStream_t s) {
+  const size_t smem = sizeof(Smem<kWords>);
+  const void* fn = reinterpret_cast<const void*>(&k_small<kWords>);
+  const uint32_t resident = radix::resident_ctas(radix::Kernel{fn, 0, kThreads, 0, smem, 1});
+  if (resident == 0) return cudaErrorInvalidConfiguration;
+  SplitArgs args = a;
+  void* params[] = {(void*)&args};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tiles < resident ? tiles : resident);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
 template <int kLevel, int kWords>
 cudaError_t launch_split_form(const SplitArgs& a, uint32_t tiles, int ctas_per_sm, cudaStream_t s) {
   const size_t smem = sizeof(Smem<kWords>);
@@ -637,6 +883,14 @@ cudaError_t launch_split(const SplitArgs& a, uint32_t bins, uint32_t tiles, int 
 
 }  // namespace split
 
+cudaError_t launch_small_split(const SplitArgs& a, uint32_t max_bins, uint32_t max_tiles, cudaStream_t s) {
+  if (!a.vt.one.on || a.ntiles1 == 0) return cudaErrorInvalidValue;
+  const uint32_t tiles = a.ntiles1 > max_tiles ? a.ntiles1 : max_tiles;
+  if (max_bins <= 64) return split::launch_small_form<2>(a, tiles, s);
+  if (max_bins <= 96) return split::launch_small_form<3>(a, tiles, s);
+  if (max_bins <= 160) return split::launch_small_form<5>(a, tiles, s);
+  return split::launch_small_form<9>(a, tiles, s);
+}
 cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s) {
   if (a.ntiles1 == 0) return cudaSuccess;
   return launch_after(split::k_row_count, a.ntiles1, split::kCountThreads, 0, s, a);

@@ -449,9 +449,14 @@ struct SplitArgs {
   uint64_t cap;               // pairs that segs, keys and values hold
   const uint64_t* total;      // the pair count
   uint32_t* ticket;           // a zero word, left zero
+  uint32_t* bar;              // two words of the radix passes' grid barrier
   uint32_t ntiles1, nrows;
   uint32_t* err;
 };
+// One view of at most kSplitSmall Gaussians in one cooperative launch
+// (max_bins: the larger of its rows and columns).
+constexpr uint32_t kSplitSmall = 32 * kSplitTile;
+cudaError_t launch_small_split(const SplitArgs& a, uint32_t max_bins, uint32_t max_tiles, cudaStream_t s);
 cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s);
 cudaError_t launch_row_scan(const SplitArgs& a, cudaStream_t s);
 // max_rows, max_cols: of any view; max_tiles: a bound on the level-2 tiles.

@@ -34,18 +34,20 @@ def same(ctx, oracle, fr):
     assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 1023, 1024, 1025, 2048, 2049, 4097, 70_001])
+@pytest.mark.parametrize("n", [1, 31, 33, 1023, 1024, 1025, 2048, 2049, 4097, 32_768, 32_769, 70_001])
 def test_item_counts(ctx, oracle, n):
     same(ctx, oracle, synth.frame_random(n, n, 333, 209, depth_ties=0.3))
 
 
+@pytest.mark.parametrize("n", [5000, 33_000])
 @pytest.mark.parametrize("cols,rows", [(1, 1), (1, 70), (32, 33), (33, 32), (64, 65), (65, 64), (96, 97), (97, 96),
                                        (160, 161), (161, 160), (224, 225), (225, 224), (256, 3), (3, 256),
                                        (256, 256), (257, 2), (2, 257)])
-def test_grid_sizes(ctx, oracle, cols, rows):
+def test_grid_sizes(ctx, oracle, cols, rows, n):
     """Rows and columns on both sides of each compiled width, 256 (the most
-    that the splits take) and 257."""
-    same(ctx, oracle, synth.frame_random(cols * 1000 + rows, 5000, 16 * cols - 7, 16 * rows - 3, max_sigma=90.0))
+    that the splits take) and 257, for the one-launch form of small frames and
+    the launch per step."""
+    same(ctx, oracle, synth.frame_random(cols * 1000 + rows, n, 16 * cols - 7, 16 * rows - 3, max_sigma=90.0))
 
 
 def covering(n, width, height, seed, small=0.0):
@@ -63,6 +65,19 @@ def test_windows_of_bins(ctx, oracle, n, width, height, small):
     """Tiles with several times the pairs that are staged at once: windows
     of whole rows or columns, in which some items have no bins."""
     same(ctx, oracle, covering(n, width, height, n, small))
+
+
+@pytest.mark.parametrize("width,height", [(4096, 48), (640, 360), (48, 4096)])
+def test_windows_of_bins_among_many(ctx, oracle, width, height):
+    """The same above the one-launch form: 1100 covering Gaussians in front of
+    34,000 small ones, so that whole tiles are covering."""
+    rng = np.random.default_rng(width)
+    front = covering(1100, width, height, 5)
+    front.gaussians["depth"] = rng.uniform(0.3, 0.4, 1100).astype(np.float32)
+    rest = synth.frame_random(6, 34_000, width, height, max_sigma=3.0)
+    rest.gaussians["depth"] += 1.0
+    g = np.concatenate([rest.gaussians, front.gaussians])[rng.permutation(35_100)]
+    same(ctx, oracle, synth.Frame(width, height, g, "front"))
 
 
 @pytest.mark.parametrize("per_sm", [2048, 4096])
