@@ -115,6 +115,7 @@ struct tdgs_context {
   Buffer os_scratch;  // onesweep sort: histograms, digit starts, tickets, look-back status
   Buffer f_dsort;     // single-launch depth sort: barrier counters, totals, rows (kept zero between launches)
   Buffer f_dos;       // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
+  Buffer f_pair;      // single-launch depth sort without offsets: intermediate pairs (with f_sdo)
   Buffer f_raw;       // its first pass's digit counts (zero between frames)
   // State that kernels keep between launches, to be cleared before its next
   // use after an error was latched on the device (a bounded wait may have
@@ -550,7 +551,7 @@ void tdgs_context_destroy(tdgs_context* ctx) {
   DeviceGuard g(ctx->device);
   drain_timings(ctx);
   for (cudaEvent_t e : ctx->free_events) cudaEventDestroy(e);
-  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort, &ctx->f_dos, &ctx->f_raw, &ctx->f_counts, &ctx->f_dkey[0],
+  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort, &ctx->f_dos, &ctx->f_raw, &ctx->f_pair, &ctx->f_counts, &ctx->f_dkey[0],
                     &ctx->f_dkey[1],    &ctx->f_dkey[2],     &ctx->f_dval[0],    &ctx->f_dval[1],
                     &ctx->f_dval[2],    &ctx->f_soff,       &ctx->f_sdo,        &ctx->f_rec3,
                     &ctx->f_conic,      &ctx->d_cams,       &ctx->diag,       &ctx->b_keys,       &ctx->b_vals,       &ctx->n_counts,
@@ -839,7 +840,8 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   if (st == TDGS_OK) st = ensure(ctx, ctx->sort_scratch, dp.scratch_words * 4, s);
   if (st == TDGS_OK && dp.resident) {
     grown = false;
-    st = ensure(ctx, ctx->f_dsort, depth_sort_scratch_words(depth_sort_grid()) * 4, s, &grown);
+    if (ctx->split) st = ensure(ctx, ctx->f_pair, static_cast<size_t>(n_all) * 8 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_dsort, depth_sort_scratch_words(depth_sort_grid()) * 4, s, &grown);
     if (st == TDGS_OK && (grown || ctx->dsort_dirty)) {
       TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_dsort.p, 0, ctx->f_dsort.bytes, s));
       ctx->dsort_dirty = false;
@@ -910,6 +912,8 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   da.v1 = dv[1];
   da.k2 = dk[2];
   da.v2 = dv[2];
+  da.pair[0] = static_cast<uint64_t*>(ctx->f_pair.p);
+  da.pair[1] = static_cast<uint64_t*>(ctx->f_sdo.p);  // written again only after the sort
   da.counts = counts;
   da.offsets = ctx->split ? nullptr : static_cast<uint32_t*>(ctx->f_soff.p);  // the interval splits take none
   uint32_t* range = ctx->norm ? static_cast<uint32_t*>(ctx->n_norm.p) : ctx->d_range;  // of the keys that are sorted

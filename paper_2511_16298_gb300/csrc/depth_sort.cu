@@ -46,10 +46,12 @@
 // each chunk scans its counts from the sum of the chunks before it: the
 // pair offsets.
 //
-// Each tile's values (pass 0: the tile counts) come into shared memory by
-// one bulk copy issued before the tile is ranked, so their latency hides
-// behind the ranking; keys and values cross the exchange as one 8-byte
-// word.
+// Keys and values cross the exchange as one 8-byte word.  Between passes they
+// are one word too when the launch ends with the order (k_depth_sort<*,
+// false>): one store and one load per key where there were two, in runs of
+// twice the bytes.  With the offsets each tile's values (pass 0: the tile
+// counts) come into shared memory by one bulk copy issued before the tile is
+// ranked, so their latency hides behind the ranking.
 //
 // A barrier is an arrival counter of its own: a CTA adds one with release
 // semantics and waits (acquire, bounded) until the count reaches the grid
@@ -233,7 +235,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
                                                  uint32_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                  const uint32_t* __restrict__ counts, uint32_t Sz, uint32_t G,
                                                  uint32_t* __restrict__ csum,
-                                                 const uint32_t* s_begin = nullptr, uint32_t nv = 0) {
+                                                 uint64_t* __restrict__ pout, const uint32_t* s_begin, uint32_t nv) {
   using S = ShapeOf<kItems>;
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   bool ok = true;
@@ -260,7 +262,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
   for (int j = 0; j < kItems; ++j)
     if (wbase + j * 32 + lane < valid) x64[pos[j]] = (static_cast<uint64_t>(hi[j]) << 32) | v[j];
   __syncthreads();
-  if (!kOffsets || !last) {
+  if constexpr (!kOffsets) {
     // (in the last pass the high word is the digit, and only the values are kept)
     const uint32_t sh = last ? 0u : shift;
 #pragma unroll
@@ -268,15 +270,26 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
       const uint32_t xp = i * kThreads + t;
       if (xp < valid) {
         const uint64_t x = x64[xp];
-        const uint32_t key = static_cast<uint32_t>(x >> 32);
+        const uint32_t key = static_cast<uint32_t>(x >> 32), val = static_cast<uint32_t>(x);
         const uint32_t dst = sm.off[(key >> sh) & mask] + xp;
+        if (dst >= n)
+          ok = false;
+        else if (last)
+          v1[dst] = val;
+        else
+          pout[dst] = nv ? (static_cast<uint64_t>(find_view(s_begin, nv, val)) << 32) | val : x;
+      }
+    }
+  } else if (!last) {
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      const uint32_t xp = i * kThreads + t;
+      if (xp < valid) {
+        const uint64_t x = x64[xp];
+        const uint32_t key = static_cast<uint32_t>(x >> 32);
+        const uint32_t dst = sm.off[(key >> shift) & mask] + xp;
         if (dst < n) {
-          if (kOffsets || !last) {
-            uint32_t out = key;
-            if constexpr (!kOffsets)
-              if (nv) out = find_view(s_begin, nv, static_cast<uint32_t>(x));
-            kout[dst] = out;
-          }
+          kout[dst] = key;
           vout[dst] = static_cast<uint32_t>(x);
         } else {
           ok = false;
@@ -648,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
   if (kOffsets && c == 0)  // this launch's chunk sums (added to after the first barrier)
     for (uint32_t i = t; i < G; i += kThreads) csum[i] = 0u;
   const uint32_t nbulk = valid & ~3u;  // values by bulk copy; the last 1-3 by plain loads
-  if (t == 0) {
+  if (kOffsets && t == 0) {
     osw::mbar_init(&s_mbar);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -683,9 +696,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     a.mask = view_pass ? kBins - 1u : mask;  // (at most 256 views)
     const uint32_t* vsrc = p == 0 ? counts : vin;
     const bool counted = kCount && p == 0;  // keys in registers, values (the counts) already staged
-    const bool unstaged = counted || (!kOffsets && p == 0);  // no values to copy in
-    const uint32_t nstaged = counted ? valid : nbulk;
-    if (t == 0) {
+    const bool unstaged = !kOffsets || counted;  // no values to copy in
+    const uint32_t nstaged = unstaged ? valid : nbulk;
+    if (kOffsets && t == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       osw::mbar_arrive(&s_mbar, unstaged ? 0u : nbulk * 4);
       if (!unstaged && nbulk) osw::bulk_g2s(vstage, vsrc + beg, nbulk * 4, &s_mbar);
@@ -699,6 +712,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
         for (int j = 0; j < kItems; ++j) {
           const uint32_t idx = wbase + j * 32 + lane;
           R.k[j] = idx < valid ? (R.k[j] == 0xffffffffu ? cull : R.k[j] - lo) : 0u;
+        }
+      } else if (!kOffsets && p > 0) {
+        // (key, value) pairs: the values wait in the staging buffer
+        const uint2* pin = reinterpret_cast<const uint2*>(A.pair[(p - 1) & 1u]) + beg;
+        uint2 x[kItems];
+#pragma unroll
+        for (int j = 0; j < kItems; ++j) {
+          const uint32_t idx = wbase + j * 32 + lane;
+          x[j] = idx < valid ? __ldcs(pin + idx) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int j = 0; j < kItems; ++j) {
+          R.k[j] = x[j].y;
+          vstage[wbase + j * 32 + lane] = x[j].x;
         }
       } else {
 #pragma unroll
@@ -768,7 +795,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
       sm.lstart[t] = st.y;
       sm.off[t] = st.x + before - st.y;
     }
-    if (!osw::mbar_wait(&s_mbar, p & 1u, err) && t == 0) (void)osw::mbar_wait(&s_mbar, p & 1u, err);
+    if constexpr (kOffsets)
+      if (!osw::mbar_wait(&s_mbar, p & 1u, err) && t == 0) (void)osw::mbar_wait(&s_mbar, p & 1u, err);
     __syncthreads();
     {
       // ranks into tile positions; this warp's counter row back to zero
@@ -783,7 +811,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
 #pragma unroll
     for (int j = 0; j < kItems; ++j) hk[j] = last ? R.d[j] : R.k[j];
     ok &= exchange_scatter<kOffsets, kItems>(sm, vstage, hk, R.r, valid, beg, nstaged, vsrc, p == 0, last, a.shift, a.mask, n, kout,
-                           vout, k1, v1, counts, Sz, G, csum, s_begin, to_view ? by_view : 0u);
+                           vout, k1, v1, counts, Sz, G, csum, A.pair[p & 1u], s_begin,
+                           to_view ? by_view : 0u);
     arrive_and_wait(scratch + (last ? kFinalSlot : 1 + p) * kLine, G, err);
   }
   if (!ok) latch_error(err, TDGS_ERR_CAPACITY, kSiteRadixRange);

@@ -363,8 +363,7 @@ cudaError_t launch_depth_pass(const DepthPlan& dp, uint32_t pass, const uint32_t
 //    receives only counts of 1023 or more.
 //  * Without (launch_depth_sort): key0 = the count kernel's depth keys,
 //    counts its tile counts, range[2..3] its range.
-//  * With offsets null the launch stops at v1: counts is not read, k1 holds
-//    intermediate keys, and several views are ordered view after view (by
+//  * With offsets null the launch stops at v1: counts is not read, and several views are ordered view after view (by
 //    depth inside each).
 struct DepthSortArgs {
   const uint32_t* key0;
@@ -373,6 +372,7 @@ struct DepthSortArgs {
   uint32_t* host_status;
   uint32_t host_seq;
   uint32_t *k1, *v1, *k2, *v2;
+  uint64_t* pair[2];  // without offsets: intermediate (key << 32 | value), n each; k1, k2 and v2 are not used
   uint32_t* counts;
   uint32_t* offsets;
   uint32_t* range;
