@@ -193,81 +193,108 @@ cudaError_t launch_scan(const uint32_t* counts, const float4* recs, const uint32
 // ------------------------------------------------------------- duplicate
 // Load-balanced expansion.  A warp owns 32 consecutive Gaussians; their
 // pairs occupy one contiguous output range (their offsets are consecutive
-// in the scan).  The warp walks that range 32 pairs at a time: lane l takes
-// pair q = chunk + l, finds the owning Gaussian by a 5-step binary search
-// over the lanes' start offsets (shuffles), and derives (ty, tx) from the
-// local index (row-major within the Gaussian's tile rectangle).  Every
+// in the scan).  The warp walks that range 32 pairs at a time, lane l taking
+// pair p = step + l.  The Gaussians with pairs lie compacted in shared memory;
+// those that start inside the step are one word of bits (one warp OR), so the
+// owner of a pair is a population count, not a search.  (ty, tx) come from the
+// local index by a float reciprocal with one exact correction step.  Every
 // store is a fully coalesced 256-byte (keys) / 128-byte (values) run.
 // kNorm: the paper's 32-bit key (Sec. IV-B), tile << 10 | q with q the
 // depth normalised to 2^10 over the visible range norm[0..1] (float bits).
+struct DupOwner {
+  uint32_t start, first, w;  // first pair (relative), first tile, columns
+  float rw;                  // 1 / columns
+};
 template <bool kNorm>
 __global__ void __launch_bounds__(256)
     k_duplicate(const float4* __restrict__ g, const uint32_t* __restrict__ offsets, uint32_t n,
                 FrameGeom fg, void* __restrict__ keys_raw, uint32_t* __restrict__ values,
                 uint32_t cap, const uint32_t* __restrict__ norm, uint32_t* err) {
+  __shared__ __align__(16) DupOwner s_owner[8][32];
+  __shared__ uint2 s_pay[8][32];  // low key word, index
   begin_launch();
   float dmin = 0.0f, scale = 0.0f;
   if constexpr (kNorm) {
     dmin = __uint_as_float(norm[0]);
     scale = norm_scale(dmin, __uint_as_float(norm[1]));
   }
-  const uint32_t lane = lane_id();
+  const uint32_t lane = lane_id(), w8 = threadIdx.x >> 5;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
   const uint32_t warps_total = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t gx = static_cast<uint32_t>(fg.gx);
   bool bad = false, over = false;
   for (uint32_t wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
        static_cast<uint64_t>(wg) * 32u < n; wg += warps_total) {
     const uint32_t i = wg * 32u + lane;
     TileRect q;
+    q.x0 = q.y0 = q.x1 = q.y1 = 0;
+    q.count = 0;
     uint64_t start = 0;
+    uint32_t low = 0;
     if (i < n) {
-      q = tile_rect(__ldg(g + i), fg);
+      const float4 rec = __ldg(g + i);
+      q = tile_rect(rec, fg);
       start = __ldg(offsets + i);
       bad |= q.invalid;
-    } else {
-      q.x0 = q.y0 = q.x1 = q.y1 = 0;
-      q.count = 0;
+      low = kNorm ? norm_depth(rec.z, dmin, scale) : __float_as_uint(rec.z);
     }
-    uint32_t depth_bits = i < n ? __float_as_uint(__ldg(&g[i].z)) : 0u;
-    if constexpr (kNorm) depth_bits = norm_depth(__uint_as_float(depth_bits), dmin, scale);
-    uint64_t end = start + q.count;
-    // warp range [begin, end_max)
-    uint64_t end_max = end;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      const uint64_t o = __shfl_xor_sync(0xffffffffu, end_max, d);
-      end_max = o > end_max ? o : end_max;
+    // the warp's range: from its first Gaussian with pairs to the end of its
+    // last one; positions relative to it, in 32 bits, none at or beyond cap
+    const uint32_t with = __ballot_sync(0xffffffffu, q.count != 0u);
+    if (with == 0u) continue;
+    const uint64_t begin = __shfl_sync(0xffffffffu, start, __ffs(with) - 1);
+    const uint64_t end = __shfl_sync(0xffffffffu, start + q.count, 31 - __clz(with));
+    if (end > cap) over = true;
+    const uint64_t stop = end < cap ? end : cap;
+    const uint64_t span = stop > begin ? stop - begin : 0;
+    const uint32_t nrel = static_cast<uint32_t>(span);  // (cap has 32 bits)
+    const uint64_t rel = start - begin;
+    const bool mine = q.count != 0u && rel < nrel;
+    const uint32_t mask = __ballot_sync(0xffffffffu, mine);
+    const uint32_t wd = static_cast<uint32_t>(q.x1 - q.x0);
+    __syncwarp();  // the last Gaussians' owners are read
+    if (mine) {
+      const uint32_t r = __popc(mask & lt);
+      s_owner[w8][r] = DupOwner{static_cast<uint32_t>(rel),
+                                static_cast<uint32_t>(q.y0) * gx + static_cast<uint32_t>(q.x0), wd,
+                                __frcp_rn(static_cast<float>(wd))};
+      s_pay[w8][r] = make_uint2(low, i);
     }
-    if (i >= n) start = end_max;  // never selected by the owner search
-    const uint64_t begin = __shfl_sync(0xffffffffu, start, 0);
-    const int32_t w = q.x1 - q.x0;
-    for (uint64_t c = begin; c < end_max; c += 32) {
-      const uint64_t p = c + lane;
-      uint32_t lo = 0;
-#pragma unroll
-      for (uint32_t step = 16; step > 0; step >>= 1) {
-        const uint64_t sc = __shfl_sync(0xffffffffu, start, lo + step);
-        if (sc <= p) lo += step;
-      }
-      const uint64_t s0 = __shfl_sync(0xffffffffu, start, lo);
-      const int32_t ow = __shfl_sync(0xffffffffu, w, lo);
-      const int32_t ox0 = __shfl_sync(0xffffffffu, q.x0, lo);
-      const int32_t oy0 = __shfl_sync(0xffffffffu, q.y0, lo);
-      const uint32_t od = __shfl_sync(0xffffffffu, depth_bits, lo);
-      if (p < end_max && ow > 0) {
-        const uint32_t j = static_cast<uint32_t>(p - s0);
-        const uint32_t ry = j / static_cast<uint32_t>(ow);
-        const uint32_t rx = j - ry * static_cast<uint32_t>(ow);
-        const uint64_t tile = static_cast<uint64_t>(oy0 + ry) * static_cast<uint64_t>(fg.gx) +
-                              static_cast<uint64_t>(ox0 + rx);
-        if (p < cap) {
-          if constexpr (kNorm)
-            static_cast<uint32_t*>(keys_raw)[p] = (static_cast<uint32_t>(tile) << 10) | od;
-          else
-            static_cast<uint64_t*>(keys_raw)[p] = (tile << 32) | od;
-          values[p] = wg * 32u + lo;
+    __syncwarp();
+    uint32_t seen = 0xffffffffu;  // owners that start before the step, less one
+    for (uint64_t p64 = 0; p64 < nrel; p64 += 32) {
+      const uint32_t p0 = static_cast<uint32_t>(p64);
+      const uint32_t at = static_cast<uint32_t>(rel) - p0;
+      const uint32_t starts = __reduce_or_sync(0xffffffffu, mine && at < 32u ? 1u << at : 0u);
+      const uint32_t src = (seen + __popc(starts & le)) & 31u;
+      seen += __popc(starts);
+      const uint32_t p = p0 + lane;
+      if (p64 + lane < nrel) {
+        const DupOwner o = s_owner[w8][src];
+        const uint2 pay = s_pay[w8][src];
+        const uint32_t j = p - o.start;
+        uint32_t ry, rx;
+        if (j < (1u << 22)) {
+          ry = __float2uint_rz(__fmul_rn(__uint2float_rn(j), o.rw));
+          rx = j - ry * o.w;
+          if (static_cast<int32_t>(rx) < 0) {
+            --ry;
+            rx += o.w;
+          } else if (rx >= o.w) {
+            ++ry;
+            rx -= o.w;
+          }
         } else {
-          over = true;
+          ry = j / o.w;
+          rx = j - ry * o.w;
         }
+        const uint32_t tile = o.first + ry * gx + rx;
+        const uint64_t dst = begin + p;
+        if constexpr (kNorm)
+          static_cast<uint32_t*>(keys_raw)[dst] = (tile << 10) | pay.x;
+        else
+          static_cast<uint64_t*>(keys_raw)[dst] = (static_cast<uint64_t>(tile) << 32) | pay.x;
+        values[dst] = pay.y;
       }
     }
   }
@@ -363,35 +390,57 @@ cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, 
 }
 
 // ---------------------------------------------------------- tile ranges
-// Identify Range: a tile's range starts where its id differs from the
-// previous key's and ends where it differs from the next key's.  ranges is
-// zeroed beforehand, so tiles without pairs stay {0, 0}.
+// Identify Range: where a key's tile differs from the previous key's, the
+// previous tile's range ends and this one's starts.  ranges is zeroed
+// beforehand, so tiles without pairs stay {0, 0}.  Each key's word with the
+// tile is read once; the previous one comes from the lane before (the first
+// lane reads it again).
 // K, kShift: 64-bit keys with the tile above bit 32, or the 32-bit
 // normalised keys with the tile above bit 10.
+constexpr int kRangeItems = 4;
 template <typename K, int kShift>
 __global__ void __launch_bounds__(256) k_tile_ranges(const K* __restrict__ keys, uint32_t m,
                                                      uint32_t num_tiles, uint2* ranges,
                                                      uint32_t* err) {
   begin_launch();
+  const uint32_t* __restrict__ words = reinterpret_cast<const uint32_t*>(keys);
+  constexpr uint32_t kStep = sizeof(K) / 4, kHigh = sizeof(K) == 8 ? 1 : 0;
+  auto tile_of = [&](uint64_t k) { return __ldg(words + k * kStep + kHigh) >> (kShift & 31); };
+  const uint32_t lane = lane_id();
+  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x * kRangeItems;
   bool bad = false;
-  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    const uint64_t t = static_cast<uint64_t>(__ldg(keys + k)) >> kShift;
-    if (t >= num_tiles) {
-      bad = true;
-      continue;
+  for (uint64_t w0 = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31u)) * kRangeItems; w0 < m;
+       w0 += stride) {
+    uint32_t t[kRangeItems];
+#pragma unroll
+    for (int u = 0; u < kRangeItems; ++u) {
+      const uint64_t k = w0 + u * 32 + lane;
+      t[u] = k < m ? tile_of(k) : 0u;
     }
-    const uint64_t prev = k > 0 ? (static_cast<uint64_t>(__ldg(keys + k - 1)) >> kShift) : ~0ull;
-    const uint64_t next = k + 1 < m ? (static_cast<uint64_t>(__ldg(keys + k + 1)) >> kShift) : ~0ull;
-    if (t != prev) ranges[t].x = k;
-    if (t != next) ranges[t].y = k + 1;
+    uint32_t last = w0 > 0 && lane == 0 ? tile_of(w0 - 1) : 0u;  // the tile before lane 0's
+#pragma unroll
+    for (int u = 0; u < kRangeItems; ++u) {
+      const uint64_t k = w0 + u * 32 + lane;
+      uint32_t prev = __shfl_up_sync(0xffffffffu, t[u], 1);
+      if (lane == 0) prev = last;
+      last = __shfl_sync(0xffffffffu, t[u], 31);
+      if (k < m) {
+        bad |= t[u] >= num_tiles;
+        if (k == 0 || t[u] != prev) {
+          if (t[u] < num_tiles) ranges[t[u]].x = static_cast<uint32_t>(k);
+          if (k > 0 && prev < num_tiles) ranges[prev].y = static_cast<uint32_t>(k);
+        }
+        if (k + 1 == m && t[u] < num_tiles) ranges[t[u]].y = m;
+      }
+    }
   }
-  if (__any_sync(0xffffffffu, bad) && lane_id() == 0) latch_error(err, TDGS_ERR_INVALID_ARGUMENT, kSiteRanges);
+  if (__any_sync(0xffffffffu, bad) && lane == 0) latch_error(err, TDGS_ERR_INVALID_ARGUMENT, kSiteRanges);
 }
 
 cudaError_t launch_tile_ranges(const uint64_t* keys, uint32_t m, uint32_t num_tiles,
                                uint2* ranges, uint32_t* err, cudaStream_t s) {
   if (m == 0) return cudaSuccess;
-  const uint32_t blocks = (m + 255) / 256;
+  const uint32_t blocks = m / (256 * kRangeItems) + 1;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
   return launch_after(k_tile_ranges<uint64_t, 32>, grid, 256, 0, s, keys, m, num_tiles, ranges, err);
 }
@@ -399,7 +448,7 @@ cudaError_t launch_tile_ranges(const uint64_t* keys, uint32_t m, uint32_t num_ti
 cudaError_t launch_tile_ranges_norm(const uint32_t* keys, uint32_t m, uint32_t num_tiles, uint2* ranges,
                                     uint32_t* err, cudaStream_t s) {
   if (m == 0) return cudaSuccess;
-  const uint32_t blocks = (m + 255) / 256;
+  const uint32_t blocks = m / (256 * kRangeItems) + 1;
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
   return launch_after(k_tile_ranges<uint32_t, 10>, grid, 256, 0, s, keys, m, num_tiles, ranges, err);
 }

@@ -170,3 +170,36 @@ def test_normalized_key(ctx, oracle, n, width, height):
     assert np.array_equal(k.cpu().numpy().view(np.uint32), ek)
     assert np.array_equal(v.cpu().numpy().view(np.uint32), ev)
     assert np.array_equal(r.cpu().numpy().view(np.uint32), er)
+
+
+@pytest.mark.parametrize("n,cap", [(1, None), (33, None), (5000, None), (5000, 1), (5000, 0.5), (70_001, None)])
+def test_duplicate_and_ranges_steps(ctx, oracle, n, cap):
+    """duplicate_keys with runs of culled Gaussians and whole-screen ones, with
+    and without room for every pair, and tile_ranges at sizes around a warp's
+    128 keys: the pairs written are the oracle's, and the missing ones are
+    reported."""
+    fr = synth.frame_random(n, n, 777, 331, max_sigma=200.0, culled=0.4)
+    ref = oracle.sort_frame(fr.gaussians, fr.width, fr.height)
+    m = ref["m"]
+    g = T.records_to_tensor(fr.gaussians, DEV)
+    off = torch.from_numpy(ref["offsets"].view(np.int32)).to(DEV)
+    room = m if cap is None else (cap if cap >= 1 else int(m * cap))
+    k, v = ctx.duplicate_keys(g, off, fr.width, fr.height, room)
+    if room < m:
+        with pytest.raises(T.TdgsError) as e:
+            ctx.sync()
+        assert e.value.status == T.CAPACITY
+    else:
+        ctx.sync()
+    assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["unsorted_keys"][:room])
+    assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["unsorted_values"][:room])
+    sk = torch.from_numpy(ref["keys"].view(np.int64)).to(DEV)
+    for mm in sorted({min(x, m) for x in (1, 31, 32, 33, 127, 128, 129, 1024, 1025, m)}):
+        r = ctx.tile_ranges(sk, fr.num_tiles, m=mm)
+        ctx.sync()
+        tiles = (ref["keys"][:mm] >> np.uint64(32)).astype(np.int64)
+        want = np.zeros((fr.num_tiles, 2), np.uint32)
+        want[:, 0] = np.searchsorted(tiles, np.arange(fr.num_tiles), "left")
+        want[:, 1] = np.searchsorted(tiles, np.arange(fr.num_tiles), "right")
+        want[want[:, 0] == want[:, 1]] = 0
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), want)
