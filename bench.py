@@ -104,14 +104,19 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-def kernel_source_sha() -> str:
-    """Hash of the sources the chunked radix pass kernels are compiled
-    from: the radix files and the device part of the internal header (its
-    host-side declarations, after the "host side" marker, do not enter the
-    kernels)."""
+# Sources of the frame's kernels besides the device part of the internal header.
+KERNEL_SOURCES = {"count_depth_order": ("depth_sort.cu", "onesweep.cuh", "radix.cuh"),
+                  "column_split": ("interval_split.cu", "radix.cuh"), "row_split": ("interval_split.cu", "radix.cuh")}
+
+
+def kernel_source_sha(kernel: str = "") -> str:
+    """Hash of the sources a kernel is compiled from (by default the chunked
+    radix pass kernels' files) and the device part of the internal header
+    (its host-side declarations, after the "host side" marker, do not enter
+    the kernels)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2511_16298_gb300", "csrc")
-    for f in ("radix.cuh", "radix.cu", "radix_frame.cu", "sort_kernels.cu"):
+    for f in KERNEL_SOURCES.get(kernel, ("radix.cuh", "radix.cu", "radix_frame.cu", "sort_kernels.cu")):
         h.update(open(os.path.join(csrc, f), "rb").read())
     hdr = open(os.path.join(csrc, "tdgs_internal.cuh"), "rb").read()
     cut = hdr.find(b"// ------------------------------------------------------------- host side")
@@ -129,7 +134,7 @@ def profiled_traffic(kernel: str):
     sha = re.search(r"source_sha256:\s*([0-9a-f]{64})", text)
     tr = re.search(r"traffic_bytes_per_launch:\s*([0-9.eE+]+)", text)
     items = re.search(r"items_per_launch:\s*([0-9]+)", text)
-    cur = kernel_source_sha()
+    cur = kernel_source_sha(kernel)
     if not (sha and tr) or sha.group(1) != cur:
         return None
     return float(tr.group(1)), int(items.group(1)) if items else None
@@ -139,8 +144,8 @@ def algorithmic_bytes(kernel: str, items: int, n: int, m: int, tiles: int, depth
     """Minimum DRAM bytes of one launch (reads + writes), per kernel.
     items = the units the launch processed (Gaussians, pairs or tiles, as
     the library's tracer reports them); n, m, tiles = the frame's sizes.
-    The fused-frame figures assume the packed (tile, depth rank) element
-    fits 32 bits, which holds for every single-frame workload timed here.
+    The tile passes' figures assume the packed (tile, depth rank) element
+    fits 32 bits.
     depth_passes: digit passes one depth_sort launch ran; negative for the
     single-launch form (all passes and the depth-order scan in one launch),
     1 for one launch per pass."""
@@ -173,6 +178,20 @@ def algorithmic_bytes(kernel: str, items: int, n: int, m: int, tiles: int, depth
         # reads no key, the last writes index and count); offsets: count in,
         # offset out
         return 16.0 * items + 16.0 * items * abs(depth_passes) + 8.0 * items
+    if kernel in ("depth_order", "count_depth_order"):  # the single launch without the offsets:
+        # key (4 B) or record (16 B) in; between passes one 8 B word out and in; the index out
+        return ((16.0 if kernel == "count_depth_order" else 4.0) + 16.0 * (abs(depth_passes) - 1) + 4.0) * items
+    # interval splits (a Gaussian has at least one segment: the floor counted here)
+    if kernel == "row_count":        # index and record in; {low key word, index} and rectangle out
+        return 32.0 * items
+    if kernel == "row_split":        # the same 12 B in; a segment and its columns out
+        return 22.0 * items
+    if kernel == "column_count":     # columns in, per segment
+        return 2.0 * n
+    if kernel == "column_split":     # segment and columns in; u64 key + u32 value out per pair
+        return 12.0 * items + 10.0 * n
+    if kernel == "small_split":      # all of the above and the ranges in one launch
+        return 32.0 * n + 12.0 * items + 8.0 * tiles
     if kernel == "scan_by_depth":    # index in, gathered count, offset out
         return 12.0 * items
     if kernel == "duplicate_by_depth":  # index, offset, record in; {depth key, index} out; 4 B per pair out
@@ -266,7 +285,8 @@ def run_ours(args, rank, world, local_rank, dist):
     ctx.sync()
     ktimes = ctx.kernel_times()
     ctx.enable_timing(False)
-    dsl = ktimes.get("depth_sort", {}).get("launches", 0) + ktimes.get("count_depth_sort", {}).get("launches", 0)
+    dsl = sum(ktimes.get(k, {}).get("launches", 0)
+              for k in ("depth_sort", "count_depth_sort", "depth_order", "count_depth_order"))
     depth_passes = -ctx.depth_passes() if dsl == args.steps else 1
     step_ms = [a.elapsed_time(b) for a, b in ev]
     dev_s = sum(step_ms) / 1e3

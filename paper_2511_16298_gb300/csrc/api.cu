@@ -64,14 +64,14 @@ enum KernelId {
   kKCount, kKScan, kKDuplicate, kKRanges, kKRadixPass,
   kKFrameCount, kKDepthSort, kKFrameScan, kKDupDepth, kKTilePass, kKTileExpand, kKPreprocess, kKBitonic, kKRender, kKPreCount, kKNormRange, kKNormDup, kKNormPass,
   kKNormRanges, kKRenderOrder, kKSortHist, kKOnesweep, kKCountDepth,
-  kKNormKeys, kKSmallSplit, kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
+  kKDepthOrder, kKCountOrder, kKNormKeys, kKSmallSplit, kKRowCount, kKRowScan, kKRowSplit, kKColCount, kKColScan, kKColSplit, kKNum
 };
 const char* const kKernelNames[kKNum] = {
     "count_tiles",  "scan",       "duplicate_keys",     "tile_ranges",    "radix_pass",
     "frame_count",  "depth_sort", "scan_by_depth", "duplicate_by_depth", "tile_sort_pass",
     "tile_expand_pass", "preprocess", "bitonic_sort", "render", "preprocess_count", "norm_range",
     "norm_duplicate", "norm_sort_pass", "norm_ranges", "render_order", "sort_histogram", "onesweep_pass",
-    "count_depth_sort", "norm_keys", "small_split", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
+    "count_depth_sort", "depth_order", "count_depth_order", "norm_keys", "small_split", "row_count", "row_scan", "row_split", "column_count", "column_scan", "column_split"};
 
 // View table as stored in device memory (SoA, fixed maximum size).
 struct ViewBlob {
@@ -931,7 +931,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
       if (ctx->early_seq == 0) ctx->early_seq = 1;  // 0: never written
       da.host_seq = ctx->early_seq;
     }
-    TDGS_TRACED(ctx, kKCountDepth, n_all, s, launch_count_depth_sort(dp.grid, dp.items, da, s));
+    TDGS_TRACED(ctx, ctx->split ? kKCountOrder : kKCountDepth, n_all, s, launch_count_depth_sort(dp.grid, dp.items, da, s));
     if (early_total) TDGS_CUDA(ctx, cudaEventRecord(ctx->ev_count, s));
     return TDGS_OK;
   }
@@ -957,7 +957,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
   if (dp.resident) {  // one launch: the sort (pass count from the depth range) and the offsets
     da.key0 = dk[0];
-    TDGS_TRACED(ctx, kKDepthSort, n_all, s, launch_depth_sort(dp.grid, dp.items, da, s));
+    TDGS_TRACED(ctx, ctx->split ? kKDepthOrder : kKDepthSort, n_all, s, launch_depth_sort(dp.grid, dp.items, da, s));
   } else if (dp.onesweep) {  // the passes that the key range needs, and the one by view
     if (n_all) {
       uint32_t* dos = static_cast<uint32_t*>(ctx->f_dos.p);
