@@ -235,8 +235,8 @@ tdgs_status tdgs_duplicate_keys(tdgs_context* ctx, const tdgs_gaussian2d* g,
  * variant chosen by tdgs_context_set_sort_variant), a onesweep LSD radix sort:
  * one launch reads the keys once for the first digit's counts, then one
  * launch per 9-bit digit reads and writes every pair once (its tiles go
- * through shared memory by bulk copy; scan blocks of the same cooperative
- * launch turn the tiles' digit counts into prefixes); every other case
+ * through shared memory by bulk copy; scan blocks of the same launch
+ * turn the tiles' digit counts into prefixes); every other case
  * takes the chunked per-digit passes.  Both give the same bytes. */
 tdgs_status tdgs_sort_pairs(tdgs_context* ctx, uint64_t* keys, uint32_t* values,
                             uint64_t* keys_alt, uint32_t* values_alt, uint32_t m,

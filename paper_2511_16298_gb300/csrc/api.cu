@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "render.cuh"
@@ -95,9 +96,48 @@ struct PendingTime {
   uint64_t items;
 };
 
+// Staged views, buffers and results of the fused frame.  The frame with the
+// normalised key runs the same code on a state of its own, so it leaves a
+// frame's results, a reservation and captured graphs alone.
+struct FrameState {
+  Buffer f_counts, f_dkey[3], f_dval[3], f_soff, f_sdo, f_rminmax, f_stream[2], f_keys, f_values, f_ranges;
+  Buffer f_rects, f_c1, f_rows, f_segs, f_cols, f_c2, f_b2;  // interval splits
+  Buffer f_dos;   // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
+  Buffer f_pair;  // single-launch depth sort without offsets: intermediate pairs (with f_sdo)
+  // f_rminmax holds first positions in its first half and one-past-last
+  // positions in its second half, kept at (all ones, zero) between frames:
+  // the ranges kernel resets what the last tile pass recorded
+  bool rminmax_dirty = true;
+  bool vtot_dirty = true;       // the view totals are to be cleared (see note_device_error)
+  ViewBlob* d_views = nullptr;  // device view table
+  ViewBlob* h_views = nullptr;  // pinned staging of the table
+  uint32_t nv = 0, n_all = 0, t_all = 0;
+  uint32_t max_gx = 0, max_gy = 0;  // over the staged views
+  bool norm = false;            // the frame with the 32-bit normalised key (by interval splits)
+  bool split = false;           // pairs by interval splits (else packed elements and tile passes)
+  uint64_t capacity = 0;        // pair capacity reserved for the asynchronous path
+  bool split_reserved = false;  // what the reservation chose
+  bool exact = false;           // a call that waits for the pair count (not an asynchronous one)
+  bool reserved = false;
+
+  bool allocate_tables() {
+    if (!d_views && cudaMalloc(&d_views, sizeof(ViewBlob)) != cudaSuccess) return false;
+    return h_views || cudaMallocHost(&h_views, sizeof(ViewBlob)) == cudaSuccess;
+  }
+  void release() {
+    for (Buffer* b : {&f_counts, &f_dkey[0], &f_dkey[1], &f_dkey[2], &f_dval[0], &f_dval[1], &f_dval[2], &f_soff,
+                      &f_sdo, &f_rminmax, &f_stream[0], &f_stream[1], &f_keys, &f_values, &f_ranges, &f_rects, &f_c1,
+                      &f_rows, &f_segs, &f_cols, &f_c2, &f_b2, &f_dos, &f_pair})
+      if (b->p) cudaFree(b->p);
+    if (d_views) cudaFree(d_views);
+    if (h_views) cudaFreeHost(h_views);
+  }
+};
+
 }  // namespace
 
-struct tdgs_context {
+struct tdgs_context : FrameState {
+  FrameState norm_state;  // swapped in for tdgs_sort_frame_normalized
   int device = 0;
   DevStatus* d_status = nullptr;
   DevStatus* h_status = nullptr;  // pinned
@@ -114,15 +154,12 @@ struct tdgs_context {
   Buffer scan_status, sort_scratch;
   Buffer os_scratch;  // onesweep sort: histograms, digit starts, tickets, look-back status
   Buffer f_dsort;     // single-launch depth sort: barrier counters, totals, rows (kept zero between launches)
-  Buffer f_dos;       // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
-  Buffer f_pair;      // single-launch depth sort without offsets: intermediate pairs (with f_sdo)
-  Buffer f_raw;       // its first pass's digit counts (zero between frames)
+  Buffer f_raw;       // onesweep depth sort: the first pass's digit counts (zero between frames)
   // State that kernels keep between launches, to be cleared before its next
   // use after an error was latched on the device (a bounded wait may have
   // given up mid-launch): the depth sort's buffers, the onesweep header, the
   // radix grid barrier words, the view totals.
-  bool dsort_dirty = true, dos_dirty = true, os_dirty = false, bar_dirty = false, vtot_dirty = true;
-  // fused-frame / multi-view buffers
+  bool dsort_dirty = true, dos_dirty = true, os_dirty = false, bar_dirty = false;
   Buffer f_rec3, f_conic;  // projected records and conics of tdgs_sort_frame_3d
   Buffer d_cams;           // cameras of the 3D calls (device)
   Buffer diag;             // barrier words of tdgs_diag_barrier_timeout
@@ -132,23 +169,9 @@ struct tdgs_context {
   bool proj_on = false;
   Buffer b_keys, b_vals;   // padded scratch of tdgs_sort_pairs_bitonic
   Buffer n_counts, n_offs, n_norm, n_keys[2], n_vals[2], n_ranges;  // tdgs_sort_frame_normalized
-  Buffer f_counts, f_dkey[3], f_dval[3], f_soff, f_sdo, f_rminmax, f_stream[2], f_keys, f_values, f_ranges;
-  Buffer f_rects, f_c1, f_rows, f_segs, f_cols, f_c2, f_b2;  // interval splits
   // depth-key range: accumulators [0..1], result [2..3], passes of the last
   // resident depth sort [4]
   uint32_t* d_range = nullptr;
-  // f_rminmax holds first positions in its first half and one-past-last
-  // positions in its second half, kept at (all ones, zero) between frames:
-  // the ranges kernel resets what the last tile pass recorded
-  bool rminmax_dirty = true;
-  ViewBlob* d_views = nullptr;  // device view table
-  ViewBlob* h_views = nullptr;  // pinned staging of the table
-  uint32_t nv = 0, n_all = 0, t_all = 0;
-  uint32_t max_gx = 0, max_gy = 0;  // over the staged views
-  bool norm = false;            // the frame with the 32-bit normalised key (by interval splits)
-  bool split = false;           // pairs by interval splits (else packed elements and tile passes)
-  uint64_t capacity = 0;        // pair capacity reserved for the asynchronous path
-  bool reserved = false;
   Tuning tuning;
   std::string last_error;
   // tracing
@@ -217,8 +240,22 @@ tdgs_status ensure(tdgs_context* ctx, Buffer& b, size_t bytes, cudaStream_t s,
 uint32_t* err_word(tdgs_context* ctx) { return &ctx->d_status->err; }
 
 void note_device_error(tdgs_context* ctx) {
-  ctx->dsort_dirty = ctx->dos_dirty = ctx->os_dirty = ctx->bar_dirty = ctx->vtot_dirty = true;
+  ctx->dsort_dirty = ctx->dos_dirty = ctx->os_dirty = ctx->bar_dirty = true;
+  ctx->vtot_dirty = ctx->norm_state.vtot_dirty = true;
 }
+
+// The normalised frame's state in place of the fused frame's, for a scope.
+class UseNormState {
+ public:
+  explicit UseNormState(tdgs_context* ctx) : ctx_(ctx) { swap(); }
+  ~UseNormState() { swap(); }
+  UseNormState(const UseNormState&) = delete;
+  UseNormState& operator=(const UseNormState&) = delete;
+
+ private:
+  void swap() { std::swap(static_cast<FrameState&>(*ctx_), ctx_->norm_state); }
+  tdgs_context* ctx_;
+};
 
 // The radix grid barrier words back to zero if an error was latched since
 // their last use.
@@ -486,8 +523,7 @@ tdgs_status tdgs_context_create(tdgs_context** out, int device) {
       cudaMallocHost(&ctx->h_status, sizeof(DevStatus)) != cudaSuccess ||
       cudaHostAlloc(&ctx->h_early, sizeof(EarlyStatus), cudaHostAllocMapped) != cudaSuccess ||
       cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_early), ctx->h_early, 0) != cudaSuccess ||
-      cudaMalloc(&ctx->d_views, sizeof(ViewBlob)) != cudaSuccess ||
-      cudaMallocHost(&ctx->h_views, sizeof(ViewBlob)) != cudaSuccess ||
+      !ctx->allocate_tables() ||
       cudaMemset(ctx->d_status, 0, sizeof(DevStatus)) != cudaSuccess ||
       cudaMemset(ctx->d_tickets, 0, 4 * sizeof(uint32_t)) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->ev_count, cudaEventDisableTiming) != cudaSuccess ||
@@ -551,18 +587,12 @@ void tdgs_context_destroy(tdgs_context* ctx) {
   DeviceGuard g(ctx->device);
   drain_timings(ctx);
   for (cudaEvent_t e : ctx->free_events) cudaEventDestroy(e);
-  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort, &ctx->f_dos, &ctx->f_raw, &ctx->f_pair, &ctx->f_counts, &ctx->f_dkey[0],
-                    &ctx->f_dkey[1],    &ctx->f_dkey[2],     &ctx->f_dval[0],    &ctx->f_dval[1],
-                    &ctx->f_dval[2],    &ctx->f_soff,       &ctx->f_sdo,        &ctx->f_rec3,
-                    &ctx->f_conic,      &ctx->d_cams,       &ctx->diag,       &ctx->b_keys,       &ctx->b_vals,       &ctx->n_counts,
+  Buffer* bufs[] = {&ctx->scan_status, &ctx->sort_scratch, &ctx->os_scratch, &ctx->f_dsort,
+                    &ctx->f_raw,        &ctx->f_rec3,       &ctx->f_conic,      &ctx->d_cams,       &ctx->diag,       &ctx->b_keys,       &ctx->b_vals,       &ctx->n_counts,
                     &ctx->n_offs,       &ctx->n_norm,       &ctx->n_keys[0],    &ctx->n_keys[1],
-                    &ctx->n_vals[0],    &ctx->n_vals[1],    &ctx->n_ranges,
-                    &ctx->f_rminmax,    &ctx->f_stream[0],   &ctx->f_stream[1],  &ctx->f_keys,
-                    &ctx->f_values,     &ctx->f_ranges,     &ctx->r_order,
-                    &ctx->f_rects,      &ctx->f_c1,         &ctx->f_rows,       &ctx->f_segs,       &ctx->f_cols,       &ctx->f_c2,
-                    &ctx->f_b2};
-  if (ctx->d_views) cudaFree(ctx->d_views);
-  if (ctx->h_views) cudaFreeHost(ctx->h_views);
+                    &ctx->n_vals[0],    &ctx->n_vals[1],    &ctx->n_ranges,     &ctx->r_order};
+  ctx->release();
+  ctx->norm_state.release();
   for (Buffer* b : bufs)
     if (b->p) cudaFree(b->p);
   if (ctx->d_status) cudaFree(ctx->d_status);
@@ -744,8 +774,9 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
 
 // One view through the interval splits: its table goes with the kernel
 // parameters (a copy to the device before the first kernel costs a small
-// frame a twentieth of its time); otherwise it is uploaded.
-bool table_in_params(const tdgs_context* ctx) { return ctx->split && ctx->nv == 1; }
+// frame a twentieth of its time); otherwise it is uploaded, as the
+// asynchronous calls' always is: a replay reads the table staged last.
+bool table_in_params(const tdgs_context* ctx) { return ctx->split && ctx->nv == 1 && ctx->exact; }
 
 ViewTable device_table(tdgs_context* ctx) {
   ViewBlob* d = ctx->d_views;
@@ -767,17 +798,24 @@ ViewTable device_table(tdgs_context* ctx) {
 // Whether the staged views' pairs come from the interval splits: images up to
 // 4096 pixels a side, and several views only up to the Gaussians that the
 // depth sort orders view after view; a tuned tile digit width asks for the
-// tile passes.
+// tile passes.  A rectangle's bounds are a byte each, hence 256 rows and
+// columns; inside that range the splits are the faster form at every size
+// measured (us a frame, tile passes and splits: 10,000 Gaussians 78 and 46,
+// 1M 239 and 145, 3M 867 and 390, 4096x2304 244 and 137, 64 views 1410 and
+// 832).
 bool splits(const tdgs_context* ctx) {
   return (ctx->nv == 1 || ctx->n_all < (1u << 30)) && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
          ctx->tuning.tile_digit_bits == 0;
 }
 
 // A view of at most kSplitSmall Gaussians and kSmallTiles tiles of segments
-// takes one launch for all of it.
+// takes one launch for all of it: kSplitSmall says where the line lies, and
+// 1024 tiles are about seven for each of the launch's blocks, one per SM (the
+// separate launch runs three per SM).
 constexpr uint32_t kSmallTiles = 1024;
 
 uint32_t split_pitch(const tdgs_context* ctx) { return (ctx->max_gx + 7u) & ~7u; }
+uint32_t split_max_rows(const tdgs_context* ctx) { return (ctx->max_gy + 7u) & ~7u; }
 uint32_t split_rows(const tdgs_context* ctx) { return ctx->h_views->row_begin[ctx->nv]; }
 // Level-2 tiles of at most m segments: full ones, and one ragged one per row.
 uint64_t split_tiles(const tdgs_context* ctx, uint64_t m) { return m / kSplitTile + split_rows(ctx); }
@@ -857,6 +895,19 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
     }
   }
   return st;
+}
+
+// Whether the staged views of at most m pairs fit the interval splits'
+// buffers as they are.  A reservation takes every batch with its counts of
+// views, Gaussians and tiles; images of other proportions, or Gaussians
+// spread over the views in another way, may need more rows or columns than it
+// sized.
+bool split_fits(const tdgs_context* ctx, uint64_t m) {
+  const size_t entries = static_cast<size_t>(split_tiles(ctx, m)) * split_pitch(ctx);
+  return ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
+         ctx->f_c1.bytes >= static_cast<size_t>(ctx->h_views->c1_begin[ctx->nv]) * 8 &&
+         ctx->f_rows.bytes >= (static_cast<size_t>(split_rows(ctx)) + 1) * 20 && ctx->f_c2.bytes >= entries * 2 &&
+         ctx->f_b2.bytes >= entries * 4;
 }
 
 // Buffers that depend on the pair count (or capacity) m.
@@ -1020,20 +1071,24 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.total = &ctx->d_status->total;
   a.ticket = ctx->d_tickets;
   a.bar = ctx->d_tickets + 2;
-  a.ntiles1 = ctx->h_views->t1_begin[ctx->nv];
+  // (a captured batch may be replayed with its Gaussians spread over the views
+  // in another way: a ragged tile per view at most)
+  a.ntiles1 = a.vt.one.on ? ctx->h_views->t1_begin[1] : ctx->n_all / kSplitTile + ctx->nv;
+  a.max_gy = split_max_rows(ctx);
+  a.c1_cap = ctx->f_c1.bytes / sizeof(uint2);
   a.err = err_word(ctx);
   const uint32_t tiles2 = static_cast<uint32_t>(split_tiles(ctx, m));
   const int cps = ctx->tuning.ctas_per_sm;
-  if (ctx->nv == 1 && n_all > 0 && n_all <= kSplitSmall && tiles2 <= kSmallTiles) {
+  if (table_in_params(ctx) && n_all > 0 && n_all <= kSplitSmall && tiles2 <= kSmallTiles) {
     TDGS_TRACED(ctx, kKSmallSplit, m, s, launch_small_split(a, std::max(ctx->max_gx, ctx->max_gy), tiles2, s));
     return TDGS_OK;
   }
   TDGS_TRACED(ctx, kKRowCount, n_all, s, launch_row_count(a, s));
   TDGS_TRACED(ctx, kKRowScan, a.nrows, s, launch_row_scan(a, s));
-  TDGS_TRACED(ctx, kKRowSplit, n_all, s, launch_row_split(a, ctx->max_gy, cps, s));
+  TDGS_TRACED(ctx, kKRowSplit, n_all, s, launch_row_split(a, a.max_gy, cps, s));
   TDGS_TRACED(ctx, kKColCount, m, s, launch_col_count(a, tiles2, s));
   TDGS_TRACED(ctx, kKColScan, a.nrows, s, launch_col_scan(a, s));
-  TDGS_TRACED(ctx, kKColSplit, m, s, launch_col_split(a, ctx->max_gx, tiles2, cps, s));
+  TDGS_TRACED(ctx, kKColSplit, m, s, launch_col_split(a, a.pitch, tiles2, cps, s));
   return TDGS_OK;
 }
 
@@ -1108,6 +1163,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
 // before the GPU runs out of work.
 tdgs_status sort_views_exact(tdgs_context* ctx, cudaStream_t s, uint32_t* m_out) {
   ctx->split = ctx->norm || splits(ctx);
+  ctx->exact = true;
   tdgs_status st = ensure_record_buffers(ctx, s);
   if (st != TDGS_OK) return st;
   st = run_front(ctx, s, true);
@@ -1359,14 +1415,14 @@ tdgs_status tdgs_sort_frame_normalized(tdgs_context* ctx, const tdgs_gaussian2d*
   if ((f.width + 15) / 16 <= kSplitMaxBins && (f.height + 15) / 16 <= kSplitMaxBins) {
     // the fused frame with normalised depths for keys; its order is that of
     // the steps below: equal keys keep the Gaussians' index order
+    UseNormState use(ctx);
+    if (!ctx->allocate_tables()) return cuda_fail(ctx, cudaGetLastError(), "view table");
     tdgs_view view{g, n, f};
     st = stage_views(ctx, &view, 1);
     if (st != TDGS_OK) return st;
-    ctx->reserved = false;
     ctx->norm = true;
     uint32_t m = 0;
     st = sort_views_exact(ctx, s, &m);
-    ctx->norm = false;
     if (st != TDGS_OK) return st;
     *sorted_keys = static_cast<const uint32_t*>(ctx->n_keys[0].p);
     *sorted_values = static_cast<const uint32_t*>(ctx->f_values.p);
@@ -1489,9 +1545,16 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
   DeviceGuard dg(ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tdgs_status st = stage_views(ctx, views, num_views);
-  if (st == TDGS_OK) ctx->split = splits(ctx);  // the asynchronous calls keep this choice
-  if (st == TDGS_OK) st = ensure_record_buffers(ctx, s);
-  if (st == TDGS_OK) st = ensure_pair_buffers(ctx, pair_capacity, s);
+  ctx->exact = false;
+  ctx->split_reserved = st == TDGS_OK && splits(ctx);  // the asynchronous calls keep this choice
+  // the tile passes' buffers too: they take a batch with the same totals whose
+  // rows or columns the splits' buffers do not hold (split_fits)
+  for (const bool split : {false, true}) {
+    if (split && !ctx->split_reserved) continue;
+    ctx->split = split;
+    if (st == TDGS_OK) st = ensure_record_buffers(ctx, s);
+    if (st == TDGS_OK) st = ensure_pair_buffers(ctx, pair_capacity, s);
+  }
   if (st != TDGS_OK) return st;
   TDGS_CUDA(ctx, cudaStreamSynchronize(s));
   ctx->capacity = pair_capacity;
@@ -1510,6 +1573,8 @@ tdgs_status tdgs_sort_views_async(tdgs_context* ctx, const tdgs_view* views, uin
   if (st != TDGS_OK) return st;
   if (ctx->n_all != n_prev || ctx->t_all != t_prev || ctx->nv != nv_prev)
     return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "views differ in shape from the reservation");
+  ctx->split = ctx->split_reserved && split_fits(ctx, ctx->capacity);
+  ctx->exact = false;
   st = run_front(ctx, s);
   if (st != TDGS_OK) return st;
   return run_back(ctx, static_cast<uint32_t>(ctx->capacity), &ctx->d_status->total, s);

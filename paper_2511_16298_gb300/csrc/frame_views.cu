@@ -3,8 +3,10 @@
 // is one frame; several views of one scene are sorted together with one
 // set of passes, each view keeping its local tile ids and its own list.
 //
-// The Gaussians of all views are sorted by depth first; every Gaussian's
-// pairs are then emitted in that depth order as packed elements
+// The Gaussians of all views are sorted by depth first.  Images of up to 4096
+// pixels a side then take the interval splits (interval_split.cu), and only
+// the count kernel here.  For larger ones, and where a digit width is tuned,
+// every Gaussian's pairs are emitted in that depth order as packed elements
 // (global tile << rbits | depth position), and a stable sort on the tile
 // bits alone yields the order by (tile, depth, index) that a stable sort of
 // the 64-bit keys defines: ties of the 64-bit key are pairs of distinct

@@ -27,6 +27,14 @@
 // and one XOR scan over the bins, whatever the intervals.  The rank of item i
 // in a bin is the number of lower bits of that bin's mask, plus the bin's
 // items in the warps before.
+//
+// Measured against the form this replaced (an expanding pass that wrote packed
+// (tile, depth rank) elements and a second pass over them, both serial in a
+// look-back chain), whole frames: 1M Gaussians at 1280x720 (10.6M pairs) 239
+// to 145 us, 3M at 1080p 867 to 390 us, 64 views 1410 to 832 us.  Two levels
+// with counts and a scan in place of one pass with a look-back: the counts
+// read 2 to 4 B per item where the look-back held every tile for the one
+// before, and no launch waits inside.
 #include "radix.cuh"
 
 namespace tdgs {
@@ -113,19 +121,41 @@ __device__ __forceinline__ Place place_of(const SplitArgs& a, uint32_t v) {
   return Place{t0, __ldg(a.t1_begin + v + 1) - t0, __ldg(a.row_begin + v), __ldg(a.c1_begin + v)};
 }
 
+// A captured batch reads its view table when it is replayed: views may have
+// other proportions or Gaussians by then, within the same totals.  The counts
+// of tiles and rows come from the table, and a view that the launches or
+// buffers have no room for is left out (k_row_scan reports it).
+__device__ __forceinline__ uint32_t tiles1_of(const SplitArgs& a) {
+  return a.vt.one.on ? a.ntiles1 : __ldg(a.t1_begin + a.vt.nv);
+}
+__device__ __forceinline__ uint32_t rows_of(const SplitArgs& a) {
+  return a.vt.one.on ? a.nrows : min(a.nrows, __ldg(a.row_begin + a.vt.nv));
+}
+__device__ __forceinline__ bool has_room(const SplitArgs& a, const Place& pl, const FrameGeom& fg) {
+  return static_cast<uint32_t>(fg.gx) <= a.pitch && static_cast<uint32_t>(fg.gy) <= a.max_gy &&
+         pl.c10 + static_cast<uint64_t>(pl.tiles) * fg.gy <= a.c1_cap;
+}
+
 // ------------------------------------------------------------ level 1 count
 // Per tile of 1024 depth positions: each Gaussian's {depth key, index} and
 // rectangle in depth order (coalesced for the later launches; the records
 // are gathered here, once), and per row its Gaussians and its pairs in the
 // tile, as differences at the first row and past the last.
+// Bound by the gather of 16 B records from L2 in depth order (four in flight
+// per thread): 12.8 us for 1M Gaussians, 28.5 us for 3M (1.0 and 1.3 TB/s of
+// 32 B sectors that hold two records).  Gathered here, the depth sort need
+// carry no rectangle or count per Gaussian, and the split reads 12 B per item
+// in order.
 __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
   __shared__ int s_d[kMaxBins + 1][2];
   __shared__ uint32_t s_w[kCountThreads / 32][2];
   begin_launch();
   const uint32_t t = threadIdx.x;
+  if (blockIdx.x >= tiles1_of(a)) return;
   const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.t1_begin, a.vt.nv, blockIdx.x);
   const Place pl = place_of(a, v);
   const ViewOf vw = view_of(a.vt, v);
+  if (!has_room(a, pl, vw.geom)) return;
   const uint32_t tl = blockIdx.x - pl.tile0, nt = pl.tiles, rec0 = vw.rec0, nrec = vw.nrec;
   const FrameGeom fg = vw.geom;
   const float4* __restrict__ g = vw.g;
@@ -134,7 +164,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
   constexpr int kPer = kTile / kCountThreads;
   const uint32_t first = tl * kTile;
   float dmin = 0.0f, scale = 0.0f;
-  if (a.keys32) {
+  if (a.norm) {
     dmin = __uint_as_float(__ldcg(a.norm));
     scale = norm_scale(dmin, __uint_as_float(__ldcg(a.norm + 1)));
   }
@@ -165,7 +195,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
     }
     a.rects[rec0 + p] = pack;
     // the low part of the pairs' keys: depth bits, or the normalised depth
-    const uint32_t low = a.keys32 ? norm_depth(rec[u].z, dmin, scale) : __float_as_uint(rec[u].z);
+    const uint32_t low = a.norm ? norm_depth(rec[u].z, dmin, scale) : __float_as_uint(rec[u].z);
     a.sdo[rec0 + p] = make_uint2(low, gi[u]);
   }
   __syncthreads();
@@ -180,6 +210,9 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
 // row its first segment, first level-2 tile and first pair.  More pairs than
 // the buffers hold (or than the depth order accounts for) latches
 // TDGS_ERR_CAPACITY and leaves nothing for the later launches to do.
+// Latency: a row's tiles in one or a few steps of 1024, one ticket, and the
+// last block's scan of the rows: 5.5 us for 45 rows of 977 tiles, 8.4 us for
+// 68 rows of 2930.
 __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
   __shared__ uint32_t s_w[kCountThreads / 32][2];
   __shared__ unsigned long long s_w64[kCountThreads / 32][2];
@@ -189,7 +222,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
   const uint32_t t = threadIdx.x, r = blockIdx.x;
   const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
   const Place pl = place_of(a, v);
-  const uint32_t nt = pl.tiles;
+  const uint32_t nt = r < rows_of(a) && has_room(a, pl, view_of(a.vt, v).geom) ? pl.tiles : 0u;
   uint2* __restrict__ col = a.c1 + pl.c10 + static_cast<size_t>(r - pl.row0) * nt;
   uint32_t segs = 0, pairs = 0;
   for (uint32_t i0 = 0; i0 < nt; i0 += kCountThreads * kPer) {
@@ -222,14 +255,17 @@ __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
     __syncthreads();
   }
   if (t == 0) {
-    a.row_tot[r] = make_uint2(segs, pairs);
+    a.row_tot[r] = make_uint2(segs, pairs);  // (one entry per block)
     __threadfence();
     s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const uint32_t nrows = gridDim.x;
+  bool room = true;
+  for (uint32_t i = t; i < a.vt.nv; i += kCountThreads) room &= has_room(a, place_of(a, i), view_of(a.vt, i).geom);
+  const uint32_t nrows = gridDim.x;  // (rows beyond the table's have no segments)
+  room = __syncthreads_and(room) && (a.vt.one.on || __ldg(a.row_begin + a.vt.nv) <= a.nrows);
   uint32_t seg0 = 0, tile0 = 0;
   unsigned long long pair0 = 0;
   for (uint32_t i0 = 0; i0 < nrows; i0 += kCountThreads) {
@@ -256,7 +292,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
     __syncthreads();
   }
   if (t == 0) {
-    const bool fits = pair0 == *a.total && pair0 <= a.cap;
+    const bool fits = room && pair0 == *a.total && pair0 <= a.cap;
     if (!fits)
       latch_error(a.err, *a.total > 0xffffffffull ? TDGS_ERR_OVERFLOW : TDGS_ERR_CAPACITY, kSiteViewsDup);
     a.row_seg[nrows] = seg0;
@@ -269,6 +305,8 @@ __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
 
 // ------------------------------------------------------------ level 2 count
 // Per tile of 1024 segments of one row: the segments that cover each column.
+// Two shared atomics per segment and one 2 B read: 8.6 us for 2.6M segments,
+// 18.8 us for 8.6M, half of it launch, search and the scan of the columns.
 __global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
   __shared__ int s_d[kMaxBins + 1];
   __shared__ uint32_t s_w[kCountThreads / 32];
@@ -311,7 +349,12 @@ __global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
 // One block per row: the first output position of every tile and column, and
 // the row's tile ranges (relative to the view's first pair; {0, 0} if
 // empty).  Thread (g, c) walks column c over the g-th share of the row's
-// tiles: once for the sums, once for the positions.
+// tiles: once for the sums, once for the positions (the second time from L1
+// or L2).  Latency of the two walks with eight loads in flight: 8.8 us for
+// 45 rows of ~58 tiles, 10.8 us for 68 of ~125.  One block per row, not the
+// count kernel's last block of a row: that made count and scan one launch,
+// but 43 and 171 us of it where these two take 17 and 30: a block in a scan
+// holds up its later tiles, so the rows end one after another.
 constexpr int kScanThreads = 1024;
 __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
   __shared__ uint32_t s_sum[kScanThreads];
@@ -319,6 +362,7 @@ __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
   begin_launch();
   if (__ldg(a.info + 1) == 0u) return;  // more pairs than the buffers hold
   const uint32_t t = threadIdx.x, r = blockIdx.x;
+  if (r >= rows_of(a)) return;
   const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
   const uint32_t gx = static_cast<uint32_t>(view_of(a.vt, v).geom.gx), y = r - place_of(a, v).row0;
   const uint32_t lp = gx <= 32 ? 5u : 32u - static_cast<uint32_t>(__clz(gx - 1));  // columns padded to 2^lp
@@ -383,6 +427,20 @@ __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
 //            positions in bin order;
 //   flush    the staged pairs in bin order: runs of consecutive addresses.
 // A tile with more pairs than the stage holds takes windows of whole bins.
+//
+// Level 2 is the frame's longest kernel and bound by instruction issue and the
+// shared-memory pipe together (10.6M pairs: 3.3 warp instructions per
+// pair, issue 60 %, LSU data pipe 68 % busy, 69 % of the warps
+// resident), not by its 127 MB of final pairs, of which 65 to 81 MB reach
+// DRAM inside the launch: 51 us, 2.5 TB/s written; 166 us for the 36M pairs of
+// a 3M-Gaussian frame, 2.6 TB/s.  Level 1: 18.6 us for 2.6M segments.  What it
+// replaced took 154 us for the 10.6M pairs (expand + one tile pass).
+// 512 threads and 1024 items, three blocks per SM, so that one block's flush
+// overlaps another's ranks.  A frame of 1M / 3M Gaussians takes longer with 256
+// threads and 512 items (1.2 / 13 us), 256 and 1024 (8 / 20), 512 and 512 (11 /
+// 33: every tile pays for its bins, and its runs are half as long).  The owner
+// search over the starts' word took the 1M column split from 75 us (each lane
+// walking its own item's bins) to 57.
 template <int kWords>  // 32 kWords bins; each lane scans kWords consecutive ones
 struct Smem {
   static constexpr int kBinsP = 32 * kWords;
@@ -548,7 +606,7 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
   begin_launch();
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   if (__ldg(a.info + 1) == 0u) return;
-  const uint32_t ntiles = kLevel == 1 ? a.ntiles1 : __ldg(a.info);
+  const uint32_t ntiles = kLevel == 1 ? tiles1_of(a) : __ldg(a.info);
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     uint32_t v, beg, cnt, bins, r = 0, tl = 0;
     Place pl;
@@ -629,6 +687,11 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
 // counts need no phase of their own: every block sums the few tiles' counts of
 // all rows for level 1, and counts all segments of its tile's row for level 2
 // (at most kSplitSmall of them: the sums are kept in 16 bits).
+// Bound by the latency of its phases and two barriers: for 10,000 Gaussians
+// (57k pairs) one launch of ~20 us in place of six (34 us), the frame 57 to
+// 46 us; 30,000 Gaussians 58 to 50 us.  From ~60,000 on the six launches are
+// as fast, since every block of level 2 counts its whole row again: the line
+// (kSplitSmall) lies below, where the 16-bit sums end too.
 // What an earlier phase wrote is read through L2 (__ldcg).  A barrier that
 // times out ends the block: the counts that size the staging are then not to
 // be trusted.
@@ -678,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_small(SplitArgs a) {
   constexpr int kPer = kTile / kThreads;
   // ---- rectangles in depth order and the rows' counts
   float dmin = 0.0f, scale = 0.0f;
-  if (a.keys32) {
+  if (a.norm) {
     dmin = __uint_as_float(__ldcg(a.norm));
     scale = norm_scale(dmin, __uint_as_float(__ldcg(a.norm + 1)));
   }
@@ -703,7 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_small(SplitArgs a) {
         atomicAdd(&s_d[q.y1][1], -w);
       }
       a.rects[p] = pack;
-      a.sdo[p] = make_uint2(a.keys32 ? norm_depth(rec.z, dmin, scale) : __float_as_uint(rec.z), gi);
+      a.sdo[p] = make_uint2(a.norm ? norm_depth(rec.z, dmin, scale) : __float_as_uint(rec.z), gi);
     }
     __syncthreads();
     unsigned long long c = t < kMaxBins ? static_cast<uint32_t>(s_d[t][0]) : 0u;

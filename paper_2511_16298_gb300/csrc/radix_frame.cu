@@ -1,6 +1,8 @@
 // Radix passes of the depth-first frame path: the depth sort of the N
-// Gaussians and the stable passes over the packed (tile, depth rank)
-// stream, the last of which expands to the final keys and indices.
+// Gaussians and, for images above 4096 pixels a side and tuned digit widths
+// (the interval splits take the rest), the stable passes over the packed
+// (tile, depth rank) stream, the last of which expands to the final keys and
+// indices.
 #include "radix.cuh"
 
 namespace tdgs {
@@ -37,7 +39,10 @@ DepthPlan plan_depth_sort(uint32_t n, int tuned_bits, int ctas_per_sm, bool offs
   if (g && nn <= depth_sort_count_capacity(g, 16)) {
     p.resident = true;
     // the smallest tile that takes the keys with one CTA per SM, and no more
-    // CTAs than it fills
+    // CTAs than it fills: a pass's time is one CTA's ranking of its tile and
+    // the wait for the others' counts (10,000 Gaussians, 16 keys per thread
+    // on all SMs and 4 on 5 of them: 44 and 27 us).  The form with the
+    // offsets keeps 16: only large images and tuned digits take it.
     p.items = 16;
     if (!offsets) {
       while (p.items > 4 && nn <= depth_sort_count_capacity(g, p.items / 2)) p.items /= 2;

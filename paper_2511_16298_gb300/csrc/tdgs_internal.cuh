@@ -317,12 +317,13 @@ cudaError_t launch_views_dup(const ViewTable& vt, const uint32_t* sorder, const 
 // keys compressed to their range (key - smallest; culled Gaussians one past
 // the largest) with as many 9-bit digits as that range needs (3 for a range
 // below 2^27, 4 at most).  When the Gaussians fit one 8192-key chunk per
-// resident CTA, the whole sort and the scan of the tile counts in depth
-// order run in one cooperative launch (launch_depth_sort).  Larger N (below
-// 2^30) take the onesweep passes over 32-bit keys (onesweep.cu): a
-// histogram launch and kDepthOnesweepPasses pass launches, each reading the
-// pass plan from the key range (passes beyond it end at once), the result
-// in buffer pair 1; the scan of the counts in depth order follows.
+// resident CTA, the whole sort and, where the tile passes follow, the scan
+// of the tile counts in depth order run in one cooperative launch
+// (launch_depth_sort).  Larger N (below 2^30) take the onesweep passes over
+// 32-bit keys (onesweep.cu): kDepthOnesweepPasses pass launches, each reading
+// the pass plan from the key range (passes beyond it end at once), the first
+// digit's counts from the count kernel, and with several views in view order
+// one more pass by view; the result is in buffer pair 1 (2 by view).
 // Otherwise one launch per pass over all 32 bits: 8-bit (4 passes) or, if
 // tuned, 11-bit (3 passes) digits.
 struct DepthPlan {
@@ -363,8 +364,8 @@ cudaError_t launch_depth_pass(const DepthPlan& dp, uint32_t pass, const uint32_t
 //    receives only counts of 1023 or more.
 //  * Without (launch_depth_sort): key0 = the count kernel's depth keys,
 //    counts its tile counts, range[2..3] its range.
-//  * With offsets null the launch stops at v1: counts is not read, and several views are ordered view after view (by
-//    depth inside each).
+//  * With offsets null the launch stops at v1: counts is not read, and
+//    several views are ordered view after view (by depth inside each).
 struct DepthSortArgs {
   const uint32_t* key0;
   ViewTable vt;
@@ -444,17 +445,22 @@ struct SplitArgs {
   uint2* ranges;
   uint64_t* keys;
   uint32_t* values;
-  uint32_t* keys32;           // not null: the 32-bit normalised keys, in place of keys
-  const uint32_t* norm;       // with keys32: smallest and largest visible depth (float bits)
+  uint32_t* keys32;           // with norm: the 32-bit normalised keys, in place of keys
+  const uint32_t* norm;       // not null: normalised keys; smallest and largest visible depth (float bits)
   uint64_t cap;               // pairs that segs, keys and values hold
   const uint64_t* total;      // the pair count
   uint32_t* ticket;           // a zero word, left zero
   uint32_t* bar;              // two words of the radix passes' grid barrier
-  uint32_t ntiles1, nrows;
+  uint32_t ntiles1, nrows;    // one view in vt.one: its tiles and rows; else the most there can be
+  uint32_t max_gy;            // most rows and (pitch) columns that the launches take
+  uint64_t c1_cap;            // entries of c1
   uint32_t* err;
 };
 // One view of at most kSplitSmall Gaussians in one cooperative launch
-// (max_bins: the larger of its rows and columns).
+// (max_bins: the larger of its rows and columns).  The line: the launch keeps
+// a row's column sums in 16 bits, and it wins only up to there (10,000
+// Gaussians 46 us a frame against 57 with the six launches, 30,000 50 against
+// 58, 60,000 equal).
 constexpr uint32_t kSplitSmall = 32 * kSplitTile;
 cudaError_t launch_small_split(const SplitArgs& a, uint32_t max_bins, uint32_t max_tiles, cudaStream_t s);
 cudaError_t launch_row_count(const SplitArgs& a, cudaStream_t s);
@@ -511,8 +517,8 @@ cudaError_t launch_radix_pass(const SortPlan& plan, uint32_t pass, const uint64_
                               uint32_t* scratch, uint32_t* bar, uint32_t* err, cudaStream_t s);
 
 // Onesweep form of tdgs_sort_pairs (onesweep.cu): one histogram launch
-// that reads the keys once, then one launch per digit pass with a
-// decoupled look-back.  Eligible for 0 < m < 2^30 pairs with all four
+// that reads the keys once, then one launch per digit pass whose scan CTAs
+// turn the tiles' counts into prefixes.  Eligible for 0 < m < 2^30 pairs with all four
 // buffers 16-byte aligned (the tiles arrive by bulk copies).  Scratch:
 // onesweep_scratch_words(m) uint32 words whose first
 // onesweep_header_words() are zero when first used (the kernels leave
@@ -529,9 +535,9 @@ cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint
                                  cudaStream_t s);
 // The same passes over the depth sort's 32-bit keys (dk[0], dv[0]: keys and
 // indices from the count kernel; range: the key range it published in
-// range[2..3]; the histogram writes the pass count to range[4]).  The pass
-// plan is read on the device: launch the histogram,
-// then passes 0 .. kDepthOnesweepPasses - 1 in order; passes the range does
+// range[2..3], and raw: the counts of the keys' low 9 bits, which it makes
+// when given depth_onesweep_prep).  The pass plan is read on the device:
+// passes 0 .. kDepthOnesweepPasses - 1 in order; passes the range does
 // not need end at once, and the last pass that runs writes dk[1], dv[1]
 // (dk[2], dv[2] hold intermediate passes).  Scratch as above for m = n,
 // separate from any other sort's while both may be in use.

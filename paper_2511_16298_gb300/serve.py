@@ -67,8 +67,9 @@ class Result:
 
 def estimate_bytes(n: int, width: int, height: int, pairs_per_gaussian: float = 24.0) -> int:
     """Conservative device footprint of one request: its records (16 B),
-    the per-Gaussian sort buffers (24 B), and per pair the two packed
-    stream buffers, the final keys and values (<= 28 B)."""
+    the per-Gaussian sort buffers (24 B), and per pair the segments or
+    packed stream buffers, the final keys and values (<= 28 B; a generous
+    pair count covers the depth sort's further buffers)."""
     tiles = ((width + 15) // 16) * ((height + 15) // 16)
     m = int(n * pairs_per_gaussian)
     return 16 * n + 24 * n + 28 * m + 24 * tiles
@@ -89,7 +90,9 @@ def _tiles(r: Request) -> int:
 def narrow_elements(n: int, tiles: int) -> bool:
     """Whether a batch of n Gaussians over `tiles` tiles (all views) sorts
     with 32-bit packed (tile, depth rank) elements and at most two 8-bit
-    tile passes -- the library's cheaper per-pair form."""
+    tile passes where it takes the tile passes (images above 4096 pixels a
+    side, or a tuned tile digit width) -- their cheaper per-pair form.  The
+    interval splits cost the same per pair on both sides of this line."""
     return _bits(n) + _bits(tiles) <= 32 and _bits(tiles) <= 16
 
 

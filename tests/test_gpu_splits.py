@@ -203,3 +203,117 @@ def test_duplicate_and_ranges_steps(ctx, oracle, n, cap):
         want[:, 1] = np.searchsorted(tiles, np.arange(fr.num_tiles), "right")
         want[want[:, 0] == want[:, 1]] = 0
         assert np.array_equal(r.cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("n", [5000, 60_000])
+def test_normalized_key_first_call(oracle, n):
+    """A context's first call: nothing is allocated yet."""
+    fr = synth.frame_random(n, n, 500, 300)
+    st, ek, ev, er = oracle.sort_frame_normalized(fr.gaussians, fr.width, fr.height)
+    assert st == 0
+    c = T.Context(0)
+    try:
+        k, v, r, m = c.sort_frame_normalized(T.records_to_tensor(fr.gaussians, DEV), fr.width, fr.height)
+        c.sync()
+        assert m == len(ek)
+        assert np.array_equal(k.cpu().numpy().view(np.uint32), ek)
+        assert np.array_equal(v.cpu().numpy().view(np.uint32), ev)
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), er)
+    finally:
+        c.close()
+
+
+def test_normalized_call_keeps_frames(ctx, oracle):
+    """A frame's results, a batch between its asynchronous call and its
+    results, and a captured batch all outlive a larger normalised-key frame on
+    the same context."""
+    a, b = synth.frame_random(1, 3000, 320, 200), synth.frame_random(2, 60_000, 1000, 700)
+    ga, gb = T.records_to_tensor(a.gaussians, DEV), T.records_to_tensor(b.gaussians, DEV)
+    ref = oracle.sort_frame(a.gaussians, a.width, a.height)
+
+    def equal(res):
+        assert res[3] == ref["m"]
+        assert np.array_equal(res[0].cpu().numpy().view(np.uint64), ref["keys"])
+        assert np.array_equal(res[1].cpu().numpy().view(np.uint32), ref["values"])
+        assert np.array_equal(res[2].cpu().numpy().view(np.uint32), ref["ranges"])
+
+    c = T.Context(0)
+    try:
+        res = c.sort_frame(ga, a.width, a.height)
+        c.sort_frame_normalized(gb, b.width, b.height)
+        equal(res)
+        views = [(ga, a.width, a.height)] * 2
+        c.reserve_views(views, 2 * ref["m"])
+        c.sort_frame_normalized(gb, b.width, b.height)
+        c.sort_views_async(views)  # (the reservation still stands)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            c.sort_views_async(views)
+        k, v, r, m = c.sort_frame_normalized(gb, b.width, b.height)
+        for x in c.views_results(2):
+            equal(x)
+        graph.replay()
+        for x in c.views_results(2):
+            equal(x)
+        st, ek, ev, er = oracle.sort_frame_normalized(b.gaussians, b.width, b.height)
+        assert st == 0 and m == len(ek)
+        assert np.array_equal(k.cpu().numpy().view(np.uint32), ek)
+        assert np.array_equal(v.cpu().numpy().view(np.uint32), ev)
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), er)
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("n,shapes,new", [
+    (20_000, [(1600, 64)], [(64, 1600)]),                              # one view, turned
+    (20_000, [(640, 160), (160, 640)], [(160, 640), (640, 160)]),      # two views exchanged
+    (20_000, [(320, 320), (320, 320)], [(6400, 16), (16, 6400)]),      # beyond the splits' 256 columns and rows
+    (700_000, [(320, 320), (320, 320)], [(640, 160), (160, 640)]),     # above one depth-sort launch
+])
+def test_reservation_takes_other_proportions(ctx, oracle, n, shapes, new):
+    """A reservation is for counts of views, Gaussians and tiles: batches with
+    the same totals in other proportions, and views with other Gaussian
+    counts, give their own results through the asynchronous call; replays of
+    the captured batch read the table staged last, and give its results or
+    report that they have no room for them."""
+    def batch(dims, split, seed):
+        ns = [n] if len(dims) == 1 else [int(n * split), 2 * n - int(n * split)]
+        return [synth.frame_random(seed + i, k, w, h, max_sigma=5.0) for i, (k, (w, h)) in enumerate(zip(ns, dims))]
+
+    def on_gpu(frames):
+        return [(T.records_to_tensor(f.gaussians, DEV), f.width, f.height) for f in frames]
+
+    def check(frames, res):
+        for f, (k, v, r, m) in zip(frames, res):
+            ref = oracle.sort_frame(f.gaussians, f.width, f.height)
+            assert ref["status"] == 0 and m == ref["m"]
+            assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
+            assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
+            assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
+
+    first, other = batch(shapes, 1.0, 1), batch(new, 0.31, 7)
+    vf, vo = on_gpu(first), on_gpu(other)
+    c = T.Context(0)
+    try:
+        cap = max(sum(x[3] for x in c.sort_views(v)) for v in (vf, vo)) + 100
+        c2 = T.Context(0)  # sized by the reservation alone
+        try:
+            c2.reserve_views(vf, cap)
+            c2.sort_views_async(vf)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                c2.sort_views_async(vf)
+            check(first, c2.views_results(len(vf)))
+            c2.sort_views_async(vo)
+            check(other, c2.views_results(len(vo)))
+            graph.replay()  # (reads the table of `other`)
+            try:
+                check(other, c2.views_results(len(vo)))
+            except T.TdgsError as e:
+                assert e.status == T.CAPACITY and new != shapes
+            c2.sort_views_async(vf)
+            check(first, c2.views_results(len(vf)))
+        finally:
+            c2.close()
+    finally:
+        c.close()
