@@ -801,8 +801,8 @@ ViewTable device_table(tdgs_context* ctx) {
 // tile passes.  A rectangle's bounds are a byte each, hence 256 rows and
 // columns; inside that range the splits are the faster form at every size
 // measured (us a frame, tile passes and splits: 10,000 Gaussians 78 and 46,
-// 1M 239 and 145, 3M 867 and 390, 4096x2304 244 and 137, 64 views 1410 and
-// 832).
+// 1M 239 and 145, 3M 867 and 390, 778,000 at an odd 4K size 244 and 137,
+// 16 views of 500,000 1410 and 832).
 bool splits(const tdgs_context* ctx) {
   return (ctx->nv == 1 || ctx->n_all < (1u << 30)) && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
          ctx->tuning.tile_digit_bits == 0;
