@@ -8,13 +8,13 @@ namespace tdgs {
 // ------------------------------------------------------------ tile count
 // One Gaussian per thread; one 128-bit load per record (Table IV packs the
 // mean, depth and radius into one 16-byte record for exactly this read).
-__global__ void __launch_bounds__(256) k_count_tiles(const float4* __restrict__ g, uint32_t n,
+__global__ void __launch_bounds__(256) k_count_tiles(const float4* g, uint32_t n,
                                                      FrameGeom fg, uint32_t* __restrict__ counts,
                                                      uint32_t* err) {
   begin_launch();
   bool bad = false;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const TileRect q = tile_rect(__ldg(g + i), fg);
+    const TileRect q = tile_rect(__ldca(g + i), fg);
     bad |= q.invalid;
     counts[i] = q.count;
   }
@@ -59,8 +59,8 @@ __device__ __forceinline__ uint64_t warp_incl_scan64(uint64_t v) {
 // kMode 0: counts[i]; 1: counts computed from recs[i]; 2: counts[gather[i]].
 template <int kMode>
 __global__ void __launch_bounds__(kScanThreads)
-    k_scan(const uint32_t* __restrict__ counts, const float4* __restrict__ recs,
-           const uint32_t* __restrict__ gather, FrameGeom fg, uint32_t n,
+    k_scan(const uint32_t* counts, const float4* recs,
+           const uint32_t* gather, FrameGeom fg, uint32_t n,
            uint32_t* __restrict__ offsets, uint64_t* status, uint32_t* ticket,
            uint32_t ticket_base, uint64_t* total64, uint32_t* total32, uint32_t* err) {
   constexpr bool kFromRecords = kMode == 1;
@@ -87,13 +87,13 @@ __global__ void __launch_bounds__(kScanThreads)
     uint32_t v = 0;
     if (idx < n) {
       if constexpr (kMode == 1) {
-        const TileRect q = tile_rect(__ldg(recs + idx), fg);
+        const TileRect q = tile_rect(__ldca(recs + idx), fg);
         bad |= q.invalid;
         v = q.count;
       } else if constexpr (kMode == 2) {
-        v = __ldg(counts + __ldg(gather + idx));
+        v = __ldca(counts + __ldca(gather + idx));
       } else {
-        v = __ldg(counts + idx);
+        v = __ldca(counts + idx);
       }
     }
     s_items[spad(p)] = v;
@@ -207,9 +207,9 @@ struct DupOwner {
 };
 template <bool kNorm>
 __global__ void __launch_bounds__(256)
-    k_duplicate(const float4* __restrict__ g, const uint32_t* __restrict__ offsets, uint32_t n,
+    k_duplicate(const float4* g, const uint32_t* offsets, uint32_t n,
                 FrameGeom fg, void* __restrict__ keys_raw, uint32_t* __restrict__ values,
-                uint32_t cap, const uint32_t* __restrict__ norm, uint32_t* err) {
+                uint32_t cap, const uint32_t* norm, uint32_t* err) {
   __shared__ __align__(16) DupOwner s_owner[8][32];
   __shared__ uint2 s_pay[8][32];  // low key word, index
   begin_launch();
@@ -232,9 +232,9 @@ __global__ void __launch_bounds__(256)
     uint64_t start = 0;
     uint32_t low = 0;
     if (i < n) {
-      const float4 rec = __ldg(g + i);
+      const float4 rec = __ldca(g + i);
       q = tile_rect(rec, fg);
-      start = __ldg(offsets + i);
+      start = __ldca(offsets + i);
       bad |= q.invalid;
       low = kNorm ? norm_depth(rec.z, dmin, scale) : __float_as_uint(rec.z);
     }
@@ -325,12 +325,12 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
 // Smallest and largest depth (float bits; positive finite depths order as
 // unsigned integers) of the Gaussians with pairs: norm[0] min, norm[1] max
 // (all ones / zero on entry).
-__global__ void __launch_bounds__(256) k_norm_range(const float4* __restrict__ g, const uint32_t* __restrict__ counts,
+__global__ void __launch_bounds__(256) k_norm_range(const float4* g, const uint32_t* counts,
                                                     uint32_t n, uint32_t* norm) {
   uint32_t lo = 0xffffffffu, hi = 0u;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (__ldg(counts + i)) {
-      const uint32_t b = __float_as_uint(__ldg(&g[i].z));
+    if (__ldca(counts + i)) {
+      const uint32_t b = __float_as_uint(__ldca(&g[i].z));
       lo = min(lo, b);
       hi = max(hi, b);
     }
@@ -354,7 +354,7 @@ cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t 
 // Four keys per thread.  The normalised depths are 0 .. 1023 whatever the
 // frame, so their range is constant.
 __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, uint32_t n,
-                                                   const uint32_t* __restrict__ range, uint32_t* __restrict__ out,
+                                                   const uint32_t* range, uint32_t* __restrict__ out,
                                                    uint32_t* __restrict__ raw) {
   __shared__ uint32_t s_raw[kRawBins + 1];
   begin_launch();
@@ -399,13 +399,13 @@ cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, 
 // normalised keys with the tile above bit 10.
 constexpr int kRangeItems = 4;
 template <typename K, int kShift>
-__global__ void __launch_bounds__(256) k_tile_ranges(const K* __restrict__ keys, uint32_t m,
+__global__ void __launch_bounds__(256) k_tile_ranges(const K* keys, uint32_t m,
                                                      uint32_t num_tiles, uint2* ranges,
                                                      uint32_t* err) {
   begin_launch();
-  const uint32_t* __restrict__ words = reinterpret_cast<const uint32_t*>(keys);
+  const uint32_t* words = reinterpret_cast<const uint32_t*>(keys);
   constexpr uint32_t kStep = sizeof(K) / 4, kHigh = sizeof(K) == 8 ? 1 : 0;
-  auto tile_of = [&](uint64_t k) { return __ldg(words + k * kStep + kHigh) >> (kShift & 31); };
+  auto tile_of = [&](uint64_t k) { return __ldca(words + k * kStep + kHigh) >> (kShift & 31); };
   const uint32_t lane = lane_id();
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x * kRangeItems;
   bool bad = false;

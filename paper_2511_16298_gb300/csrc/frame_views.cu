@@ -128,16 +128,16 @@ __global__ void __launch_bounds__(256, kProject ? 4 : 6)
         if constexpr (kProject) {
           float4 co;
           if (vt.nv == 1) {
-            proj::project(__ldg(pj.g + i), __ldg(pj.cov + 2 * static_cast<size_t>(i)),
-                          __ldg(pj.cov + 2 * static_cast<size_t>(i) + 1), pj.cam0, lim0, rec[u], co);
+            proj::project(__ldca(pj.g + i), __ldca(pj.cov + 2 * static_cast<size_t>(i)),
+                          __ldca(pj.cov + 2 * static_cast<size_t>(i) + 1), pj.cam0, lim0, rec[u], co);
           } else {
-            proj::project(__ldg(pj.g + l), __ldg(pj.cov + 2 * static_cast<size_t>(l)),
-                          __ldg(pj.cov + 2 * static_cast<size_t>(l) + 1), s_cam[vv[u]], s_lim[vv[u]], rec[u], co);
+            proj::project(__ldca(pj.g + l), __ldca(pj.cov + 2 * static_cast<size_t>(l)),
+                          __ldca(pj.cov + 2 * static_cast<size_t>(l) + 1), s_cam[vv[u]], s_lim[vv[u]], rec[u], co);
           }
           pj.rec[i] = rec[u];
           pj.conic[i] = co;
         } else {
-          rec[u] = __ldg(s_g[vv[u]] + l);
+          rec[u] = __ldca(s_g[vv[u]] + l);
         }
       }
     }
@@ -267,8 +267,8 @@ __device__ __forceinline__ void store_quad(K* dst, const K (&e)[4], uint32_t val
 
 template <typename K>
 __global__ void __launch_bounds__(256)
-    k_views_dup(ViewTable vt, const uint32_t* __restrict__ sorder,
-                const uint32_t* __restrict__ soff, uint32_t n_all, uint32_t rbits,
+    k_views_dup(ViewTable vt, const uint32_t* sorder,
+                const uint32_t* soff, uint32_t n_all, uint32_t rbits,
                 K* __restrict__ out, uint32_t cap, uint2* __restrict__ sdo, uint32_t* err) {
   __shared__ uint32_t s_begin[kMaxViews + 1];
   __shared__ const float4* s_g[kMaxViews];
@@ -300,13 +300,13 @@ __global__ void __launch_bounds__(256)
     q.count = 0;
     uint64_t start = 0;
     uint32_t first = 0, gx = 1;
-    const uint32_t gi = j < n_all ? __ldg(sorder + j) : 0xffffffffu;
+    const uint32_t gi = j < n_all ? __ldca(sorder + j) : 0xffffffffu;
     if (gi < n_all) {  // a depth order that is not a permutation is never followed out of bounds
       const uint32_t v = vt.nv == 1 ? 0u : find_view(s_begin, vt.nv, gi);
       const FrameGeom fg = s_geom[v];
-      const float4 rec = __ldg(s_g[v] + (gi - s_begin[v]));
+      const float4 rec = __ldca(s_g[v] + (gi - s_begin[v]));
       q = tile_rect(rec, fg);
-      start = __ldg(soff + j);
+      start = __ldca(soff + j);
       gx = static_cast<uint32_t>(fg.gx);
       first = s_tb[v] + static_cast<uint32_t>(q.y0) * gx + static_cast<uint32_t>(q.x0);
       // the depth key of the count kernel, beside the record index

@@ -55,11 +55,11 @@ static_assert(kTile <= kStage, "one bin of a tile fits the stage");
 
 // Largest i < n with begin[i] <= x (begin ascending, begin[0] <= x), by the
 // whole warp: 32 probes at a time.
-__device__ __forceinline__ uint32_t warp_find(const uint32_t* __restrict__ begin, uint32_t n, uint32_t x) {
+__device__ __forceinline__ uint32_t warp_find(const uint32_t* begin, uint32_t n, uint32_t x) {
   uint32_t lo = 0, len = n;
   while (len > 1) {
     const uint32_t step = (len + 31) / 32, at = lane_id() * step;
-    const bool le = at < len && __ldg(begin + lo + at) <= x;
+    const bool le = at < len && __ldca(begin + lo + at) <= x;
     const uint32_t k = 31u - __clz(__ballot_sync(0xffffffffu, le) | 1u);
     lo += k * step;
     len = min(step, len - k * step);
@@ -117,8 +117,8 @@ struct Place {
 };
 __device__ __forceinline__ Place place_of(const SplitArgs& a, uint32_t v) {
   if (a.vt.one.on) return Place{0u, a.ntiles1, 0u, 0u};
-  const uint32_t t0 = __ldg(a.t1_begin + v);
-  return Place{t0, __ldg(a.t1_begin + v + 1) - t0, __ldg(a.row_begin + v), __ldg(a.c1_begin + v)};
+  const uint32_t t0 = __ldca(a.t1_begin + v);
+  return Place{t0, __ldca(a.t1_begin + v + 1) - t0, __ldca(a.row_begin + v), __ldca(a.c1_begin + v)};
 }
 
 // A captured batch reads its view table when it is replayed: views may have
@@ -126,10 +126,10 @@ __device__ __forceinline__ Place place_of(const SplitArgs& a, uint32_t v) {
 // of tiles and rows come from the table, and a view that the launches or
 // buffers have no room for is left out (k_row_scan reports it).
 __device__ __forceinline__ uint32_t tiles1_of(const SplitArgs& a) {
-  return a.vt.one.on ? a.ntiles1 : __ldg(a.t1_begin + a.vt.nv);
+  return a.vt.one.on ? a.ntiles1 : __ldca(a.t1_begin + a.vt.nv);
 }
 __device__ __forceinline__ uint32_t rows_of(const SplitArgs& a) {
-  return a.vt.one.on ? a.nrows : min(a.nrows, __ldg(a.row_begin + a.vt.nv));
+  return a.vt.one.on ? a.nrows : min(a.nrows, __ldca(a.row_begin + a.vt.nv));
 }
 __device__ __forceinline__ bool has_room(const SplitArgs& a, const Place& pl, const FrameGeom& fg) {
   return static_cast<uint32_t>(fg.gx) <= a.pitch && static_cast<uint32_t>(fg.gy) <= a.max_gy &&
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
   if (!has_room(a, pl, vw.geom)) return;
   const uint32_t tl = blockIdx.x - pl.tile0, nt = pl.tiles, rec0 = vw.rec0, nrec = vw.nrec;
   const FrameGeom fg = vw.geom;
-  const float4* __restrict__ g = vw.g;
+  const float4* g = vw.g;
   for (uint32_t b = t; b <= kMaxBins; b += kCountThreads) s_d[b][0] = s_d[b][1] = 0;
   __syncthreads();
   constexpr int kPer = kTile / kCountThreads;
@@ -173,11 +173,11 @@ __global__ void __launch_bounds__(kCountThreads) k_row_count(SplitArgs a) {
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
     const uint32_t p = first + u * kCountThreads + t;
-    gi[u] = p < nrec ? __ldg(a.sorder + rec0 + p) - rec0 : 0xffffffffu;
+    gi[u] = p < nrec ? __ldca(a.sorder + rec0 + p) - rec0 : 0xffffffffu;
   }
 #pragma unroll
   for (int u = 0; u < kPer; ++u)  // an order that is not a permutation is never followed out of bounds
-    rec[u] = gi[u] < nrec ? __ldg(g + gi[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    rec[u] = gi[u] < nrec ? __ldca(g + gi[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
     const uint32_t p = first + u * kCountThreads + t;
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kCountThreads) k_row_scan(SplitArgs a) {
   bool room = true;
   for (uint32_t i = t; i < a.vt.nv; i += kCountThreads) room &= has_room(a, place_of(a, i), view_of(a.vt, i).geom);
   const uint32_t nrows = gridDim.x;  // (rows beyond the table's have no segments)
-  room = __syncthreads_and(room) && (a.vt.one.on || __ldg(a.row_begin + a.vt.nv) <= a.nrows);
+  room = __syncthreads_and(room) && (a.vt.one.on || __ldca(a.row_begin + a.vt.nv) <= a.nrows);
   uint32_t seg0 = 0, tile0 = 0;
   unsigned long long pair0 = 0;
   for (uint32_t i0 = 0; i0 < nrows; i0 += kCountThreads) {
@@ -312,17 +312,17 @@ __global__ void __launch_bounds__(kCountThreads) k_col_count(SplitArgs a) {
   __shared__ uint32_t s_w[kCountThreads / 32];
   begin_launch();
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
-  const uint32_t ntiles = __ldg(a.info);
+  const uint32_t ntiles = __ldca(a.info);
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint32_t r = warp_find(a.row_tile, a.nrows, tile);
-    const uint32_t beg = __ldg(a.row_seg + r) + (tile - __ldg(a.row_tile + r)) * kTile;
-    const uint32_t end = min(beg + kTile, __ldg(a.row_seg + r + 1));
+    const uint32_t beg = __ldca(a.row_seg + r) + (tile - __ldca(a.row_tile + r)) * kTile;
+    const uint32_t end = min(beg + kTile, __ldca(a.row_seg + r + 1));
     constexpr int kPer = kTile / kCountThreads;
     uint32_t x[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const uint32_t p = beg + u * kCountThreads + t;
-      x[u] = p < end ? __ldg(a.cols + p) : 0xffffffffu;
+      x[u] = p < end ? __ldca(a.cols + p) : 0xffffffffu;
     }
     for (uint32_t b = t; b <= kMaxBins; b += kCountThreads) s_d[b] = 0;
     __syncthreads();
@@ -360,21 +360,21 @@ __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
   __shared__ uint32_t s_sum[kScanThreads];
   __shared__ uint32_t s_w[kScanThreads / 32];
   begin_launch();
-  if (__ldg(a.info + 1) == 0u) return;  // more pairs than the buffers hold
+  if (__ldca(a.info + 1) == 0u) return;  // more pairs than the buffers hold
   const uint32_t t = threadIdx.x, r = blockIdx.x;
   if (r >= rows_of(a)) return;
   const uint32_t v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
   const uint32_t gx = static_cast<uint32_t>(view_of(a.vt, v).geom.gx), y = r - place_of(a, v).row0;
   const uint32_t lp = gx <= 32 ? 5u : 32u - static_cast<uint32_t>(__clz(gx - 1));  // columns padded to 2^lp
   const uint32_t c = t & ((1u << lp) - 1u), g = t >> lp, groups = kScanThreads >> lp;
-  const uint32_t tile0 = __ldg(a.row_tile + r), nt = __ldg(a.row_tile + r + 1) - tile0;
+  const uint32_t tile0 = __ldca(a.row_tile + r), nt = __ldca(a.row_tile + r + 1) - tile0;
   const uint32_t per = (nt + groups - 1) / groups;
   const uint32_t lo = min(g * per, nt), hi = min(lo + per, nt);
-  const uint16_t* __restrict__ cnt = a.c2 + static_cast<size_t>(tile0) * a.pitch + c;
+  const uint16_t* cnt = a.c2 + static_cast<size_t>(tile0) * a.pitch + c;
   uint32_t sum = 0;
   if (c < gx) {
 #pragma unroll 8
-    for (uint32_t i = lo; i < hi; ++i) sum += __ldg(cnt + static_cast<size_t>(i) * a.pitch);
+    for (uint32_t i = lo; i < hi; ++i) sum += __ldca(cnt + static_cast<size_t>(i) * a.pitch);
   }
   s_sum[t] = sum;
   __syncthreads();
@@ -394,11 +394,11 @@ __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
     if (w < cw && t < (1u << lp)) incl += s_w[w];
   __syncthreads();
   if (t < (1u << lp)) {
-    const uint32_t start = __ldg(a.row_pair + r) + incl - total;
+    const uint32_t start = __ldca(a.row_pair + r) + incl - total;
     s_sum[t] = start;
     if (c < gx) {
       const uint32_t pb = a.vt.pbeg[v];
-      a.ranges[(a.vt.one.on ? 0u : __ldg(a.vt.tile_begin + v)) + y * gx + c] =
+      a.ranges[(a.vt.one.on ? 0u : __ldca(a.vt.tile_begin + v)) + y * gx + c] =
           total ? make_uint2(start - pb, start + total - pb) : make_uint2(0u, 0u);
     }
   }
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kScanThreads) k_col_scan(SplitArgs a) {
 #pragma unroll 8
     for (uint32_t i = lo; i < hi; ++i) {
       out[static_cast<size_t>(i) * a.pitch] = run;
-      run += __ldg(cnt + static_cast<size_t>(i) * a.pitch);
+      run += __ldca(cnt + static_cast<size_t>(i) * a.pitch);
     }
   }
 }
@@ -605,8 +605,8 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
   S& s = *reinterpret_cast<S*>(smem);
   begin_launch();
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
-  if (__ldg(a.info + 1) == 0u) return;
-  const uint32_t ntiles = kLevel == 1 ? tiles1_of(a) : __ldg(a.info);
+  if (__ldca(a.info + 1) == 0u) return;
+  const uint32_t ntiles = kLevel == 1 ? tiles1_of(a) : __ldca(a.info);
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     uint32_t v, beg, cnt, bins, r = 0, tl = 0;
     Place pl;
@@ -622,8 +622,8 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
       r = warp_find(a.row_tile, a.nrows, tile);
       v = a.vt.nv == 1 ? 0u : warp_find(a.row_begin, a.vt.nv, r);
       pl = place_of(a, v);
-      beg = __ldg(a.row_seg + r) + (tile - __ldg(a.row_tile + r)) * kTile;
-      cnt = min(kTile, __ldg(a.row_seg + r + 1) - beg);
+      beg = __ldca(a.row_seg + r) + (tile - __ldca(a.row_tile + r)) * kTile;
+      cnt = min(kTile, __ldca(a.row_seg + r + 1) - beg);
       bins = static_cast<uint32_t>(view_of(a.vt, v).geom.gx);
     }
     // ---- load
@@ -634,17 +634,17 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
       lo[b] = hi[b] = 0u;
       if (i < cnt) {
         if constexpr (kLevel == 1) {
-          const uint32_t q = __ldg(a.rects + beg + i);
+          const uint32_t q = __ldca(a.rects + beg + i);
           lo[b] = (q >> 16) & 0xffu;
           hi[b] = (q >> 24) + 1u;
           if (hi[b] <= lo[b]) lo[b] = hi[b] = 0u;
-          s.pay[i] = __ldg(a.sdo + beg + i);
+          s.pay[i] = __ldca(a.sdo + beg + i);
           s.cols[i] = static_cast<uint16_t>(q);
         } else {
-          const uint32_t q = __ldg(a.cols + beg + i);
+          const uint32_t q = __ldca(a.cols + beg + i);
           lo[b] = q & 0xffu;
           hi[b] = (q >> 8) + 1u;
-          s.pay[i] = __ldg(a.segs + beg + i);
+          s.pay[i] = __ldca(a.segs + beg + i);
         }
       }
     }
@@ -657,12 +657,12 @@ __global__ void __launch_bounds__(kThreads, kWords > 5 ? 2 : 3) k_split(SplitArg
         c[i] = base[i] = 0u;
         if (b < bins) {
           if constexpr (kLevel == 1) {
-            const uint2 x = __ldg(a.c1 + pl.c10 + static_cast<size_t>(b) * pl.tiles + tl);
+            const uint2 x = __ldca(a.c1 + pl.c10 + static_cast<size_t>(b) * pl.tiles + tl);
             c[i] = x.x;
-            base[i] = x.y + __ldg(a.row_seg + pl.row0 + b);
+            base[i] = x.y + __ldca(a.row_seg + pl.row0 + b);
           } else {
-            c[i] = __ldg(a.c2 + static_cast<size_t>(tile) * a.pitch + b);
-            base[i] = __ldg(a.b2 + static_cast<size_t>(tile) * a.pitch + b);
+            c[i] = __ldca(a.c2 + static_cast<size_t>(tile) * a.pitch + b);
+            base[i] = __ldca(a.b2 + static_cast<size_t>(tile) * a.pitch + b);
           }
         }
         sum += c[i];
@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_small(SplitArgs a) {
   const FrameGeom fg = a.vt.one.geom;
   const uint32_t n = a.vt.one.n, nt = a.ntiles1;
   const uint32_t gx = static_cast<uint32_t>(fg.gx), gy = static_cast<uint32_t>(fg.gy);
-  const float4* __restrict__ g = a.vt.one.g;
+  const float4* g = a.vt.one.g;
   constexpr int kPer = kTile / kThreads;
   // ---- rectangles in depth order and the rows' counts
   float dmin = 0.0f, scale = 0.0f;
@@ -752,8 +752,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_small(SplitArgs a) {
     for (int u = 0; u < kPer; ++u) {
       const uint32_t p = tile * kTile + u * kThreads + t;
       if (p >= n) continue;
-      const uint32_t gi = __ldg(a.sorder + p);
-      const float4 rec = gi < n ? __ldg(g + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const uint32_t gi = __ldca(a.sorder + p);
+      const float4 rec = gi < n ? __ldca(g + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
       const TileRect q = tile_rect(rec, fg);
       uint32_t pack = kEmptyRect;
       if (q.count) {

@@ -173,7 +173,7 @@ struct PassArgs {
 // into L2 while it counts.  Few blocks (4 per SM) keep the final global
 // atomics on the counters few.
 constexpr int kHistThreads = 512;
-__global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const uint64_t* __restrict__ keys, HistArgs a) {
+__global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const uint64_t* keys, HistArgs a) {
   __shared__ uint32_t h[kBins];
   __shared__ uint32_t s_warp[kHistThreads / 32];
   __shared__ bool s_last;
@@ -320,7 +320,7 @@ __device__ __forceinline__ void rank_in_warps(const TileBuf<KeyOf<kMode>>& tb, u
 // the next pass's digits; the counts reach hist_next when it finishes.
 template <int kMode, int kModeN>
 __global__ void __launch_bounds__(kThreads, 2)
-    k_onesweep_pass(const KeyOf<kMode>* __restrict__ kin, const uint32_t* __restrict__ vin,
+    k_onesweep_pass(const KeyOf<kMode>* kin, const uint32_t* vin,
                     KeyOf<kMode>* __restrict__ kout, uint32_t* __restrict__ vout, PassArgs a) {
   using K = KeyOf<kMode>;
   constexpr bool kSwz = kMode == kDigitSpan;  // per-digit tables in swizzled slots
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       in = a.pass == 0 ? 0u : (((dd.passes - a.pass) & 1u) ? 2u : 1u);
     }
     if (to_view)
-      for (uint32_t v = threadIdx.x; v <= a.nv; v += kThreads) s_begin[v] = __ldg(a.rec_begin + v);
+      for (uint32_t v = threadIdx.x; v <= a.nv; v += kThreads) s_begin[v] = __ldca(a.rec_begin + v);
     kin = a.dk[in];
     vin = a.dv[in];
     kout = a.dk[out];
@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     g0 = cta_excl_scan(h0 + h1, s_warp);
     g1 = g0 + h0;
   } else if (a.gstart) {
-    g0 = __ldg(a.gstart + 2 * t);
-    g1 = __ldg(a.gstart + 2 * t + 1);
+    g0 = __ldca(a.gstart + 2 * t);
+    g1 = __ldca(a.gstart + 2 * t + 1);
   } else {
     const uint32_t h0 = __ldcg(a.hist + 2 * t), h1 = __ldcg(a.hist + 2 * t + 1);
     g0 = cta_excl_scan(h0 + h1, s_warp);

@@ -196,7 +196,7 @@ __device__ __forceinline__ void scan_tiles(uint32_t* __restrict__ status, uint32
 // Exclusive prefix of digits 2t and 2t+1 for tile `tile` > 0: the inclusive
 // prefix the scan CTAs wrote for tile - 1 (bounded wait).
 template <uint32_t kBins>
-__device__ __forceinline__ void wait_prefix(const uint32_t* __restrict__ status, uint32_t tile, uint32_t t,
+__device__ __forceinline__ void wait_prefix(const uint32_t* status, uint32_t tile, uint32_t t,
                                             uint32_t& e0, uint32_t& e1, uint32_t* err) {
   const uint32_t* row = status + static_cast<size_t>(tile - 1) * kBins + 2 * t;
   uint2 w = ld_relaxed_v2(row);

@@ -11,14 +11,14 @@ namespace tdgs {
 namespace {
 
 __global__ void __launch_bounds__(256)
-    k_preprocess(const float4* __restrict__ g, const float4* __restrict__ cov, uint32_t n, CameraDev cam,
+    k_preprocess(const float4* g, const float4* cov, uint32_t n, CameraDev cam,
                  float4* __restrict__ rec, float4* __restrict__ conic) {
   begin_launch();
   const float2 lim = proj::slope_limits(cam);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float4 p = __ldg(g + i);
-    const float4 c0 = __ldg(cov + 2 * static_cast<size_t>(i));
-    const float4 c1 = __ldg(cov + 2 * static_cast<size_t>(i) + 1);
+    const float4 p = __ldca(g + i);
+    const float4 c0 = __ldca(cov + 2 * static_cast<size_t>(i));
+    const float4 c1 = __ldca(cov + 2 * static_cast<size_t>(i) + 1);
     float4 out, co;
     proj::project(p, c0, c1, cam, lim, out, co);
     rec[i] = out;

@@ -133,7 +133,7 @@ __device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, floa
 // is empty).  Positions come from the exclusive bucket scan, so they are a
 // permutation of 0 .. tiles-1.
 __global__ void __launch_bounds__(kOrderThreads)
-    k_render_order(const uint2* __restrict__ ranges, uint32_t tiles, uint32_t* __restrict__ order) {
+    k_render_order(const uint2* ranges, uint32_t tiles, uint32_t* __restrict__ order) {
   begin_launch();
   __shared__ uint32_t s_max[kOrderThreads / 32];
   __shared__ uint32_t s_cnt[kOrderBuckets];
@@ -189,9 +189,9 @@ __global__ void __launch_bounds__(kOrderThreads)
 
 
 __global__ void __launch_bounds__(kRenderThreads, 6)
-    k_render(const float4* __restrict__ rec, const float4* __restrict__ conic, const float* __restrict__ rgb,
-             const uint32_t* __restrict__ values, const uint2* __restrict__ ranges,
-             const uint32_t* __restrict__ order, uint32_t gx, uint32_t width,
+    k_render(const float4* rec, const float4* conic, const float* rgb,
+             const uint32_t* values, const uint2* ranges,
+             const uint32_t* order, uint32_t gx, uint32_t width,
              uint32_t height, float3 bg, uint32_t n, float* __restrict__ image, uint32_t* err) {
   // staged Gaussians, two 16-byte loads per step: (x, y, cut, -c/2) and
   // (-a/2, -b, opacity, -); cut = the exponent below which alpha < 1/255; a
@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(kRenderThreads, 6)
         s_mask[t] = 0;
         s_rgb[t] = make_float4(0.f, 0.f, 0.f, 0.f);
       } else {
-        const float4 q = __ldg(rec + g);
-        const float4 c = __ldg(conic + g);
+        const float4 q = __ldca(rec + g);
+        const float4 c = __ldca(conic + g);
         // opacity * exp(power) < 1/255 exactly when power < -ln(255 opacity):
         // far pixels skip the exponential (the 1/255 test below stays)
         const float cut = c.w > 0.0f ? -__logf(255.0f * c.w) : __int_as_float(0x7f800000);
@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(kRenderThreads, 6)
         s_g1[t] = make_float4(-0.5f * c.x, -c.y, c.w, 0.f);
         s_mask[t] = static_cast<uint8_t>(warp_mask(q.x, q.y, c, cut, __uint2float_rn(tx), __uint2float_rn(ty),
                                                  ellipse));
-        s_rgb[t] = make_float4(__ldg(rgb + 3 * static_cast<size_t>(g)), __ldg(rgb + 3 * static_cast<size_t>(g) + 1),
-                               __ldg(rgb + 3 * static_cast<size_t>(g) + 2), 0.f);
+        s_rgb[t] = make_float4(__ldca(rgb + 3 * static_cast<size_t>(g)), __ldca(rgb + 3 * static_cast<size_t>(g) + 1),
+                               __ldca(rgb + 3 * static_cast<size_t>(g) + 2), 0.f);
       }
     }
     __syncthreads();

@@ -130,6 +130,11 @@ __device__ __forceinline__ void st_release(uint64_t* p, uint64_t v) {
 // (griddepcontrol.launch_dependents): blocks that wait on SMs where others
 // still run measured slower (1M frame 146 -> 153 us, 3M 403 -> 454, sorting
 // 10.5M pairs 486 -> 505; plain launches 165, - and 513).
+// Such a kernel reads memory by plain loads, __ldca, __ldcg or __ldcs, which
+// stay below the wait (it clobbers memory, and volatile assembly keeps its
+// order), never by __ldg or through a const __restrict__ pointer: the
+// read-only path holds only for data that no one writes while the kernel is
+// resident, and its loads may be moved above the wait.
 __device__ __forceinline__ void begin_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
