@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kHistThreads) k_onesweep_hist(const uint64_t* 
   bool bad = false;
   for (uint64_t base = static_cast<uint64_t>(blockIdx.x) * kStep; base < m; base += stride) {
     if (t == 0 && base + stride < m)  // the next step's keys into L2 while this step counts
-      radix::prefetch_l2(keys + base + stride, (min(static_cast<uint64_t>(kStep), m - (base + stride))) * 8);
+      radix::prefetch_l2(keys + base + stride, static_cast<uint32_t>(min(static_cast<uint64_t>(kStep), m - (base + stride))));
     const uint64_t i0 = base + 8 * t;
     uint64_t k[8];
     if (vec && i0 + 8 <= m) {
@@ -475,8 +475,8 @@ __global__ void __launch_bounds__(kThreads, 2)
       rank_in_warps<kMode, kModeN>(tb, valid, dg, my_wh, r, dgn, hn);
       if (t == 0 && nxt < ntiles) {
         const uint32_t nf = nxt * kTileKeys, nv = min(kTileKeys, m - nf);
-        radix::prefetch_l2(kin + nf, static_cast<uint64_t>(nv) * 8);
-        if (!iota) radix::prefetch_l2(vin + nf, static_cast<uint64_t>(nv) * 4);
+        radix::prefetch_l2(kin + nf, nv);
+        if (!iota) radix::prefetch_l2(vin + nf, nv);
       }
       __syncthreads();
       // ---- per-digit counts (column t holds digits 2t and 2t+1), prefixes over warps

@@ -57,11 +57,12 @@ __device__ __forceinline__ void st_release32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Hint: bring [p, p + bytes) into L2 with one bulk prefetch (the 16-byte
-// aligned part of it; nothing is read into registers or shared memory).
-__device__ __forceinline__ void prefetch_l2(const void* p, uint64_t bytes) {
+// Hint: bring the n elements at p into L2 with one bulk prefetch (the 16-byte
+// aligned part of them; nothing is read into registers or shared memory).
+template <typename T>
+__device__ __forceinline__ void prefetch_l2(const T* p, uint32_t n) {
   const uint64_t a = reinterpret_cast<uint64_t>(p);
-  const uint64_t lo = (a + 15) & ~15ull, hi = (a + bytes) & ~15ull;
+  const uint64_t lo = (a + 15) & ~15ull, hi = (a + static_cast<uint64_t>(n) * sizeof(T)) & ~15ull;
   if (hi > lo)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"(static_cast<uint32_t>(hi - lo))
                  : "memory");
@@ -854,10 +855,10 @@ __global__ void __launch_bounds__(kThreads, (PassShape<K, kVals, kExpand, kBits,
   }
   // (chunk_bases starts and ends with a block barrier)
   if constexpr (kVals)  // the first tile's values, while the histogram is built
-    if (t == 0 && end > beg) prefetch_l2(vin + beg, static_cast<uint64_t>(min(kTileKeys, end - beg)) * 4);
+    if (t == 0 && end > beg) prefetch_l2(vin + beg, min(kTileKeys, end - beg));
   chunk_bases<K, S::kBins, kThreads>(kin, a, beg, end, d31, sm.base, sm.lstart, s_warp, s_vtile);
   if (t == 0 && end > beg)  // the first tile's keys again: phase 1 read the whole chunk since
-    prefetch_l2(kin + beg, static_cast<uint64_t>(min(kTileKeys, end - beg)) * sizeof(K));
+    prefetch_l2(kin + beg, min(kTileKeys, end - beg));
 
   // ---- phase 3: stable rank + scatter, tile by tile; while a tile is
   // processed, the next one's keys and values are prefetched into L2
@@ -868,8 +869,8 @@ __global__ void __launch_bounds__(kThreads, (PassShape<K, kVals, kExpand, kBits,
     const uint32_t tb = beg + i * kTileKeys;
     if (t == 0 && tb + kTileKeys < end) {
       const uint32_t cnt = min(kTileKeys, end - (tb + kTileKeys));
-      prefetch_l2(kin + tb + kTileKeys, static_cast<uint64_t>(cnt) * sizeof(K));
-      if constexpr (kVals) prefetch_l2(vin + tb + kTileKeys, static_cast<uint64_t>(cnt) * 4);
+      prefetch_l2(kin + tb + kTileKeys, cnt);
+      if constexpr (kVals) prefetch_l2(vin + tb + kTileKeys, cnt);
     }
     ok &= rank_and_scatter<true, S, K, kVals, kExpand, kBits, kItems>(
         kin + tb, kVals ? vin + tb : nullptr, kTileKeys, m, a, d31, sm, s_warp, s_vrec, s_vtile, kout_raw, vout);
