@@ -259,7 +259,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
       if (!kOffsets && first) {
         v[j] = tb + idx;
       } else {
-        const uint32_t x = idx < nstaged ? vstage[idx] : __ldg(vsrc + tb + idx);
+        const uint32_t x = idx < nstaged ? vstage[idx] : __ldcg(vsrc + tb + idx);
         v[j] = first ? (tb + idx) | (min(x, kCntEscape) << kValueBits) : x;
       }
     }
@@ -326,7 +326,7 @@ __device__ __forceinline__ bool exchange_scatter(const radix::Smem<uint32_t>& sm
         const uint32_t dst = sm.off[static_cast<uint32_t>(x >> 32)] + xp;
         if (dst < n && rec < n) {
           uint32_t c1 = w >> kValueBits;
-          if (c1 == kCntEscape) c1 = __ldg(counts + rec);
+          if (c1 == kCntEscape) c1 = __ldcg(counts + rec);
           cnt[i] = c1;
           v1[dst] = rec;
           k1[dst] = c1;
@@ -707,7 +707,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_depth_sort(DepthSortArgs A) {
     const bool unstaged = !kOffsets || counted;  // no values to copy in
     const uint32_t nstaged = unstaged ? valid : nbulk;
     if (kOffsets && t == 0) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      // the staging buffer was read, and the values were written by other
+      // CTAs of this launch, through ordinary accesses: both before the copy
+      asm volatile("fence.proxy.async;" ::: "memory");
       osw::mbar_arrive(&s_mbar, unstaged ? 0u : nbulk * 4);
       if (!unstaged && nbulk) osw::bulk_g2s(vstage, vsrc + beg, nbulk * 4, &s_mbar);
     }

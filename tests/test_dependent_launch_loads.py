@@ -29,3 +29,14 @@ def test_every_dependent_launch_waits():
         waits = {re.search(r"\b(k_\w+)\s*\(", k).group(1): "begin_launch();" in k for k in kernels}
         for name in re.findall(r"launch_after\((?:\w+::)?(k_\w+)", code):
             assert waits[name], name
+
+
+def test_depth_sort_reads_its_own_launch_coherently():
+    """The single-launch depth sort writes counts and values that other blocks
+    of the launch read: only the records, which it never writes, may take the
+    read-only path, and the bulk copy of the values follows a proxy fence over
+    global memory too."""
+    code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "depth_sort.cu")).read())
+    assert re.findall(r"__ldg\((\w+)", code) == ["s_g"]
+    copy = code.index("bulk_g2s(")
+    assert code.rindex("fence.proxy.async;", 0, copy) > code.rindex("mbar_init(", 0, copy)
