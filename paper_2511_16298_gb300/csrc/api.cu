@@ -115,7 +115,10 @@ struct FrameState {
   uint32_t max_gx = 0, max_gy = 0;  // over the staged views
   bool norm = false;            // the frame with the 32-bit normalised key (by interval splits)
   bool split = false;           // pairs by interval splits (else packed elements and tile passes)
-  uint64_t capacity = 0;        // pair capacity reserved for the asynchronous path
+  // What tdgs_reserve_views sized the buffers for: an asynchronous batch has
+  // the same counts of views, Gaussians and tiles and no more pairs.
+  uint32_t reserved_nv = 0, reserved_n = 0, reserved_t = 0;
+  uint64_t capacity = 0;
   bool split_reserved = false;  // what the reservation chose
   bool exact = false;           // a call that waits for the pair count (not an asynchronous one)
   bool reserved = false;
@@ -726,22 +729,41 @@ uint32_t bits_for(uint64_t count) {  // smallest b with count <= 2^b
   return b;
 }
 
-// Validate the views, fill the pinned staging table and the totals.
-tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) {
+// Validate the views and total their Gaussians and tiles; nothing is staged.
+tdgs_status check_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv, uint32_t* n, uint32_t* t) {
   if (nv == 0 || nv > kMaxViews) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "view count out of range");
   if (!views) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null views");
-  ViewBlob* h = ctx->h_views;
-  uint64_t n_all = 0, t_all = 0, t1 = 0, rows = 0, c1 = 0;
-  ctx->max_gx = ctx->max_gy = 0;
+  uint64_t n_all = 0, t_all = 0;
   for (uint32_t v = 0; v < nv; ++v) {
     const tdgs_view& w = views[v];
     if (w.f.width == 0 || w.f.height == 0) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "empty image");
     if (w.n && !w.g) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null pointer");
     if (!aligned(w.g, 16)) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "misaligned pointer");
+    n_all += w.n;
+    t_all += tdgs_num_tiles(w.f);
+  }
+  if (n_all > 0xffffffffull || t_all > 0xffffffffull)
+    return fail(ctx, TDGS_ERR_OVERFLOW, "too many Gaussians or tiles in one batch");
+  *n = static_cast<uint32_t>(n_all);
+  *t = static_cast<uint32_t>(t_all);
+  return TDGS_OK;
+}
+
+// Validate the views, fill the pinned staging table and the totals.  Views
+// that are refused leave both as they were.
+tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) {
+  uint32_t n_total = 0, t_total = 0;
+  if (tdgs_status st = check_views(ctx, views, nv, &n_total, &t_total); st != TDGS_OK) return st;
+  ViewBlob* h = ctx->h_views;
+  uint32_t n_all = 0, t_all = 0;
+  uint64_t t1 = 0, rows = 0, c1 = 0;
+  ctx->max_gx = ctx->max_gy = 0;
+  for (uint32_t v = 0; v < nv; ++v) {
+    const tdgs_view& w = views[v];
     h->g[v] = reinterpret_cast<const float4*>(w.g);
     h->geom[v] = make_geom(w.f);
-    h->rec_begin[v] = static_cast<uint32_t>(n_all);
-    h->tile_begin[v] = static_cast<uint32_t>(t_all);
+    h->rec_begin[v] = n_all;
+    h->tile_begin[v] = t_all;
     h->nt[v] = tdgs_num_tiles(w.f);
     h->vtot[v] = 0;
     h->n[v] = w.n;
@@ -758,17 +780,15 @@ tdgs_status stage_views(tdgs_context* ctx, const tdgs_view* views, uint32_t nv) 
     rows += gy;
     c1 += static_cast<uint64_t>(tiles1) * gy;
   }
-  if (n_all > 0xffffffffull || t_all > 0xffffffffull)
-    return fail(ctx, TDGS_ERR_OVERFLOW, "too many Gaussians or tiles in one batch");
   std::memset(h->n + nv, 0, sizeof(h->n) - nv * sizeof(h->n[0]));
-  h->rec_begin[nv] = static_cast<uint32_t>(n_all);
-  h->tile_begin[nv] = static_cast<uint32_t>(t_all);
+  h->rec_begin[nv] = n_total;
+  h->tile_begin[nv] = t_total;
   h->t1_begin[nv] = static_cast<uint32_t>(t1);
   h->row_begin[nv] = static_cast<uint32_t>(rows);
   h->c1_begin[nv] = static_cast<uint32_t>(c1);
   ctx->nv = nv;
-  ctx->n_all = static_cast<uint32_t>(n_all);
-  ctx->t_all = static_cast<uint32_t>(t_all);
+  ctx->n_all = n_total;
+  ctx->t_all = t_total;
   return TDGS_OK;
 }
 
@@ -1545,8 +1565,10 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
   DeviceGuard dg(ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tdgs_status st = stage_views(ctx, views, num_views);
+  if (st != TDGS_OK) return st;
+  ctx->reserved = false;  // an allocation that fails leaves no reservation
   ctx->exact = false;
-  ctx->split_reserved = st == TDGS_OK && splits(ctx);  // the asynchronous calls keep this choice
+  ctx->split_reserved = splits(ctx);  // the asynchronous calls keep this choice
   // the tile passes' buffers too: they take a batch with the same totals whose
   // rows or columns the splits' buffers do not hold (split_fits)
   for (const bool split : {false, true}) {
@@ -1557,6 +1579,9 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
   }
   if (st != TDGS_OK) return st;
   TDGS_CUDA(ctx, cudaStreamSynchronize(s));
+  ctx->reserved_nv = ctx->nv;
+  ctx->reserved_n = ctx->n_all;
+  ctx->reserved_t = ctx->t_all;
   ctx->capacity = pair_capacity;
   ctx->reserved = true;
   return TDGS_OK;
@@ -1568,11 +1593,15 @@ tdgs_status tdgs_sort_views_async(tdgs_context* ctx, const tdgs_view* views, uin
   if (!ctx->reserved) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "call tdgs_reserve_views first");
   DeviceGuard dg(ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const uint32_t n_prev = ctx->n_all, t_prev = ctx->t_all, nv_prev = ctx->nv;
-  tdgs_status st = stage_views(ctx, views, num_views);
+  uint32_t n = 0, t = 0;
+  tdgs_status st = check_views(ctx, views, num_views, &n, &t);
   if (st != TDGS_OK) return st;
-  if (ctx->n_all != n_prev || ctx->t_all != t_prev || ctx->nv != nv_prev)
+  // before anything is staged: a refused batch leaves the context, and the
+  // table that replays read, as they were
+  if (n != ctx->reserved_n || t != ctx->reserved_t || num_views != ctx->reserved_nv)
     return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "views differ in shape from the reservation");
+  st = stage_views(ctx, views, num_views);
+  if (st != TDGS_OK) return st;
   ctx->split = ctx->split_reserved && split_fits(ctx, ctx->capacity);
   ctx->exact = false;
   st = run_front(ctx, s);

@@ -1,0 +1,95 @@
+"""Reservations of asynchronous batches: what a refused batch or a failed
+reservation leaves behind."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2511_16298_gb300 import synth
+from paper_2511_16298_gb300 import tdgs as T
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture
+def ctx():
+    from paper_2511_16298_gb300 import build
+    build.build()
+    c = T.Context(0)
+    yield c
+    c.close()
+
+
+def on_gpu(frames):
+    return [(T.records_to_tensor(f.gaussians, DEV), f.width, f.height) for f in frames]
+
+
+def check(oracle, frames, results):
+    assert len(frames) == len(results)
+    for f, (k, v, r, m) in zip(frames, results):
+        ref = oracle.sort_frame(f.gaussians, f.width, f.height)
+        assert ref["status"] == 0 and m == ref["m"]
+        assert np.array_equal(k.cpu().numpy().view(np.uint64), ref["keys"])
+        assert np.array_equal(v.cpu().numpy().view(np.uint32), ref["values"])
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), ref["ranges"])
+
+
+def refused(ctx, views):
+    with pytest.raises(T.TdgsError) as e:
+        ctx.sort_views_async(views)
+    assert e.value.status == T.INVALID_ARGUMENT
+
+
+def capture(ctx, views):
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.sort_views_async(views)
+    return graph
+
+
+@pytest.mark.parametrize("n,size", [(3000, (640, 360)), (3000, (4800, 64))])
+def test_refused_batches_stay_refused(ctx, oracle, n, size):
+    """Batches of other counts (more Gaussians, more tiles, more views) are
+    refused each time, and the reserved batch and its captured graph then give
+    their own results: through the splits and the tile passes."""
+    small = [synth.frame_random(i, n, *size) for i in range(2)]
+    larger = [[synth.frame_random(5, n + 50_000, *size), small[1]],
+              [small[0], synth.frame_random(6, n, size[0] * 2, size[1])], small + small[:1]]
+    vs = on_gpu(small)
+    cap = sum(oracle.sort_frame(f.gaussians, f.width, f.height)["m"] for f in small)
+    ctx.reserve_views(vs, cap)
+    ctx.sort_views_async(vs)
+    graph = capture(ctx, vs)
+    for frames in larger:
+        vl = on_gpu(frames)
+        refused(ctx, vl)
+        refused(ctx, vl)
+        graph.replay()
+        check(oracle, small, ctx.views_results(2))
+        ctx.sort_views_async(vs)
+        check(oracle, small, ctx.views_results(2))
+
+
+def test_failed_reservation_is_none(ctx, oracle):
+    """A reservation for which there is no memory leaves none, not the one
+    before with its buffers given up; arguments that are refused leave the one
+    before."""
+    frames = [synth.frame_random(1, 5000, 300, 200)]
+    vs = on_gpu(frames)
+    m = oracle.sort_frame(frames[0].gaussians, 300, 200)["m"]
+    ctx.reserve_views(vs, m)
+    with pytest.raises(T.TdgsError):
+        ctx.reserve_views([(vs[0][0], 0, 200)], m)
+    ctx.sort_views_async(vs)
+    check(oracle, frames, ctx.views_results(1))
+    torch.cuda.empty_cache()
+    hold = torch.empty(max(0, torch.cuda.mem_get_info()[0] - (24 << 30)), dtype=torch.uint8, device=DEV)
+    with pytest.raises(T.TdgsError) as e:
+        ctx.reserve_views(vs, 0xffffffff)
+    assert e.value.status == T.OUT_OF_MEMORY
+    refused(ctx, vs)
+    del hold
+    torch.cuda.empty_cache()
+    ctx.reserve_views(vs, m)
+    ctx.sort_views_async(vs)
+    check(oracle, frames, ctx.views_results(1))
