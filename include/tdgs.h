@@ -130,6 +130,8 @@ tdgs_status tdgs_context_set_sort_variant(tdgs_context* ctx, int variant);
 /* Further tuning knobs of a context (value 0, or -1 for the sort variant,
  * restores the built-in choice); out-of-range keys or values return
  * TDGS_ERR_INVALID_ARGUMENT.
+ * An asynchronous batch (tdgs_sort_views_async) keeps the knobs that its
+ * reservation was made with.
  *   TDGS_TUNE_SORT_VARIANT     pass kernel of tdgs_sort_pairs (as above)
  *   TDGS_TUNE_TILE_DIGIT_BITS  widest digit (4..12) of the frame's passes
  *                              over the tile bits (built-in: no such passes

@@ -120,6 +120,8 @@ struct FrameState {
   uint32_t reserved_nv = 0, reserved_n = 0, reserved_t = 0;
   uint64_t capacity = 0;
   bool split_reserved = false;  // what the reservation chose
+  Tuning tuning_reserved;       // its knobs: launches and scratch of the asynchronous batches
+  Tuning knobs;                 // of the call at hand: the context's, or the reservation's
   bool exact = false;           // a call that waits for the pair count (not an asynchronous one)
   bool reserved = false;
 
@@ -825,7 +827,7 @@ ViewTable device_table(tdgs_context* ctx) {
 // 16 views of 500,000 1410 and 832).
 bool splits(const tdgs_context* ctx) {
   return (ctx->nv == 1 || ctx->n_all < (1u << 30)) && ctx->max_gx <= kSplitMaxBins && ctx->max_gy <= kSplitMaxBins &&
-         ctx->tuning.tile_digit_bits == 0;
+         ctx->knobs.tile_digit_bits == 0;
 }
 
 // A view of at most kSplitSmall Gaussians and kSmallTiles tiles of segments
@@ -844,7 +846,7 @@ uint64_t split_tiles(const tdgs_context* ctx, uint64_t m) { return m / kSplitTil
 bool by_view(const tdgs_context* ctx) { return ctx->split && ctx->nv > 1; }
 
 DepthPlan depth_plan(const tdgs_context* ctx) {
-  return plan_depth_sort(ctx->n_all, ctx->tuning.depth_digit_bits, ctx->tuning.ctas_per_sm, !ctx->split,
+  return plan_depth_sort(ctx->n_all, ctx->knobs.depth_digit_bits, ctx->knobs.ctas_per_sm, !ctx->split,
                          by_view(ctx));
 }
 
@@ -865,7 +867,7 @@ Shape shape_of(const tdgs_context* ctx) {
   // tuned: one pass, but its scatter writes runs of about one element per
   // digit, which costs more than a second pass); the bits are split evenly
   // over the passes
-  const uint32_t dmax = ctx->tuning.tile_digit_bits > 0 ? static_cast<uint32_t>(ctx->tuning.tile_digit_bits) : 8u;
+  const uint32_t dmax = ctx->knobs.tile_digit_bits > 0 ? static_cast<uint32_t>(ctx->knobs.tile_digit_bits) : 8u;
   sh.npass = sh.tbits <= dmax ? 1u : (sh.tbits + dmax - 1) / dmax;
   sh.w0 = (sh.tbits + sh.npass - 1) / std::max(1u, sh.npass);
   sh.kbits = stream_kernel_bits(sh.w0);
@@ -947,7 +949,7 @@ tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
   const size_t esz = sh.wide ? 8 : 4;
   for (int b = 0; b < 2 && st == TDGS_OK; ++b) st = ensure(ctx, ctx->f_stream[b], m * esz + 16, s);
   const uint32_t mm = static_cast<uint32_t>(m ? m : 1);
-  const int cps = ctx->tuning.ctas_per_sm;
+  const int cps = ctx->knobs.ctas_per_sm;
   const uint32_t g0 = stream_grid(sh.wide, false, sh.kbits, mm, cps), g1 = stream_grid(sh.wide, true, sh.klast, mm, cps);
   if (g0 == 0 || g1 == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the tile sort failed");
   if (st == TDGS_OK)
@@ -1098,7 +1100,7 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.c1_cap = ctx->f_c1.bytes / sizeof(uint2);
   a.err = err_word(ctx);
   const uint32_t tiles2 = static_cast<uint32_t>(split_tiles(ctx, m));
-  const int cps = ctx->tuning.ctas_per_sm;
+  const int cps = ctx->knobs.ctas_per_sm;
   if (table_in_params(ctx) && n_all > 0 && n_all <= kSplitSmall && tiles2 <= kSmallTiles) {
     TDGS_TRACED(ctx, kKSmallSplit, m, s, launch_small_split(a, std::max(ctx->max_gx, ctx->max_gy), tiles2, s));
     return TDGS_OK;
@@ -1155,7 +1157,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
     sp.wide = sh.wide;
     sp.expand = last;
     sp.bits = last ? sh.klast : sh.kbits;
-    sp.grid = stream_grid(sh.wide, last, sp.bits, m, ctx->tuning.ctas_per_sm);
+    sp.grid = stream_grid(sh.wide, last, sp.bits, m, ctx->knobs.ctas_per_sm);
     sp.kin = st[p & 1];
     sp.kout = last ? ctx->f_keys.p : st[(p + 1) & 1];
     sp.vout = last ? static_cast<uint32_t*>(ctx->f_values.p) : nullptr;
@@ -1182,6 +1184,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
 // sort and the scan run; the back half is then enqueued with the exact M
 // before the GPU runs out of work.
 tdgs_status sort_views_exact(tdgs_context* ctx, cudaStream_t s, uint32_t* m_out) {
+  ctx->knobs = ctx->tuning;
   ctx->split = ctx->norm || splits(ctx);
   ctx->exact = true;
   tdgs_status st = ensure_record_buffers(ctx, s);
@@ -1568,6 +1571,7 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
   if (st != TDGS_OK) return st;
   ctx->reserved = false;  // an allocation that fails leaves no reservation
   ctx->exact = false;
+  ctx->knobs = ctx->tuning_reserved = ctx->tuning;
   ctx->split_reserved = splits(ctx);  // the asynchronous calls keep this choice
   // the tile passes' buffers too: they take a batch with the same totals whose
   // rows or columns the splits' buffers do not hold (split_fits)
@@ -1602,6 +1606,7 @@ tdgs_status tdgs_sort_views_async(tdgs_context* ctx, const tdgs_view* views, uin
     return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "views differ in shape from the reservation");
   st = stage_views(ctx, views, num_views);
   if (st != TDGS_OK) return st;
+  ctx->knobs = ctx->tuning_reserved;
   ctx->split = ctx->split_reserved && split_fits(ctx, ctx->capacity);
   ctx->exact = false;
   st = run_front(ctx, s);

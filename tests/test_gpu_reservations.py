@@ -93,3 +93,29 @@ def test_failed_reservation_is_none(ctx, oracle):
     ctx.reserve_views(vs, m)
     ctx.sort_views_async(vs)
     check(oracle, frames, ctx.views_results(1))
+
+
+@pytest.mark.parametrize("dims,new", [([(320, 320), (320, 320)], [(6400, 16), (16, 6400)]),  # splits, then not
+                                      ([(4800, 64), (4800, 64)], [(64, 4800), (4800, 64)])])  # tile passes both
+def test_knobs_set_after_the_reservation(ctx, oracle, dims, new):
+    """Batches keep the knobs of their reservation, which sized the scratch: a
+    wider tile digit and more blocks set later wait for the next one."""
+    first = [synth.frame_random(i, 20_000, w, h, max_sigma=5.0) for i, (w, h) in enumerate(dims)]
+    other = [synth.frame_random(7 + i, 20_000, w, h, max_sigma=5.0) for i, (w, h) in enumerate(new)]
+    vf, vo = on_gpu(first), on_gpu(other)
+    cap = max(sum(oracle.sort_frame(f.gaussians, f.width, f.height)["m"] for f in x) for x in (first, other))
+    ctx.apply_tuning({"tile_digit_bits": 0, "ctas_per_sm": 1})
+    ctx.reserve_views(vf, cap)
+    try:
+        ctx.apply_tuning({"tile_digit_bits": 12, "ctas_per_sm": 8})
+        for _ in range(2):
+            ctx.sort_views_async(vo)
+            check(oracle, other, ctx.views_results(2))
+            ctx.sort_views_async(vf)
+            check(oracle, first, ctx.views_results(2))
+        ctx.reserve_views(vf, cap)
+        ctx.sort_views_async(vo)
+        check(oracle, other, ctx.views_results(2))
+        check(oracle, first, ctx.sort_views(vf))
+    finally:
+        ctx.apply_tuning({"tile_digit_bits": 0, "ctas_per_sm": 0})
