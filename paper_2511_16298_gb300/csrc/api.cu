@@ -1115,12 +1115,14 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
 }
 
 // Steps after: duplication, tile passes, ranges.  m = exact pair count, or
-// the reserved capacity with m_dev pointing at the device count.
+// the reserved capacity with m_dev pointing at the device count.  Without
+// pairs there is nothing to do but the ranges; for a capacity of zero the
+// kernels that compare the count with it come first.
 tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaStream_t s) {
-  if (m == 0) {
+  const bool none = m == 0 && ctx->exact;
+  if (none || (m == 0 && !ctx->split))
     TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_ranges.p, 0, static_cast<size_t>(ctx->t_all) * 8, s));
-    return TDGS_OK;
-  }
+  if (none) return TDGS_OK;
   if (ctx->split) return run_back_split(ctx, m, s);
   const ViewTable vt = device_table(ctx);
   const Shape sh = shape_of(ctx);
@@ -1137,6 +1139,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
   TDGS_TRACED(ctx, kKDupDepth, n_all, s,
               launch_views_dup(vt, sorder, static_cast<uint32_t*>(ctx->f_soff.p), n_all, sh.rbits, st[0],
                                sh.wide, m, sdo, err_word(ctx), s));
+  if (m == 0) return TDGS_OK;
   // One pass over the whole tile id writes the ranges from its digit
   // totals; with several passes the last one records each tile's first and
   // last position and a small kernel turns them into ranges.

@@ -119,3 +119,25 @@ def test_knobs_set_after_the_reservation(ctx, oracle, dims, new):
         check(oracle, first, ctx.sort_views(vf))
     finally:
         ctx.apply_tuning({"tile_digit_bits": 0, "ctas_per_sm": 0})
+
+
+@pytest.mark.parametrize("width,height", [(640, 360), (4800, 64)])
+@pytest.mark.parametrize("views", [1, 3])
+def test_capacity_of_zero(ctx, width, height, views):
+    """A reservation for no pairs takes batches without any, and reports the
+    others, through the splits and the tile passes."""
+    frames = [synth.frame_random(i, 2500, width, height) for i in range(views)]
+    vs = on_gpu(frames)
+    ctx.reserve_views(vs, 0)
+    for _ in range(2):
+        ctx.sort_views_async(vs)
+        with pytest.raises(T.TdgsError) as e:  # (no result is read)
+            ctx.views_results(views)
+        assert e.value.status == T.CAPACITY
+    for g, _, _ in vs:
+        g[:, 3] = 0  # radius: culled
+    ctx.sort_views_async(vs)
+    graph = capture(ctx, vs)
+    graph.replay()
+    for k, v, r, m in ctx.views_results(views):
+        assert m == 0 and k.numel() == 0 and not r.any()
