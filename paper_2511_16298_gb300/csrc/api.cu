@@ -104,6 +104,10 @@ struct FrameState {
   Buffer f_rects, f_c1, f_rows, f_segs, f_cols, f_c2, f_b2;  // interval splits
   Buffer f_dos;   // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
   Buffer f_pair;  // single-launch depth sort without offsets: intermediate pairs (with f_sdo)
+  // Scratch of a frame's passes and scan, apart from that of the step calls
+  // and of the other state: only a frame or reservation on this state moves
+  // what a captured batch was given.
+  Buffer f_scratch, f_scan;
   // f_rminmax holds first positions in its first half and one-past-last
   // positions in its second half, kept at (all ones, zero) between frames:
   // the ranges kernel resets what the last tile pass recorded
@@ -132,7 +136,7 @@ struct FrameState {
   void release() {
     for (Buffer* b : {&f_counts, &f_dkey[0], &f_dkey[1], &f_dkey[2], &f_dval[0], &f_dval[1], &f_dval[2], &f_soff,
                       &f_sdo, &f_rminmax, &f_stream[0], &f_stream[1], &f_keys, &f_values, &f_ranges, &f_rects, &f_c1,
-                      &f_rows, &f_segs, &f_cols, &f_c2, &f_b2, &f_dos, &f_pair})
+                      &f_rows, &f_segs, &f_cols, &f_c2, &f_b2, &f_dos, &f_pair, &f_scratch, &f_scan})
       if (b->p) cudaFree(b->p);
     if (d_views) cudaFree(d_views);
     if (h_views) cudaFreeHost(h_views);
@@ -347,14 +351,14 @@ tdgs_status traced(tdgs_context* ctx, KernelId id, uint64_t items, cudaStream_t 
 
 tdgs_status do_scan(tdgs_context* ctx, KernelId id, const uint32_t* counts, const float4* recs,
                     const uint32_t* gather, FrameGeom fg, uint32_t n, uint32_t* offsets,
-                    uint64_t* total64, uint32_t* total32, cudaStream_t s) {
-  // scan_status: the tile ticket in word 0, then one status word per tile;
+                    uint64_t* total64, uint32_t* total32, Buffer& status, cudaStream_t s) {
+  // status: the tile ticket in word 0, then one status word per tile;
   // one memset clears both
   const uint32_t tiles = (n + kScanTileItems - 1) / kScanTileItems;
-  tdgs_status st = ensure(ctx, ctx->scan_status, static_cast<size_t>(tiles) * 8 + 8, s);
+  tdgs_status st = ensure(ctx, status, static_cast<size_t>(tiles) * 8 + 8, s);
   if (st != TDGS_OK) return st;
-  TDGS_CUDA(ctx, cudaMemsetAsync(ctx->scan_status.p, 0, static_cast<size_t>(tiles) * 8 + 8, s));
-  uint64_t* words = static_cast<uint64_t*>(ctx->scan_status.p);
+  TDGS_CUDA(ctx, cudaMemsetAsync(status.p, 0, static_cast<size_t>(tiles) * 8 + 8, s));
+  uint64_t* words = static_cast<uint64_t*>(status.p);
   TDGS_TRACED(ctx, id, n, s,
               launch_scan(counts, recs, gather, fg, n, offsets, words + 1, reinterpret_cast<uint32_t*>(words), 0u,
                           total64, total32, err_word(ctx), s));
@@ -643,7 +647,7 @@ tdgs_status tdgs_scan(tdgs_context* ctx, const uint32_t* counts, uint32_t n, uin
   if (!counts || !offsets) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null pointer");
   if (!aligned(counts, 4) || !aligned(offsets, 4) || (total_dev && !aligned(total_dev, 4)))
     return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "misaligned pointer");
-  return do_scan(ctx, kKScan, counts, nullptr, nullptr, FrameGeom{}, n, offsets, nullptr, total_dev, s);
+  return do_scan(ctx, kKScan, counts, nullptr, nullptr, FrameGeom{}, n, offsets, nullptr, total_dev, ctx->scan_status, s);
 }
 
 tdgs_status tdgs_duplicate_keys(tdgs_context* ctx, const tdgs_gaussian2d* g,
@@ -893,11 +897,13 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_rows, (static_cast<size_t>(split_rows(ctx)) + 1) * 20 + 16, s);
   }
   const uint32_t n_all = ctx->n_all;
-  const uint32_t tiles = (n_all + kScanTileItems - 1) / kScanTileItems;
-  if (st == TDGS_OK) st = ensure(ctx, ctx->scan_status, static_cast<size_t>(tiles) * 8 + 8, s);
   const DepthPlan dp = depth_plan(ctx);
   if (dp.grid == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the depth sort failed");
-  if (st == TDGS_OK) st = ensure(ctx, ctx->sort_scratch, dp.scratch_words * 4, s);
+  if (!ctx->split && !dp.resident) {  // the scan of the counts in depth order
+    const uint32_t tiles = (n_all + kScanTileItems - 1) / kScanTileItems;
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_scan, static_cast<size_t>(tiles) * 8 + 8, s);
+  }
+  if (st == TDGS_OK) st = ensure(ctx, ctx->f_scratch, dp.scratch_words * 4, s);
   if (st == TDGS_OK && dp.resident) {
     grown = false;
     if (ctx->split) st = ensure(ctx, ctx->f_pair, static_cast<size_t>(n_all) * 8 + 16, s);
@@ -953,7 +959,7 @@ tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
   const uint32_t g0 = stream_grid(sh.wide, false, sh.kbits, mm, cps), g1 = stream_grid(sh.wide, true, sh.klast, mm, cps);
   if (g0 == 0 || g1 == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the tile sort failed");
   if (st == TDGS_OK)
-    st = ensure(ctx, ctx->sort_scratch,
+    st = ensure(ctx, ctx->f_scratch,
                 std::max(stream_scratch_words(sh.wide, false, sh.kbits, g0),
                          stream_scratch_words(sh.wide, true, sh.klast, g1)) * 4,
                 s);
@@ -1027,7 +1033,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   }
   if (ctx->norm) TDGS_TRACED(ctx, kKNormKeys, n_all, s, launch_norm_keys(dk[0], n_all, ctx->d_range, range, dp.onesweep ? raw : nullptr, s));
   const uint32_t dpasses = dp.passes;
-  uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
+  uint32_t* scratch = static_cast<uint32_t*>(ctx->f_scratch.p);
   if (dp.resident) {  // one launch: the sort (pass count from the depth range) and the offsets
     da.key0 = dk[0];
     TDGS_TRACED(ctx, ctx->split ? kKDepthOrder : kKDepthSort, n_all, s, launch_depth_sort(dp.grid, dp.items, da, s));
@@ -1048,7 +1054,7 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   }
   if (n_all && !dp.resident && !ctx->split) {
     tdgs_status st = do_scan(ctx, kKFrameScan, counts, nullptr, dv[dp.result], FrameGeom{}, n_all,
-                             static_cast<uint32_t*>(ctx->f_soff.p), &ctx->d_status->total, nullptr, s);
+                             static_cast<uint32_t*>(ctx->f_soff.p), &ctx->d_status->total, nullptr, ctx->f_scan, s);
     if (st != TDGS_OK) return st;
   } else if (n_all == 0) {
     TDGS_CUDA(ctx, cudaMemsetAsync(&ctx->d_status->total, 0, 8, s));
@@ -1130,7 +1136,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
   const uint32_t dres = depth_plan(ctx).result;
   const uint32_t* sorder = static_cast<uint32_t*>(ctx->f_dval[dres].p);
   uint2* sdo = static_cast<uint2*>(ctx->f_sdo.p);
-  uint32_t* scratch = static_cast<uint32_t*>(ctx->sort_scratch.p);
+  uint32_t* scratch = static_cast<uint32_t*>(ctx->f_scratch.p);
   uint32_t* bar = ctx->d_tickets + 2;
   void* st[2] = {ctx->f_stream[0].p, ctx->f_stream[1].p};
   const size_t half = ctx->f_rminmax.bytes / 8;  // tiles the buffer holds
@@ -1474,7 +1480,8 @@ tdgs_status tdgs_sort_frame_normalized(tdgs_context* ctx, const tdgs_gaussian2d*
     TDGS_CUDA(ctx, cudaMemsetAsync(norm, 0xff, 4, s));
     TDGS_CUDA(ctx, cudaMemsetAsync(norm + 1, 0, 4, s));
     TDGS_TRACED(ctx, kKNormRange, n, s, launch_norm_range(g4, counts, n, norm, s));
-    st = do_scan(ctx, kKScan, counts, nullptr, nullptr, FrameGeom{}, n, offs, &ctx->d_status->total, nullptr, s);
+    st = do_scan(ctx, kKScan, counts, nullptr, nullptr, FrameGeom{}, n, offs, &ctx->d_status->total, nullptr,
+                 ctx->scan_status, s);
     if (st != TDGS_OK) return st;
     TDGS_CUDA(ctx, cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
     TDGS_CUDA(ctx, cudaStreamSynchronize(s));

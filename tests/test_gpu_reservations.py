@@ -141,3 +141,35 @@ def test_capacity_of_zero(ctx, width, height, views):
     graph.replay()
     for k, v, r, m in ctx.views_results(views):
         assert m == 0 and k.numel() == 0 and not r.any()
+
+
+@pytest.mark.parametrize("n", [3000, 700_000])  # the single-launch depth sort, and the passes with their scan
+def test_captured_tile_passes_keep_their_scratch(ctx, oracle, n):
+    """A captured batch through the tile passes outlives larger calls that
+    take scratch of their own: normalised frames of both kinds, a scan and a
+    sort by the chunked passes."""
+    frames = [synth.frame_random(i, n, 4800, 64, max_sigma=5.0) for i in range(2)]
+    vs = on_gpu(frames)
+    ctx.reserve_views(vs, sum(oracle.sort_frame(f.gaussians, f.width, f.height)["m"] for f in frames))
+    ctx.sort_views_async(vs)
+    graph = capture(ctx, vs)
+    for width, height in ((640, 360), (4800, 64)):
+        f = synth.frame_random(9, 3 * n, width, height, max_sigma=5.0)
+        st, ek, ev, er = oracle.sort_frame_normalized(f.gaussians, width, height)
+        k, v, r, m = ctx.sort_frame_normalized(T.records_to_tensor(f.gaussians, DEV), width, height)
+        assert st == 0 and m == len(ek)
+        assert np.array_equal(k.cpu().numpy().view(np.uint32), ek)
+        assert np.array_equal(v.cpu().numpy().view(np.uint32), ev)
+    counts = torch.randint(0, 9, (9 * n,), dtype=torch.int32, device=DEV)
+    off, _ = ctx.scan(counts)
+    assert torch.equal(off[1:].long(), torch.cumsum(counts.long(), 0)[:-1])
+    keys = torch.randint(0, 1 << 44, (9 * n,), dtype=torch.int64, device=DEV)
+    vals = torch.arange(9 * n, dtype=torch.int32, device=DEV)
+    want, order = torch.sort(keys, stable=True)
+    ctx.set_sort_variant(0)
+    sk, sv = ctx.sort_pairs(keys, vals, 12)
+    ctx.set_sort_variant(-1)
+    assert torch.equal(sk, want) and torch.equal(sv.long(), order)
+    for _ in range(2):
+        graph.replay()
+        check(oracle, frames, ctx.views_results(2))
