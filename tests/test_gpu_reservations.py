@@ -173,3 +173,36 @@ def test_captured_tile_passes_keep_their_scratch(ctx, oracle, n):
     for _ in range(2):
         graph.replay()
         check(oracle, frames, ctx.views_results(2))
+
+
+@pytest.mark.parametrize("shapes,new,fits", [
+    ([(640, 160), (160, 640)], [(160, 640), (640, 160)], True),   # as many rows and columns at most
+    ([(640, 160), (160, 640)], [(480, 160), (160, 800)], False),  # more rows in one view
+    ([(320, 320), (320, 320)], [(640, 160), (160, 640)], False),  # wider and taller
+    ([(1600, 64)], [(64, 1600)], False),
+    ([(320, 320), (320, 320)], [(6400, 16), (16, 6400)], False),  # beyond the splits
+])
+def test_replays_of_other_proportions(ctx, oracle, shapes, new, fits):
+    """A captured batch replayed over the table of a later one: its results
+    where the captured launches have room for its rows and columns, and a
+    report where they have not."""
+    first = [synth.frame_random(i, 9000, w, h, max_sigma=5.0) for i, (w, h) in enumerate(shapes)]
+    ns = [18_000] if len(new) == 1 else [7000, 11_000]
+    other = [synth.frame_random(5 + i, k * len(shapes) // 2, w, h, max_sigma=5.0)
+             for i, (k, (w, h)) in enumerate(zip(ns, new))]
+    vf, vo = on_gpu(first), on_gpu(other)
+    ctx.reserve_views(vf, max(sum(oracle.sort_frame(f.gaussians, f.width, f.height)["m"] for f in x)
+                              for x in (first, other)))
+    ctx.sort_views_async(vf)
+    graph = capture(ctx, vf)
+    ctx.sort_views_async(vo)
+    check(oracle, other, ctx.views_results(len(vo)))
+    graph.replay()
+    if fits:
+        check(oracle, other, ctx.views_results(len(vo)))
+    else:
+        with pytest.raises(T.TdgsError) as e:
+            ctx.views_results(len(vo))
+        assert e.value.status == T.CAPACITY
+    ctx.sort_views_async(vf)
+    check(oracle, first, ctx.views_results(len(vf)))
