@@ -86,8 +86,10 @@ static_assert(kWarpW * kWarpH == 32 && 2 * kWarpW == 16 && 4 * kWarpH == 16, "ei
 // staging thread 110 instructions, so only tiles of more than one batch take
 // it (render of 700k Gaussians: 400x300 88 -> 84 us, 20k at 320x180 29 -> 27,
 // but 4K with 86 Gaussians a tile 455 -> 467).  Flatter conics, Q not positive
-// definite, or anything not finite reach every warp.  K < 0: no pixel passes
-// the cut test (no warp).
+// definite or not finite, and means that are no number reach every warp (the
+// exponent of such a mean is no number either, which no test of a pixel
+// leaves out; the clamps here would take it for a coordinate).  K < 0: no
+// pixel passes the cut test (no warp).
 __device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, float cut, float tx0, float ty0,
                                               bool ellipse) {
   const float K = -2.0f * cut;
@@ -96,6 +98,7 @@ __device__ __forceinline__ uint32_t warp_mask(float mx, float my, float4 c, floa
   const float ac = c.x * c.z;
   const float det = fmaf(-c.y, c.y, ac);
   if (!(c.x > 0.0f && c.z > 0.0f && det > 1e-3f * ac && K < 1e30f)) return all;
+  if (isnan(mx) || isnan(my)) return all;
   const float hy2 = __fdividef(K * c.x, det) * 1.0201f;
   const float hx2 = __fdividef(K * c.z, det) * 1.0201f;
   if (!(hy2 < 1e30f && hx2 < 1e30f)) return all;
