@@ -411,6 +411,16 @@ tdgs_status tdgs_render(tdgs_context* ctx, const tdgs_gaussian2d* records, const
  * fault or hang is involved. */
 tdgs_status tdgs_diag_barrier_timeout(tdgs_context* ctx, void* stream);
 
+/* Failure-detection check of the onesweep passes: tdgs_sort_pairs with the
+ * blocks left out that turn the tiles' digit counts into prefixes, as if
+ * another stream's kernel held the SMs that they wait for.  Each tile then
+ * adds up the counts before it once its wait for a prefix has run out (a few
+ * ms each), and the result is the same.  For the sorts that take these passes
+ * (else TDGS_ERR_INVALID_ARGUMENT). */
+tdgs_status tdgs_diag_sort_pairs(tdgs_context* ctx, uint64_t* keys, uint32_t* values, uint64_t* keys_alt,
+                                 uint32_t* values_alt, uint32_t m, uint32_t tile_bits, uint32_t flags,
+                                 int* result_in_alt, void* stream);
+
 /* ------------------------------------------------- scan without allocation */
 
 /* The exclusive scan of tdgs_scan (offsets, total, 64-bit overflow check)

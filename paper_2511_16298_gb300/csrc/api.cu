@@ -367,7 +367,7 @@ tdgs_status do_scan(tdgs_context* ctx, KernelId id, const uint32_t* counts, cons
 
 tdgs_status do_sort(tdgs_context* ctx, uint64_t* keys, uint32_t* values, uint64_t* keys_alt,
                     uint32_t* values_alt, uint32_t m, uint32_t tile_bits, uint32_t flags,
-                    int* result_in_alt, cudaStream_t s) {
+                    int* result_in_alt, cudaStream_t s, bool scan = true) {
   *result_in_alt = 0;
   if (m == 0) return TDGS_OK;
   if (tdgs_status st0 = clear_barrier_if_dirty(ctx, s); st0 != TDGS_OK) return st0;
@@ -386,7 +386,7 @@ tdgs_status do_sort(tdgs_context* ctx, uint64_t* keys, uint32_t* values, uint64_
     uint32_t* vout = values_alt;
     for (uint32_t p = 0; p < plan.passes; ++p) {
       TDGS_TRACED(ctx, kKOnesweep, m, s,
-                  launch_onesweep_pass(plan, p, kin, vin, kout, vout, m, scratch, err_word(ctx), s));
+                  launch_onesweep_pass(plan, p, kin, vin, kout, vout, m, scratch, err_word(ctx), s, scan));
       std::swap(kin, kout);
       std::swap(vin, vout);
     }
@@ -424,6 +424,24 @@ tdgs_status read_and_clear_error(tdgs_context* ctx, cudaStream_t s) {
     return fail(ctx, static_cast<tdgs_status>(e),
                 std::string("error latched on the device by ") + site_name(ctx->h_status->site));
   }
+  return TDGS_OK;
+}
+
+// The arguments of tdgs_sort_pairs.
+tdgs_status check_pairs(tdgs_context* ctx, const uint64_t* keys, const uint32_t* values, const uint64_t* keys_alt,
+                        const uint32_t* values_alt, uint32_t m, uint32_t tile_bits, uint32_t flags,
+                        int* result_in_alt) {
+  if (!ctx || !result_in_alt) return TDGS_ERR_INVALID_ARGUMENT;
+  *result_in_alt = 0;
+  if (tile_bits > 32) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "tile_bits > 32");
+  if (flags & ~TDGS_SORT_DEPTH_POSITIVE) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "unknown flag");
+  if (m == 0) return TDGS_OK;
+  if (!keys || !values || !keys_alt || !values_alt)
+    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null pointer");
+  if (!aligned(keys, 8) || !aligned(keys_alt, 8) || !aligned(values, 4) || !aligned(values_alt, 4))
+    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "misaligned pointer");
+  if (keys == keys_alt || values == values_alt)
+    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "alternate buffers must differ");
   return TDGS_OK;
 }
 
@@ -673,20 +691,25 @@ tdgs_status tdgs_sort_pairs(tdgs_context* ctx, uint64_t* keys, uint32_t* values,
                             uint64_t* keys_alt, uint32_t* values_alt, uint32_t m,
                             uint32_t tile_bits, uint32_t flags, int* result_in_alt,
                             void* stream) {
-  if (!ctx || !result_in_alt) return TDGS_ERR_INVALID_ARGUMENT;
-  *result_in_alt = 0;
-  if (tile_bits > 32) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "tile_bits > 32");
-  if (flags & ~TDGS_SORT_DEPTH_POSITIVE) return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "unknown flag");
-  if (m == 0) return TDGS_OK;
-  if (!keys || !values || !keys_alt || !values_alt)
-    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "null pointer");
-  if (!aligned(keys, 8) || !aligned(keys_alt, 8) || !aligned(values, 4) || !aligned(values_alt, 4))
-    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "misaligned pointer");
-  if (keys == keys_alt || values == values_alt)
-    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "alternate buffers must differ");
+  const tdgs_status st =
+      check_pairs(ctx, keys, values, keys_alt, values_alt, m, tile_bits, flags, result_in_alt);
+  if (st != TDGS_OK || m == 0) return st;
   DeviceGuard dg(ctx->device);
   return do_sort(ctx, keys, values, keys_alt, values_alt, m, tile_bits, flags, result_in_alt,
                  static_cast<cudaStream_t>(stream));
+}
+
+tdgs_status tdgs_diag_sort_pairs(tdgs_context* ctx, uint64_t* keys, uint32_t* values, uint64_t* keys_alt,
+                                 uint32_t* values_alt, uint32_t m, uint32_t tile_bits, uint32_t flags,
+                                 int* result_in_alt, void* stream) {
+  const tdgs_status st =
+      check_pairs(ctx, keys, values, keys_alt, values_alt, m, tile_bits, flags, result_in_alt);
+  if (st != TDGS_OK || m == 0) return st;
+  if (ctx->tuning.sort_variant >= 0 || !onesweep_eligible(m, keys, values, keys_alt, values_alt))
+    return fail(ctx, TDGS_ERR_INVALID_ARGUMENT, "not a sort by the onesweep passes");
+  DeviceGuard dg(ctx->device);
+  return do_sort(ctx, keys, values, keys_alt, values_alt, m, tile_bits, flags, result_in_alt,
+                 static_cast<cudaStream_t>(stream), false);
 }
 
 tdgs_status tdgs_sort_pairs_bitonic(tdgs_context* ctx, const uint64_t* keys_in, const uint32_t* values_in,

@@ -27,9 +27,10 @@
 // high word, or spanning both (tdgs_sort_pairs), and 32-bit depth keys
 // compressed to their range, whose pass plan each launch reads from the
 // range on the device.  Tickets keep the waits deadlock-free: a tile only
-// waits on tiles with smaller tickets, and ranking (which publishes the
-// counts) never waits on another CTA.  Every wait is bounded and latches
-// TDGS_ERR_TIMEOUT when it runs out; every scatter is checked against the
+// waits on tiles with smaller tickets, whose counts it adds up itself if the
+// scan CTAs do not, and ranking (which publishes the counts) never waits on
+// another CTA.  Every wait is bounded: one that runs out latches
+// TDGS_ERR_TIMEOUT (or ends a scan CTA); every scatter is checked against the
 // pair count.
 #include <mutex>
 #include <type_traits>
@@ -140,6 +141,7 @@ struct HistArgs {
 
 struct PassArgs {
   uint32_t m, ntiles;
+  uint32_t nscan;          // scan CTAs: kScanCtas, or none (a diagnostic)
   Digit dg;
   Digit dgn;               // the next pass's digit (counted while ranking)
   const uint32_t* gstart;  // [kBins] this pass's digit starts (pass 0), or null
@@ -311,11 +313,13 @@ __device__ __forceinline__ void rank_in_warps(const TileBuf<KeyOf<kMode>>& tb, u
 // k_(i-1) (ranked one iteration earlier) from the scan CTAs and scatters
 // that tile.  The prefix is needed a whole ranking phase after the counts
 // went out, so the scan has (nearly always) produced it.  Ranking never
-// waits for another CTA, so every tile with a ticket publishes its counts
-// and the scan always completes.  The grid has no more CTAs than are resident
-// at once, and the scan CTAs come first in it: they run alongside whichever
-// others do, and a CTA that is not resident yet holds no ticket.  (A
-// cooperative launch would start only after the launch before it has ended.)
+// waits for another CTA, a CTA that is not resident yet holds no ticket, and a
+// tile whose prefix does not come adds up the counts before it (wait_prefix):
+// the tiles end in ticket order with whatever CTAs are resident, the scan
+// CTAs among them or not.  So the launch need not be cooperative (which would
+// start only after the launch before it has ended, and with all CTAs at once),
+// and other streams' kernels may hold any part of the GPU.  The scan CTAs come
+// first in the grid, so that they usually start first.
 // While ranking, the CTA also counts
 // the next pass's digits; the counts reach hist_next when it finishes.
 template <int kMode, int kModeN>
@@ -378,8 +382,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 
   const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
   const uint32_t m = a.m, ntiles = a.ntiles;
-  if (blockIdx.x < kScanCtas) {
-    scan_tiles<kBins>(a.status, ntiles, blockIdx.x, a.err, reinterpret_cast<uint32_t*>(smem));
+  if (blockIdx.x < a.nscan) {
+    scan_tiles<kBins>(a.status, ntiles, blockIdx.x, reinterpret_cast<uint32_t*>(smem));
     return;
   }
   uint16_t* my_wh = wh + warp * kBins;
@@ -671,7 +675,7 @@ cudaError_t launch_pass(Fn fn, const K* kin, const uint32_t* vin, K* kout, uint3
   constexpr bool depth = sizeof(K) == 4;
   const uint32_t resident = pass_grid(depth);
   if (resident < 2 * kScanCtas) return cudaErrorInvalidConfiguration;
-  const uint32_t grid = (a.ntiles < resident - kScanCtas ? a.ntiles : resident - kScanCtas) + kScanCtas;
+  const uint32_t grid = (a.ntiles < resident - kScanCtas ? a.ntiles : resident - kScanCtas) + a.nscan;
   const size_t smem = pass_smem(depth);
   if (cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem)) != cudaSuccess)
@@ -750,11 +754,12 @@ cudaError_t launch_onesweep_hist(const SortPlan& plan, const uint64_t* keys, uin
 
 cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint64_t* kin, const uint32_t* vin,
                                  uint64_t* kout, uint32_t* vout, uint32_t m, uint32_t* scratch, uint32_t* err,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, bool scan) {
   using namespace onesweep;
   PassArgs a{};
   a.m = m;
   a.ntiles = (m + kTileKeys - 1) / kTileKeys;
+  a.nscan = scan ? kScanCtas : 0u;
   a.dg = make_digit(plan.shift[pass], plan.mask[pass], plan.drop31);
   const bool has_next = pass + 1 < plan.passes;
   if (has_next) a.dgn = make_digit(plan.shift[pass + 1], plan.mask[pass + 1], plan.drop31);
@@ -789,6 +794,7 @@ cudaError_t launch_depth_onesweep_pass(uint32_t pass, uint32_t* const dk[3], uin
   PassArgs a{};
   a.m = n;
   a.ntiles = (n + kTileKeys - 1) / kTileKeys;
+  a.nscan = kScanCtas;
   a.nv = nv;
   a.rec_begin = rec_begin;
   // the device drops the next pass's counts and status when this pass is

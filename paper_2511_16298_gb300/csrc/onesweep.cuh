@@ -104,9 +104,10 @@ __device__ __forceinline__ uint32_t cta_excl_scan(uint32_t v, uint32_t* s_warp) 
 // consumed in order: running sums plus the sums of the warps before give
 // each row its inclusive prefix, which overwrites its counts.  The next
 // round starts at the first row not consumed (after a short sleep when no
-// pair moved).  The scan waits only on counts, which every tile publishes
-// without waiting on anything, so it always finishes (the wait is
-// bounded).  Spreading the digits over several CTAs spreads the status
+// pair moved).  The scan only saves work: tiles that wait too long for a
+// prefix add up the counts themselves (look_back), so a scan CTA that finds
+// no counts for kSpinLimit rounds (other streams' kernels may hold the SMs
+// that the tiles' CTAs need) leaves, and nothing is wrong.  Spreading the digits over several CTAs spreads the status
 // traffic (about 4 KB per tile) over several SMs.
 constexpr uint32_t kSegRows = 8;  // rows per warp and round
 static_assert(kWarps * kSegRows == 64, "scan layout");
@@ -117,7 +118,7 @@ constexpr uint32_t scan_ctas() {
 }
 template <uint32_t kBins>
 __device__ __forceinline__ void scan_tiles(uint32_t* __restrict__ status, uint32_t ntiles, uint32_t c,
-                                           uint32_t* err, uint32_t* sm) {
+                                           uint32_t* sm) {
   uint32_t(*s_stop)[32] = reinterpret_cast<uint32_t(*)[32]>(sm);
   uint32_t(*s_sum0)[32] = reinterpret_cast<uint32_t(*)[32]>(sm + kWarps * 32);
   uint32_t(*s_sum1)[32] = reinterpret_cast<uint32_t(*)[32]>(sm + 2 * kWarps * 32);
@@ -184,17 +185,46 @@ __device__ __forceinline__ void scan_tiles(uint32_t* __restrict__ status, uint32
     run1 += all1;
     // no pair of the CTA moved: wait a little (bounded)
     if (!__syncthreads_or(used != 0 || k >= ntiles)) {
-      if (++idle > kSpinLimit) {
-        latch_error(err, TDGS_ERR_TIMEOUT, kSiteBarrier);
-        return;
-      }
+      if (++idle > kSpinLimit) return;
       __nanosleep(64);
     }
   }
 }
 
+// Exclusive prefix of digits 2t and 2t+1 for tile `tile` > 0 from the rows
+// before it: counts down to the first inclusive prefix, or to tile 0.  Every
+// row before it belongs to a tile whose ticket a resident CTA holds, and is
+// published once that CTA has the prefixes of its earlier tiles: the tiles
+// end in ticket order, with or without the scan CTAs.  (The wait for a row is
+// bounded all the same.)
+template <uint32_t kBins>
+__device__ __forceinline__ uint2 look_back(const uint32_t* status, uint32_t tile, uint32_t t, uint32_t* err) {
+  uint2 e = make_uint2(0u, 0u);
+  bool open0 = true, open1 = true;
+  uint32_t spins = 0;
+  for (uint32_t j = tile; j > 0 && (open0 || open1);) {
+    const uint2 w = ld_relaxed_v2(status + static_cast<size_t>(j - 1) * kBins + 2 * t);
+    if ((w.x & ~kCountMask) == 0 || (w.y & ~kCountMask) == 0) {
+      if (++spins > kSpinLimit) {
+        latch_error(err, TDGS_ERR_TIMEOUT, kSiteBarrier);
+        break;
+      }
+      __nanosleep(64);
+      continue;
+    }
+    if (open0) e.x += w.x & kCountMask;
+    if (open1) e.y += w.y & kCountMask;
+    open0 &= (w.x & ~kCountMask) != kFlagP;
+    open1 &= (w.y & ~kCountMask) != kFlagP;
+    --j;
+  }
+  return e;
+}
+
 // Exclusive prefix of digits 2t and 2t+1 for tile `tile` > 0: the inclusive
-// prefix the scan CTAs wrote for tile - 1 (bounded wait).
+// prefix the scan CTAs write for tile - 1, or, after kPatience polls (a few
+// ms; a prefix takes microseconds), the sum of the rows before.
+constexpr uint32_t kPatience = 1u << 12;
 template <uint32_t kBins>
 __device__ __forceinline__ void wait_prefix(const uint32_t* status, uint32_t tile, uint32_t t,
                                             uint32_t& e0, uint32_t& e1, uint32_t* err) {
@@ -202,8 +232,8 @@ __device__ __forceinline__ void wait_prefix(const uint32_t* status, uint32_t til
   uint2 w = ld_relaxed_v2(row);
   uint32_t spins = 0;
   while ((w.x & ~kCountMask) != kFlagP || (w.y & ~kCountMask) != kFlagP) {
-    if (++spins > kSpinLimit) {
-      latch_error(err, TDGS_ERR_TIMEOUT, kSiteBarrier);
+    if (++spins > kPatience) {
+      w = look_back<kBins>(status, tile, t, err);
       break;
     }
     __nanosleep(32);

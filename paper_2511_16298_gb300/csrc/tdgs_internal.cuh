@@ -537,7 +537,7 @@ cudaError_t launch_onesweep_hist(const SortPlan& plan, const uint64_t* keys, uin
                                  uint32_t* err, cudaStream_t s);
 cudaError_t launch_onesweep_pass(const SortPlan& plan, uint32_t pass, const uint64_t* kin, const uint32_t* vin,
                                  uint64_t* kout, uint32_t* vout, uint32_t m, uint32_t* scratch, uint32_t* err,
-                                 cudaStream_t s);
+                                 cudaStream_t s, bool scan);  // scan false: without the scan CTAs (a diagnostic)
 // The same passes over the depth sort's 32-bit keys (dk[0], dv[0]: keys and
 // indices from the count kernel; range: the key range it published in
 // range[2..3], and raw: the counts of the keys' low 9 bits, which it makes

@@ -99,6 +99,7 @@ def lib():
                 "tdgs_scan": ([P, P, u32, P, P, P], st),
                 "tdgs_duplicate_keys": ([P, P, P, u32, F, P, P, u32, P], st),
                 "tdgs_sort_pairs": ([P, P, P, P, P, u32, u32, u32, ctypes.POINTER(i32), P], st),
+                "tdgs_diag_sort_pairs": ([P, P, P, P, P, u32, u32, u32, ctypes.POINTER(i32), P], st),
                 "tdgs_tile_ranges": ([P, P, u32, u32, P, P], st),
                 "tdgs_sort_frame": ([P, P, u32, F, ctypes.POINTER(P), ctypes.POINTER(P),
                                      ctypes.POINTER(P), ctypes.POINTER(u32), P], st),
@@ -303,18 +304,26 @@ class Context:
                                               _stream(self.device)), "tdgs_duplicate_keys")
         return keys, values
 
-    def sort_pairs(self, keys, values, tile_bits: int, flags: int = 0, keys_alt=None,
-                   values_alt=None):
-        """Sort in place through the alternate buffers; returns the
-        (keys, values) tensors that hold the sorted result."""
+    def _sort_pairs(self, name, keys, values, tile_bits, flags, keys_alt, values_alt):
         m = keys.shape[0]
         keys_alt = torch.empty_like(keys) if keys_alt is None else keys_alt
         values_alt = torch.empty_like(values) if values_alt is None else values_alt
         alt = ctypes.c_int(0)
-        self._check(lib().tdgs_sort_pairs(self._h, _ptr(keys), _ptr(values), _ptr(keys_alt),
-                                          _ptr(values_alt), m, tile_bits, flags, ctypes.byref(alt),
-                                          _stream(self.device)), "tdgs_sort_pairs")
+        self._check(getattr(lib(), name)(self._h, _ptr(keys), _ptr(values), _ptr(keys_alt),
+                                         _ptr(values_alt), m, tile_bits, flags, ctypes.byref(alt),
+                                         _stream(self.device)), name)
         return (keys_alt, values_alt) if alt.value else (keys, values)
+
+    def sort_pairs(self, keys, values, tile_bits: int, flags: int = 0, keys_alt=None,
+                   values_alt=None):
+        """Sort in place through the alternate buffers; returns the
+        (keys, values) tensors that hold the sorted result."""
+        return self._sort_pairs("tdgs_sort_pairs", keys, values, tile_bits, flags, keys_alt, values_alt)
+
+    def diag_sort_pairs(self, keys, values, tile_bits: int, flags: int = 0):
+        """Failure-detection check: sort_pairs without the blocks that make
+        the tiles' prefixes."""
+        return self._sort_pairs("tdgs_diag_sort_pairs", keys, values, tile_bits, flags, None, None)
 
     def diag_barrier_timeout(self):
         """Failure-detection check: a grid barrier one block never reaches;
