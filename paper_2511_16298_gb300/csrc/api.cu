@@ -354,7 +354,7 @@ tdgs_status do_scan(tdgs_context* ctx, KernelId id, const uint32_t* counts, cons
                     uint64_t* total64, uint32_t* total32, Buffer& status, cudaStream_t s) {
   // status: the tile ticket in word 0, then one status word per tile;
   // one memset clears both
-  const uint32_t tiles = (n + kScanTileItems - 1) / kScanTileItems;
+  const uint32_t tiles = ceil_div(n, kScanTileItems);
   tdgs_status st = ensure(ctx, status, static_cast<size_t>(tiles) * 8 + 8, s);
   if (st != TDGS_OK) return st;
   TDGS_CUDA(ctx, cudaMemsetAsync(status.p, 0, static_cast<size_t>(tiles) * 8 + 8, s));
@@ -923,7 +923,7 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   const DepthPlan dp = depth_plan(ctx);
   if (dp.grid == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the depth sort failed");
   if (!ctx->split && !dp.resident) {  // the scan of the counts in depth order
-    const uint32_t tiles = (n_all + kScanTileItems - 1) / kScanTileItems;
+    const uint32_t tiles = ceil_div(n_all, kScanTileItems);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_scan, static_cast<size_t>(tiles) * 8 + 8, s);
   }
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_scratch, dp.scratch_words * 4, s);

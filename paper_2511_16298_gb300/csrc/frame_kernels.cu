@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(256) k_count_tiles(const float4* g, uint32_t n
                                                      uint32_t* err) {
   begin_launch();
   bool bad = false;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const TileRect q = tile_rect(__ldca(g + i), fg);
     bad |= q.invalid;
     counts[i] = q.count;
@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256) k_count_tiles(const float4* g, uint32_t n
 cudaError_t launch_count_tiles(const float4* g, uint32_t n, FrameGeom fg, uint32_t* counts,
                                uint32_t* err, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t blocks = (n + 255) / 256;
+  const uint32_t blocks = ceil_div(n, 256);
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
   return launch_after(k_count_tiles, grid, 256, 0, s, g, n, fg, counts, err);
 }
@@ -183,7 +183,7 @@ cudaError_t launch_scan(const uint32_t* counts, const float4* recs, const uint32
                         FrameGeom fg, uint32_t n, uint32_t* offsets, uint64_t* status,
                         uint32_t* ticket, uint32_t ticket_base, uint64_t* total64,
                         uint32_t* total32, uint32_t* err, cudaStream_t s) {
-  const uint32_t tiles = (n + kScanTileItems - 1) / kScanTileItems;
+  const uint32_t tiles = ceil_div(n, kScanTileItems);
   if (tiles == 0) return cudaSuccess;
   const auto fn = recs ? k_scan<1> : gather ? k_scan<2> : k_scan<0>;
   return launch_after(fn, tiles, kScanThreads, 0, s, counts, recs, gather, fg, n, offsets, status, ticket, ticket_base,
@@ -306,8 +306,8 @@ cudaError_t launch_duplicate(const float4* g, const uint32_t* offsets, uint32_t 
                              FrameGeom fg, uint64_t* keys, uint32_t* values, uint32_t cap,
                              uint32_t* err, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t warps = (n + 31) / 32;
-  const uint32_t blocks = (warps + 7) / 8;
+  const uint32_t warps = ceil_div(n, 32);
+  const uint32_t blocks = ceil_div(warps, 8);
   const uint32_t grid = blocks < 152u * 32u ? blocks : 152u * 32u;
   return launch_after(k_duplicate<false>, grid, 256, 0, s, g, offsets, n, fg, keys, values, cap, nullptr, err);
 }
@@ -316,8 +316,8 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
                                   uint32_t* keys, uint32_t* values, uint32_t cap, const uint32_t* norm,
                                   uint32_t* err, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t warps = (n + 31) / 32;
-  const uint32_t blocks = (warps + 7) / 8;
+  const uint32_t warps = ceil_div(n, 32);
+  const uint32_t blocks = ceil_div(warps, 8);
   const uint32_t grid = blocks < 152u * 32u ? blocks : 152u * 32u;
   return launch_after(k_duplicate<true>, grid, 256, 0, s, g, offsets, n, fg, keys, values, cap, norm, err);
 }
@@ -328,7 +328,7 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
 __global__ void __launch_bounds__(256) k_norm_range(const float4* g, const uint32_t* counts,
                                                     uint32_t n, uint32_t* norm) {
   uint32_t lo = 0xffffffffu, hi = 0u;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (__ldca(counts + i)) {
       const uint32_t b = __float_as_uint(__ldca(&g[i].z));
       lo = min(lo, b);
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(256) k_norm_range(const float4* g, const uint3
 
 cudaError_t launch_norm_range(const float4* g, const uint32_t* counts, uint32_t n, uint32_t* norm, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t blocks = (n + 255) / 256;
+  const uint32_t blocks = ceil_div(n, 256);
   const uint32_t grid = blocks < 152u * 8u ? blocks : 152u * 8u;
   k_norm_range<<<grid, 256, 0, s>>>(g, counts, n, norm);
   return cudaGetLastError();
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(256) k_norm_keys(uint32_t* __restrict__ keys, 
 cudaError_t launch_norm_keys(uint32_t* keys, uint32_t n, const uint32_t* range, uint32_t* out, uint32_t* raw,
                              cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  return launch_after(k_norm_keys, (n + 1023) / 1024, 256, 0, s, keys, n, range, out, raw);
+  return launch_after(k_norm_keys, ceil_div(n, 1024), 256, 0, s, keys, n, range, out, raw);
 }
 
 // ---------------------------------------------------------- tile ranges

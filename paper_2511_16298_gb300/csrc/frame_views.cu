@@ -229,7 +229,7 @@ cudaError_t launch_views_count(const ViewTable& vt, uint32_t n_all, uint32_t* co
                                uint64_t* total, uint32_t* range, void* host_status, cudaStream_t s,
                                const DepthPrep& prep, const Proj3D* proj) {
   const uint32_t per_block = 256u * (proj ? 2u : static_cast<uint32_t>(kCountUnroll));
-  const uint32_t blocks = (n_all + per_block - 1) / per_block;
+  const uint32_t blocks = ceil_div(n_all, per_block);
   // four blocks per SM: every block ends with up to 513 global atomics, on the
   // same words as all others' (3M records: 8 per SM 37 us, 4 31, 2 36)
   const uint32_t grid = blocks < 1u ? 1u : (blocks < 152u * 4u ? blocks : 152u * 4u);
@@ -406,7 +406,7 @@ cudaError_t launch_views_dup(const ViewTable& vt, const uint32_t* sorder, const 
                              uint32_t n_all, uint32_t rbits, void* out, bool wide, uint32_t cap,
                              uint2* sdo, uint32_t* err, cudaStream_t s) {
   if (n_all == 0) return cudaSuccess;
-  const uint32_t warps = (n_all + 31) / 32;
+  const uint32_t warps = ceil_div(n_all, 32);
   const uint32_t blocks = (warps + 7) / 8;
   const uint32_t grid = blocks < 152u * 32u ? blocks : 152u * 32u;
   if (wide)

@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(256)
                  float4* __restrict__ rec, float4* __restrict__ conic) {
   begin_launch();
   const float2 lim = proj::slope_limits(cam);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float4 p = __ldca(g + i);
     const float4 c0 = __ldca(cov + 2 * static_cast<size_t>(i));
     const float4 c1 = __ldca(cov + 2 * static_cast<size_t>(i) + 1);
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256)
 cudaError_t launch_preprocess(const float4* g, const float4* cov, uint32_t n, const CameraDev& cam, float4* rec,
                               float4* conic, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t blocks = (n + 255) / 256;
+  const uint32_t blocks = ceil_div(n, 256);
   const uint32_t grid = blocks < 152u * 16u ? blocks : 152u * 16u;
   return launch_after(k_preprocess, grid, 256, 0, s, g, cov, n, cam, rec, conic);
 }

@@ -145,6 +145,9 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
 }
 
 // ------------------------------------------------------------- host side
+// Blocks, warps or tiles of `per` items each that hold n items.
+constexpr uint32_t ceil_div(uint64_t n, uint32_t per) { return static_cast<uint32_t>((n + per - 1) / per); }
+
 // Launch of a kernel that starts with begin_launch().
 template <typename... Params, typename... Args>
 cudaError_t launch_after(void (*kernel)(Params...), uint32_t grid, int threads, size_t smem, cudaStream_t s,
