@@ -652,14 +652,16 @@ void pass_layout(onesweep::PassArgs& a, uint32_t pass, bool has_next, uint32_t* 
   a.status_next = has_next ? st + ((pass + 1) & 1u) * rows : nullptr;
 }
 
-// 4096 keys per block and step, at most 4 blocks per SM; above 4M keys at least
-// 4 steps per block (fewer global atomics on the 512 counters), below one (a
-// block's steps are a serial chain: 0.8M pairs 118.6 -> 117.0 us a sort)
+// 4096 keys per block and step, at most 4 blocks per SM; from 2M keys on at
+// least 4 steps per block (fewer global atomics on the 512 counters), below
+// one (a block's steps are a serial chain).  us a sort with one and four: 0.1M
+// pairs 53.9 and 58.0, 0.8M 99 and 101, 1.5M 121.5 and 122, 2.5M 152.2 and
+// 150.1, 4M 200 and 197, 6M 273 and 270, equal from 10M (the most blocks).
 uint32_t hist_grid(uint32_t m) {
   int sms = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
-  const uint32_t kPerBlock = (m >= (1u << 22) ? 4 : 1) * 8 * onesweep::kHistThreads;
+  const uint32_t kPerBlock = (m >= (1u << 21) ? 4 : 1) * 8 * onesweep::kHistThreads;
   uint32_t grid = static_cast<uint32_t>((static_cast<uint64_t>(m) + kPerBlock - 1) / kPerBlock);
   const uint32_t cap = static_cast<uint32_t>(sms) * 4;
   if (grid > cap) grid = cap;

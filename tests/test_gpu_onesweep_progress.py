@@ -89,3 +89,14 @@ def test_two_streams_at_once(oracle):
     finally:
         for c in ctx:
             c.close()
+
+
+@pytest.mark.parametrize("m", [(1 << 21) - 1, 1 << 21, (1 << 21) + 4097])
+def test_histogram_with_one_and_four_steps(m):
+    """Both sides of the size from which a histogram block takes four steps."""
+    keys, vals = pairs(m, 44, m)
+    want, order = torch.sort(keys, stable=True)
+    with T.Context(0) as ctx:
+        k, v = ctx.sort_pairs(keys, vals, 12)
+        ctx.sync()
+        assert torch.equal(k, want) and torch.equal(v.long(), order)
