@@ -365,7 +365,8 @@ tdgs_status tdgs_context_projected(tdgs_context* ctx, const tdgs_gaussian2d** re
  * tdgs_sort_frame wherever that happens (it is lossy by design).  At most
  * 2^20 tiles (else TDGS_ERR_INVALID_ARGUMENT).  Outputs: device pointers into
  * context-owned buffers (m keys, m values, tdgs_num_tiles(f) ranges), valid
- * until the next call on the context; host *m_out.  Waits once (pair count). */
+ * until the next call on the context; host *m_out.  Waits once (pair count).
+ * The context keeps a second set of a frame's buffers for these frames. */
 tdgs_status tdgs_sort_frame_normalized(tdgs_context* ctx, const tdgs_gaussian2d* g, uint32_t n, tdgs_frame f,
                                        const uint32_t** sorted_keys, const uint32_t** sorted_values,
                                        const tdgs_range** ranges, uint32_t* m_out, void* stream);
@@ -481,7 +482,12 @@ tdgs_status tdgs_sort_views(tdgs_context* ctx, const tdgs_view* views, uint32_t 
                             tdgs_view_result* results, void* stream);
 
 /* Allocate everything a batch of this shape needs (same view count, total
- * Gaussians and total tiles) for up to pair_capacity pairs.  Waits. */
+ * Gaussians and total tiles) for up to pair_capacity pairs.  Waits.
+ * The buffers serve both ways to the pairs (interval splits and tile passes:
+ * a batch with the same totals in other proportions may need the other one):
+ * at most about 30 bytes per pair and 60 per Gaussian, and a quarter more
+ * for growth.  Arguments that are refused leave an earlier reservation as it
+ * was; an allocation that fails leaves none. */
 tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32_t num_views,
                                uint64_t pair_capacity, void* stream);
 
@@ -490,7 +496,12 @@ tdgs_status tdgs_reserve_views(tdgs_context* ctx, const tdgs_view* views, uint32
  * count from device memory.  Requires tdgs_reserve_views with the same
  * shape.  A batch with more pairs than the reserved capacity latches
  * TDGS_ERR_CAPACITY (reserve more and run again).  The view table is read
- * from a host staging buffer the context owns, refreshed by each call. */
+ * from a host staging buffer the context owns, refreshed by each call that
+ * takes the batch (a refused one leaves it).  A captured batch may be
+ * replayed until the next tdgs_reserve_views, tdgs_sort_frame(_3d) or
+ * tdgs_sort_views(_3d) on the context, which restage the table and may move
+ * the buffers; the step calls, tdgs_sort_frame_normalized and tdgs_render
+ * leave it alone. */
 tdgs_status tdgs_sort_views_async(tdgs_context* ctx, const tdgs_view* views, uint32_t num_views,
                                   void* stream);
 

@@ -100,8 +100,10 @@ struct PendingTime {
 // normalised key runs the same code on a state of its own, so it leaves a
 // frame's results, a reservation and captured graphs alone.
 struct FrameState {
+  // f_stream: the two forms' intermediate pairs (packed elements between tile
+  // passes; or the segments, and the segments' columns)
   Buffer f_counts, f_dkey[3], f_dval[3], f_soff, f_sdo, f_rminmax, f_stream[2], f_keys, f_values, f_ranges;
-  Buffer f_rects, f_c1, f_rows, f_segs, f_cols, f_c2, f_b2;  // interval splits
+  Buffer f_rects, f_c1, f_rows, f_c2, f_b2;  // interval splits
   Buffer f_dos;   // onesweep depth sort (large N): histograms, digit starts, tickets, look-back status
   Buffer f_pair;  // single-launch depth sort without offsets: intermediate pairs (with f_sdo)
   // Scratch of a frame's passes and scan, apart from that of the step calls
@@ -136,7 +138,7 @@ struct FrameState {
   void release() {
     for (Buffer* b : {&f_counts, &f_dkey[0], &f_dkey[1], &f_dkey[2], &f_dval[0], &f_dval[1], &f_dval[2], &f_soff,
                       &f_sdo, &f_rminmax, &f_stream[0], &f_stream[1], &f_keys, &f_values, &f_ranges, &f_rects, &f_c1,
-                      &f_rows, &f_segs, &f_cols, &f_c2, &f_b2, &f_dos, &f_pair, &f_scratch, &f_scan})
+                      &f_rows, &f_c2, &f_b2, &f_dos, &f_pair, &f_scratch, &f_scan})
       if (b->p) cudaFree(b->p);
     if (d_views) cudaFree(d_views);
     if (h_views) cudaFreeHost(h_views);
@@ -902,29 +904,40 @@ Shape shape_of(const tdgs_context* ctx) {
   return sh;
 }
 
-// Buffers that depend only on the record and tile counts.
+// Buffers that depend only on the record and tile counts: those that the
+// staged views' depth sort and pair path use.
 tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
   const size_t n4 = static_cast<size_t>(ctx->n_all) * 4 + 16;
   tdgs_status st = TDGS_OK;
-  for (Buffer* b : {&ctx->f_counts, &ctx->f_dkey[0], &ctx->f_dkey[1], &ctx->f_dkey[2], &ctx->f_dval[0],
-                    &ctx->f_dval[1], &ctx->f_dval[2], &ctx->f_soff})
-    if (st == TDGS_OK) st = ensure(ctx, *b, n4, s);
-  if (st == TDGS_OK) st = ensure(ctx, ctx->f_sdo, static_cast<size_t>(ctx->n_all) * 8 + 16, s);
-  bool grown = false;
-  if (st == TDGS_OK) st = ensure(ctx, ctx->f_rminmax, static_cast<size_t>(ctx->t_all) * 8 + 16, s, &grown);
-  if (grown) ctx->rminmax_dirty = true;
-  if (st == TDGS_OK) st = ensure(ctx, ctx->f_ranges, static_cast<size_t>(ctx->t_all) * 8 + 16, s);
-  if (st == TDGS_OK && ctx->split) {
-    st = ensure(ctx, ctx->f_rects, n4, s);
-    if (st == TDGS_OK) st = ensure(ctx, ctx->f_c1, static_cast<size_t>(ctx->h_views->c1_begin[ctx->nv]) * 8 + 16, s);
-    if (st == TDGS_OK) st = ensure(ctx, ctx->f_rows, (static_cast<size_t>(split_rows(ctx)) + 1) * 20 + 16, s);
-  }
-  const uint32_t n_all = ctx->n_all;
   const DepthPlan dp = depth_plan(ctx);
   if (dp.grid == 0) return fail(ctx, TDGS_ERR_CUDA, "device query for the depth sort failed");
-  if (!ctx->split && !dp.resident) {  // the scan of the counts in depth order
-    const uint32_t tiles = ceil_div(n_all, kScanTileItems);
-    if (st == TDGS_OK) st = ensure(ctx, ctx->f_scan, static_cast<size_t>(tiles) * 8 + 8, s);
+  const uint32_t n_all = ctx->n_all;
+  bool grown = false;
+  auto need = [&](bool used, Buffer& b, size_t bytes) {
+    if (used && st == TDGS_OK) st = ensure(ctx, b, bytes, s, &grown);
+  };
+  // the single launch counts by itself, and makes the order alone from 8-byte
+  // pairs; the first onesweep pass makes its own indices
+  const bool order_only = dp.resident && ctx->split;
+  need(!dp.resident || ctx->proj_on || ctx->norm, ctx->f_dkey[0], n4);
+  need(!order_only, ctx->f_dkey[1], n4);
+  need(!order_only && (dp.resident || dp.onesweep), ctx->f_dkey[2], n4);
+  need(!dp.resident && !dp.onesweep, ctx->f_dval[0], n4);
+  need(true, ctx->f_dval[1], n4);
+  need(!order_only && (dp.resident || dp.onesweep), ctx->f_dval[2], n4);
+  need(true, ctx->f_sdo, static_cast<size_t>(n_all) * 8 + 16);
+  need(true, ctx->f_ranges, static_cast<size_t>(ctx->t_all) * 8 + 16);
+  if (ctx->split) {
+    need(true, ctx->f_rects, n4);
+    need(true, ctx->f_c1, static_cast<size_t>(ctx->h_views->c1_begin[ctx->nv]) * 8 + 16);
+    need(true, ctx->f_rows, (static_cast<size_t>(split_rows(ctx)) + 1) * 20 + 16);
+  } else {
+    need(true, ctx->f_counts, n4);
+    need(true, ctx->f_soff, n4);
+    need(!dp.resident, ctx->f_scan, static_cast<size_t>(ceil_div(n_all, kScanTileItems)) * 8 + 8);
+    grown = false;
+    need(true, ctx->f_rminmax, static_cast<size_t>(ctx->t_all) * 8 + 16);
+    if (grown) ctx->rminmax_dirty = true;
   }
   if (st == TDGS_OK) st = ensure(ctx, ctx->f_scratch, dp.scratch_words * 4, s);
   if (st == TDGS_OK && dp.resident) {
@@ -968,8 +981,8 @@ tdgs_status ensure_pair_buffers(tdgs_context* ctx, uint64_t m, cudaStream_t s) {
   if (ctx->split) {
     // every segment has a pair: at most m segments
     const size_t entries = static_cast<size_t>(split_tiles(ctx, m)) * split_pitch(ctx);
-    if (st == TDGS_OK) st = ensure(ctx, ctx->f_segs, m * 8 + 16, s);
-    if (st == TDGS_OK) st = ensure(ctx, ctx->f_cols, m * 2 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_stream[0], m * 8 + 16, s);
+    if (st == TDGS_OK) st = ensure(ctx, ctx->f_stream[1], m * 2 + 16, s);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_c2, entries * 2 + 16, s);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_b2, entries * 4 + 16, s);
     return st;
@@ -1106,8 +1119,8 @@ tdgs_status run_back_split(tdgs_context* ctx, uint32_t m, cudaStream_t s) {
   a.row_tile = a.row_seg + a.nrows + 1;
   a.row_pair = a.row_tile + a.nrows + 1;
   a.info = a.row_pair + a.nrows;
-  a.segs = static_cast<uint2*>(ctx->f_segs.p);
-  a.cols = static_cast<uint16_t*>(ctx->f_cols.p);
+  a.segs = static_cast<uint2*>(ctx->f_stream[0].p);
+  a.cols = static_cast<uint16_t*>(ctx->f_stream[1].p);
   a.c2 = static_cast<uint16_t*>(ctx->f_c2.p);
   a.b2 = static_cast<uint32_t*>(ctx->f_b2.p);
   a.pitch = split_pitch(ctx);

@@ -65,14 +65,17 @@ class Result:
     checksum: int = 0
 
 
-def estimate_bytes(n: int, width: int, height: int, pairs_per_gaussian: float = 24.0) -> int:
-    """Conservative device footprint of one request: its records (16 B),
-    the per-Gaussian sort buffers (24 B), and per pair the segments or
-    packed stream buffers, the final keys and values (<= 28 B; a generous
-    pair count covers the depth sort's further buffers)."""
+def estimate_bytes(n: int, width: int, height: int, pairs_per_gaussian: Optional[float] = None) -> int:
+    """Conservative device footprint of one request: its records (16 B per
+    Gaussian) and the library's buffers, which grow by a quarter more than
+    they need: per Gaussian the depth sort's keys and indices, rectangles and
+    counts (<= 40 B), per pair the final keys and values and the segments
+    between (<= 23.5 B; images above 4096 pixels: packed elements, 28 B), and
+    the tile ranges.  The default counts 21.9 (18.4) pairs per Gaussian."""
     tiles = ((width + 15) // 16) * ((height + 15) // 16)
-    m = int(n * pairs_per_gaussian)
-    return 16 * n + 24 * n + 28 * m + 24 * tiles
+    pair, usual = (23.5, 21.9) if max(width, height) <= 4096 else (28.0, 18.4)
+    pairs = usual if pairs_per_gaussian is None else pairs_per_gaussian
+    return 16 * n + int(1.25 * n * (40 + pair * pairs)) + 24 * tiles
 
 
 Executor = Callable[[int, Sequence[Request]], Sequence[Result]]

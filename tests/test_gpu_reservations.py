@@ -206,3 +206,27 @@ def test_replays_of_other_proportions(ctx, oracle, shapes, new, fits):
         assert e.value.status == T.CAPACITY
     ctx.sort_views_async(vf)
     check(oracle, first, ctx.views_results(len(vf)))
+
+
+@pytest.mark.parametrize("n,width,height,sigma", [(4_000_000, 1280, 720, 0.5), (1_000_000, 1280, 720, 6.0),
+                                                  (4_000_000, 4800, 1024, 0.5), (4_000_000, 4096, 4096, 0.5)])
+def test_estimated_footprint(n, width, height, sigma):
+    """The server's estimate bounds what a request holds, with few and with
+    many pairs per Gaussian, and so does the documented size of a
+    reservation."""
+    from paper_2511_16298_gb300 import build, serve
+    build.build()
+    f = synth.frame_random(1, n, width, height, max_sigma=sigma)
+    slack = 48 << 20  # allocations come in steps of 2 MB
+    g = T.records_to_tensor(f.gaussians, DEV)
+    with T.Context(0) as c:
+        free = torch.cuda.mem_get_info()[0]
+        m = c.sort_frame(g, width, height)[3]
+        c.sync()
+        used = free - torch.cuda.mem_get_info()[0]
+        assert used + 16 * n <= serve.estimate_bytes(n, width, height, m / n) + slack, (used, m)
+    with T.Context(0) as c:
+        free = torch.cuda.mem_get_info()[0]
+        c.reserve_views([(g, width, height)], m)
+        used = free - torch.cuda.mem_get_info()[0]
+        assert used <= 1.25 * (60 * n + 30 * m) + slack, (used, m)
