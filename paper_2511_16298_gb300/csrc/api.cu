@@ -268,14 +268,28 @@ class UseNormState {
   tdgs_context* ctx_;
 };
 
-// The radix grid barrier words back to zero if an error was latched since
-// their last use.
-tdgs_status clear_barrier_if_dirty(tdgs_context* ctx, cudaStream_t s) {
-  if (ctx->bar_dirty) {
-    TDGS_CUDA(ctx, cudaMemsetAsync(ctx->d_tickets + 2, 0, 2 * sizeof(uint32_t), s));
-    ctx->bar_dirty = false;
+// Work on a stream that is being captured runs when the graph is replayed,
+// not before the next call.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// State kept between launches back to zero if it may not be (`dirty`); it
+// stays so marked if that only happens in a graph.
+tdgs_status clear_if_dirty(tdgs_context* ctx, bool& dirty, void* p, size_t bytes, cudaStream_t s) {
+  if (dirty) {
+    TDGS_CUDA(ctx, cudaMemsetAsync(p, 0, bytes, s));
+    dirty = capturing(s);
   }
   return TDGS_OK;
+}
+
+// The radix grid barrier words, after an error.
+tdgs_status clear_barrier_if_dirty(tdgs_context* ctx, cudaStream_t s) {
+  return clear_if_dirty(ctx, ctx->bar_dirty, ctx->d_tickets + 2, 2 * sizeof(uint32_t), s);
 }
 
 cudaEvent_t take_event(tdgs_context* ctx) {
@@ -379,8 +393,9 @@ tdgs_status do_sort(tdgs_context* ctx, uint64_t* keys, uint32_t* values, uint64_
     tdgs_status st = ensure(ctx, ctx->os_scratch, onesweep_scratch_words(m) * 4, s, &grown);
     if (st != TDGS_OK) return st;
     uint32_t* scratch = static_cast<uint32_t*>(ctx->os_scratch.p);
-    if (grown || ctx->os_dirty) TDGS_CUDA(ctx, cudaMemsetAsync(scratch, 0, onesweep_header_words() * 4, s));
-    ctx->os_dirty = false;
+    ctx->os_dirty |= grown;
+    st = clear_if_dirty(ctx, ctx->os_dirty, scratch, onesweep_header_words() * 4, s);
+    if (st != TDGS_OK) return st;
     TDGS_TRACED(ctx, kKSortHist, m, s, launch_onesweep_hist(plan, keys, m, scratch, err_word(ctx), s));
     uint64_t* kin = keys;
     uint32_t* vin = values;
@@ -944,19 +959,13 @@ tdgs_status ensure_record_buffers(tdgs_context* ctx, cudaStream_t s) {
     grown = false;
     if (ctx->split) st = ensure(ctx, ctx->f_pair, static_cast<size_t>(n_all) * 8 + 16, s);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_dsort, depth_sort_scratch_words(depth_sort_grid()) * 4, s, &grown);
-    if (st == TDGS_OK && (grown || ctx->dsort_dirty)) {
-      TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_dsort.p, 0, ctx->f_dsort.bytes, s));
-      ctx->dsort_dirty = false;
-    }
+    ctx->dsort_dirty |= grown;
   }
   if (st == TDGS_OK && dp.onesweep) {
     grown = false;
     st = ensure(ctx, ctx->f_dos, onesweep_scratch_words(n_all ? n_all : 1, by_view(ctx)) * 4, s, &grown);
     if (st == TDGS_OK) st = ensure(ctx, ctx->f_raw, (kRawBins + 1) * 4, s, &grown);
-    if (st == TDGS_OK && (grown || ctx->dos_dirty)) {
-      TDGS_CUDA(ctx, cudaMemsetAsync(ctx->f_raw.p, 0, (kRawBins + 1) * 4, s));
-      ctx->dos_dirty = false;
-    }
+    ctx->dos_dirty |= grown;
   }
   return st;
 }
@@ -1013,13 +1022,18 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
   } else if (ctx->vtot_dirty) {
     TDGS_CUDA(ctx, cudaMemsetAsync(ctx->d_views->vtot, 0, sizeof(ctx->d_views->vtot), s));
   }
-  ctx->vtot_dirty = false;
+  ctx->vtot_dirty = ctx->vtot_dirty && capturing(s);
   uint32_t* counts = static_cast<uint32_t*>(ctx->f_counts.p);
   uint32_t* dk[3] = {static_cast<uint32_t*>(ctx->f_dkey[0].p), static_cast<uint32_t*>(ctx->f_dkey[1].p),
                      static_cast<uint32_t*>(ctx->f_dkey[2].p)};
   uint32_t* dv[3] = {static_cast<uint32_t*>(ctx->f_dval[0].p), static_cast<uint32_t*>(ctx->f_dval[1].p),
                      static_cast<uint32_t*>(ctx->f_dval[2].p)};
   const DepthPlan dp = depth_plan(ctx);
+  // state that launches leave as they found it, unless an error ended one
+  tdgs_status st = TDGS_OK;
+  if (dp.resident) st = clear_if_dirty(ctx, ctx->dsort_dirty, ctx->f_dsort.p, ctx->f_dsort.bytes, s);
+  if (dp.onesweep) st = clear_if_dirty(ctx, ctx->dos_dirty, ctx->f_raw.p, (kRawBins + 1) * 4, s);
+  if (st != TDGS_OK) return st;
   DepthSortArgs da{};
   da.vt = vt;
   da.total = &ctx->d_status->total;
@@ -1089,8 +1103,8 @@ tdgs_status run_front(tdgs_context* ctx, cudaStream_t s, bool early_total = fals
     }
   }
   if (n_all && !dp.resident && !ctx->split) {
-    tdgs_status st = do_scan(ctx, kKFrameScan, counts, nullptr, dv[dp.result], FrameGeom{}, n_all,
-                             static_cast<uint32_t*>(ctx->f_soff.p), &ctx->d_status->total, nullptr, ctx->f_scan, s);
+    st = do_scan(ctx, kKFrameScan, counts, nullptr, dv[dp.result], FrameGeom{}, n_all,
+                 static_cast<uint32_t*>(ctx->f_soff.p), &ctx->d_status->total, nullptr, ctx->f_scan, s);
     if (st != TDGS_OK) return st;
   } else if (n_all == 0) {
     TDGS_CUDA(ctx, cudaMemsetAsync(&ctx->d_status->total, 0, 8, s));
@@ -1220,7 +1234,7 @@ tdgs_status run_back(tdgs_context* ctx, uint32_t m, const uint64_t* m_dev, cudaS
     TDGS_TRACED(ctx, last ? kKTileExpand : kKTilePass, m, s, launch_stream_pass(sp, scratch, bar, err_word(ctx), s));
     shift += width;
   }
-  if (!single) ctx->rminmax_dirty = false;  // the last pass turned them into ranges and reset them
+  if (!single) ctx->rminmax_dirty = capturing(s);  // the last pass turned them into ranges and reset them
   return TDGS_OK;
 }
 

@@ -230,3 +230,25 @@ def test_estimated_footprint(n, width, height, sigma):
         c.reserve_views([(g, width, height)], m)
         used = free - torch.cuda.mem_get_info()[0]
         assert used <= 1.25 * (60 * n + 30 * m) + slack, (used, m)
+
+
+@pytest.mark.parametrize("n,size", [(3000, (640, 360)), (3000, (4800, 64)), (700_000, (640, 360)),
+                                    (700_000, (4800, 64))])
+def test_first_call_is_a_capture(ctx, oracle, n, size):
+    """A context whose first batch is captured and not yet replayed: what that
+    batch clears is still to be cleared for the calls that run first (a batch
+    outside the graph, or a frame of a second context)."""
+    frames = [synth.frame_random(i, n, *size, max_sigma=5.0) for i in range(2)]
+    vs = on_gpu(frames)
+    cap = sum(oracle.sort_frame(f.gaussians, f.width, f.height)["m"] for f in frames)
+    ctx.reserve_views(vs, cap)
+    graph = capture(ctx, vs)
+    ctx.sort_views_async(vs)
+    check(oracle, frames, ctx.views_results(2))
+    graph.replay()
+    check(oracle, frames, ctx.views_results(2))
+    with T.Context(0) as c:
+        c.reserve_views(vs, cap)
+        capture(c, vs)
+        check(oracle, frames[:1], [c.sort_frame(*vs[0])])
+        check(oracle, frames, c.sort_views(vs))
