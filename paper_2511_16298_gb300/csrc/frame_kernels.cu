@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(256) k_count_tiles(const float4* g, uint32_t n
                                                      uint32_t* err) {
   begin_launch();
   bool bad = false;
-  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = next_of(i, gridDim.x * blockDim.x, n)) {
     const TileRect q = tile_rect(__ldca(g + i), fg);
     bad |= q.invalid;
     counts[i] = q.count;
@@ -328,7 +328,7 @@ cudaError_t launch_duplicate_norm(const float4* g, const uint32_t* offsets, uint
 __global__ void __launch_bounds__(256) k_norm_range(const float4* g, const uint32_t* counts,
                                                     uint32_t n, uint32_t* norm) {
   uint32_t lo = 0xffffffffu, hi = 0u;
-  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = next_of(i, gridDim.x * blockDim.x, n)) {
     if (__ldca(counts + i)) {
       const uint32_t b = __float_as_uint(__ldca(&g[i].z));
       lo = min(lo, b);

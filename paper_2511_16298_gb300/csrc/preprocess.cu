@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(256)
                  float4* __restrict__ rec, float4* __restrict__ conic) {
   begin_launch();
   const float2 lim = proj::slope_limits(cam);
-  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = next_of(i, gridDim.x * blockDim.x, n)) {
     const float4 p = __ldca(g + i);
     const float4 c0 = __ldca(cov + 2 * static_cast<size_t>(i));
     const float4 c1 = __ldca(cov + 2 * static_cast<size_t>(i) + 1);

@@ -144,6 +144,13 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
+// The next index of a grid-stride loop over n items, n past the last one (the
+// sum may exceed 32 bits; 64-bit indexes took k_preprocess from 40 to 48
+// registers).
+__device__ __forceinline__ uint32_t next_of(uint32_t i, uint32_t stride, uint32_t n) {
+  return n - i > stride ? i + stride : n;
+}
+
 // ------------------------------------------------------------- host side
 // Blocks, warps or tiles of `per` items each that hold n items.
 constexpr uint32_t ceil_div(uint64_t n, uint32_t per) { return static_cast<uint32_t>((n + per - 1) / per); }
