@@ -216,6 +216,7 @@ __device__ __forceinline__ uint2 look_back(const uint32_t* status, uint32_t tile
     if (open1) e.y += w.y & kCountMask;
     open0 &= (w.x & ~kCountMask) != kFlagP;
     open1 &= (w.y & ~kCountMask) != kFlagP;
+    spins = 0;  // the limit is for one row
     --j;
   }
   return e;
